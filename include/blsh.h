@@ -284,12 +284,13 @@ BLSH_API int blsh_srp_sparse_q16_cols(blsh_ctx *ctx, const int64_t *indptr, cons
  * [ sum_c X[i][c] R[c][j] >= 0 ], each bit equal to the sign of the FP64 sum
  * over c = 0..d-1 in order.
  * With a workspace (blsh_srp_dense_workspace bytes, 256-byte aligned; nonzero
- * when d is a multiple of 64 and bits a multiple of 256) the projection runs
- * on the tensor cores: X and R are split into BF16 pairs hi + lo and
+ * when bits is a multiple of 256 and d at most 4096) the projection runs
+ * on the tensor cores (d padded to a multiple of 64 with zeros; a width that
+ * is no multiple of 64 takes the CUDA cores when the workspace is smaller): X and R are split into BF16 pairs hi + lo and
  * hi*hi + hi*lo + lo*hi is accumulated in FP32; every product with
  * |p| <= margin * |x_i| * |r_j| is recomputed in FP32 with a rigorous bound
  * and, where that cannot decide it, in FP64.  margin is raised to the
- * tensor-core error bound (about (2^-14 + 3 d 2^-22) * 1.25) when smaller;
+ * tensor-core error bound (about (2^-14 + 3 d 2^-22) * 1.25, d padded) when smaller;
  * pass 0 for that bound.  Without a workspace (or for other shapes) the
  * projection runs in FP32 on the CUDA cores with the same rechecks.
  * X and R 16-byte aligned; bits a multiple of 32, at most 4096. */

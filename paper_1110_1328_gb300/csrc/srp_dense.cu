@@ -1,7 +1,8 @@
 // srp_dense.cu -- sign random projections of dense rows (Section 4.2, "LSH
 // family"): bit j of row i = [x_i . r_j >= 0].
 //
-// Tensor-core path (d a multiple of 64, bits a multiple of 256):
+// Tensor-core path (bits a multiple of 256, any d up to 4096: K is padded with
+// zeros to Kpad, the next multiple of 64):
 //   1. srp_dense_prep: X and R become BF16 pairs hi + lo with
 //      hi = bf16(v), lo = bf16(v - hi) (|v - hi - lo| <= 2^-16 |v|), written in
 //      the tile layout the tensor cores read (128- and 256-row tiles of 64
@@ -20,13 +21,19 @@
 //      definition -- so every bit is exact whenever the margin bounds the
 //      tensor-core error.
 // The error of step 2 is at most 3.1 * 2^-16 sum|x_i r_ij| from the split
-// plus the FP32 accumulation of 3d products; the rigorous margin used when
-// the caller passes margin <= 0 is (2^-14 + 3 d 2^-22) * 1.25, applied to
+// plus the FP32 accumulation of 3 Kpad products; the rigorous margin used when
+// the caller passes margin <= 0 is (2^-14 + 3 Kpad 2^-22) * 1.25, applied to
 // |x| |r| >= sum|x_i r_ij|.
+//
+// A width that is no multiple of 64 takes the same path since the padding
+// costs at most one K stage, while the CUDA cores need 2 d operations a sign
+// at 1/50 of the tensor rate: 99,991 x 300 x 1,024 bits took 36.4 ms on the
+// CUDA cores' kernel of that time, 332 us here.
 //
 // Every other shape uses srp_dense_simt_kernel (hashing.cu): FP32 sums with
 // the same kind of bound and an FP64 recheck.
 #include <cuda_bf16.h>
+#include <math.h>
 
 #include <atomic>
 
@@ -55,23 +62,94 @@ __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)_
 
 // ---- preparation --------------------------------------------------------------
 
-// One warp per row of X (rows >= N are zero-filled up to the padded tile);
-// lanes take 4 consecutive values at a time.  xnorm: |x| in FP32 rounded up.
-__global__ void srp_dense_prep_x(const float *__restrict__ X, long long N, long long Npad, int d,
-                                 unsigned char *__restrict__ Xh, unsigned char *__restrict__ Xl,
-                                 float *__restrict__ xnorm) {
-    const int lane = threadIdx.x & 31;
-    const int KT = d / BK;
-    const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
-    for (long long r = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < Npad; r += warps) {
+// One launch prepares both operands and clears the recheck queue's count: the
+// first r_blocks CTAs take 32 columns of R each, the others the rows of X.
+//
+// R: a CTA walks K in stages of 64: a 64 x 32 tile is read in 128-byte rows,
+// turned in shared memory, and each thread writes eight K values of a column
+// (16 bytes of the hi and lo operands, which are N-major rows of K values, and
+// 32 bytes of Rt, FP32 R transposed, read by the rechecks).  One thread per
+// column, with its 2-byte stores 128 bytes apart, had taken 133 us at
+// 384 x 1,024 (of a 169 us call for 1,000 rows) and 102 us at 256 x 1,024;
+// this form takes 11 us, both operands together, for those 1,000 rows.
+// X: one warp per row (rows >= N are zero-filled up to the padded tile), four
+// consecutive values a lane at a time (VEC: d a multiple of 4, so that every
+// row starts on 16 bytes).
+// xnorm, rnorm: |x_i|, |r_j| in FP32 rounded up, infinity outside
+// [1e-15, 1e18] (norm_or_inf): inside it no partial sum of the tensor cores
+// can overflow (each is at most |x_i| |r_j| <= 1e36) and no underflow of a
+// split or a product comes near margin |x_i| |r_j| >= 3e-34; outside it an
+// infinite bound sends every sign to the recheck.
+constexpr int kPrepCols = 32;
+__device__ __forceinline__ float norm_or_inf(float ss) {
+    const float n = __fsqrt_ru(ss) * 1.0001f;
+    return n >= 1e-15f && n <= 1e18f ? n : INFINITY;
+}
+
+template <bool VEC>
+__global__ void __launch_bounds__(256) srp_dense_prep(
+    const float *__restrict__ X, long long N, long long Npad, int d, int KT, unsigned char *__restrict__ Xh,
+    unsigned char *__restrict__ Xl, float *__restrict__ xnorm, const float *__restrict__ R, int bits,
+    unsigned char *__restrict__ Rh, unsigned char *__restrict__ Rl, float *__restrict__ rnorm,
+    float *__restrict__ Rt, int r_blocks, unsigned long long *qcount) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if ((int)blockIdx.x < r_blocks) {
+        __shared__ float tile[BK][kPrepCols + 1];
+        if (blockIdx.x == 0 && threadIdx.x == 0) *qcount = 0ull;
+        const int j0 = blockIdx.x * kPrepCols;
+        const int c = threadIdx.x >> 3, q = threadIdx.x & 7;   // this thread's column and 16-byte chunk
+        const int j = j0 + c;
+        const int nt = j / BN, jj = j % BN;
+        float ss = 0.0f;
+        for (int kt = 0; kt < KT; ++kt) {
+#pragma unroll
+            for (int i = 0; i < BK / 8; ++i) {
+                const int kk = warp + 8 * i, k = kt * BK + kk;
+                tile[kk][lane] = k < d ? __ldg(R + (size_t)k * bits + j0 + lane) : 0.0f;
+            }
+            __syncthreads();
+            __align__(16) __nv_bfloat16 hi[8], lo[8];
+            __align__(16) float v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                v[i] = tile[8 * q + i][c];
+                hi[i] = __float2bfloat16_rn(v[i]);
+                lo[i] = __float2bfloat16_rn(v[i] - __bfloat162float(hi[i]));
+                ss = __fmaf_ru(v[i], v[i], ss);
+            }
+            const size_t off = ((size_t)nt * KT + kt) * TILE_B + swz_offset(jj, 8 * q);
+            *reinterpret_cast<uint4 *>(Rh + off) = *reinterpret_cast<const uint4 *>(hi);
+            *reinterpret_cast<uint4 *>(Rl + off) = *reinterpret_cast<const uint4 *>(lo);
+            float4 *t = reinterpret_cast<float4 *>(Rt + (size_t)j * (KT * BK) + kt * BK + 8 * q);
+            t[0] = make_float4(v[0], v[1], v[2], v[3]);
+            t[1] = make_float4(v[4], v[5], v[6], v[7]);
+            __syncthreads();
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) ss = __fadd_ru(ss, __shfl_xor_sync(kFull, ss, o));
+        if (q == 0) rnorm[j] = norm_or_inf(ss);
+        return;
+    }
+    const long long warps = (long long)(gridDim.x - r_blocks) * (blockDim.x >> 5);
+    for (long long r = (long long)(blockIdx.x - r_blocks) * (blockDim.x >> 5) + warp; r < Npad; r += warps) {
         const long long mt = r / BM;
         const int rr = (int)(r % BM);
         float ss = 0.0f;
-        for (int k0 = 4 * lane; k0 < d; k0 += 128) {
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (r < N) v = __ldg(reinterpret_cast<const float4 *>(X + (size_t)r * d + k0));
-            const float a[4] = {v.x, v.y, v.z, v.w};
-            __nv_bfloat16 hi[4], lo[4];
+        for (int k0 = 4 * lane; k0 < KT * BK; k0 += 128) {
+            float a[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            if (r < N) {
+                if (VEC) {
+                    if (k0 < d) {
+                        const float4 v = __ldg(reinterpret_cast<const float4 *>(X + (size_t)r * d + k0));
+                        a[0] = v.x; a[1] = v.y; a[2] = v.z; a[3] = v.w;
+                    }
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        if (k0 + i < d) a[i] = __ldg(X + (size_t)r * d + k0 + i);
+                }
+            }
+            __align__(8) __nv_bfloat16 hi[4], lo[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 hi[i] = __float2bfloat16_rn(a[i]);
@@ -85,32 +163,8 @@ __global__ void srp_dense_prep_x(const float *__restrict__ X, long long N, long 
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) ss = __fadd_ru(ss, __shfl_xor_sync(kFull, ss, o));
-        if (lane == 0) xnorm[r] = __fsqrt_ru(ss) * 1.0001f;
+        if (lane == 0) xnorm[r] = norm_or_inf(ss);
     }
-}
-
-// One thread per column j of R (bits): its d values become row j of the B
-// operand (B is stored N-major rows of K values) and row j of Rt (FP32 R
-// transposed, read by the rechecks).  rnorm: |r_j| rounded up.
-__global__ void srp_dense_prep_r(const float *__restrict__ R, int d, int bits, unsigned char *__restrict__ Rh,
-                                 unsigned char *__restrict__ Rl, float *__restrict__ rnorm,
-                                 float *__restrict__ Rt) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= bits) return;
-    const int KT = d / BK;
-    const int nt = j / BN, jj = j % BN;
-    float ss = 0.0f;
-    for (int k = 0; k < d; ++k) {
-        const float v = __ldg(R + (size_t)k * bits + j);
-        const __nv_bfloat16 hi = __float2bfloat16_rn(v);
-        const __nv_bfloat16 lo = __float2bfloat16_rn(v - __bfloat162float(hi));
-        ss = __fmaf_ru(v, v, ss);
-        Rt[(size_t)j * d + k] = v;   // column j of R, contiguous, for the rechecks
-        const size_t tile = ((size_t)nt * KT + k / BK) * TILE_B;
-        *reinterpret_cast<__nv_bfloat16 *>(Rh + tile + swz_offset(jj, k % BK)) = hi;
-        *reinterpret_cast<__nv_bfloat16 *>(Rl + tile + swz_offset(jj, k % BK)) = lo;
-    }
-    rnorm[j] = __fsqrt_ru(ss) * 1.0001f;
 }
 
 // ---- tcgen05 / mbarrier / bulk-copy helpers ------------------------------------
@@ -247,7 +301,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) srp_dense_tc_persistent(
     __shared__ __align__(8) unsigned long long mma_done;
     __shared__ unsigned tmem_base;
     __shared__ volatile int s_fail;
-    const int KT = d / BK;
+    const int KT = (d + BK - 1) / BK;
     const int tiles_n = bits / BN;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -424,25 +478,36 @@ __global__ void __launch_bounds__(kTcThreads, 1) srp_dense_tc_persistent(
 // Queued signs: eight lanes per (row, bit).  Three stages, each with a
 // rigorous bound:
 //   FP32 partial sums, lane g of the group taking the 16-byte pieces 8i + g
-//   of both rows (any summation order errs by at most (d+8) u sum|p|);
+//   of both rows into four chains of at most ceil(d/32) FMAs, joined by two
+//   and then three additions: no term passes through more than
+//   ceil(d/32) + 5 roundings, so the sum errs by at most that many u sum|p|;
 //   if undecided, FP64 partial sums of the exact products, lane g owning
-//   coordinates [g d/8, (g+1) d/8) (error at most
+//   coordinates [g per, (g+1) per), per = ceil(d/8) (error at most
 //   (d+8) 2^-53 sum|p|, so a sign it decides is the sign of the exact sum and
 //   of the oracle's sum, which errs by less);
 //   if still undecided (exact ties such as zero rows), the FP64 sum over
 //   coordinates 0..d-1 in order, lane g continuing lane g-1's running sum --
 //   exactly the oracle's sum.
+// The FP64 stage costs a warp about fifty times the FP32 one (the FP64 pipe is
+// narrow) and runs when any of its four signs needs it, so the first bound
+// decides the time: counting the chains' own lengths instead of d + 8
+// roundings leaves 1/19 as many signs at d = 256.  1e6 x 256 x 1,024 bits with
+// the margin 1e-3 (1.3e7 queued signs): 2,374 us before, 2,077 now (the gathers of 2 KB a sign are left).
+// VEC: d a multiple of 4 (16-byte loads of X).
+template <bool VEC>
 __global__ void __launch_bounds__(256) srp_dense_recheck_kernel(const uint2 *__restrict__ queue,
                                                                 unsigned long long qcap,
                                                                 const unsigned long long *qcount,
                                                                 const float *__restrict__ X,
-                                                                const float *__restrict__ Rt, int d, int bits,
+                                                                const float *__restrict__ Rt, int d, int ldr, int bits,
                                                                 uint32_t *__restrict__ sig,
                                                                 blsh_dev_scratch *scratch) {
     const unsigned long long total = *qcount;
     const unsigned long long n = total < qcap ? total : qcap;
     const int lane = threadIdx.x & 31, g = lane & 7;
-    const int per = d >> 3;   // coordinates per lane (d is a multiple of 64)
+    const int per = (d + 7) >> 3;   // coordinates per lane of the FP64 stages
+    const int lo = g * per < d ? g * per : d, hi = lo + per < d ? lo + per : d;
+    const float roundings = (float)((d + 31) / 32 + 6);
     const unsigned long long groups = (unsigned long long)gridDim.x * (blockDim.x >> 3);
     unsigned long long done = 0, zeros = 0;
     const unsigned long long warp_first = (((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3) & ~3ull;
@@ -451,19 +516,23 @@ __global__ void __launch_bounds__(256) srp_dense_recheck_kernel(const uint2 *__r
         const bool live = it < n;
         uint2 rj = make_uint2(0u, 0u);
         if (live) rj = queue[it];
-        const float *xr = X + (size_t)rj.x * d, *rr = Rt + (size_t)rj.y * d;
-        const float *x = xr + g * per;
-        const float *r = rr + g * per;
+        const float *xr = X + (size_t)rj.x * d, *rr = Rt + (size_t)rj.y * ldr;
         float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f;
-        // FP32 stage: the group's eight lanes read 128 contiguous bytes of each
-        // row per step (lane g the 16 bytes at 4 (8 i + g)); the bound holds
-        // for any order of the terms
+        // the group's eight lanes read 128 contiguous bytes of each row per
+        // step (lane g the 16 bytes at 4 (8 i + g))
         if (live)
 #pragma unroll 4
-            for (int i = 0; i < per / 4; ++i) {
-                const int c = (8 * i + g) * 4;
-                const float4 u = __ldg(reinterpret_cast<const float4 *>(xr + c));
-                const float4 v = __ldg(reinterpret_cast<const float4 *>(rr + c));
+            for (int c = 4 * g; c < d; c += 32) {
+                float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (VEC) {
+                    u = __ldg(reinterpret_cast<const float4 *>(xr + c));
+                } else {
+                    u.x = __ldg(xr + c);
+                    if (c + 1 < d) u.y = __ldg(xr + c + 1);
+                    if (c + 2 < d) u.z = __ldg(xr + c + 2);
+                    if (c + 3 < d) u.w = __ldg(xr + c + 3);
+                }
+                const float4 v = __ldg(reinterpret_cast<const float4 *>(rr + c));   // zeros past d
                 a0 = __fmaf_rn(u.x, v.x, a0); a1 = __fmaf_rn(u.y, v.y, a1);
                 a2 = __fmaf_rn(u.z, v.z, a2); a3 = __fmaf_rn(u.w, v.w, a3);
                 m0 = __fmaf_rn(fabsf(u.x), fabsf(v.x), m0); m1 = __fmaf_rn(fabsf(u.y), fabsf(v.y), m1);
@@ -475,14 +544,14 @@ __global__ void __launch_bounds__(256) srp_dense_recheck_kernel(const uint2 *__r
             acc += __shfl_xor_sync(kFull, acc, o);
             mag += __shfl_xor_sync(kFull, mag, o);
         }
-        const float bound = 1.25f * (float)(d + 8) * 5.9604644775390625e-8f * mag + (float)(d + 8) * 1.4e-45f;
+        const float bound = 1.25f * roundings * 5.9604644775390625e-8f * mag + (float)(d + 8) * 1.4e-45f;
         bool decided = !live || fabsf(acc) > bound;
         bool bit = acc >= 0.0f;
         if (__any_sync(kFull, !decided)) {
             double p = 0.0, q = 0.0;
             if (!decided)
-                for (int c = 0; c < per; ++c) {
-                    const double t = (double)__ldg(x + c) * (double)__ldg(r + c);
+                for (int c = lo; c < hi; ++c) {
+                    const double t = (double)__ldg(xr + c) * (double)__ldg(rr + c);
                     p += t;
                     q += fabs(t);
                 }
@@ -498,7 +567,7 @@ __global__ void __launch_bounds__(256) srp_dense_recheck_kernel(const uint2 *__r
                 double s = 0.0;
                 for (int step = 0; step < 8; ++step) {
                     if (g == step && !decided64)
-                        for (int c = 0; c < per; ++c) s += (double)__ldg(x + c) * (double)__ldg(r + c);
+                        for (int c = lo; c < hi; ++c) s += (double)__ldg(xr + c) * (double)__ldg(rr + c);
                     s = __shfl_sync(kFull, s, (lane & 24) | step);
                 }
                 if (!decided64) {
@@ -531,7 +600,8 @@ unsigned long long queue_cap(long long N, int bits) {
     return c < (1ull << 20) ? ((1ull << 20) < all ? (1ull << 20) : all) : c;
 }
 
-DenseLayout dense_layout(long long N, int d, int bits) {
+DenseLayout dense_layout(long long N, int d0, int bits) {
+    const int d = (d0 + BK - 1) / BK * BK;   // K padded to whole stages
     const long long Npad = (N + BM - 1) / BM * BM;
     DenseLayout L;
     size_t o = 0;
@@ -550,7 +620,7 @@ DenseLayout dense_layout(long long N, int d, int bits) {
 }
 
 bool tc_shape(long long N, int d, int bits) {
-    return N > 0 && d % BK == 0 && bits % BN == 0 && d <= 4096 && (N + BM - 1) / BM <= 65535;
+    return N > 0 && bits % BN == 0 && d <= 4096 && (N + BM - 1) / BM <= 65535;
 }
 
 }  // namespace
@@ -573,25 +643,28 @@ extern "C" int blsh_srp_dense(blsh_ctx *ctx, const float *X, int64_t N, int32_t 
     if (!workspace || !tc_shape(N, d, bits) || !blsh_aligned(X, 16) || !blsh_aligned(R, 16))
         return blsh_srp_dense_simt(ctx, X, N, d, R, bits, sig, s);
     const DenseLayout L = dense_layout(N, d, bits);
-    if (workspace_bytes < L.total || !blsh_aligned(workspace, 256))
+    if (workspace_bytes < L.total || !blsh_aligned(workspace, 256)) {
+        // widths that are no multiple of 64 need no workspace
+        if (d % BK) return blsh_srp_dense_simt(ctx, X, N, d, R, bits, sig, s);
         return blsh_fail(ctx, BLSH_ETRUNC, "workspace needs %zu bytes, 256-byte aligned", L.total);
+    }
+    const int KT = (d + BK - 1) / BK;
     // the margin must cover the tensor-core error: split 3.1 * 2^-16, FP32
-    // accumulation of 3d products at 2^-22 each, with a 25% slack
-    const float rigorous = 1.25f * (4.0f * 1.52587890625e-5f + 3.0f * (float)d * 2.384185791015625e-7f);
+    // accumulation of 3 Kpad products at 2^-22 each, with a 25% slack
+    const float rigorous = 1.25f * (4.0f * 1.52587890625e-5f + 3.0f * (float)(KT * BK) * 2.384185791015625e-7f);
     const float m = margin > rigorous ? margin : rigorous;
     unsigned char *ws = (unsigned char *)workspace;
     const long long Npad = (N + BM - 1) / BM * BM;
-    blsh_time_start(ctx, s);
-    srp_dense_prep_x<<<(unsigned)((Npad + 7) / 8 < 65535ll * 8 ? (Npad + 7) / 8 : 65535ll * 8), 256, 0, s>>>(
-        X, N, Npad, d, ws + L.xh, ws + L.xl, (float *)(ws + L.xn));
-    BLSH_LAUNCHED(ctx, "srp_dense_prep_x");
-    blsh_time_start(ctx, s);
-    srp_dense_prep_r<<<(bits + 127) / 128, 128, 0, s>>>(R, d, bits, ws + L.rh, ws + L.rl, (float *)(ws + L.rn),
-                                                        (float *)(ws + L.rt));
-    BLSH_LAUNCHED(ctx, "srp_dense_prep_r");
     unsigned long long *qcount = (unsigned long long *)(ws + L.qc);
     uint2 *queue = (uint2 *)(ws + L.q);
-    BLSH_CUDA(ctx, cudaMemsetAsync(qcount, 0, sizeof(unsigned long long), s));
+    const int r_blocks = bits / kPrepCols;
+    const unsigned x_blocks = (unsigned)((Npad + 7) / 8 < 65535ll * 8 ? (Npad + 7) / 8 : 65535ll * 8);
+    const bool vec = d % 4 == 0;
+    blsh_time_start(ctx, s);
+    (vec ? srp_dense_prep<true> : srp_dense_prep<false>)<<<r_blocks + x_blocks, 256, 0, s>>>(
+        X, N, Npad, d, KT, ws + L.xh, ws + L.xl, (float *)(ws + L.xn), R, bits, ws + L.rh, ws + L.rl,
+        (float *)(ws + L.rn), (float *)(ws + L.rt), r_blocks, qcount);
+    BLSH_LAUNCHED(ctx, "srp_dense_prep");
     const size_t smem = (size_t)STAGES * STAGE_BYTES + 1024 + (size_t)bits * sizeof(float);
     const size_t smem_max = (size_t)STAGES * STAGE_BYTES + 1024 + 4096 * sizeof(float);   // bits <= 4096
     static std::atomic<unsigned long long> opted{0};
@@ -608,8 +681,8 @@ extern "C" int blsh_srp_dense(blsh_ctx *ctx, const float *X, int64_t N, int32_t 
                                                           sig, queue, L.qcap, qcount, X, R, tiles, ctx->scratch);
     BLSH_LAUNCHED(ctx, "srp_dense_tc_persistent");
     blsh_time_start(ctx, s);
-    srp_dense_recheck_kernel<<<ctx->sm_count * 8, 256, 0, s>>>(queue, L.qcap, qcount, X, (float *)(ws + L.rt), d,
-                                                                 bits, sig, ctx->scratch);
+    (vec ? srp_dense_recheck_kernel<true> : srp_dense_recheck_kernel<false>)<<<ctx->sm_count * 8, 256, 0, s>>>(
+        queue, L.qcap, qcount, X, (float *)(ws + L.rt), d, KT * BK, bits, sig, ctx->scratch);
     BLSH_LAUNCHED(ctx, "srp_dense_recheck_kernel");
     return BLSH_OK;
 }
