@@ -659,56 +659,125 @@ __global__ void __launch_bounds__(256) gaussian_codes_kernel(unsigned long long 
     }
 }
 
-// Dense rows X [N][d] against R [d][bits], the same FP32 sums with the same
-// error bound and FP64 recheck (coordinates in order 0..d-1).  One CTA per
-// row; the row is staged in shared memory.
+// Dense rows X [N][d] against R [d][bits] on the CUDA cores: the shapes the
+// tensor-core path does not take (bits no multiple of 256, no workspace,
+// unaligned rows).  A CTA of 256 threads forms a tile of 8 RT rows by 128
+// columns, K in stages of 32 staged in shared memory (X turned, so that a
+// thread reads its RT rows' values of a coordinate in 16-byte loads that the
+// whole warp shares); thread t owns rows RT (t / 32) .. and columns
+// 4 (t % 32) .. +3.  With RT = 8 a coordinate costs a thread 32 FMAs for
+// three 16-byte shared loads, and R is read from L2 once per 64 rows; the
+// former kernel (one row per CTA, R streamed from L2 for every row, a second
+// FMA per product for the error bound) was bound by those reads: 99,991 x 300
+// x 1,024 bits took 36.4 ms, 2.69 ms here; 1,659 x 100 x 512 bits 208 us, 34 us here.
+//
+// Error bound: a stage's chain of at most 32 FMAs, then the stage totals
+// added in order, so no product passes through more than 32 + ceil(d/32)
+// roundings, and sum|x_i r_ij| <= |x| |r_j| (norms formed from the staged
+// values, every operation rounded up): a sum of magnitude above 1.25 times
+// that many u |x| |r_j| (plus the underflow terms) has the sign of the exact
+// sum.  The others, about 1 in 10^4, are summed in FP64 over coordinates
+// 0..d-1 in order, which is the definition.
+constexpr int kSimtK = 32;
+constexpr int kSimtCols = 128;
+
+template <int RT>
 __global__ void __launch_bounds__(256) srp_dense_simt_kernel(const float *__restrict__ X, long long N, int d,
-                                                             const float *__restrict__ R, int bits, int per_thread,
+                                                             const float *__restrict__ R, int bits, int col_tiles,
                                                              uint32_t *__restrict__ sig, blsh_dev_scratch *scratch) {
-    extern __shared__ float xs[];
-    const int T = blockDim.x;
-    const int t = threadIdx.x;
+    constexpr int ROWS = 8 * RT;
+    __shared__ __align__(16) float xs[kSimtK][ROWS + 4];      // [k][row]
+    __shared__ __align__(16) float rs[kSimtK][kSimtCols];
+    __shared__ float xn[ROWS], rn[kSimtCols];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const long long rt = blockIdx.x / col_tiles;
+    const int j0 = (int)(blockIdx.x - rt * col_tiles) * kSimtCols;
+    const long long row0 = rt * ROWS;
+    const int ncols = bits - j0 < kSimtCols ? bits - j0 : kSimtCols;   // a multiple of 32
+    float tot[RT][4];
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tot[i][c] = 0.0f;
+    float nrm = 0.0f;   // threads 0 .. ROWS-1: their row's squared norm; 128 .. 255: their column's
+    for (int k0 = 0; k0 < d; k0 += kSimtK) {
+        __syncthreads();
+        for (int r = w; r < ROWS; r += 8) {
+            const long long row = row0 + r;
+            xs[lane][r] = row < N && k0 + lane < d ? __ldg(X + (size_t)row * d + k0 + lane) : 0.0f;
+        }
+        for (int i = t; i < kSimtK * kSimtCols; i += 256) {
+            const int k = i / kSimtCols, c = i % kSimtCols;
+            rs[k][c] = k0 + k < d && c < ncols ? __ldg(R + (size_t)(k0 + k) * bits + j0 + c) : 0.0f;
+        }
+        __syncthreads();
+        if (t < ROWS) {
+#pragma unroll
+            for (int k = 0; k < kSimtK; ++k) nrm = __fmaf_ru(xs[k][t], xs[k][t], nrm);
+        } else if (t >= 128) {
+#pragma unroll
+            for (int k = 0; k < kSimtK; ++k) nrm = __fmaf_ru(rs[k][t - 128], rs[k][t - 128], nrm);
+        }
+        float acc[RT][4];
+#pragma unroll
+        for (int i = 0; i < RT; ++i)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[i][c] = 0.0f;
+#pragma unroll 8
+        for (int k = 0; k < kSimtK; ++k) {
+            const float4 r = *reinterpret_cast<const float4 *>(&rs[k][4 * lane]);
+            float x[RT];
+#pragma unroll
+            for (int i = 0; i < RT; i += 4) {
+                const float4 v = *reinterpret_cast<const float4 *>(&xs[k][RT * w + i]);
+                x[i] = v.x; x[i + 1] = v.y; x[i + 2] = v.z; x[i + 3] = v.w;
+            }
+#pragma unroll
+            for (int i = 0; i < RT; ++i) {
+                acc[i][0] = __fmaf_rn(x[i], r.x, acc[i][0]);
+                acc[i][1] = __fmaf_rn(x[i], r.y, acc[i][1]);
+                acc[i][2] = __fmaf_rn(x[i], r.z, acc[i][2]);
+                acc[i][3] = __fmaf_rn(x[i], r.w, acc[i][3]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < RT; ++i)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) tot[i][c] = __fadd_rn(tot[i][c], acc[i][c]);
+    }
+    if (t < ROWS) xn[t] = __fsqrt_ru(nrm);
+    else if (t >= 128) rn[t - 128] = __fsqrt_ru(nrm);
+    __syncthreads();
     const int words = bits >> 5;
+    const float u = 1.25f * (float)(kSimtK + (d + kSimtK - 1) / kSimtK) * 5.9604644775390625e-8f;
+    const float tiny = (float)d * 2.9e-45f;
+    const bool loose = (float)d * 5.9604644775390625e-8f > 0.05f;   // the 1.25 slack needs d u <= 0.05
     unsigned long long rechecked = 0, zeros = 0;
-    for (long long row = blockIdx.x; row < N; row += gridDim.x) {
-        __syncthreads();
-        for (int c = t; c < d; c += T) xs[c] = __ldg(X + (size_t)row * d + c);
-        __syncthreads();
-        float acc[kSrpMaxPerThread], mag[kSrpMaxPerThread];
 #pragma unroll
-        for (int u = 0; u < kSrpMaxPerThread; ++u) acc[u] = mag[u] = 0.0f;
-        for (int c = 0; c < d; ++c) {
-            const float v = xs[c];
-            const float *Rrow = R + (size_t)c * bits + t;
+    for (int i = 0; i < RT; ++i) {
+        const long long row = row0 + RT * w + i;
+        const float ux = u * xn[RT * w + i];
+        uint32_t nib = 0;
 #pragma unroll
-            for (int u = 0; u < kSrpMaxPerThread; ++u) {
-                if (u < per_thread) {
-                    const float r = __ldg(Rrow + u * T);
-                    acc[u] = __fmaf_rn(v, r, acc[u]);
-                    mag[u] = __fmaf_rn(fabsf(v), fabsf(r), mag[u]);
-                }
+        for (int c = 0; c < 4; ++c) {
+            const int col = 4 * lane + c;
+            bool bit = tot[i][c] >= 0.0f;
+            if (row < N && col < ncols && (loose || !(fabsf(tot[i][c]) > ux * rn[col] + tiny))) {
+                double dd = 0.0;
+                for (int k = 0; k < d; ++k)
+                    dd += (double)__ldg(X + (size_t)row * d + k) * (double)__ldg(R + (size_t)k * bits + j0 + col);
+                bit = dd >= 0.0;
+                ++rechecked;
+                zeros += dd == 0.0;
             }
+            nib |= (uint32_t)bit << c;
         }
-        const float n = (float)d;
-        const int w = t >> 5;
-#pragma unroll
-        for (int u = 0; u < kSrpMaxPerThread; ++u) {
-            if (u < per_thread) {
-                const float bound = 1.25f * n * 5.9604644775390625e-8f * mag[u] + n * 1.4e-45f;
-                bool bit;
-                if (fabsf(acc[u]) > bound) {
-                    bit = acc[u] >= 0.0f;
-                } else {
-                    double dd = 0.0;
-                    for (int c = 0; c < d; ++c) dd += (double)xs[c] * (double)__ldg(R + (size_t)c * bits + t + u * T);
-                    bit = dd >= 0.0;
-                    ++rechecked;
-                    zeros += dd == 0.0;
-                }
-                const unsigned word = __ballot_sync(kFull, bit);
-                if ((t & 31) == 0) sig[(size_t)row * words + w + u * (T >> 5)] = word;
-            }
-        }
+        // eight lanes' nibbles form a word
+        uint32_t word = nib << (4 * (lane & 7));
+        word |= __shfl_xor_sync(kFull, word, 1);
+        word |= __shfl_xor_sync(kFull, word, 2);
+        word |= __shfl_xor_sync(kFull, word, 4);
+        if ((lane & 7) == 0 && row < N && 4 * lane < ncols) sig[(size_t)row * words + (j0 >> 5) + (lane >> 3)] = word;
     }
     if (rechecked) atomicAdd(&scratch->counters[2], rechecked);
     if (zeros) atomicAdd(&scratch->counters[3], zeros);
@@ -875,18 +944,16 @@ extern "C" int blsh_srp_sparse(blsh_ctx *ctx, const int64_t *indptr, const uint3
 int blsh_srp_dense_simt(blsh_ctx *ctx, const float *X, int64_t N, int32_t d, const float *R, int32_t bits,
                         uint32_t *sig, cudaStream_t s) {
     int per_thread = 0;
-    const int T = srp_threads(bits, &per_thread);
+    srp_threads(bits, &per_thread);
     if (per_thread > kSrpMaxPerThread) return blsh_fail(ctx, BLSH_EINVAL, "bits/32 needs a divisor in 2..8");
-    const size_t smem = sizeof(float) * (size_t)d;
-    if (smem > 48 * 1024) {
-        if (smem > ctx->smem_optin) return blsh_fail(ctx, BLSH_EINVAL, "d too large");
-        BLSH_CUDA(ctx, cudaFuncSetAttribute(srp_dense_simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)smem));
-    }
-    const long long cap = (long long)ctx->sm_count * 16;
-    const unsigned grid = (unsigned)(N < cap ? N : cap);
+    if (sizeof(float) * (size_t)d > ctx->smem_optin) return blsh_fail(ctx, BLSH_EINVAL, "d too large");
+    // 64-row tiles where they give every SM at least two, else 32-row ones
+    const int col_tiles = (bits + kSimtCols - 1) / kSimtCols;
+    const bool wide = (N + 63) / 64 * col_tiles >= 2ll * ctx->sm_count;
+    const long long tiles = (wide ? (N + 63) / 64 : (N + 31) / 32) * col_tiles;   // N < 2^32, so < 2^31
     blsh_time_start(ctx, s);
-    srp_dense_simt_kernel<<<grid, T, smem, s>>>(X, N, d, R, bits, per_thread, sig, ctx->scratch);
+    (wide ? srp_dense_simt_kernel<8> : srp_dense_simt_kernel<4>)<<<(unsigned)tiles, 256, 0, s>>>(
+        X, N, d, R, bits, col_tiles, sig, ctx->scratch);
     BLSH_LAUNCHED(ctx, "srp_dense_simt_kernel");
     return BLSH_OK;
 }
