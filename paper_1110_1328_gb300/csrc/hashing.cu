@@ -9,25 +9,81 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 constexpr uint32_t kP31 = 0x7fffffffu;   // 2^31 - 1
 
-// (a x + b) mod (2^31 - 1) for a, b < 2^31 - 1 and any 32-bit x, exactly:
-// v < 2^63, and 2^31 = 1 (mod p) lets a fold of the high bits onto the low
-// 31 bits bring v below 2^32 + 2^31, a second fold (in 32 bits) below
-// 2^31 + 2, then one conditional subtraction.
-__device__ __forceinline__ uint32_t mod_mersenne31(uint32_t a, uint32_t b, uint32_t x) {
-    const unsigned long long v = (unsigned long long)a * x + b;
-    const unsigned long long r = (v & kP31) + (v >> 31);
-    const uint32_t h = ((uint32_t)r & kP31) + (uint32_t)(r >> 31);
-    return h >= kP31 ? h - kP31 : h;
+// v mod (2^31 - 1) for any 32-bit v.
+__device__ __forceinline__ uint32_t mod_p31(uint32_t v) {
+    const uint32_t f = (v & kP31) + (v >> 31);   // at most 2^31
+    return f >= kP31 ? f - kP31 : f;
 }
 
-// One warp per set; lane l owns hashes l, l+32, ..., l+32(HPL-1) of the
-// current tile of 32*HPL hashes and keeps their running minima in
-// registers.  The set's elements are read 32 at a time (coalesced) and
-// broadcast with shuffles.  Sets longer than kBigSet are left to
-// minhash_big_kernel.
-constexpr long long kBigSet = 2048;
+// The running minimum of (a x + b) mod p, p = 2^31 - 1, for a, b, x < p, given
+// a2 = 2a and b2 = 2b: with v = a x + b < p (p - 1) + p, the high word of 2v is
+// v >> 31 < p and the low word is 2 (v mod 2^31), so r = high + low / 2 is
+// congruent to v and below 2p: the residue is r or r - p, and where r < p the
+// difference wraps to a larger number, so the three-way minimum takes the
+// right one.  Four instructions (multiply-add to 64 bits, shift-and-add,
+// subtract, minimum) against about twelve for folding twice and subtracting
+// under a test; the integer pipe is what this kernel waits for.
+__device__ __forceinline__ uint32_t min_hash31(uint32_t mn, uint32_t a2, uint32_t b2, uint32_t x) {
+    const unsigned long long v2 = (unsigned long long)a2 * x + b2;
+    const uint32_t r = (uint32_t)(v2 >> 32) + ((uint32_t)v2 >> 1);
+    return __vimin3_u32(mn, r, r - kP31);
+}
 
-constexpr long long kBigChunk = 4096;   // elements of a long set per CTA task
+// Minima over elements [s, e) of the hashes whose a2, b2 the lanes hold:
+// elements are read 32 at a time, one per lane, and broadcast; a partial
+// block repeats its last element (a minimum does not change) up to a multiple
+// of four, so that the loop runs four elements at a time.
+template <int HPL>
+__device__ __forceinline__ void min_hash_run(const uint32_t *__restrict__ indices, long long s, long long e,
+                                             const uint32_t (&a2)[HPL], const uint32_t (&b2)[HPL],
+                                             uint32_t (&mn)[HPL]) {
+    const int lane = threadIdx.x & 31;
+    for (long long e0 = s; e0 < e; e0 += 32) {
+        const int cnt = (int)min(32ll, e - e0);
+        const uint32_t mine = mod_p31(__ldg(indices + e0 + min(lane, cnt - 1)));
+        for (int l = 0; l < cnt; l += 4) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t x = __shfl_sync(kFull, mine, l + q);   // lanes past cnt hold the last element
+#pragma unroll
+                for (int u = 0; u < HPL; ++u) mn[u] = min_hash31(mn[u], a2[u], b2[u], x);
+            }
+        }
+    }
+}
+
+// One warp per (set, tile of 32 HPL hashes): lane l owns hashes l, l + 32, ...
+// of tile blockIdx.y and keeps their running minima in registers.  A warp
+// alone takes about 46 ns an element, so sets longer than kBigSet are queued
+// in chunks of kBigChunk elements for minhash_big_kernel: the degrees of a
+// graph follow a power law, and a set of 150,000 elements would hold up one
+// warp for milliseconds.
+// 1e6 neighbour lists (mean 27) x 256 hashes, both kernels: 4.77 ms with
+// twelve instructions a hash and long sets spread over whole CTAs, 1.66 now
+// (4.2e12 hashes/s; 4.9e12 where every set has 64 elements or more, the
+// rate of the 64-bit multiply-add and the four others at this mix).
+constexpr long long kBigSet = 256;
+constexpr long long kBigChunk = 256;   // elements of a long set per warp task
+
+// Queues the chunks of a long set [s, e) for one tile of hashes (one warp);
+// false if the queue is full: the set is then hashed by its own warp.
+__device__ __forceinline__ bool queue_long_set(long long i, long long s, long long e, unsigned tile, unsigned tiles,
+                                               blsh_dev_scratch *scratch, uint2 *__restrict__ big) {
+    const int lane = threadIdx.x & 31;
+    const unsigned long long chunks = (unsigned long long)(e - s + kBigChunk - 1) / kBigChunk;
+    unsigned long long slot = 0;
+    if (lane == 0) slot = atomicAdd(&scratch->work3, chunks);
+    slot = __shfl_sync(kFull, slot, 0);
+    if (slot + chunks <= BLSH_RECHECK_CAP) {
+        for (unsigned long long c = lane; c < chunks; c += 32)
+            big[slot + c] = make_uint2((uint32_t)i, (uint32_t)c * tiles + tile);
+        return true;
+    }
+    // entries of the queue that this set reserved but does not fill
+    for (unsigned long long c = slot + lane; c < slot + chunks && c < BLSH_RECHECK_CAP; c += 32)
+        big[c] = make_uint2(0u, 0xffffffffu);
+    return false;
+}
 
 template <int HPL>
 __global__ void __launch_bounds__(256) minhash_kernel(const int64_t *__restrict__ indptr,
@@ -36,100 +92,107 @@ __global__ void __launch_bounds__(256) minhash_kernel(const int64_t *__restrict_
                                                       const uint32_t *__restrict__ B, uint32_t *__restrict__ sig,
                                                       blsh_dev_scratch *scratch, uint2 *__restrict__ big) {
     const int lane = threadIdx.x & 31;
+    const int h0 = blockIdx.y * 32 * HPL + lane;
+    uint32_t a2[HPL], b2[HPL];
+#pragma unroll
+    for (int u = 0; u < HPL; ++u) {
+        a2[u] = 2u * mod_p31(__ldg(A + h0 + 32 * u));
+        b2[u] = 2u * mod_p31(__ldg(B + h0 + 32 * u));
+    }
     const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
     for (long long i = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < N; i += warps) {
         const long long s = __ldg(indptr + i), e = __ldg(indptr + i + 1);
-        if (e - s > kBigSet) {
-            // a long set: its row starts at the identity of min, the chunks of
-            // minhash_big_kernel lower it; queued unless the queue is full
-            for (int k = lane; k < n_hashes; k += 32) sig[(size_t)i * n_hashes + k] = 0xffffffffu;
-            unsigned long long slot = 0;
-            if (lane == 0) slot = atomicAdd(&scratch->work3, 1ull);
-            slot = __shfl_sync(kFull, slot, 0);
-            if (slot < BLSH_RECHECK_CAP) {
-                if (lane == 0) big[slot] = make_uint2((uint32_t)i, (uint32_t)((e - s + kBigChunk - 1) / kBigChunk));
-                continue;
-            }
-        }
-        for (int t0 = 0; t0 < n_hashes; t0 += 32 * HPL) {
-            uint32_t a[HPL], b[HPL], mn[HPL];
+        uint32_t mn[HPL];
 #pragma unroll
-            for (int u = 0; u < HPL; ++u) {
-                a[u] = __ldg(A + t0 + 32 * u + lane);
-                b[u] = __ldg(B + t0 + 32 * u + lane);
-                mn[u] = 0xffffffffu;
-            }
-            for (long long e0 = s; e0 < e; e0 += 32) {
-                const uint32_t mine = e0 + lane < e ? __ldg(indices + e0 + lane) : 0u;
-                const int cnt = (int)min(32ll, e - e0);
-                for (int l = 0; l < cnt; ++l) {
-                    const uint32_t x = __shfl_sync(kFull, mine, l);
+        for (int u = 0; u < HPL; ++u) mn[u] = 0xffffffffu;
+        // a long set: its part of the row starts at the identity of min, the
+        // chunks lower it
+        const bool queued = e - s > kBigSet && queue_long_set(i, s, e, blockIdx.y, gridDim.y, scratch, big);
+        if (!queued) min_hash_run<HPL>(indices, s, e, a2, b2, mn);
 #pragma unroll
-                    for (int u = 0; u < HPL; ++u) mn[u] = min(mn[u], mod_mersenne31(a[u], b[u], x));
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < HPL; ++u) sig[(size_t)i * n_hashes + t0 + 32 * u + lane] = mn[u];
-        }
+        for (int u = 0; u < HPL; ++u) sig[(size_t)i * n_hashes + h0 + 32 * u] = mn[u];
     }
 }
 
-// Sets longer than kBigSet, queued by minhash_kernel as (set, chunks of
-// kBigChunk elements).  Every CTA walks the queue and takes the chunks of
-// each set that fall to it (chunk c of queue entry q goes to CTA
-// (c + 7919 q) mod gridDim), so one set with thousands of elements is
-// hashed by many SMs.  In a chunk, warp w takes every 32nd block of 32
-// elements; the warps' minima meet in shared memory, and the chunk's minima
-// in the set's row in global memory (atomicMin: the minimum does not depend
-// on the order).
+// The same for few sets: a CTA per (set, tile), its eight warps taking an
+// eighth of the elements each, their minima joined in shared memory.
 template <int HPL>
-__global__ void __launch_bounds__(1024) minhash_big_kernel(const int64_t *__restrict__ indptr,
-                                                           const uint32_t *__restrict__ indices, int n_hashes,
-                                                           const uint32_t *__restrict__ A,
-                                                           const uint32_t *__restrict__ B,
-                                                           uint32_t *__restrict__ sig, const blsh_dev_scratch *scratch,
-                                                           const uint2 *__restrict__ big) {
-    __shared__ uint32_t smin[32 * HPL];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+__global__ void __launch_bounds__(256) minhash_cta_kernel(const int64_t *__restrict__ indptr,
+                                                          const uint32_t *__restrict__ indices, int n_hashes,
+                                                          const uint32_t *__restrict__ A,
+                                                          const uint32_t *__restrict__ B, uint32_t *__restrict__ sig,
+                                                          blsh_dev_scratch *scratch, uint2 *__restrict__ big) {
+    __shared__ uint32_t red[8][32 * HPL];
+    __shared__ bool s_queued;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int h0 = blockIdx.y * 32 * HPL;
+    const long long i = blockIdx.x;
+    const long long s = __ldg(indptr + i), e = __ldg(indptr + i + 1);
+    uint32_t a2[HPL], b2[HPL], mn[HPL];
+#pragma unroll
+    for (int u = 0; u < HPL; ++u) {
+        a2[u] = 2u * mod_p31(__ldg(A + h0 + 32 * u + lane));
+        b2[u] = 2u * mod_p31(__ldg(B + h0 + 32 * u + lane));
+        mn[u] = 0xffffffffu;
+    }
+    bool queued = false;
+    if (e - s > 8 * kBigSet) {
+        if (warp == 0) {
+            const bool q = queue_long_set(i, s, e, blockIdx.y, gridDim.y, scratch, big);
+            if (lane == 0) s_queued = q;
+        }
+        __syncthreads();
+        queued = s_queued;
+    }
+    if (!queued) {
+        const long long piece = (e - s + 7) >> 3;
+        const long long s0 = s + warp * piece, e0 = s0 + piece < e ? s0 + piece : e;
+        min_hash_run<HPL>(indices, s0, e0, a2, b2, mn);
+    }
+#pragma unroll
+    for (int u = 0; u < HPL; ++u) red[warp][32 * u + lane] = mn[u];
+    __syncthreads();
+    if (threadIdx.x < 32 * HPL) {
+        uint32_t m = red[0][threadIdx.x];
+#pragma unroll
+        for (int w = 1; w < 8; ++w) m = min(m, red[w][threadIdx.x]);
+        sig[(size_t)i * n_hashes + h0 + threadIdx.x] = m;
+    }
+}
+
+// The queued chunks of long sets, a warp each: entry (set, chunk * tiles +
+// tile); the chunk's minima meet in the set's row in global memory (atomicMin:
+// the minimum does not depend on the order).
+template <int HPL>
+__global__ void __launch_bounds__(256) minhash_big_kernel(const int64_t *__restrict__ indptr,
+                                                          const uint32_t *__restrict__ indices, int n_hashes,
+                                                          const uint32_t *__restrict__ A,
+                                                          const uint32_t *__restrict__ B,
+                                                          uint32_t *__restrict__ sig, const blsh_dev_scratch *scratch,
+                                                          const uint2 *__restrict__ big) {
+    const int lane = threadIdx.x & 31;
+    const unsigned tiles = (unsigned)n_hashes / (32u * HPL);
     const unsigned long long total = scratch->work3;
     const unsigned long long nq = total < BLSH_RECHECK_CAP ? total : BLSH_RECHECK_CAP;
-    const unsigned G = gridDim.x;
-    for (unsigned long long qi = 0; qi < nq; ++qi) {
-        const uint2 ent = big[qi];
-        const long long i = ent.x;
-        const unsigned chunks = ent.y;
-        const unsigned first = (unsigned)((blockIdx.x + (unsigned long long)G * chunks - (qi * 7919ull) % G) % G);
-        for (unsigned c = first; c < chunks; c += G) {
-            const long long s0 = __ldg(indptr + i) + (long long)c * kBigChunk;
-            const long long e1 = __ldg(indptr + i + 1);
-            const long long e = e1 < s0 + kBigChunk ? e1 : s0 + kBigChunk;
-            for (int t0 = 0; t0 < n_hashes; t0 += 32 * HPL) {
-                __syncthreads();
-                for (int k = threadIdx.x; k < 32 * HPL; k += blockDim.x) smin[k] = 0xffffffffu;
-                __syncthreads();
-                uint32_t a[HPL], b[HPL], mn[HPL];
+    const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+    for (unsigned long long q = (unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < nq;
+         q += warps) {
+        const uint2 ent = big[q];
+        if (ent.y == 0xffffffffu) continue;
+        const unsigned c = ent.y / tiles;
+        const int h0 = (int)(ent.y - c * tiles) * 32 * HPL + lane;
+        const long long s = __ldg(indptr + ent.x) + (long long)c * kBigChunk;
+        const long long e = min(s + kBigChunk, (long long)__ldg(indptr + ent.x + 1));
+        uint32_t a2[HPL], b2[HPL], mn[HPL];
 #pragma unroll
-                for (int u = 0; u < HPL; ++u) {
-                    a[u] = __ldg(A + t0 + 32 * u + lane);
-                    b[u] = __ldg(B + t0 + 32 * u + lane);
-                    mn[u] = 0xffffffffu;
-                }
-                for (long long e0 = s0 + 32ll * warp; e0 < e; e0 += 32ll * nwarps) {
-                    const uint32_t mine = e0 + lane < e ? __ldg(indices + e0 + lane) : 0u;
-                    const int cnt = (int)min(32ll, e - e0);
-                    for (int l = 0; l < cnt; ++l) {
-                        const uint32_t x = __shfl_sync(kFull, mine, l);
-#pragma unroll
-                        for (int u = 0; u < HPL; ++u) mn[u] = min(mn[u], mod_mersenne31(a[u], b[u], x));
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < HPL; ++u) atomicMin(&smin[32 * u + lane], mn[u]);
-                __syncthreads();
-                for (int k = threadIdx.x; k < 32 * HPL; k += blockDim.x)
-                    atomicMin(&sig[(size_t)i * n_hashes + t0 + k], smin[k]);
-            }
+        for (int u = 0; u < HPL; ++u) {
+            a2[u] = 2u * mod_p31(__ldg(A + h0 + 32 * u));
+            b2[u] = 2u * mod_p31(__ldg(B + h0 + 32 * u));
+            mn[u] = 0xffffffffu;
         }
+        min_hash_run<HPL>(indices, s, e, a2, b2, mn);
+#pragma unroll
+        for (int u = 0; u < HPL; ++u) atomicMin(&sig[(size_t)ent.x * n_hashes + h0 + 32 * u], mn[u]);
     }
 }
 
@@ -868,16 +931,24 @@ int srp_threads(int bits, int *per_thread) {
 
 // minhash_kernel over every set, then minhash_big_kernel over the long sets
 // the first one queued.
-template <int WV>
-int minhash_launch(blsh_ctx *ctx, cudaStream_t s, unsigned grid, unsigned big_grid, const int64_t *indptr,
-                   const uint32_t *indices, int64_t N, int n_hashes, const uint32_t *a, const uint32_t *b,
-                   uint32_t *sig, uint2 *big) {
+template <int HPL>
+int minhash_launch(blsh_ctx *ctx, cudaStream_t s, const int64_t *indptr, const uint32_t *indices, int64_t N,
+                   int n_hashes, const uint32_t *a, const uint32_t *b, uint32_t *sig, uint2 *big) {
     blsh_dev_scratch *scr = ctx->scratch;
+    const unsigned tiles = (unsigned)(n_hashes / (32 * HPL));
+    const long long blocks = (N + 7) / 8, cap = (long long)ctx->sm_count * 32;
     blsh_time_start(ctx, s);
-    minhash_kernel<WV><<<grid, 256, 0, s>>>(indptr, indices, N, n_hashes, a, b, sig, scr, big);
+    // a CTA per set where a warp per set would give an SM fewer than 32: then
+    // the longest set's chain decides (2,000 sets, mean 50, longest 837, x 256
+    // hashes: 124 us with a warp per set, 23 us with a CTA)
+    if (N * tiles < 32ll * ctx->sm_count)
+        minhash_cta_kernel<HPL><<<dim3((unsigned)N, tiles), 256, 0, s>>>(indptr, indices, n_hashes, a, b, sig, scr, big);
+    else
+        minhash_kernel<HPL><<<dim3((unsigned)(blocks < cap ? blocks : cap), tiles), 256, 0, s>>>(
+            indptr, indices, N, n_hashes, a, b, sig, scr, big);
     BLSH_LAUNCHED(ctx, "minhash_kernel");
     blsh_time_start(ctx, s);
-    minhash_big_kernel<WV><<<big_grid, 1024, 0, s>>>(indptr, indices, n_hashes, a, b, sig, scr, big);
+    minhash_big_kernel<HPL><<<ctx->sm_count * 4, 256, 0, s>>>(indptr, indices, n_hashes, a, b, sig, scr, big);
     BLSH_LAUNCHED(ctx, "minhash_big_kernel");
     return BLSH_OK;
 }
@@ -893,20 +964,16 @@ extern "C" int blsh_minhash(blsh_ctx *ctx, const int64_t *indptr, const uint32_t
     if (N == 0) return BLSH_OK;
     blsh_device_guard g(ctx->device);
     cudaStream_t s = blsh_stream(stream);
-    const long long blocks_needed = (N + 7) / 8;
-    const long long cap = (long long)ctx->sm_count * 8;
-    const unsigned grid = (unsigned)(blocks_needed < cap ? blocks_needed : cap);
     const int words = n_hashes / 32;
-    const unsigned big_grid = (unsigned)ctx->sm_count * 2;
     // long sets go to minhash_big_kernel through the context's work queue
     uint2 *big = ctx->recheck_queue;
     BLSH_CUDA(ctx, cudaMemsetAsync(&ctx->scratch->work3, 0, sizeof(unsigned long long), s));
-    const int wv = words % 8 == 0 ? 8 : words % 4 == 0 ? 4 : words % 2 == 0 ? 2 : 1;
-    switch (wv) {
-    case 8: return minhash_launch<8>(ctx, s, grid, big_grid, indptr, indices, N, n_hashes, a, b, sig, big);
-    case 4: return minhash_launch<4>(ctx, s, grid, big_grid, indptr, indices, N, n_hashes, a, b, sig, big);
-    case 2: return minhash_launch<2>(ctx, s, grid, big_grid, indptr, indices, N, n_hashes, a, b, sig, big);
-    default: return minhash_launch<1>(ctx, s, grid, big_grid, indptr, indices, N, n_hashes, a, b, sig, big);
+    const int hpl = words % 8 == 0 ? 8 : words % 4 == 0 ? 4 : words % 2 == 0 ? 2 : 1;   // hashes a lane
+    switch (hpl) {
+    case 8: return minhash_launch<8>(ctx, s, indptr, indices, N, n_hashes, a, b, sig, big);
+    case 4: return minhash_launch<4>(ctx, s, indptr, indices, N, n_hashes, a, b, sig, big);
+    case 2: return minhash_launch<2>(ctx, s, indptr, indices, N, n_hashes, a, b, sig, big);
+    default: return minhash_launch<1>(ctx, s, indptr, indices, N, n_hashes, a, b, sig, big);
     }
 }
 
