@@ -621,7 +621,7 @@ extern "C" int blsh_verify_lite(blsh_ctx *ctx, const blsh_tables *tab, const uin
     A.lsim = nullptr;
     A.cap_levels = A.levels;
     A.need = nullptr;
-    const blsh_plan plan = blsh_plan_for(ctx, tab);
+    const blsh_plan plan = blsh_plan_for(ctx, tab, P);
     A.grab = (plan.grab + 31) / 32 * 32;
     int rc = blsh_launch_verify(ctx, A, plan, s);
     if (rc) return rc;
@@ -720,7 +720,7 @@ int verify_both(blsh_ctx *ctx, const blsh_tables *tab, int32_t hash_limit, const
     A.lsim = sim;
     A.cap_levels = hash_limit / p.k;
     A.need = need;
-    const blsh_plan plan = blsh_plan_for(ctx, tab);
+    const blsh_plan plan = blsh_plan_for(ctx, tab, P);
     A.grab = (plan.grab + 31) / 32 * 32;
     blsh_device_guard g(ctx->device);
     cudaStream_t s = blsh_stream(stream);

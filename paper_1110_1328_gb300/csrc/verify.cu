@@ -1142,11 +1142,19 @@ int dispatch(blsh_ctx *ctx, const VerifyArgs &A, const blsh_plan &plan, int kind
 
 }  // namespace
 
-blsh_plan blsh_default_plan(int kind) {
+// The plan of a caller who has not tuned one, for up to P pairs: the plain
+// form, the fastest for every k, size and kind measured (Algorithms 1 and 2
+// together, plain against persistent: 2.7e7 cosine pairs, k = 32: 240 against
+// 471 us, k = 64: 334 / 448, k = 128: 319 / 444; 6e5 pairs 54 / 58; 1.4e7
+// Jaccard pairs, k = 32: four lanes a pair 467 / 524, one 542, eight 775 / 865;
+// k = 64: 555 / 638, 913, 938 / 1,079; 176 pairs 31 / 41).  Cosine calls over
+// fewer than 65,536 pairs, where the two forms take the same time, keep the
+// persistent one.
+blsh_plan blsh_default_plan(int kind, long long P) {
     blsh_plan p;
-    p.mode = BLSH_PLAN_PERSISTENT;
-    p.group = kind == BLSH_COSINE ? 1 : 8;
-    p.block = 256;
+    p.mode = kind == BLSH_COSINE && P < 65536 ? BLSH_PLAN_PERSISTENT : BLSH_PLAN_PLAIN;
+    p.group = kind == BLSH_COSINE ? 1 : 4;
+    p.block = kind == BLSH_COSINE ? 256 : 128;
     p.grab = kind == BLSH_COSINE ? 128 : 32;
     p.ctas_per_sm = 0;
     return p;
@@ -1252,8 +1260,8 @@ int blsh_make_verify_args(blsh_ctx *ctx, const blsh_tables *tab, const uint32_t 
 // The plan the autotuner chose for these tables, else the default.  (A
 // plan stored for destroyed tables whose address was reused may not fit the
 // new tables' kind and k; the default is used then.)
-blsh_plan blsh_plan_for(blsh_ctx *ctx, const blsh_tables *tab) {
-    blsh_plan plan = blsh_default_plan(tab->p.kind);
+blsh_plan blsh_plan_for(blsh_ctx *ctx, const blsh_tables *tab, long long P) {
+    blsh_plan plan = blsh_default_plan(tab->p.kind, P);
     std::lock_guard<std::mutex> lk(ctx->mu);
     auto it = ctx->plans.find(tab);
     if (it != ctx->plans.end() && blsh_check_plan(it->second, tab->p.kind, tab->p.k) == BLSH_OK) plan = it->second;
@@ -1284,7 +1292,7 @@ extern "C" int blsh_verify(blsh_ctx *ctx, const blsh_tables *tab, const uint32_t
                            uint8_t *status, uint16_t *n_used, uint16_t *m, float *est, uint64_t *stop_hist,
                            void *stream) {
     if (!ctx || !tab) return BLSH_EINVAL;
-    const blsh_plan plan = blsh_plan_for(ctx, tab);
+    const blsh_plan plan = blsh_plan_for(ctx, tab, P);
     return blsh_verify_plan(ctx, tab, &plan, pairs, P, P_dev, sig, N, sig_words, status, n_used, m, est,
                             stop_hist, stream);
 }
@@ -1332,7 +1340,7 @@ int tune_plans(blsh_ctx *ctx, const blsh_tables *tab, const uint32_t *pairs, int
     BLSH_CUDA(ctx, cudaEventCreate(&e0));
     BLSH_CUDA(ctx, cudaEventCreate(&e1));
     float best_ms = 1e30f;
-    blsh_plan best_plan = blsh_default_plan(kind);
+    blsh_plan best_plan = blsh_default_plan(kind, P);
     int rc = BLSH_OK;
     for (const blsh_plan &p : cands) {
         rc = blsh_verify_plan(ctx, tab, &p, pairs, P, nullptr, sig, N, sig_words, status, n_used, m, est,
@@ -1391,7 +1399,7 @@ extern "C" int blsh_autotune_k(blsh_ctx *ctx, const blsh_params *params, const i
             return blsh_fail(ctx, BLSH_EINVAL, "chunk size %d: not 32, 64 or 128, or not dividing n_max", ks[i]);
     blsh_device_guard g(ctx->device);
     blsh_tables *best_tab = nullptr;
-    blsh_plan best_plan = blsh_default_plan(params->kind);
+    blsh_plan best_plan = blsh_default_plan(params->kind, P);
     float best_ms = 1e30f;
     int rc = BLSH_OK;
     for (int i = 0; i < n_ks && rc == BLSH_OK; ++i) {

@@ -56,9 +56,9 @@ struct VerifyArgs {
 // those computed so far (blsh_verify_resume finishes it).
 
 int blsh_launch_verify(blsh_ctx *ctx, const VerifyArgs &A, const blsh_plan &plan, cudaStream_t s);
-blsh_plan blsh_default_plan(int kind);
+blsh_plan blsh_default_plan(int kind, long long P);
 int blsh_check_plan(const blsh_plan &plan, int kind, int k);
 int blsh_make_verify_args(blsh_ctx *ctx, const blsh_tables *tab, const uint32_t *pairs, int64_t P,
                           const int64_t *P_dev, const uint32_t *sig, int64_t N, int32_t sig_words, uint8_t *status,
                           uint16_t *n_used, uint16_t *m, float *est, uint64_t *stop_hist, VerifyArgs &A);
-blsh_plan blsh_plan_for(blsh_ctx *ctx, const blsh_tables *tab);
+blsh_plan blsh_plan_for(blsh_ctx *ctx, const blsh_tables *tab, long long P);
