@@ -13,10 +13,10 @@
 //      (cosine: ceil((t - 1e-9) 2^48); sets: ceil(t |x| - 1e-9)).  The
 //      unindexed prefix then cannot lift a similarity to t, so every pair that
 //      reaches t shares an indexed feature of its first row.  Rows of up to
-//      32 elements: a warp, lane = element, each lane's bound the sum over the
-//      elements that precede or equal it (shuffles); up to 4096: a CTA sorts
-//      (order key, position) in shared memory and scans; longer rows index
-//      every feature;
+//      128 elements: a warp, each element's bound the sum over the elements
+//      that precede or equal it (one broadcast read of shared memory each); up
+//      to 4096: a CTA sorts (order key, position) in shared memory and scans;
+//      longer rows index every feature;
 //   3. the inverted index: a key (feature, row) per indexed nonzero (padding
 //      for the others), radix-sorted, so that a feature's list holds its rows
 //      in increasing order, and each feature's list bounds from a scan of the
@@ -27,6 +27,15 @@
 //      writes each prefix with coalesced stores);
 //   5. the keys are radix-sorted, and the distinct ones are written as pairs
 //      (x, y) in increasing order.
+//
+// Where N^2 <= 4096 max_dups (and N <= 2^19) steps 3 to 5 need no sort: the
+// rows of every feature are listed in any order, and a CTA per row x sets bit
+// y of an N-bit map in shared memory for every y > x in the lists of x's
+// indexed features; the map's set bits, in order, are x's candidates (counted
+// first, then written at scanned offsets).  A map costs N / 32 words per row
+// and pass (0.3 ps a word), the sort about 50 ps a key, which is where the
+// line lies.  20,000 tf-idf rows (2.4e7 keys, 1.7e7 pairs): 1.96 ms by sorting,
+// 0.86 ms with the maps.
 #include "common.cuh"
 #include "radix.cuh"
 #include "scan.cuh"
@@ -34,8 +43,9 @@
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kShortRow = 32;
+constexpr int kShortRow = 128;
 constexpr int kLongRow = 4096;
+constexpr long long kMapRows = 1ll << 19;   // bit maps of up to 64 KB
 constexpr double kTwo48 = 281474976710656.0;
 constexpr long long kTermCap = 1ll << 50;
 
@@ -86,11 +96,18 @@ __global__ void __launch_bounds__(256) ap_stats_kernel(ApArgs A, long long nnz) 
     if (bad) blsh_dev_error(A.scratch, BLSH_ERANGE, 0, bad);
 }
 
-// Rows of up to kShortRow elements (one warp per row, lane = element) and
-// rows longer than kLongRow (every feature indexed); the rows in between are
-// left to ap_prefix_cta_kernel.
+// Rows of up to kShortRow elements (one warp per row, up to kShortRow / 32
+// elements a lane) and rows longer than kLongRow (every feature indexed); the
+// rows in between are left to ap_prefix_cta_kernel.  The bound at an element
+// is the sum of the weights that precede it in the global order and its own:
+// n^2 comparisons, which a warp does faster than a CTA sorts while n <= 128
+// (20,000 rows, mean 57: 208 us with a CTA for every row above 32 elements,
+// 52 and 98 us with this).
 __global__ void __launch_bounds__(256) ap_prefix_warp_kernel(ApArgs A) {
+    __shared__ ulonglong2 s_kw[8][kShortRow];   // order key, weight
+    constexpr int EPL = kShortRow / 32;
     const int lane = threadIdx.x & 31;
+    ulonglong2 *kw = s_kw[threadIdx.x >> 5];
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     for (long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < A.N; row += nw) {
         const long long s = __ldg(A.indptr + row), n = __ldg(A.indptr + row + 1) - s;
@@ -99,25 +116,35 @@ __global__ void __launch_bounds__(256) ap_prefix_warp_kernel(ApArgs A) {
             continue;
         }
         if (n == 0 || n > kShortRow) continue;
-        uint32_t f = 0;
-        unsigned long long key = ~0ull;
-        long long w = 0;
-        if (lane < n) {
-            f = __ldg(A.indices + s + lane);
-            if (f < A.dim) {
-                key = ap_key(A, f);
-                w = ap_weight(A, s + lane, f);
+        unsigned long long key[EPL];
+        long long b[EPL];
+        __syncwarp();                              // the previous row has been read
+#pragma unroll
+        for (int u = 0; u < EPL; ++u) {
+            const int i = lane + 32 * u;
+            key[u] = ~0ull;
+            b[u] = 0;
+            long long w = 0;
+            if (i < n) {
+                const uint32_t f = __ldg(A.indices + s + i);
+                if (f < A.dim) {
+                    key[u] = ap_key(A, f);
+                    w = ap_weight(A, s + i, f);
+                }
+                kw[i] = make_ulonglong2(key[u], (unsigned long long)w);
             }
         }
-        // bound including this element: the weights of the elements that
-        // precede it in the global order, and its own
-        long long b = 0;
-        for (int j = 0; j < n; ++j) {
-            const unsigned long long kj = __shfl_sync(kFull, key, j);
-            const long long wj = __shfl_sync(kFull, w, j);
-            if (kj <= key) b += wj;
+        __syncwarp();
+        for (int j = 0; j < (int)n; ++j) {
+            const ulonglong2 v = kw[j];
+#pragma unroll
+            for (int u = 0; u < EPL; ++u)
+                if (v.x <= key[u]) b[u] += (long long)v.y;
         }
-        if (lane < n) A.indexed[s + lane] = b >= ap_threshold(A, n);
+        const long long thr = ap_threshold(A, n);
+#pragma unroll
+        for (int u = 0; u < EPL; ++u)
+            if (lane + 32 * u < n) A.indexed[s + lane + 32 * u] = b[u] >= thr;
     }
 }
 
@@ -314,9 +341,102 @@ __global__ void __launch_bounds__(256) ap_write_kernel(const unsigned long long 
     }
 }
 
+// ---- candidates by bit maps ---------------------------------------------------
+
+// Every feature's rows, in any order: post[fstart[f] .. fstart[f + 1]).
+__global__ void __launch_bounds__(256) ap_post_kernel(ApArgs A, const uint32_t *fstart, uint32_t *cursor,
+                                                      uint32_t *post) {
+    const int lane = threadIdx.x & 31;
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < A.N; row += nw) {
+        const long long s = __ldg(A.indptr + row), e = __ldg(A.indptr + row + 1);
+        for (long long i = s + lane; i < e; i += 32) {
+            const uint32_t f = __ldg(A.indices + i);
+            if (f < A.dim) post[__ldg(fstart + f) + atomicAdd(cursor + f, 1u)] = (uint32_t)row;
+        }
+    }
+}
+
+// One CTA per row x (grid-stride).  MAP_COUNT: cnt[x] = the number of distinct
+// y > x in the lists of x's indexed features.  MAP_WRITE: the pairs (x, y), y
+// increasing, from offset cnt[x] (after the scan).  Both MAP_COUNT and
+// MAP_DUPS (which forms no map) add the number of (feature, y) met to
+// *dup_total, the number of keys the sorting form would have.
+enum { MAP_DUPS, MAP_COUNT, MAP_WRITE };
+template <int MODE>
+__global__ void __launch_bounds__(256) ap_map_kernel(ApArgs A, const uint32_t *fstart, const uint32_t *post,
+                                                     unsigned long long *cnt, unsigned long long *dup_total,
+                                                     long long max_dups, uint32_t *pairs, long long cap) {
+    extern __shared__ uint32_t map[];   // [(N + 31) / 32], zero between rows
+    __shared__ unsigned s_cnt;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (MODE == MAP_WRITE && (long long)*dup_total > max_dups) return;   // no pairs: the buffer was too small
+    const int words = (int)((A.N + 31) >> 5);
+    if (MODE != MAP_DUPS)
+        for (int i = threadIdx.x; i < words; i += blockDim.x) map[i] = 0;
+    if (threadIdx.x == 0) s_cnt = 0;
+    unsigned long long dups = 0;
+    for (long long x = blockIdx.x; x < A.N; x += gridDim.x) {
+        const long long s = __ldg(A.indptr + x), e = __ldg(A.indptr + x + 1);
+        if (MODE != MAP_DUPS) __syncthreads();   // the map is clear
+        for (long long i = s + warp; i < e; i += 8) {
+            if (!A.indexed[i]) continue;
+            const uint32_t f = __ldg(A.indices + i);
+            if (f >= A.dim) continue;
+            const uint32_t l1 = __ldg(fstart + f + 1);
+            for (uint32_t l = __ldg(fstart + f) + lane; l < l1; l += 32) {
+                const uint32_t y = __ldg(post + l);
+                if (y > x) {
+                    if (MODE != MAP_DUPS) atomicOr(map + (y >> 5), 1u << (y & 31));
+                    ++dups;
+                }
+            }
+        }
+        if (MODE == MAP_DUPS) continue;
+        __syncthreads();
+        const int w0 = (int)((x + 1) >> 5);
+        if (MODE == MAP_COUNT) {
+            unsigned c = 0;
+            for (int i = w0 + threadIdx.x; i < words; i += blockDim.x) {
+                c += __popc(map[i]);
+                map[i] = 0;
+            }
+            c = __reduce_add_sync(kFull, c);
+            if (lane == 0 && c) atomicAdd(&s_cnt, c);
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                cnt[x] = s_cnt;
+                s_cnt = 0;
+            }
+        } else {
+            long long base = (long long)cnt[x];
+            const long long end = (long long)cnt[x + 1];
+            for (int i0 = w0; i0 < words && base < end; i0 += blockDim.x) {
+                const int i = i0 + threadIdx.x;
+                uint32_t m = 0;
+                if (i < words) {
+                    m = map[i];
+                    map[i] = 0;
+                }
+                unsigned total;
+                long long o = base + blsh_scan::block_exclusive<unsigned>((unsigned)__popc(m), &total);
+                base += total;
+                for (; m; m &= m - 1, ++o)
+                    if (o < cap) reinterpret_cast<uint2 *>(pairs)[o] = make_uint2((uint32_t)x, 32u * i + __ffs(m) - 1u);
+            }
+        }
+    }
+    if (MODE != MAP_WRITE) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) dups += __shfl_xor_sync(kFull, dups, o);
+        if (lane == 0 && dups) atomicAdd(dup_total, dups);
+    }
+}
+
 // n_pairs = the number of distinct keys; truncation and an undersized key
 // buffer are reported on the device.
-__global__ void ap_finish_kernel(const uint32_t *mark_total, const unsigned long long *dup_total, long long dup_cap,
+template <typename T>
+__global__ void ap_finish_kernel(const T *mark_total, const unsigned long long *dup_total, long long dup_cap,
                                  long long cap, int64_t *n_pairs, int64_t *n_dups, blsh_dev_scratch *scratch) {
     const long long dups = (long long)*dup_total;
     if (n_dups) *n_dups = dups;
@@ -452,6 +572,51 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
     blsh_time_start(ctx, s);
     ap_prefix_cta_kernel<<<(unsigned)sms * 4, kCtaThreads, 0, s>>>(A);
     BLSH_LAUNCHED(ctx, "ap_prefix_cta_kernel");
+    // bit maps where they cost less than sorting the keys (see the top of the
+    // file), and for a count-only call, which then forms no map
+    const bool count_only = cap == 0 || max_dups == 0;
+    if (N <= kMapRows && (count_only || N * N <= 4096 * max_dups)) {
+        uint32_t *fstart = (uint32_t *)(ws + L.fcnt), *cursor = fstart + dim + 1;   // in the (dim + 1) * 8 bytes
+        uint32_t *post = (uint32_t *)(ws + L.ik0);
+        BLSH_CUDA(ctx, cudaMemsetAsync(cursor, 0, dim * 4, s));
+        BLSH_CUDA(ctx, cudaMemsetAsync(dup_total, 0, 8, s));
+        blsh_time_start(ctx, s);
+        BLSH_CUDA(ctx, blsh_scan::exclusive_scan<uint32_t>(A.df, fstart, dim, (uint32_t *)partial64, fstart + dim, s));
+        ctx->launches.fetch_add(3, std::memory_order_relaxed);
+        blsh_time_stop(ctx, "exclusive scan (3 launches)");
+        blsh_time_start(ctx, s);
+        ap_post_kernel<<<grid_for(N, 8), 256, 0, s>>>(A, fstart, cursor, post);
+        BLSH_LAUNCHED(ctx, "ap_post_kernel");
+        const unsigned grid = (unsigned)(N < (long long)sms * 8 ? N : (long long)sms * 8);
+        if (count_only) {
+            blsh_time_start(ctx, s);
+            ap_map_kernel<MAP_DUPS><<<grid, 256, 0, s>>>(A, fstart, post, nullptr, dup_total, 0, nullptr, 0);
+            BLSH_LAUNCHED(ctx, "ap_map_kernel (keys)");
+            ap_count_only_kernel<<<1, 1, 0, s>>>(dup_total, n_pairs, n_dups);
+            BLSH_LAUNCHED(ctx, "ap_count_only_kernel");
+            return BLSH_OK;
+        }
+        const size_t smem = (size_t)((N + 31) / 32) * 4;
+        if (smem > 48 * 1024) {
+            BLSH_CUDA(ctx, cudaFuncSetAttribute(ap_map_kernel<MAP_COUNT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)(kMapRows / 8)));
+            BLSH_CUDA(ctx, cudaFuncSetAttribute(ap_map_kernel<MAP_WRITE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)(kMapRows / 8)));
+        }
+        blsh_time_start(ctx, s);
+        ap_map_kernel<MAP_COUNT><<<grid, 256, smem, s>>>(A, fstart, post, ycnt, dup_total, max_dups, nullptr, 0);
+        BLSH_LAUNCHED(ctx, "ap_map_kernel (count pass)");
+        blsh_time_start(ctx, s);
+        BLSH_CUDA(ctx, blsh_scan::exclusive_scan<unsigned long long>(ycnt, ycnt, N, partial64, ycnt + N, s));
+        ctx->launches.fetch_add(3, std::memory_order_relaxed);
+        blsh_time_stop(ctx, "exclusive scan (3 launches)");
+        blsh_time_start(ctx, s);
+        ap_map_kernel<MAP_WRITE><<<grid, 256, smem, s>>>(A, fstart, post, ycnt, dup_total, max_dups, pairs, cap);
+        BLSH_LAUNCHED(ctx, "ap_map_kernel (write pass)");
+        ap_finish_kernel<<<1, 1, 0, s>>>(ycnt + N, dup_total, max_dups, cap, n_pairs, n_dups, ctx->scratch);
+        BLSH_LAUNCHED(ctx, "ap_finish_kernel");
+        return BLSH_OK;
+    }
     // 3. the inverted index
     const int xbits = bits_for(N);
     const int key_bits = xbits + bits_for(dim);

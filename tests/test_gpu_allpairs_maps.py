@@ -1,0 +1,86 @@
+"""GPU parity of the prefix-filter candidates on both sides of their dispatch:
+bit maps where the keys are many for the number of rows, sorted keys where
+they are few, at map sizes around a word and a block, rows around the lengths
+where the prefix computation changes, and truncated outputs.  Pair for pair
+against the CPU oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+import synth
+
+pytestmark = pytest.mark.gpu
+dev = torch.device("cuda")
+
+
+def rows_csr(lens, dim, seed, values):
+    rng = np.random.default_rng(seed)
+    rows = [np.sort(rng.choice(dim, n, replace=False)).astype(np.uint32) for n in lens]
+    indptr = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    vals = None
+    if values:
+        v = [rng.uniform(0.1, 1.0, n) for n in lens]
+        vals = np.concatenate([x / max(np.linalg.norm(x), 1e-9) for x in v]).astype(np.float32)
+    return synth.CSR(indptr, np.concatenate(rows) if rows else np.zeros(0, np.uint32), vals, dim)
+
+
+def candidates(B, ctx, csr, t, kind, cap_less=0):
+    ip = torch.from_numpy(csr.indptr).to(dev)
+    ix = torch.from_numpy(csr.indices.view(np.int32)).to(dev)
+    val = None if kind == O.JACCARD else torch.from_numpy(csr.values).to(dev)
+    N, nnz = csr.n, int(csr.indptr[-1])
+    n_pairs, n_dups = (torch.zeros(1, dtype=torch.int64, device=dev) for _ in range(2))
+    ws = torch.full((B.blsh_allpairs_workspace(N, nnz, csr.dim, 0),), 0xEE, dtype=torch.uint8, device=dev)
+    B.blsh_allpairs_candidates(ctx, ip, ix, val, csr.dim, t, kind, None, n_pairs, ws, 0, n_dups)
+    assert B.blsh_status(ctx) == 0
+    dups = int(n_dups.item())
+    if dups == 0:
+        return np.zeros((0, 2), np.uint32), 0, []
+    ws = torch.full((B.blsh_allpairs_workspace(N, nnz, csr.dim, dups),), 0xEE, dtype=torch.uint8, device=dev)
+    pairs = torch.full((max(1, dups - cap_less), 2), -1, dtype=torch.int32, device=dev)
+    B.blsh_timing_begin(ctx)
+    B.blsh_allpairs_candidates(ctx, ip, ix, val, csr.dim, t, kind, pairs, n_pairs, ws, dups, n_dups)
+    names = [n for n, _ in B.blsh_timing_end(ctx)]
+    assert B.blsh_status(ctx) == (B.ETRUNC if int(n_pairs.item()) > pairs.shape[0] else 0)
+    assert int(n_dups.item()) == dups
+    return pairs.cpu().numpy().view(np.uint32), int(n_pairs.item()), names
+
+
+@pytest.mark.parametrize("n", [2, 31, 32, 33, 257, 8200])
+@pytest.mark.parametrize("kind", [O.JACCARD, O.COSINE])
+def test_maps(B, ctx, n, kind):
+    rng = np.random.default_rng(n)
+    csr = rows_csr(rng.integers(0 if n > 2 else 20, 30, n), 300, n, kind == O.COSINE)
+    want = O.allpairs_candidates(csr, 0.4, kind)
+    got, k, names = candidates(B, ctx, csr, 0.4, kind)
+    assert k == len(want) and np.array_equal(got[:k], want)
+    assert (n == 2 and not names) or "ap_map_kernel (write pass)" in names   # (two rows may share no feature)
+
+
+@pytest.mark.parametrize("kind", [O.JACCARD, O.COSINE])
+def test_sorted_keys(B, ctx, kind):
+    csr = rows_csr(np.full(3000, 6), 200000, 4, kind == O.COSINE)
+    want = O.allpairs_candidates(csr, 0.3, kind)
+    assert len(want) > 0
+    got, k, names = candidates(B, ctx, csr, 0.3, kind)
+    assert k == len(want) and np.array_equal(got[:k], want)
+    assert "digit_scatter_kernel" in names
+
+
+@pytest.mark.parametrize("kind", [O.JACCARD, O.COSINE])
+def test_row_lengths_of_the_prefix(B, ctx, kind):
+    csr = rows_csr([1, 31, 32, 33, 64, 96, 97, 127, 128, 129, 200, 4096, 4097, 0, 128, 128], 6000, 5, kind == O.COSINE)
+    for t in (0.2, 0.7):
+        want = O.allpairs_candidates(csr, t, kind)
+        got, k, _ = candidates(B, ctx, csr, t, kind)
+        assert k == len(want) and np.array_equal(got[:k], want)
+
+
+def test_truncated_map_output(B, ctx):
+    csr = rows_csr(np.full(300, 20), 200, 6, False)
+    want = O.allpairs_candidates(csr, 0.5, O.JACCARD)
+    dups = len(candidates(B, ctx, csr, 0.5, O.JACCARD)[0])
+    less = dups - len(want) + 11
+    got, k, _ = candidates(B, ctx, csr, 0.5, O.JACCARD, cap_less=less)
+    assert k == len(want) and np.array_equal(got, want[:-11])
