@@ -35,7 +35,9 @@
 // first, then written at scanned offsets).  A map costs N / 32 words per row
 // and pass (0.3 ps a word), the sort about 50 ps a key, which is where the
 // line lies.  20,000 tf-idf rows (2.4e7 keys, 1.7e7 pairs): 1.96 ms by sorting,
-// 0.86 ms with the maps.
+// 0.55 ms with the maps.
+#include <type_traits>
+
 #include "common.cuh"
 #include "radix.cuh"
 #include "scan.cuh"
@@ -98,12 +100,13 @@ __global__ void __launch_bounds__(256) ap_stats_kernel(ApArgs A, long long nnz) 
 
 // Rows of up to kShortRow elements (one warp per row, up to kShortRow / 32
 // elements a lane) and rows longer than kLongRow (every feature indexed); the
-// rows in between are left to ap_prefix_cta_kernel.  The bound at an element
+// rows in between are listed for ap_prefix_cta_kernel (at most nnz / 129 of
+// them).  The bound at an element
 // is the sum of the weights that precede it in the global order and its own:
 // n^2 comparisons, which a warp does faster than a CTA sorts while n <= 128
 // (20,000 rows, mean 57: 208 us with a CTA for every row above 32 elements,
-// 52 and 98 us with this).
-__global__ void __launch_bounds__(256) ap_prefix_warp_kernel(ApArgs A) {
+// 47 and 56 us with this).
+__global__ void __launch_bounds__(256) ap_prefix_warp_kernel(ApArgs A, uint32_t *mid, unsigned *n_mid) {
     __shared__ ulonglong2 s_kw[8][kShortRow];   // order key, weight
     constexpr int EPL = kShortRow / 32;
     const int lane = threadIdx.x & 31;
@@ -115,7 +118,11 @@ __global__ void __launch_bounds__(256) ap_prefix_warp_kernel(ApArgs A) {
             for (long long i = lane; i < n; i += 32) A.indexed[s + i] = 1;
             continue;
         }
-        if (n == 0 || n > kShortRow) continue;
+        if (n > kShortRow) {
+            if (lane == 0) mid[atomicAdd(n_mid, 1u)] = (uint32_t)row;   // for ap_prefix_cta_kernel
+            continue;
+        }
+        if (n == 0) continue;
         unsigned long long key[EPL];
         long long b[EPL];
         __syncwarp();                              // the previous row has been read
@@ -135,12 +142,19 @@ __global__ void __launch_bounds__(256) ap_prefix_warp_kernel(ApArgs A) {
             }
         }
         __syncwarp();
-        for (int j = 0; j < (int)n; ++j) {
-            const ulonglong2 v = kw[j];
+        auto sums = [&](auto used) {               // elements per lane that the row fills
+            constexpr int U = decltype(used)::value;
+#pragma unroll 4
+            for (int j = 0; j < (int)n; ++j) {
+                const ulonglong2 v = kw[j];
 #pragma unroll
-            for (int u = 0; u < EPL; ++u)
-                if (v.x <= key[u]) b[u] += (long long)v.y;
-        }
+                for (int u = 0; u < U; ++u)
+                    if (v.x <= key[u]) b[u] += (long long)v.y;
+            }
+        };
+        if (n <= 32) sums(std::integral_constant<int, 1>{});
+        else if (n <= 64) sums(std::integral_constant<int, 2>{});
+        else sums(std::integral_constant<int, EPL>{});
         const long long thr = ap_threshold(A, n);
 #pragma unroll
         for (int u = 0; u < EPL; ++u)
@@ -151,13 +165,15 @@ __global__ void __launch_bounds__(256) ap_prefix_warp_kernel(ApArgs A) {
 // Rows of kShortRow+1 .. kLongRow elements, one CTA per row: (key, position)
 // sorted in shared memory (bitonic), the weights scanned in that order.
 constexpr int kCtaThreads = 256;
-__global__ void __launch_bounds__(kCtaThreads) ap_prefix_cta_kernel(ApArgs A) {
+__global__ void __launch_bounds__(kCtaThreads) ap_prefix_cta_kernel(ApArgs A, const uint32_t *mid,
+                                                                     const unsigned *n_mid) {
     __shared__ unsigned long long s_key[kLongRow];
     __shared__ uint16_t s_pos[kLongRow];
     __shared__ long long s_part[kCtaThreads / 32];
-    for (long long row = blockIdx.x; row < A.N; row += gridDim.x) {
+    const unsigned rows = *n_mid;
+    for (unsigned q = blockIdx.x; q < rows; q += gridDim.x) {
+        const long long row = mid[q];
         const long long s = __ldg(A.indptr + row), n = __ldg(A.indptr + row + 1) - s;
-        if (n <= kShortRow || n > kLongRow) continue;
         int m = 1;
         while (m < n) m <<= 1;
         __syncthreads();
@@ -357,7 +373,8 @@ __global__ void __launch_bounds__(256) ap_post_kernel(ApArgs A, const uint32_t *
     }
 }
 
-// One CTA per row x (grid-stride).  MAP_COUNT: cnt[x] = the number of distinct
+// One CTA per row x, rows from a counter (the work of a row varies a hundredfold
+// with its features' frequencies).  MAP_COUNT: cnt[x] = the number of distinct
 // y > x in the lists of x's indexed features.  MAP_WRITE: the pairs (x, y), y
 // increasing, from offset cnt[x] (after the scan).  Both MAP_COUNT and
 // MAP_DUPS (which forms no map) add the number of (feature, y) met to
@@ -366,9 +383,10 @@ enum { MAP_DUPS, MAP_COUNT, MAP_WRITE };
 template <int MODE>
 __global__ void __launch_bounds__(256) ap_map_kernel(ApArgs A, const uint32_t *fstart, const uint32_t *post,
                                                      unsigned long long *cnt, unsigned long long *dup_total,
-                                                     long long max_dups, uint32_t *pairs, long long cap) {
+                                                     long long max_dups, uint32_t *pairs, long long cap,
+                                                     unsigned *next_row) {
     extern __shared__ uint32_t map[];   // [(N + 31) / 32], zero between rows
-    __shared__ unsigned s_cnt;
+    __shared__ unsigned s_cnt, s_row[2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (MODE == MAP_WRITE && (long long)*dup_total > max_dups) return;   // no pairs: the buffer was too small
     const int words = (int)((A.N + 31) >> 5);
@@ -376,19 +394,37 @@ __global__ void __launch_bounds__(256) ap_map_kernel(ApArgs A, const uint32_t *f
         for (int i = threadIdx.x; i < words; i += blockDim.x) map[i] = 0;
     if (threadIdx.x == 0) s_cnt = 0;
     unsigned long long dups = 0;
-    for (long long x = blockIdx.x; x < A.N; x += gridDim.x) {
+    for (int turn = 0;; turn ^= 1) {
+        if (threadIdx.x == 0) s_row[turn] = atomicAdd(next_row, 1u);
+        __syncthreads();                         // the row is there, the map is clear
+        const uint32_t x = s_row[turn];          // N < 2^31
+        if (x >= A.N) break;
         const long long s = __ldg(A.indptr + x), e = __ldg(A.indptr + x + 1);
-        if (MODE != MAP_DUPS) __syncthreads();   // the map is clear
-        for (long long i = s + warp; i < e; i += 8) {
-            if (!A.indexed[i]) continue;
-            const uint32_t f = __ldg(A.indices + i);
-            if (f >= A.dim) continue;
-            const uint32_t l1 = __ldg(fstart + f + 1);
-            for (uint32_t l = __ldg(fstart + f) + lane; l < l1; l += 32) {
-                const uint32_t y = __ldg(post + l);
-                if (y > x) {
-                    if (MODE != MAP_DUPS) atomicOr(map + (y >> 5), 1u << (y & 31));
-                    ++dups;
+        // 32 features' list bounds at a time, one per lane (so that their
+        // dependent loads overlap); each warp walks every eighth list, four
+        // loads in flight
+        for (long long i0 = s; i0 < e; i0 += 32) {
+            uint32_t l0 = 0, l1 = 0;
+            if (i0 + lane < e && A.indexed[i0 + lane]) {
+                const uint32_t f = __ldg(A.indices + i0 + lane);
+                if (f < A.dim) {
+                    l0 = __ldg(fstart + f);
+                    l1 = __ldg(fstart + f + 1);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t begin = __shfl_sync(kFull, l0, 8 * q + warp), end = __shfl_sync(kFull, l1, 8 * q + warp);
+                for (uint32_t l = begin + lane; l < end + lane; l += 128) {   // (warp-uniform trip count)
+                    uint32_t y[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) y[k] = l + 32 * k < end ? __ldg(post + l + 32 * k) : 0u;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (y[k] > x) {
+                            if (MODE != MAP_DUPS) atomicOr(map + (y[k] >> 5), 1u << (y[k] & 31));
+                            ++dups;
+                        }
                 }
             }
         }
@@ -422,7 +458,7 @@ __global__ void __launch_bounds__(256) ap_map_kernel(ApArgs A, const uint32_t *f
                 long long o = base + blsh_scan::block_exclusive<unsigned>((unsigned)__popc(m), &total);
                 base += total;
                 for (; m; m &= m - 1, ++o)
-                    if (o < cap) reinterpret_cast<uint2 *>(pairs)[o] = make_uint2((uint32_t)x, 32u * i + __ffs(m) - 1u);
+                    if (o < cap) reinterpret_cast<uint2 *>(pairs)[o] = make_uint2(x, 32u * i + __ffs(m) - 1u);
             }
         }
     }
@@ -562,24 +598,26 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
 
     // 1. statistics
     BLSH_CUDA(ctx, cudaMemsetAsync(A.df, 0, L.indexed - L.df, s));   // df and maxabs
+    BLSH_CUDA(ctx, cudaMemsetAsync(ws + L.grand, 0, 64, s));         // the totals and counters
     blsh_time_start(ctx, s);
     ap_stats_kernel<<<grid_for(nnz, 256), 256, 0, s>>>(A, nnz);
     BLSH_LAUNCHED(ctx, "ap_stats_kernel");
     // 2. indexed features
     blsh_time_start(ctx, s);
-    ap_prefix_warp_kernel<<<grid_for(N, 8), 256, 0, s>>>(A);
+    uint32_t *mid = (uint32_t *)(ws + L.ik1);                 // rows of 129 .. 4,096 elements
+    unsigned *n_mid = (unsigned *)(ws + L.grand + 48);
+    ap_prefix_warp_kernel<<<grid_for(N, 8), 256, 0, s>>>(A, mid, n_mid);
     BLSH_LAUNCHED(ctx, "ap_prefix_warp_kernel");
     blsh_time_start(ctx, s);
-    ap_prefix_cta_kernel<<<(unsigned)sms * 4, kCtaThreads, 0, s>>>(A);
+    ap_prefix_cta_kernel<<<(unsigned)sms * 4, kCtaThreads, 0, s>>>(A, mid, n_mid);
     BLSH_LAUNCHED(ctx, "ap_prefix_cta_kernel");
     // bit maps where they cost less than sorting the keys (see the top of the
     // file), and for a count-only call, which then forms no map
     const bool count_only = cap == 0 || max_dups == 0;
-    if (N <= kMapRows && (count_only || N * N <= 4096 * max_dups)) {
+    if (N <= kMapRows && nnz < (1ll << 31) && (count_only || N * N <= 4096 * max_dups)) {
         uint32_t *fstart = (uint32_t *)(ws + L.fcnt), *cursor = fstart + dim + 1;   // in the (dim + 1) * 8 bytes
         uint32_t *post = (uint32_t *)(ws + L.ik0);
         BLSH_CUDA(ctx, cudaMemsetAsync(cursor, 0, dim * 4, s));
-        BLSH_CUDA(ctx, cudaMemsetAsync(dup_total, 0, 8, s));
         blsh_time_start(ctx, s);
         BLSH_CUDA(ctx, blsh_scan::exclusive_scan<uint32_t>(A.df, fstart, dim, (uint32_t *)partial64, fstart + dim, s));
         ctx->launches.fetch_add(3, std::memory_order_relaxed);
@@ -590,7 +628,8 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
         const unsigned grid = (unsigned)(N < (long long)sms * 8 ? N : (long long)sms * 8);
         if (count_only) {
             blsh_time_start(ctx, s);
-            ap_map_kernel<MAP_DUPS><<<grid, 256, 0, s>>>(A, fstart, post, nullptr, dup_total, 0, nullptr, 0);
+            ap_map_kernel<MAP_DUPS><<<grid, 256, 0, s>>>(A, fstart, post, nullptr, dup_total, 0, nullptr, 0,
+                                                                n_mid + 1);
             BLSH_LAUNCHED(ctx, "ap_map_kernel (keys)");
             ap_count_only_kernel<<<1, 1, 0, s>>>(dup_total, n_pairs, n_dups);
             BLSH_LAUNCHED(ctx, "ap_count_only_kernel");
@@ -604,14 +643,16 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
                                                 (int)(kMapRows / 8)));
         }
         blsh_time_start(ctx, s);
-        ap_map_kernel<MAP_COUNT><<<grid, 256, smem, s>>>(A, fstart, post, ycnt, dup_total, max_dups, nullptr, 0);
+        ap_map_kernel<MAP_COUNT><<<grid, 256, smem, s>>>(A, fstart, post, ycnt, dup_total, max_dups, nullptr, 0,
+                                                             n_mid + 1);
         BLSH_LAUNCHED(ctx, "ap_map_kernel (count pass)");
         blsh_time_start(ctx, s);
         BLSH_CUDA(ctx, blsh_scan::exclusive_scan<unsigned long long>(ycnt, ycnt, N, partial64, ycnt + N, s));
         ctx->launches.fetch_add(3, std::memory_order_relaxed);
         blsh_time_stop(ctx, "exclusive scan (3 launches)");
         blsh_time_start(ctx, s);
-        ap_map_kernel<MAP_WRITE><<<grid, 256, smem, s>>>(A, fstart, post, ycnt, dup_total, max_dups, pairs, cap);
+        ap_map_kernel<MAP_WRITE><<<grid, 256, smem, s>>>(A, fstart, post, ycnt, dup_total, max_dups, pairs, cap,
+                                                             n_mid + 2);
         BLSH_LAUNCHED(ctx, "ap_map_kernel (write pass)");
         ap_finish_kernel<<<1, 1, 0, s>>>(ycnt + N, dup_total, max_dups, cap, n_pairs, n_dups, ctx->scratch);
         BLSH_LAUNCHED(ctx, "ap_finish_kernel");
