@@ -618,10 +618,7 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
         uint32_t *fstart = (uint32_t *)(ws + L.fcnt), *cursor = fstart + dim + 1;   // in the (dim + 1) * 8 bytes
         uint32_t *post = (uint32_t *)(ws + L.ik0);
         BLSH_CUDA(ctx, cudaMemsetAsync(cursor, 0, dim * 4, s));
-        blsh_time_start(ctx, s);
-        BLSH_CUDA(ctx, blsh_scan::exclusive_scan<uint32_t>(A.df, fstart, dim, (uint32_t *)partial64, fstart + dim, s));
-        ctx->launches.fetch_add(3, std::memory_order_relaxed);
-        blsh_time_stop(ctx, "exclusive scan (3 launches)");
+        if (const int rc = blsh_scan::run<uint32_t>(ctx, A.df, fstart, dim, (uint32_t *)partial64, fstart + dim, s)) return rc;
         blsh_time_start(ctx, s);
         ap_post_kernel<<<grid_for(N, 8), 256, 0, s>>>(A, fstart, cursor, post);
         BLSH_LAUNCHED(ctx, "ap_post_kernel");
@@ -646,10 +643,7 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
         ap_map_kernel<MAP_COUNT><<<grid, 256, smem, s>>>(A, fstart, post, ycnt, dup_total, max_dups, nullptr, 0,
                                                              n_mid + 1);
         BLSH_LAUNCHED(ctx, "ap_map_kernel (count pass)");
-        blsh_time_start(ctx, s);
-        BLSH_CUDA(ctx, blsh_scan::exclusive_scan<unsigned long long>(ycnt, ycnt, N, partial64, ycnt + N, s));
-        ctx->launches.fetch_add(3, std::memory_order_relaxed);
-        blsh_time_stop(ctx, "exclusive scan (3 launches)");
+        if (const int rc = blsh_scan::run<unsigned long long>(ctx, ycnt, ycnt, N, partial64, ycnt + N, s)) return rc;
         blsh_time_start(ctx, s);
         ap_map_kernel<MAP_WRITE><<<grid, 256, smem, s>>>(A, fstart, post, ycnt, dup_total, max_dups, pairs, cap,
                                                              n_mid + 2);
@@ -675,20 +669,14 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
         if (rc) return rc;
     }
     // feature list starts: exclusive scan of the per-feature counts (dim + 1 entries)
-    blsh_time_start(ctx, s);
-    BLSH_CUDA(ctx, blsh_scan::exclusive_scan<unsigned long long>(fcnt, fcnt, dim + 1, partial64, grand64, s));
-    ctx->launches.fetch_add(3, std::memory_order_relaxed);
-    blsh_time_stop(ctx, "exclusive scan (3 launches)");
+    if (const int rc = blsh_scan::run<unsigned long long>(ctx, fcnt, fcnt, dim + 1, partial64, grand64, s)) return rc;
     const unsigned long long xmask = (1ull << xbits) - 1ull;
     // 4. candidate keys: count, scan, write
     blsh_time_start(ctx, s);
     ap_emit_kernel<false><<<grid_for(N, 8), 256, 0, s>>>(A, ik[cur], fcnt, xmask, ycnt, nullptr, 0);
     BLSH_LAUNCHED(ctx, "ap_emit_kernel (count pass)");
     BLSH_CUDA(ctx, cudaMemsetAsync(ycnt + N, 0, 8, s));
-    blsh_time_start(ctx, s);
-    BLSH_CUDA(ctx, blsh_scan::exclusive_scan<unsigned long long>(ycnt, ycnt, N + 1, partial64, dup_total, s));
-    ctx->launches.fetch_add(3, std::memory_order_relaxed);
-    blsh_time_stop(ctx, "exclusive scan (3 launches)");
+    if (const int rc = blsh_scan::run<unsigned long long>(ctx, ycnt, ycnt, N + 1, partial64, dup_total, s)) return rc;
     if (cap == 0 || max_dups == 0) {
         ap_count_only_kernel<<<1, 1, 0, s>>>(dup_total, n_pairs, n_dups);
         BLSH_LAUNCHED(ctx, "ap_count_only_kernel");
@@ -717,10 +705,7 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
     blsh_time_start(ctx, s);
     ap_mark_kernel<<<grid_for(max_dups, 256), 256, 0, s>>>(ck[kc], max_dups, mark);
     BLSH_LAUNCHED(ctx, "ap_mark_kernel");
-    blsh_time_start(ctx, s);
-    BLSH_CUDA(ctx, blsh_scan::exclusive_scan<uint32_t>(mark, pos, max_dups, (uint32_t *)partial64, grand32, s));
-    ctx->launches.fetch_add(3, std::memory_order_relaxed);
-    blsh_time_stop(ctx, "exclusive scan (3 launches)");
+    if (const int rc = blsh_scan::run<uint32_t>(ctx, mark, pos, max_dups, (uint32_t *)partial64, grand32, s)) return rc;
     blsh_time_start(ctx, s);
     ap_write_kernel<<<grid_for(max_dups, 256), 256, 0, s>>>(ck[kc], mark, pos, max_dups, pairs, cap);
     BLSH_LAUNCHED(ctx, "ap_write_kernel");

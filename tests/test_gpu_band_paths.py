@@ -1,0 +1,104 @@
+"""GPU parity of LSH banding at the edges of its forms: object counts around
+the one-CTA-per-band sort and the tiles of the large one, key rows that are
+the signature rows themselves and packed ones (1-, 2- and 4-byte lanes, up to
+128 bytes), buckets shorter and longer than the staged rows and batches, with
+the full keep record, a partial one and none.  The candidate set is the
+oracle's; cosine pairs come in order of (band, key, x, y)."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+
+pytestmark = pytest.mark.gpu
+dev = torch.device("cuda")
+
+
+def candidates(B, ctx, sig, kind, rows, bands, rec_bytes):
+    N = sig.shape[0]
+    t = torch.from_numpy(np.ascontiguousarray(sig).view(np.int32)).to(dev)
+    full = B.blsh_lsh_candidates_workspace(N, kind, rows, bands)
+    base = full - 64 * N * bands
+    ws = torch.full((base + min(rec_bytes, 64 * N * bands),), 0xA5, dtype=torch.uint8, device=dev)
+    n = torch.zeros(1, dtype=torch.int64, device=dev)
+    B.blsh_lsh_candidates(ctx, t, kind, rows, bands, None, n, ws)
+    assert B.blsh_status(ctx) == (B.ETRUNC if int(n.item()) else 0)
+    pairs = torch.full((max(1, int(n.item())), 2), -1, dtype=torch.int32, device=dev)
+    B.blsh_lsh_candidates(ctx, t, kind, rows, bands, pairs, n, ws)
+    assert B.blsh_status(ctx) == 0
+    return pairs[: int(n.item())].cpu().numpy().view(np.uint32)
+
+
+def packed(p):
+    return (p[:, 0].astype(np.uint64) << np.uint64(32)) | p[:, 1]
+
+
+def cosine_keys(sig, rows, bands):
+    bits = np.unpackbits(np.ascontiguousarray(sig).view(np.uint8), axis=1, bitorder="little")
+    w = (1 << np.arange(rows, dtype=np.uint64))
+    return np.stack([(bits[:, b * rows:(b + 1) * rows].astype(np.uint64) * w).sum(1) for b in range(bands)], 1)
+
+
+def near_duplicates(rng, N, words, flip):
+    """Rows drawn around N / 20 centres, every bit flipped with probability flip."""
+    centres = rng.integers(0, 1 << 32, (max(1, N // 20), words), dtype=np.uint64).astype(np.uint32)
+    noise = np.packbits(rng.random((N, 32 * words)) < flip, axis=1).view(np.uint32)
+    return centres[rng.integers(0, len(centres), N)] ^ noise
+
+
+@pytest.mark.parametrize("N", [2, 31, 33, 300, 4096, 4097, 6001])
+@pytest.mark.parametrize("rows,bands", [(8, 5), (8, 64), (16, 3), (16, 62), (32, 2), (5, 13), (12, 33), (20, 17), (6, 1)])
+def test_cosine(B, ctx, N, rows, bands):
+    rng = np.random.default_rng(N + rows)
+    sig = near_duplicates(rng, N, 32, 0.02)
+    want = O.lsh_candidates(sig, O.COSINE, rows, bands)
+    got = candidates(B, ctx, sig, 1, rows, bands, 1 << 40)
+    assert len(got) == len(want) and np.array_equal(np.sort(packed(got)), np.sort(packed(want)))
+    if len(got):
+        key = cosine_keys(sig, rows, bands)
+        same = key[got[:, 0]] == key[got[:, 1]]
+        band = same.argmax(1)
+        k = key[got[:, 0], band]
+        assert same.any(1).all() and (got[:, 0] < got[:, 1]).all()
+        order = np.lexsort((got[:, 1], got[:, 0], k, band))
+        assert np.array_equal(order, np.arange(len(got)))
+    for rec in (0, 8 * N):
+        assert np.array_equal(candidates(B, ctx, sig, 1, rows, bands, rec), got)
+
+
+@pytest.mark.parametrize("N", [2, 40, 4096, 4097, 6001])
+@pytest.mark.parametrize("rows,bands", [(1, 1), (1, 3), (2, 16), (3, 32), (2, 40)])
+def test_jaccard(B, ctx, N, rows, bands):
+    rng = np.random.default_rng(N + bands)
+    # values with a power law: a few long buckets and many short ones
+    sig = np.minimum(rng.zipf(1.3, (N, 96)), N).astype(np.uint32)
+    if rows == 1:
+        sig = (sig + rng.integers(0, max(1, N // 50), (N, 96))).astype(np.uint32)
+    want = O.lsh_candidates(sig, O.JACCARD, rows, bands)
+    got = candidates(B, ctx, sig, 0, rows, bands, 1 << 40)
+    assert len(got) == len(want) and np.array_equal(np.sort(packed(got)), np.sort(packed(want)))
+    for rec in (0, 8 * N):
+        assert np.array_equal(candidates(B, ctx, sig, 0, rows, bands, rec), got)
+
+
+@pytest.mark.parametrize("kind,rows,bands", [(1, 8, 5), (1, 16, 62), (1, 12, 20), (0, 2, 4), (0, 2, 32)])
+def test_long_buckets(B, ctx, kind, rows, bands):
+    """Buckets of thousands of objects, cut into segments: 4,500 of 5,200
+    objects agree on the last band, a third of those on band 1 as well."""
+    rng = np.random.default_rng(rows + bands)
+    N = 5200
+    sig = rng.integers(0, 1 << 32, (N, 64), dtype=np.uint64).astype(np.uint32)
+    chosen = rng.permutation(N)[:4500]
+    for band, who in ((bands - 1, chosen), (1, chosen[::3])):
+        if kind == 0:
+            sig[np.ix_(who, np.arange(band * rows, (band + 1) * rows))] = 7
+        else:
+            bits = np.unpackbits(sig.view(np.uint8), axis=1, bitorder="little")
+            bits[np.ix_(who, np.arange(band * rows, (band + 1) * rows))] = 1
+            sig = np.packbits(bits, axis=1, bitorder="little").view(np.uint32)
+    want = O.lsh_candidates(sig, O.COSINE if kind else O.JACCARD, rows, bands)
+    assert len(want) > 10_000_000
+    got = candidates(B, ctx, sig, kind, rows, bands, 1 << 40)
+    assert len(got) == len(want) and np.array_equal(np.sort(packed(got)), np.sort(packed(want)))
+    for rec in (0, 64 * N):   # no record: every chunk by its own warp, in the same order
+        assert np.array_equal(candidates(B, ctx, sig, kind, rows, bands, rec), got)
