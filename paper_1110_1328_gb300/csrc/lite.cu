@@ -37,6 +37,7 @@ struct LiteArgs {
     double *sim;
     blsh_dev_scratch *scratch;
     int vec;                  // status is 16-byte aligned
+    long long N;
     const long long *norm2;   // cosine: each row's sum of fixed_term(v, v), or NULL (formed per pair)
 };
 
@@ -92,7 +93,7 @@ __device__ __forceinline__ long long lower_bound(const uint32_t *L, long long n,
     return lo;
 }
 
-constexpr int kLiteStage = 512;   // longer-row elements a warp stages in shared memory
+constexpr int kLiteStage = 512;   // half the elements a warp stages in shared memory
 
 // The sums of one survivor's exact similarity (the whole warp): rows
 // x = [ax, ax+na) and y = [ay, ay+nb) of the CSR; D_out = the intersection
@@ -100,12 +101,12 @@ constexpr int kLiteStage = 512;   // longer-row elements a warp stages in shared
 // squared norms.  The shorter row's elements are spread over the lanes and each
 // is looked up in the longer row by binary search: with the longer row held
 // one element per lane (at most 32 elements: the search steps are shuffles),
-// staged in the warp's shared memory (at most kLiteStage), or read from
-// global memory.  No search touches global memory unless the longer row has
-// more than kLiteStage elements.
+// staged in the warp's shared memory, a tile at a time.  (Searching rows of
+// more than 512 elements in global memory, two lookups in flight, took 62 us
+// for 3,600 survivors whose longest rows have some 900 elements; 42 now.)
 template <bool COSINE>
 __device__ __forceinline__ void lite_exact_one(const LiteArgs &A, long long ax, long long na, long long ay,
-                                               long long nb, bool have_norms, uint32_t *w_idx, float *w_val,
+                                               long long nb, bool have_norms, uint32_t *w_idx,
                                                long long &D_out, long long &Nx_out, long long &Ny_out) {
     const int lane = threadIdx.x & 31;
     // the shorter row S, the longer row L (the sums below do not depend on
@@ -150,39 +151,58 @@ __device__ __forceinline__ void lite_exact_one(const LiteArgs &A, long long ax, 
             }
         }
     } else {
-        const uint32_t *Lidx = A.indices + l0;
-        const float *Lval = COSINE ? A.values + l0 : nullptr;
-        __syncwarp();                                      // the previous survivor is done with the stage
-        if (nl <= kLiteStage) {
-            for (long long i = lane; i < nl; i += 32) {
-                w_idx[i] = __ldg(A.indices + l0 + i);
-                if (COSINE) {
-                    const float v = __ldg(A.values + l0 + i);
-                    w_val[i] = v;
-                    if (!have_norms) Nl += fixed_term(v, v);
-                }
-            }
-            __syncwarp();
-            Lidx = w_idx;
-            if (COSINE) Lval = w_val;
-        } else if (COSINE && !have_norms) {
+        // the longer row's indices through the warp's stage, kTile at a time;
+        // the shorter row's elements up to the tile's last are looked up in it
+        // four per lane (their loads, searches and values overlap: a warp that
+        // forms one survivor has nothing else to wait behind)
+        constexpr int kTile = 2 * kLiteStage;
+        long long sp = 0;                                  // the shorter row's elements done
+        for (long long tb = 0; tb < nl && (sp < ns || (COSINE && !have_norms)); tb += kTile) {
+            const int tn = (int)(nl - tb < kTile ? nl - tb : kTile);
+            __syncwarp();                                  // the previous tile is done with the stage
 #pragma unroll 4
-            for (long long i = lane; i < nl; i += 32) {
-                const float v = __ldg(A.values + l0 + i);
-                Nl += fixed_term(v, v);
-            }
-        }
-#pragma unroll 2
-        for (long long i = lane; i < ns; i += 32) {
-            const uint32_t v = __ldg(A.indices + s0 + i);
-            const long long pos = lower_bound(Lidx, nl, v);
-            const bool hit = pos < nl && Lidx[pos] == v;
-            if (!COSINE) {
-                inter += hit;
-            } else {
-                const float sv = __ldg(A.values + s0 + i);
-                if (hit) D += fixed_term(sv, Lval[pos]);
-                if (!have_norms) Ns += fixed_term(sv, sv);
+            for (int i = lane; i < tn; i += 32) w_idx[i] = __ldg(A.indices + l0 + tb + i);
+            if (COSINE && !have_norms)
+#pragma unroll 4
+                for (int i = lane; i < tn; i += 32) {
+                    const float v = __ldg(A.values + l0 + tb + i);
+                    Nl += fixed_term(v, v);
+                }
+            __syncwarp();
+            const uint32_t last = w_idx[tn - 1];
+            const bool final_tile = tb + tn >= nl;
+            for (bool more = sp < ns; more;) {
+                uint32_t v[4];
+                bool in[4];
+                int pos[4];
+                unsigned taken = 0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const long long i = sp + 32 * u + lane;
+                    v[u] = i < ns ? __ldg(A.indices + s0 + i) : 0u;
+                    in[u] = i < ns && (final_tile || v[u] <= last);
+                    pos[u] = 0;
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) taken += __popc(__ballot_sync(kFull, in[u]));
+                for (int step = kTile / 2; step > 0; step >>= 1)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (pos[u] + step <= tn && w_idx[pos[u] + step - 1] < v[u]) pos[u] += step;
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const bool hit = in[u] && pos[u] < tn && w_idx[pos[u]] == v[u];
+                    if (!COSINE) {
+                        inter += hit;
+                    } else {
+                        const long long i = s0 + sp + 32 * u + lane;
+                        const float sv = in[u] && (hit || !have_norms) ? __ldg(A.values + i) : 0.0f;
+                        if (hit) D += fixed_term(sv, __ldg(A.values + l0 + tb + pos[u]));
+                        if (!have_norms && in[u]) Ns += fixed_term(sv, sv);
+                    }
+                }
+                sp += taken;
+                more = taken == 128 && sp < ns;            // the rest lies past this tile, or none is left
             }
         }
     }
@@ -302,15 +322,242 @@ __device__ __forceinline__ double lite_similarity(long long D, long long Nx, lon
     return __ddiv_rn(__ll2double_rn(D), __dsqrt_rn(__dmul_rn(__ll2double_rn(Nx), __ll2double_rn(Ny))));
 }
 
+// The sums of a batch of survivors (this lane's, if `mine`: rows [ax, ex) and
+// [ay, ey), each below 2^26 elements), the elements of their shorter rows dealt over the
+// lanes: element t of the batch goes to lane t mod 32, whatever survivor it
+// belongs to, and is looked up in that survivor's longer row by binary search
+// -- in shared memory where that row has at most kFlatStage elements and the
+// batch's rows fit the stage (copied asynchronously, all at once), in global
+// memory otherwise.  Hits are listed, and 32 at a time read their values and
+// add their terms to the survivors' sums in shared memory, in three limbs of
+// 24, 24 and 16 bits (32-bit adds are native there), carried into a 64-bit sum
+// before they can overflow.
+// A warp per survivor spent 430 issue slots on each (broadcasts of the bounds,
+// a search of six shuffle rounds and a 64-bit reduction over 32 lanes, for 8.9
+// elements on average).  4.6e7 survivors of 5e6 documents: 16.7 ms, 10.0
+// here.
+constexpr int kFlatStage = 127;    // (seven halvings)
+constexpr int kFlatMin = 8;        // survivors in a batch from which it is formed this way
+constexpr int kFlatCarry = 8;      // hit rounds (of 32) between carries: 256 times 2^24 - 1 fits a limb
+// a warp's limbs [3][32], rows [32] uint4, lengths [32] uint2, hits [64] uint2, in words
+constexpr int kFlatWords = 96 + 128 + 64 + 128;
+
+__device__ __forceinline__ void copy16_async(uint32_t *dst, const uint32_t *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+template <bool COSINE>
+__device__ __forceinline__ long long lite_flat(const LiteArgs &A, bool mine, long long ax, long long ex, long long ay,
+                                               long long ey, long long nnz, uint32_t *stage, uint32_t *flat) {
+    const int lane = threadIdx.x & 31;
+    uint32_t *limbs = flat;
+    uint4 *rows = reinterpret_cast<uint4 *>(flat + 96);            // [32]: first elements of S and L
+    uint2 *lens = reinterpret_cast<uint2 *>(flat + 96 + 128);      // [32]: |L|, its place in the stage (~0: none)
+    uint2 *hits = lens + 32;                                       // [64]: owner | element of S << 5, element of L
+    long long s0 = ax, l0 = ay;
+    unsigned ns = mine ? (unsigned)(ex - ax) : 0u, nl = mine ? (unsigned)(ey - ay) : 0u;
+    if (nl < ns) {
+        s0 = ay;
+        l0 = ax;
+        const unsigned t = ns;
+        ns = nl;
+        nl = t;
+    }
+    // staged rows: those of up to kFlatStage elements, while they fit (copied
+    // in whole 16-byte blocks, which must lie inside the index array); their
+    // survivors come first, so that few rounds mix the two kinds of lookup
+    const unsigned phase = ((unsigned)((uintptr_t)(A.indices + l0) >> 2)) & 3u;   // words into its block
+    const unsigned blocks = (phase + nl + 3) >> 2;
+    const bool fits = nl != 0 && nl <= kFlatStage && l0 - phase >= 0 && l0 - phase + 4ll * blocks <= nnz;
+    const unsigned want = fits ? 4 * blocks : 0u;
+    const unsigned lt = (1u << lane) - 1u;
+    unsigned at = want;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(kFull, at, o);
+        if (lane >= o) at += v;
+    }
+    const bool staged = want != 0 && at <= 2 * kLiteStage;
+    const unsigned sm = __ballot_sync(kFull, staged);
+    const int slot = staged ? __popc(sm & lt) : __popc(sm) + __popc(~sm & lt);
+    __syncwarp();                                  // the previous batch is done with the stage and the limbs
+    limbs[slot] = ns;
+    rows[slot] = make_uint4((unsigned)s0, (unsigned)(s0 >> 32), (unsigned)l0, (unsigned)(l0 >> 32));
+    lens[slot] = make_uint2(nl, staged ? at - want + phase : ~0u);
+    __syncwarp();
+    const unsigned slot_ns = limbs[lane];
+    unsigned off = slot_ns;                        // the slot's first element in the batch
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned v = __shfl_up_sync(kFull, off, o);
+        if (lane >= o) off += v;
+    }
+    const unsigned total = __shfl_sync(kFull, off, 31);
+    off -= slot_ns;
+    limbs[lane] = limbs[32 + lane] = limbs[64 + lane] = 0;
+    __syncwarp();
+    // four rows at a time, eight lanes and 128 bytes each
+    const int n_staged = __popc(sm);
+#pragma unroll 1
+    for (int r = lane >> 3; r < n_staged; r += 4) {
+        const uint2 ln = lens[r];
+        const uint4 rw = rows[r];
+        const unsigned ph = ln.y & 3u, nb = (ph + ln.x + 3) >> 2;   // stage places start on 16 bytes, plus phase
+        const uint32_t *src = A.indices + (((long long)rw.w << 32 | rw.z) - ph);
+        uint32_t *dst = stage + (ln.y - ph);
+#pragma unroll 1
+        for (unsigned e = lane & 7; e < nb; e += 8) copy16_async(dst + 4 * e, src + 4 * e);
+    }
+    long long D = 0;
+    auto carry = [&]() {                           // the limbs into the slot's sum (lane = slot)
+        __syncwarp();
+        D += (long long)limbs[lane];
+        if (COSINE)
+            D += (long long)(((unsigned long long)limbs[32 + lane] << 24) +
+                             ((unsigned long long)(long long)(int)limbs[64 + lane] << 48));
+        limbs[lane] = limbs[32 + lane] = limbs[64 + lane] = 0;
+        __syncwarp();
+    };
+    // the terms of hits [h0, h0 + m), a lane each
+    unsigned rounds = 0;
+    auto add_hits = [&](int h0, int m) {
+        __syncwarp();
+        if (lane < m) {
+            const uint2 h = hits[h0 + lane];
+            const int o = (int)(h.x & 31u);
+            if (COSINE) {
+                const uint4 rw = rows[o];
+                const long long term = fixed_term(__ldg(A.values + ((long long)rw.y << 32 | rw.x) + (h.x >> 5)),
+                                                  __ldg(A.values + ((long long)rw.w << 32 | rw.z) + h.y));
+                atomicAdd(limbs + o, (uint32_t)term & 0xffffffu);
+                atomicAdd(limbs + 32 + o, (uint32_t)((unsigned long long)term >> 24) & 0xffffffu);
+                atomicAdd(limbs + 64 + o, (uint32_t)(int)(term >> 48));
+            } else {
+                atomicAdd(limbs + o, 1u);
+            }
+        }
+        if (++rounds % kFlatCarry == 0) carry();
+    };
+    // element t of the batch: its survivor, its place there and its value (the
+    // next round's are loaded before this round's are looked up)
+    auto element = [&](unsigned t, int &o, unsigned &e, uint32_t &v) {
+        o = 0;                                     // the last lane whose offset is <= t
+#pragma unroll
+        for (int step = 16; step > 0; step >>= 1) {
+            const unsigned oc = __shfl_sync(kFull, off, o + step);
+            if (oc <= t) o += step;
+        }
+        e = t - __shfl_sync(kFull, off, o);
+        v = 0;
+        if (t < total) {
+            const uint4 rw = rows[o];
+            v = __ldg(A.indices + ((long long)rw.y << 32 | rw.x) + e);
+        }
+    };
+    int o;
+    unsigned e;
+    uint32_t v;
+    element(lane, o, e, v);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    int n_hits = 0;
+    for (unsigned t0 = 0; t0 < total; t0 += 32) {
+        int o2 = 0;
+        unsigned e2 = 0;
+        uint32_t v2 = 0;
+        if (t0 + 32 < total) element(t0 + 32 + lane, o2, e2, v2);
+        bool hit = false;
+        unsigned lo = 0;
+        if (t0 + lane < total) {
+            const uint2 ln = lens[o];
+            // lo = the elements of L below v, by halving steps without branches
+            if (ln.y != ~0u) {
+                const uint32_t *L = stage + ln.y;
+#pragma unroll
+                for (unsigned step = (kFlatStage + 1) / 2; step > 0; step >>= 1)
+                    if (lo + step <= ln.x && L[lo + step - 1] < v) lo += step;
+                hit = lo < ln.x && L[lo] == v;
+            } else {
+                const uint4 rw = rows[o];
+                const uint32_t *L = A.indices + ((long long)rw.w << 32 | rw.z);
+                for (unsigned step = ln.x ? 1u << (31 - __clz(ln.x)) : 0u; step > 0; step >>= 1)
+                    if (lo + step <= ln.x && __ldg(L + lo + step - 1) < v) lo += step;
+                hit = lo < ln.x && __ldg(L + lo) == v;
+            }
+        }
+        const unsigned hm = __ballot_sync(kFull, hit);
+        if (COSINE && hit) {                       // the values it will read, on their way meanwhile
+            const uint4 rw = rows[o];
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(A.values + ((long long)rw.y << 32 | rw.x) + e));
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(A.values + ((long long)rw.w << 32 | rw.z) + lo));
+        }
+        if (hit) hits[n_hits + __popc(hm & ((1u << lane) - 1u))] = make_uint2((unsigned)o | e << 5, lo);
+        n_hits += __popc(hm);
+        if (n_hits >= 32) {
+            n_hits -= 32;
+            add_hits(n_hits, 32);
+        }
+        o = o2;
+        e = e2;
+        v = v2;
+    }
+    if (n_hits) add_hits(0, n_hits);
+    carry();
+    return __shfl_sync(kFull, D, slot);
+}
+
+struct LiteSums {
+    long long D, Nx, Ny;
+};
+
+// The sums of the survivors of the lanes in `todo`, segments of the warp or the
+// whole warp on each; Nx and Ny as they come in when the norms are formed.
+template <bool COSINE>
+__device__ __forceinline__ LiteSums lite_few(const LiteArgs &A, unsigned todo, long long ax, long long ex, long long ay,
+                                          long long ey, bool have_norms, LiteSums in, uint32_t *w_idx) {
+    const int lane = threadIdx.x & 31;
+    LiteSums my = in;
+    // survivors whose rows are short share the warp: four at a time when
+    // both rows have at most 8 elements, two when at most 16 (a group too
+    // small to fill the segments joins the next wider one)
+    const long long longest = ex - ax > ey - ay ? ex - ax : ey - ay;
+    unsigned s8 = __ballot_sync(kFull, longest <= 8) & todo;
+    unsigned s16 = __ballot_sync(kFull, longest <= 16) & ~s8 & todo;
+    if (__popc(s8) < 3) {
+        s16 |= s8;
+        s8 = 0u;
+    }
+    if (__popc(s16) < 2) s16 = 0u;
+    if (s8) lite_segments<COSINE, 8>(A, s8, ax, ex, ay, ey, have_norms, my.D, my.Nx, my.Ny);
+    if (s16) lite_segments<COSINE, 16>(A, s16, ax, ex, ay, ey, have_norms, my.D, my.Nx, my.Ny);
+    for (todo &= ~(s8 | s16); todo; todo &= todo - 1) {
+        const int i = __ffs(todo) - 1;
+        const long long a0 = __shfl_sync(kFull, ax, i), a1 = __shfl_sync(kFull, ex, i);
+        const long long b0 = __shfl_sync(kFull, ay, i), b1 = __shfl_sync(kFull, ey, i);
+        long long D = 0, Nx = 0, Ny = 0;
+        lite_exact_one<COSINE>(A, a0, a1 - a0, b0, b1 - b0, have_norms, w_idx, D, Nx, Ny);
+        if (lane == i) {
+            my.D = D;
+            if (!have_norms) {
+                my.Nx = Nx;
+                my.Ny = Ny;
+            }
+        }
+    }
+    return my;
+}
+
 // Up to 32 survivors, survivor my_q of lane l (-1: none): their pairs, row
 // bounds and (when formed) squared norms are loaded by all lanes at once, so
-// those dependent loads overlap across the batch; then the warp forms the
-// survivors' sums one after the other, and finally every lane turns its own
-// survivor's sums into the similarity and writes it with the verdict.
+// those dependent loads overlap across the batch; then the warp forms their
+// sums, and finally every lane turns its own survivor's sums into the
+// similarity and writes it with the verdict.
 template <bool COSINE>
 __device__ __forceinline__ void lite_batch(const LiteArgs &A, long long my_q, bool have_norms, uint32_t *w_idx,
-                                           float *w_val) {
-    long long ax = 0, ex = 0, ay = 0, ey = 0, nx = 0, ny = 0;
+                                           uint32_t *flat) {
+    long long ax = 0, ex = 0, ay = 0, ey = 0;
+    LiteSums my = {0, 0, 0};
     if (my_q >= 0) {
         const uint2 pr = __ldg(A.pairs + my_q);
         ax = __ldg(A.indptr + pr.x);
@@ -318,62 +565,33 @@ __device__ __forceinline__ void lite_batch(const LiteArgs &A, long long my_q, bo
         ay = __ldg(A.indptr + pr.y);
         ey = __ldg(A.indptr + pr.y + 1);
         if (have_norms) {
-            nx = __ldg(A.norm2 + pr.x);
-            ny = __ldg(A.norm2 + pr.y);
+            my.Nx = __ldg(A.norm2 + pr.x);
+            my.Ny = __ldg(A.norm2 + pr.y);
         }
     }
-    const int lane = threadIdx.x & 31;
-    // lane i keeps survivor i's sums
-    long long myD = 0, myNx = nx, myNy = ny;
-    // survivors whose rows are short share the warp: four at a time when
-    // both rows have at most 8 elements, two when at most 16 (a group too
-    // small to fill the segments joins the next wider one)
     unsigned todo = __ballot_sync(kFull, my_q >= 0);
-    {
-        const long long longest = ex - ax > ey - ay ? ex - ax : ey - ay;
-        unsigned s8 = __ballot_sync(kFull, my_q >= 0 && longest <= 8);
-        unsigned s16 = __ballot_sync(kFull, my_q >= 0 && longest <= 16) & ~s8;
-        if (__popc(s8) < 3) {
-            s16 |= s8;
-            s8 = 0u;
-        }
-        if (__popc(s16) < 2) s16 = 0u;
-        if (s8) lite_segments<COSINE, 8>(A, s8, ax, ex, ay, ey, have_norms, myD, myNx, myNy);
-        if (s16) lite_segments<COSINE, 16>(A, s16, ax, ex, ay, ey, have_norms, myD, myNx, myNy);
-        todo &= ~(s8 | s16);
+    if ((!COSINE || have_norms) && __popc(todo) >= kFlatMin) {
+        // rows of 2^26 elements and more are left to lite_few
+        const bool mine = my_q >= 0 && ((ex - ax) | (ey - ay)) < (1ll << 26);
+        my.D = lite_flat<COSINE>(A, mine, ax, ex, ay, ey, __ldg(A.indptr + A.N), w_idx, flat);
+        todo &= ~__ballot_sync(kFull, mine);
     }
-    for (; todo; todo &= todo - 1) {
-        const int i = __ffs(todo) - 1;
-        const long long a0 = __shfl_sync(kFull, ax, i), a1 = __shfl_sync(kFull, ex, i);
-        const long long b0 = __shfl_sync(kFull, ay, i), b1 = __shfl_sync(kFull, ey, i);
-        long long D = 0, Nx = 0, Ny = 0;
-        lite_exact_one<COSINE>(A, a0, a1 - a0, b0, b1 - b0, have_norms, w_idx, w_val, D, Nx, Ny);
-        if (lane == i) {
-            myD = D;
-            if (!have_norms) {
-                myNx = Nx;
-                myNy = Ny;
-            }
-        }
-    }
+    if (todo) my = lite_few<COSINE>(A, todo, ax, ex, ay, ey, have_norms, my, w_idx);
     if (my_q >= 0) {
-        const double s = lite_similarity<COSINE>(myD, myNx, myNy, ex - ax, ey - ay);
+        const double s = lite_similarity<COSINE>(my.D, my.Nx, my.Ny, ex - ax, ey - ay);
         A.sim[my_q] = s;
         A.status[my_q] = s > A.t ? BLSH_LITE_ACCEPT : BLSH_LITE_REJECT;
     }
 }
 
 // Each row's sum of fixed_term(v, v) (the squared norm of the exact cosine,
-// an integer: independent of the order of the terms).  One warp per group of
-// 32 consecutive rows: lane l holds the end of row l of the group, the warp
-// reads the group's nonzeros 32 at a time (four such reads in flight), finds
-// each element's row by a binary search of the lanes' row ends (shuffles),
-// sums the terms of each row's run of lanes by a segmented scan, and the
-// run's last lane adds the run's sum into the row's 64-bit sum in shared
-// memory (one adding lane per row and read, so no two lanes collide).  Formed
-// only when there are more survivors than half the rows (the collection pass
-// has counted them); otherwise each survivor forms its two norms itself,
-// which is less work.
+// an integer: independent of the order of the terms).  Eight lanes per row,
+// four rows a warp; the lanes' sums meet in three shuffle steps.  (A warp over
+// 128 consecutive elements with a search for every element's row and a
+// segmented scan took 147 instructions per 32 elements: 1.27 ms for 1.4e8
+// nonzeros, 0.97 here.)  Formed only when there are more survivors than
+// half the rows (the collection pass has counted them); otherwise each
+// survivor forms its two norms itself, which is less work.
 __global__ void __launch_bounds__(256) row_norm2_kernel(const int64_t *__restrict__ indptr,
                                                         const float *__restrict__ values, long long N,
                                                         long long *__restrict__ norm2,
@@ -381,81 +599,64 @@ __global__ void __launch_bounds__(256) row_norm2_kernel(const int64_t *__restric
     const bool form = scratch->work3 * 2ull > (unsigned long long)N;
     if (blockIdx.x == 0 && threadIdx.x == 0) scratch->norm2_valid = form ? 1u : 0u;
     if (!form) return;
-    __shared__ unsigned long long part[8][32];
-    const int lane = threadIdx.x & 31;
-    unsigned long long *sum = part[threadIdx.x >> 5];
-    const long long groups = (N + 31) >> 5;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long g = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < groups; g += nwarps) {
-        const long long r0 = g << 5;
-        const int nr = (int)(N - r0 < 32 ? N - r0 : 32);
-        const long long s = __ldg(indptr + r0);
-        // lanes past the last row repeat its end (the ends stay nondecreasing)
-        const long long end = __ldg(indptr + r0 + (lane < nr ? lane + 1 : nr));
-        const long long e = __shfl_sync(kFull, end, 31);
-        sum[lane] = 0ull;
-        __syncwarp();
-        for (long long c = s; c < e; c += 128) {
+    const int g = threadIdx.x & 7;
+    const long long stride = (long long)gridDim.x * (blockDim.x >> 3);
+    // (the trip count is the same for the whole warp)
+    const long long first = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3;
+    for (long long w0 = first & ~3ll; w0 < N; w0 += stride) {
+        const long long row = w0 + (first & 3);
+        long long s = 0, e = 0;
+        if (row < N) {
+            s = __ldg(indptr + row);
+            e = __ldg(indptr + row + 1);
+        }
+        long long sum = 0;
+        for (long long i = s + g; i < e; i += 32) {
             float v[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const long long i = c + 32 * u + lane;
-                v[u] = i < e ? __ldg(values + i) : 0.0f;
-            }
+            for (int u = 0; u < 4; ++u) v[u] = i + 8 * u < e ? __ldg(values + i + 8 * u) : 0.0f;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const long long i = c + 32 * u + lane;
-                if (c + 32 * u >= e) break;                 // warp-uniform
-                int row = 0;                                // rows of the group ending at or before i
-#pragma unroll
-                for (int step = 16; step > 0; step >>= 1)
-                    if (__shfl_sync(kFull, end, row + step - 1) <= i) row += step;
-                unsigned long long term = i < e ? (unsigned long long)fixed_term(v[u], v[u]) : 0ull;
-                // inclusive sums over the lanes of the same row (rows are
-                // nondecreasing across the lanes)
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned long long tv = __shfl_up_sync(kFull, term, o);
-                    const int tr = __shfl_up_sync(kFull, row, o);
-                    if (lane >= o && tr == row) term += tv;
-                }
-                const int next_row = __shfl_down_sync(kFull, row, 1);
-                if (i < e && (lane == 31 || i + 1 == e || next_row != row)) sum[row] += term;
-                __syncwarp();
-            }
+            for (int u = 0; u < 4; ++u)
+                if (i + 8 * u < e) sum += fixed_term(v[u], v[u]);
         }
-        __syncwarp();
-        if (lane < nr) norm2[r0 + lane] = (long long)sum[lane];
-        __syncwarp();
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
+        if (g == 0 && row < N) norm2[row] = sum;
     }
 }
 
+// per warp: the staging area (4 KB), lite_flat's area, a survivor list (a tile's 512 and up to 31 before them)
+constexpr int kLiteWarpWords = 2 * kLiteStage + kFlatWords + 272;
+static_assert(kLiteWarpWords % 4 == 0, "16-byte rows");
+
 template <bool COSINE>
-__global__ void __launch_bounds__(256) lite_exact_kernel(const LiteArgs A) {
+__global__ void __launch_bounds__(256, 4) lite_exact_kernel(const LiteArgs A) {
     long long P = A.P;
     if (A.P_dev) {
         const long long pd = *A.P_dev;
         P = pd < 0 ? 0 : (pd < P ? pd : P);
     }
+    if (A.scratch->work3 <= BLSH_LITE_QUEUE_CAP) return;   // every survivor was queued
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
-    // per warp: the longer row's indices and values, when it has at most
-    // kLiteStage elements (binary searches then run in shared memory), and
-    // the survivors of the current tile (offsets within it)
+    // per warp: the stage for longer rows' indices, lite_flat's area, and the
+    // survivors of the current tile (offsets within it)
     extern __shared__ uint32_t lite_smem[];
-    uint32_t *w_idx = lite_smem + warp * 2 * kLiteStage;
-    float *w_val = reinterpret_cast<float *>(w_idx + kLiteStage);
-    uint16_t *w_list = reinterpret_cast<uint16_t *>(lite_smem + (blockDim.x >> 5) * 2 * kLiteStage) + warp * 512;
+    uint32_t *w_idx = lite_smem + warp * kLiteWarpWords;
+    uint32_t *flat = w_idx + 2 * kLiteStage;
+    uint16_t *w_list = reinterpret_cast<uint16_t *>(flat + kFlatWords);
     const bool have_norms = COSINE && A.norm2 && A.scratch->norm2_valid;
     // A warp takes kLiteGrab tiles of 512 statuses per grab of the work
-    // counter; a lane reads 16 statuses with one 16-byte load; the tile's
-    // survivors are listed in shared memory and computed 32 at a time.
+    // counter; a lane reads 16 statuses with one 16-byte load; the tiles'
+    // survivors are listed in shared memory and computed 32 at a time, what is
+    // left of a tile with the next one's.
     for (;;) {
         unsigned long long grab = 0;
         if (lane == 0) grab = atomicAdd(&A.scratch->work2, 1ull);
         grab = __shfl_sync(kFull, grab, 0);
         const long long g0 = (long long)grab * kLiteGrab * 512;
         if (g0 >= P) break;
+        int listed = 0;                                    // survivors waiting, at most 31 between tiles
         for (int tt = 0; tt < kLiteGrab; ++tt) {
             const long long q0 = g0 + 512ll * tt;
             if (q0 >= P) break;
@@ -476,15 +677,18 @@ __global__ void __launch_bounds__(256) lite_exact_kernel(const LiteArgs A) {
             }
             const int total = __shfl_sync(kFull, incl, 31);
             if (total == 0) continue;
-            __syncwarp();                                  // the previous tile's list has been read
-            int slot = incl - c;
-            for (uint32_t b = surv; b; b &= b - 1) w_list[slot++] = (uint16_t)(16 * lane + __ffs(b) - 1);
+            __syncwarp();                                  // the previous batch's part of the list has been read
+            int slot = listed + incl - c;
+            for (uint32_t b = surv; b; b &= b - 1) w_list[slot++] = (uint16_t)(512 * tt + 16 * lane + __ffs(b) - 1);
             __syncwarp();
-            for (int b0 = 0; b0 < total; b0 += 32) {
-                const long long q = b0 + lane < total ? q0 + w_list[b0 + lane] : -1;
-                lite_batch<COSINE>(A, q, have_norms, w_idx, w_val);
+            listed += total;
+            while (listed >= 32) {
+                listed -= 32;
+                lite_batch<COSINE>(A, g0 + w_list[listed + lane], have_norms, w_idx, flat);
             }
         }
+        if (listed) lite_batch<COSINE>(A, lane < listed ? g0 + w_list[lane] : -1, have_norms, w_idx, flat);
+        __syncwarp();
     }
 }
 
@@ -538,17 +742,17 @@ __global__ void __launch_bounds__(256) lite_collect_kernel(const LiteArgs A, uns
     }
 }
 
-// The queued survivors, one per warp at a time in grid-stride order: the
+// The queued survivors, a batch per warp at a time from a counter: the
 // survivors of one dense tile (a bucket of near-duplicates) spread over many
-// warps.
+// warps, and a warp with long rows takes fewer batches.
 template <bool COSINE>
-__global__ void __launch_bounds__(256) lite_queue_kernel(const LiteArgs A, const unsigned long long *queue) {
+__global__ void __launch_bounds__(256, 4) lite_queue_kernel(const LiteArgs A, const unsigned long long *queue) {
     const unsigned long long total = A.scratch->work3;
     const unsigned long long n = total < BLSH_LITE_QUEUE_CAP ? total : BLSH_LITE_QUEUE_CAP;
     extern __shared__ uint32_t lite_smem[];
     const int lane = threadIdx.x & 31;
-    uint32_t *w_idx = lite_smem + (threadIdx.x >> 5) * 2 * kLiteStage;
-    float *w_val = reinterpret_cast<float *>(w_idx + kLiteStage);
+    uint32_t *w_idx = lite_smem + (threadIdx.x >> 5) * kLiteWarpWords;
+    uint32_t *flat = w_idx + 2 * kLiteStage;
     const bool have_norms = COSINE && A.norm2 && A.scratch->norm2_valid;
     // bs consecutive queue entries per warp at a time (one per lane): 32, or
     // fewer when the survivors are too few to give every warp a full batch
@@ -556,10 +760,13 @@ __global__ void __launch_bounds__(256) lite_queue_kernel(const LiteArgs A, const
     const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
     unsigned long long bs = (n + nwarps - 1) / nwarps;
     bs = bs < 1 ? 1 : (bs > 32 ? 32 : bs);
-    for (unsigned long long base = (((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * bs; base < n;
-         base += nwarps * bs) {
+    for (;;) {
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(&A.scratch->work, bs);
+        base = __shfl_sync(kFull, base, 0);
+        if (base >= n) break;
         const long long q = lane < bs && base + lane < n ? (long long)queue[base + lane] : -1;
-        lite_batch<COSINE>(A, q, have_norms, w_idx, w_val);
+        lite_batch<COSINE>(A, q, have_norms, w_idx, flat);
     }
 }
 
@@ -647,28 +854,32 @@ int lite_exact_pass(blsh_ctx *ctx, const uint2 *pairs, int64_t P, const long lon
     L.sim = sim;
     L.scratch = ctx->scratch;
     L.vec = blsh_aligned(status, 16);
+    L.N = N;
     L.norm2 = nullptr;
     // the rows' squared norms once per call, in the buffer blsh_ctx_reserve
     // allocated; with more rows than were reserved each survivor forms its
     // two sums itself (no allocation here: this is a hot call)
     if (values && N > 0 && ctx->norm2_cap >= N) L.norm2 = (const long long *)ctx->norm2;
     // survivors: queued (balanced over warps), then any beyond the queue in place
-    BLSH_CUDA(ctx, cudaMemsetAsync(&ctx->scratch->work2, 0, 2 * sizeof(unsigned long long), s));   // work2, work3
+    BLSH_CUDA(ctx, cudaMemsetAsync(&ctx->scratch->work, 0, 3 * sizeof(unsigned long long), s));   // work, work2, work3
     unsigned long long *queue = ctx->lite_queue;
     blsh_time_start(ctx, s);
     lite_collect_kernel<<<ctx->sm_count * 8, 256, 0, s>>>(L, queue);
     BLSH_LAUNCHED(ctx, "lite_collect_kernel");
     if (L.norm2) {
-        const long long blocks = (N + 255) / 256, cap = (long long)ctx->sm_count * 8;   // 32 rows per warp
+        const long long blocks = (N + 31) / 32, cap = (long long)ctx->sm_count * 32;   // 32 rows a CTA
         blsh_time_start(ctx, s);
         row_norm2_kernel<<<(unsigned)(blocks < cap ? blocks : cap), 256, 0, s>>>(
             indptr, values, N, const_cast<long long *>(L.norm2), ctx->scratch);
         BLSH_LAUNCHED(ctx, "row_norm2_kernel");
     }
     int occ = 0;
-    // per warp of the CTA's 8: the staging area (4 KB) and a tile's survivor list (1 KB)
-    const size_t smem = 8 * (2 * kLiteStage * sizeof(uint32_t) + 512 * sizeof(uint16_t));
+    const size_t smem = 8 * kLiteWarpWords * sizeof(uint32_t);
     if (values) {
+        BLSH_CUDA(ctx, cudaFuncSetAttribute(lite_queue_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)smem));
+        BLSH_CUDA(ctx, cudaFuncSetAttribute(lite_exact_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)smem));
         BLSH_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, lite_queue_kernel<true>, 256, smem));
         blsh_time_start(ctx, s);
         lite_queue_kernel<true><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L, queue);
@@ -677,6 +888,10 @@ int lite_exact_pass(blsh_ctx *ctx, const uint2 *pairs, int64_t P, const long lon
         lite_exact_kernel<true><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L);
         BLSH_LAUNCHED(ctx, "lite_exact_kernel");
     } else {
+        BLSH_CUDA(ctx, cudaFuncSetAttribute(lite_queue_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)smem));
+        BLSH_CUDA(ctx, cudaFuncSetAttribute(lite_exact_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)smem));
         BLSH_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, lite_queue_kernel<false>, 256, smem));
         blsh_time_start(ctx, s);
         lite_queue_kernel<false><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L, queue);
