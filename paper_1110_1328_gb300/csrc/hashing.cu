@@ -1,5 +1,7 @@
 // hashing.cu -- the signature producers: minhash (Section 4.1, "LSH family")
 // and sign random projections of sparse rows (Section 4.2, "LSH family").
+#include <stddef.h>
+
 #include <type_traits>
 
 #include "common.cuh"
@@ -219,9 +221,7 @@ __device__ __forceinline__ float r_fp32(const uint16_t *R, size_t i) {
 }
 
 constexpr int kSrpMaxPerThread = 16;
-constexpr int kSrpLooseRow = 256;   // rows up to this length use the 2^15 sum|v| magnitude bound (two-byte codes)
-constexpr int kSrpBatch = 8;
-constexpr int kSrpGrab = 8;         // (row, piece) items a CTA of srp_sparse4_kernel takes per grab
+constexpr int kSrpBatch = 8;        // gathers issued together
 constexpr int kSrpChunk = 256;
 
 template <typename RT>
@@ -344,244 +344,396 @@ __device__ __forceinline__ unsigned long long f2_codes(uint32_t w) {
                    __int_as_float((int)__byte_perm(w, 0x4b00u, 0x5432)));
 }
 
-// The same computation when bits is a multiple of 128: thread t owns the
-// groups of four columns t, t+T, ... of each row of R (bits 4t..4t+3,
-// 4(t+T).., ...), so every load moves 16 bytes (float R) or 8 bytes (RT =
-// uint16_t: the two-byte codes of Section 4.3) and a warp reads 512 or 256
-// contiguous bytes.  A row's indices and values are read 32 at a time, one
-// per lane (coalesced), and reach the other lanes by shuffles; the gathers
-// of several nonzeros are issued together, so a long row is not a chain of
-// dependent loads, and no barrier is needed.  Every column keeps its sum and
-// the sum of the products' magnitudes for the error bound.  The sum is formed
-// in blocks of 32 nonzeros (a block's FMA chain, then the block added to the
-// total), so a column's result carries at most min(n, 32) + ceil(n / 32)
-// roundings in any chain rather than n: a long row leaves far fewer signs to
-// the FP64 recheck.  The four bits of
-// a group form a nibble; eight lanes OR their nibbles into one signature
-// word with shuffles.  CTAs take (row, piece of 4 V T columns) items from a
-// counter, kSrpGrab at a time (a fixed share per CTA when there are few).
-template <int V, typename RT>
-__global__ void __launch_bounds__(256) srp_sparse4_kernel(const int64_t *__restrict__ indptr,
-                                                          const uint32_t *__restrict__ indices,
-                                                          const float *__restrict__ values, long long N,
-                                                          const RT *__restrict__ R, long long dim, int bits,
-                                                          int col_first, int pieces,
-                                                          const uint8_t *__restrict__ row_mask,
-                                                          uint32_t *__restrict__ sig, blsh_dev_scratch *scratch,
-                                                          uint2 *__restrict__ queue, int grab) {
-    // columns col_first .. col_first + pieces 4 V T - 1 of the signatures of
-    // the rows row_mask selects (all rows when it is NULL); a CTA works on
-    // one (row, piece of 4 V T columns) at a time, so that a few selected
-    // rows still spread over many CTAs
-    const int T = blockDim.x;
-    const int t = threadIdx.x;
-    const int lane = t & 31;
-    const int words = bits >> 5;
-    unsigned long long rechecked = 0, zeros = 0, bad = 0;
-    // items are handed out `grab` at a time from a counter: row lengths
-    // follow a power law (a single row can hold more work than a thousand
-    // average ones), and a fixed share per CTA left most of the GPU idle
-    // while the CTAs that drew the longest rows finished
-    // (grab == 0: a fixed share per CTA, items blockIdx.x, blockIdx.x +
-    // gridDim.x, ...: few items per CTA, where a counter would cost more
-    // than it balances)
-    __shared__ unsigned long long s_next;
-    const long long items = N * pieces;
-    long long next_static = blockIdx.x;
-    for (;;) {
-        long long g0, g1;
-        if (grab > 0) {
-            __syncthreads();                               // every thread has read the previous grab
-            if (threadIdx.x == 0) s_next = atomicAdd(&scratch->hash_work, (unsigned long long)grab);
-            __syncthreads();
-            g0 = (long long)s_next;
-            g1 = g0 + grab < items ? g0 + grab : items;
+// The same computation when bits is a multiple of 128 and R is aligned for it:
+// a warp per (row, piece of 32 CPL columns), a lane owning CPL neighbouring
+// columns -- 16 bytes of a row of R a load (four floats, or eight two-byte
+// codes of Section 4.3; four codes where the columns are no multiple of 256 or
+// R lies on 8 bytes only).
+//
+// A grab of G rows comes from a counter: row lengths follow a power law, and a
+// fixed share per warp left most of the GPU idle behind the longest rows.  The
+// rows' bounds are read a lane each, a row's indices and values 32 at a time
+// (coalesced, the next row's first ones ahead of time) and broadcast by
+// shuffles, and the gathers of kSrpBatch nonzeros are issued together.  Rows of
+// more than kSrpLongRow nonzeros are listed for srp_long_kernel: one of 7,700
+// is a millisecond of one warp's time.
+//
+// Pieces: `outer` of them one after the other over all the rows, `inner` of
+// them for a row at a time.  Where R exceeds L2 the columns are walked piece by
+// piece (outer), so that a slice of R that fits L2 is gathered from at a time;
+// otherwise all of a row's pieces follow each other (inner), which reads its
+// indices once.
+//
+// The sum is formed in blocks of 32 nonzeros (a block's FMA chain, then the
+// block added to the total), so a column's result carries at most min(n, 32) +
+// ceil(n / 32) roundings in any chain rather than n.  Two-byte codes are summed
+// as q - 2^15 in paired FP32 instructions, exactly decoded, in units of 2^-12;
+// |q - 2^15| <= 2^15 bounds their magnitudes by 2^15 sum|v_i|, about ten times
+// looser than each column's own sum, but rows are short here and it saves two
+// paired FMAs and four masks a nonzero.  Float columns keep their own sums.
+//
+// What bounds it: the latency of the gathers of R's rows (one a nonzero, from
+// L2 or HBM), so as many as the registers allow are in flight; with 64
+// registers (four CTAs an SM) and eight gathers a batch the rows' kernel takes
+// 4.37 ms on the 5e6 rows below, with 79 registers 6.46 ms, with four a batch
+// 4.45 ms, with five CTAs 4.66 ms, and with the codes staged in shared memory
+// by asynchronous copies 4.78 ms.
+//
+// 5e6 rows, 1.4e8 nonzeros, the first 256 columns of two-byte codes: 11.5 ms
+// with four codes a lane and long rows left to single warps, now 4.37 ms + 3.15
+// ms for the rows of more than 256 nonzeros; 20,000 rows x 2,048 columns of
+// floats (R of 820 MB) 607 us, now 506 us + 55 us.
+constexpr int kSrpLongRow = 256;
+
+// Where a call's rows and columns lie, and its queues.
+struct SrpArgs {
+    const int64_t *indptr;
+    const uint32_t *indices;
+    const float *values;
+    long long N, dim;
+    int bits, col_first, outer, inner;
+    const uint8_t *row_mask;   // rows to project (NULL: all)
+    uint32_t *sig;
+    blsh_dev_scratch *scratch;
+    uint2 *queue;              // undecided signs, for srp_recheck_kernel
+    unsigned long long *longs; // rows of more than kSrpLongRow nonzeros (BLSH_LITE_QUEUE_CAP of them)
+};
+
+// A lane's CPL columns: their sums of a block, then of the row.
+template <typename RT, int CPL>
+struct SrpCols;
+template <int CPL>
+struct SrpCols<uint16_t, CPL> {
+    static constexpr int W = CPL / 2;   // 32-bit words of codes
+    unsigned long long acc[W], tot[W];
+    uint32_t raw[kSrpBatch][W];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int i = 0; i < W; ++i) acc[i] = tot[i] = 0ull;
+    }
+    __device__ __forceinline__ void load(int b, const uint16_t *p) {
+        if constexpr (W == 4) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(p));
+            raw[b][0] = v.x; raw[b][1] = v.y; raw[b][2] = v.z; raw[b][3] = v.w;
         } else {
-            g0 = next_static;
-            g1 = g0 + 1;
-            next_static += gridDim.x;
+            const uint2 v = __ldg(reinterpret_cast<const uint2 *>(p));
+            raw[b][0] = v.x; raw[b][1] = v.y;
         }
-        if (g0 >= items) break;
-        for (long long item = g0; item < g1; ++item) {
-            const long long row = pieces == 1 ? item : item / pieces;   // (a 64-bit division is a long call)
-            const int col0 = col_first + (int)(item - row * pieces) * 4 * V * T;
-            if (row_mask && !row_mask[row]) continue;
-            const long long s = __ldg(indptr + row), e = __ldg(indptr + row + 1);
-            constexpr bool Q16 = sizeof(RT) == 2;
-            float acc[4 * V], mag[4 * V], tot[4 * V];
+    }
+    // the decoded value of code q is (q - 2^15) 2^-12: (2^23 + q) - (2^23 + 2^15), exact
+    __device__ __forceinline__ void add(int b, float v) {
+        const unsigned long long off2 = f2_pack(-8421376.0f, -8421376.0f), v2 = f2_pack(v, v);
 #pragma unroll
-            for (int u = 0; u < 4 * V; ++u) acc[u] = mag[u] = tot[u] = 0.0f;
-            // two-byte codes: the same sums kept as pairs of columns (one 64-bit
-            // register each) for the paired instructions, unpacked once per row
-            unsigned long long acc2[2 * V], mag2[2 * V], tot2[2 * V];
+        for (int i = 0; i < W; ++i) acc[i] = f2_fma(v2, f2_add(f2_codes(raw[b][i]), off2), acc[i]);
+    }
+    // with the magnitudes' sums in mag (pairs)
+    __device__ __forceinline__ void add(int b, float v, unsigned long long (&mag)[W]) {
+        const unsigned long long off2 = f2_pack(-8421376.0f, -8421376.0f), v2 = f2_pack(v, v);
+        const unsigned long long av2 = f2_pack(fabsf(v), fabsf(v));
 #pragma unroll
-            for (int u = 0; u < 2 * V; ++u) acc2[u] = mag2[u] = tot2[u] = 0ull;
-            // Rows of at most kSrpLooseRow nonzeros (two-byte codes): the
-            // magnitude bound 2^15 sum|v_i| (every decoded code has |q - 2^15| <=
-            // 2^15) instead of each column's sum|v_i| |q_ij - 2^15|; about ten
-            // times looser, but the blocked sums keep short rows' bounds small,
-            // and it saves two paired FMAs and four masks per nonzero
-            const bool loose = Q16 && e - s <= kSrpLooseRow;
-            float sav = 0.0f;
-            // the row's nonzeros 32 at a time: lane l of every warp loads entry
-            // l (coalesced), then the gathers of kSrpBatch / V entries are issued
-            // together (their indices come by shuffle), so that a long row is not
-            // a chain of dependent loads
-            constexpr int NB = kSrpBatch / V > 0 ? kSrpBatch / V : 1;
-            for (long long k0 = s; k0 < e; k0 += 32) {
-                const int cnt = e - k0 < 32 ? (int)(e - k0) : 32;
-                uint32_t my_ix = 0;
-                float my_v = 0.0f;
-                if (lane < cnt) {
-                    my_ix = __ldg(indices + k0 + lane);
-                    my_v = __ldg(values + k0 + lane);
-                    if (my_ix >= dim) {   // malformed entry: counted once, contributes nothing
-                        bad += t < 32;
+        for (int i = 0; i < W; ++i) {
+            const unsigned long long d = f2_add(f2_codes(raw[b][i]), off2);
+            acc[i] = f2_fma(v2, d, acc[i]);
+            mag[i] = f2_fma(av2, d & 0x7fffffff7fffffffull, mag[i]);
+        }
+    }
+    __device__ __forceinline__ void end_block() {
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            tot[i] = f2_add(tot[i], acc[i]);
+            acc[i] = 0ull;
+        }
+    }
+    __device__ __forceinline__ void totals(float (&t)[CPL]) const {
+#pragma unroll
+        for (int i = 0; i < W; ++i) f2_unpack(tot[i], t[2 * i], t[2 * i + 1]);
+    }
+};
+template <int CPL>
+struct SrpCols<float, CPL> {
+    static_assert(CPL == 4, "16-byte loads of four columns");
+    float acc[4], tot[4];
+    float4 raw[kSrpBatch];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc[i] = tot[i] = 0.0f;
+    }
+    __device__ __forceinline__ void load(int b, const float *p) { raw[b] = __ldg(reinterpret_cast<const float4 *>(p)); }
+    __device__ __forceinline__ void add(int b, float v, float (&mag)[4]) {
+        const float av = fabsf(v);
+        const float r[4] = {raw[b].x, raw[b].y, raw[b].z, raw[b].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            acc[i] = __fmaf_rn(v, r[i], acc[i]);
+            mag[i] = __fmaf_rn(av, fabsf(r[i]), mag[i]);
+        }
+    }
+    __device__ __forceinline__ void end_block() {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            tot[i] = __fadd_rn(tot[i], acc[i]);
+            acc[i] = 0.0f;
+        }
+    }
+    __device__ __forceinline__ void totals(float (&t)[4]) const {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) t[i] = tot[i];
+    }
+};
+
+// The column sums' error bound: `chain` roundings in the longest chain (with
+// its 25% slack good while n u <= 0.05), and up to 2n roundings near underflow.
+__device__ __forceinline__ float srp_bound(float chain, float mag, float n) {
+    return 1.25f * chain * 5.9604644775390625e-8f * mag + n * 1.4e-45f;
+}
+
+// An undecided sign: queued for srp_recheck_kernel (bit left 0), or summed in
+// line if the queue is full.
+template <typename RT>
+__device__ __forceinline__ bool srp_undecided(const SrpArgs &A, const RT *R, long long row, long long s, long long e,
+                                              int j, unsigned long long &rechecked, unsigned long long &zeros) {
+    const unsigned long long slot = atomicAdd(&A.scratch->recheck_count, 1ull);
+    if (slot < BLSH_RECHECK_CAP) {
+        A.queue[slot] = make_uint2((uint32_t)row, (uint32_t)j);
+        return false;
+    }
+    const double d = srp_recheck_fp64<RT>(A.indices, A.values, s, e, R, A.dim, A.bits, j);
+    ++rechecked;
+    zeros += d == 0.0;
+    return d >= 0.0;
+}
+
+template <typename RT, int CPL>
+__global__ void __launch_bounds__(256, 4) srp_sparse4_kernel(const SrpArgs A, const RT *__restrict__ R, int G) {
+    constexpr bool Q16 = sizeof(RT) == 2;
+    constexpr int PC = 32 * CPL;   // columns of a piece
+    const int lane = threadIdx.x & 31;
+    const int words = A.bits >> 5;
+    unsigned long long rechecked = 0, zeros = 0, bad = 0;
+    const long long groups = (A.N + G - 1) / G;
+    const unsigned long long items = (unsigned long long)groups * A.outer;
+    for (;;) {
+        unsigned long long item = 0;
+        if (lane == 0) item = atomicAdd(&A.scratch->hash_work, 1ull);
+        item = __shfl_sync(kFull, item, 0);
+        if (item >= items) break;
+        const int outer = A.outer == 1 ? 0 : (int)(item / (unsigned long long)groups);
+        const long long r0 = ((long long)item - outer * groups) * G;
+        // this grab's rows, a lane each
+        long long my_s = 0;
+        int my_len = 0;
+        bool sel = false;
+        if (lane < G && r0 + lane < A.N && (!A.row_mask || A.row_mask[r0 + lane])) {
+            my_s = __ldg(A.indptr + r0 + lane);
+            const long long len = __ldg(A.indptr + r0 + lane + 1) - my_s;
+            sel = len <= kSrpLongRow;
+            my_len = sel ? (int)len : 0;
+            if (!sel && outer == 0) {
+                const unsigned long long slot = atomicAdd(&A.scratch->work3, 1ull);
+                if (slot < BLSH_LITE_QUEUE_CAP) A.longs[slot] = (unsigned long long)(r0 + lane);
+            }
+        }
+        unsigned todo = __ballot_sync(kFull, sel);
+        uint32_t nx_ix = 0;
+        float nx_v = 0.0f;
+        auto first_block = [&](int l) {   // row l's first 32 nonzeros
+            const long long s = __shfl_sync(kFull, my_s, l);
+            const int len = __shfl_sync(kFull, my_len, l);
+            nx_ix = 0;
+            nx_v = 0.0f;
+            if (lane < len) {
+                nx_ix = __ldg(A.indices + s + lane);
+                nx_v = __ldg(A.values + s + lane);
+            }
+        };
+        if (todo) first_block(__ffs(todo) - 1);
+        while (todo) {
+            const int l = __ffs(todo) - 1;
+            todo &= todo - 1;
+            const long long row = r0 + l, s = __shfl_sync(kFull, my_s, l);
+            const int len = __shfl_sync(kFull, my_len, l);
+            uint32_t ix0 = nx_ix;
+            float v0 = nx_v;
+            if (todo) first_block(__ffs(todo) - 1);
+            // malformed entries: counted once, contribute nothing
+            auto check = [&](uint32_t &ix, float &v, bool count) {
+                if (ix >= A.dim) {
+                    bad += count;
+                    ix = 0;
+                    v = 0.0f;
+                }
+            };
+            check(ix0, v0, outer == 0);
+            for (int p = 0; p < A.inner; ++p) {
+                const int col0 = A.col_first + (outer * A.inner + p) * PC;
+                const RT *Rc = R + col0 + CPL * lane;
+                SrpCols<RT, CPL> c;
+                c.clear();
+                [[maybe_unused]] float mag[CPL];
+#pragma unroll
+                for (int i = 0; i < CPL; ++i) mag[i] = 0.0f;
+                float sav = 0.0f;   // this lane's part of sum|v|
+                for (int k0 = 0; k0 < len; k0 += 32) {
+                    uint32_t my_ix = ix0;
+                    float my_v = v0;
+                    if (k0) {
                         my_ix = 0;
                         my_v = 0.0f;
-                    }
-                }
-                if constexpr (Q16) {
-                    // the decoded value of code q is (q - 2^15) 2^-12: (2^23 + q) - (2^23 + 2^15),
-                    // exact, with the sums kept in units of 2^-12
-                    const unsigned long long off2 = f2_pack(-8421376.0f, -8421376.0f);
-                    auto chunk = [&](auto with_mag) {
-                        constexpr bool kMag = decltype(with_mag)::value;
-                        for (int u0 = 0; u0 < cnt; u0 += NB) {
-                            uint2 qb[NB][V];
-                            float vb[NB];
-#pragma unroll
-                            for (int b = 0; b < NB; ++b) {
-                                const uint32_t ix = __shfl_sync(kFull, my_ix, (u0 + b) & 31);
-                                vb[b] = __shfl_sync(kFull, my_v, (u0 + b) & 31);   // 0 past the row's end
-                                const uint2 *Rrow = reinterpret_cast<const uint2 *>(R + (size_t)ix * bits + col0) + t;
-#pragma unroll
-                                for (int g = 0; g < V; ++g) qb[b][g] = __ldg(Rrow + g * T);
-                            }
-#pragma unroll
-                            for (int b = 0; b < NB; ++b) {
-                                const unsigned long long v2 = f2_pack(vb[b], vb[b]);
-                                const unsigned long long av2 = f2_pack(fabsf(vb[b]), fabsf(vb[b]));
-                                if (!kMag) sav += fabsf(vb[b]);
-#pragma unroll
-                                for (int g = 0; g < V; ++g) {
-                                    const unsigned long long d01 = f2_add(f2_codes(qb[b][g].x), off2);
-                                    const unsigned long long d23 = f2_add(f2_codes(qb[b][g].y), off2);
-                                    acc2[2 * g] = f2_fma(v2, d01, acc2[2 * g]);
-                                    acc2[2 * g + 1] = f2_fma(v2, d23, acc2[2 * g + 1]);
-                                    if (kMag) {
-                                        mag2[2 * g] = f2_fma(av2, d01 & 0x7fffffff7fffffffull, mag2[2 * g]);
-                                        mag2[2 * g + 1] = f2_fma(av2, d23 & 0x7fffffff7fffffffull, mag2[2 * g + 1]);
-                                    }
-                                }
-                            }
+                        if (k0 + lane < len) {
+                            my_ix = __ldg(A.indices + s + k0 + lane);
+                            my_v = __ldg(A.values + s + k0 + lane);
+                            check(my_ix, my_v, outer == 0 && p == 0);
                         }
-                    };
-                    if (loose) chunk(std::false_type{});
-                    else chunk(std::true_type{});
-                    // the block of (at most) 32 nonzeros into the total
-#pragma unroll
-                    for (int u = 0; u < 2 * V; ++u) {
-                        tot2[u] = f2_add(tot2[u], acc2[u]);
-                        acc2[u] = 0ull;
                     }
-                } else {   // float R: 16-byte loads of four columns
-                    for (int u0 = 0; u0 < cnt; u0 += NB) {
-                        float4 r[NB][V];
-                        float vb[NB];
+                    if (Q16) sav += fabsf(my_v);
+                    const int cnt = len - k0 < 32 ? len - k0 : 32;
+                    for (int u0 = 0; u0 < cnt; u0 += kSrpBatch) {
+                        float vb[kSrpBatch];
 #pragma unroll
-                        for (int b = 0; b < NB; ++b) {
+                        for (int b = 0; b < kSrpBatch; ++b) {   // (past the row's end: row 0 of R times 0)
                             const uint32_t ix = __shfl_sync(kFull, my_ix, (u0 + b) & 31);
-                            vb[b] = __shfl_sync(kFull, my_v, (u0 + b) & 31);   // 0 past the row's end
-                            const float4 *Rrow = reinterpret_cast<const float4 *>(R + (size_t)ix * bits + col0) + t;
-#pragma unroll
-                            for (int g = 0; g < V; ++g) r[b][g] = __ldg(Rrow + g * T);
+                            vb[b] = __shfl_sync(kFull, my_v, (u0 + b) & 31);
+                            c.load(b, Rc + (size_t)ix * A.bits);
                         }
 #pragma unroll
-                        for (int b = 0; b < NB; ++b) {
-                            const float v = vb[b], av = fabsf(v);
-#pragma unroll
-                            for (int g = 0; g < V; ++g) {
-                                acc[4 * g + 0] = __fmaf_rn(v, r[b][g].x, acc[4 * g + 0]);
-                                acc[4 * g + 1] = __fmaf_rn(v, r[b][g].y, acc[4 * g + 1]);
-                                acc[4 * g + 2] = __fmaf_rn(v, r[b][g].z, acc[4 * g + 2]);
-                                acc[4 * g + 3] = __fmaf_rn(v, r[b][g].w, acc[4 * g + 3]);
-                                mag[4 * g + 0] = __fmaf_rn(av, fabsf(r[b][g].x), mag[4 * g + 0]);
-                                mag[4 * g + 1] = __fmaf_rn(av, fabsf(r[b][g].y), mag[4 * g + 1]);
-                                mag[4 * g + 2] = __fmaf_rn(av, fabsf(r[b][g].z), mag[4 * g + 2]);
-                                mag[4 * g + 3] = __fmaf_rn(av, fabsf(r[b][g].w), mag[4 * g + 3]);
-                            }
+                        for (int b = 0; b < kSrpBatch; ++b) {
+                            if constexpr (Q16) c.add(b, vb[b]);
+                            else c.add(b, vb[b], mag);
                         }
                     }
-#pragma unroll
-                    for (int u = 0; u < 4 * V; ++u) {
-                        tot[u] = __fadd_rn(tot[u], acc[u]);
-                        acc[u] = 0.0f;
-                    }
+                    c.end_block();
                 }
-            }
-            if constexpr (sizeof(RT) == 2) {
+                float t[CPL];
+                c.totals(t);
+                if (Q16) {
 #pragma unroll
-                for (int u = 0; u < 2 * V; ++u) {
-                    f2_unpack(tot2[u], tot[2 * u], tot[2 * u + 1]);
-                    f2_unpack(mag2[u], mag[2 * u], mag[2 * u + 1]);
+                    for (int o = 16; o > 0; o >>= 1) sav += __shfl_xor_sync(kFull, sav, o);
                 }
-                if (loose) {
+                const float n = (float)len;
+                const float chain = fminf(n, 32.0f) + (float)((len + 31) >> 5);
+                uint32_t word = 0;
 #pragma unroll
-                    for (int u = 0; u < 4 * V; ++u) mag[u] = 32768.0f * sav;
+                for (int i = 0; i < CPL; ++i) {
+                    bool bit = t[i] >= 0.0f;
+                    if (!(fabsf(t[i]) > srp_bound(chain, Q16 ? 32768.0f * sav : mag[i], n)))
+                        bit = srp_undecided<RT>(A, R, row, s, s + len, col0 + CPL * lane + i, rechecked, zeros);
+                    word |= (uint32_t)bit << i;
                 }
-            }
-            // the row length through a 32-bit integer (a 64-bit conversion would run
-            // on the narrow FP64 pipe); rows past 2^30 count as 2^30, which is long
-            const int len = (int)(e - s < (1ll << 30) ? e - s : (1ll << 30));
-            const float n = (float)len;
-            const bool long_row = n * 5.9604644775390625e-8f > 0.05f;   // the 1.25 slack needs n u <= 0.05
-            // Roundings in a column's sum: a block's chain (at most 32 FMAs, error
-            // <= gamma_32 of its magnitudes) and the chain of block totals (at
-            // most ceil(n / 32) - 1 adds), so |sum - exact| <= (gamma_32 +
-            // gamma_nb + gamma_32 gamma_nb) sum|p|, below 1.12 (min(n, 32) + nb) u
-            // mag when n u <= 0.05 (mag, the computed sum of magnitudes, is within
-            // gamma_n of sum|p|); each rounding near underflow adds at most 2^-150,
-            // and there are at most 2n of them.
-            const float kround = fminf(n, 32.0f) + (float)((len + 31) >> 5);
+                // 32 / CPL lanes' bits form a word
+                word <<= CPL * (lane & (32 / CPL - 1));
 #pragma unroll
-            for (int g = 0; g < V; ++g) {
-                uint32_t nib = 0;
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const int u = 4 * g + c;
-                    const float bound = 1.25f * kround * 5.9604644775390625e-8f * mag[u] + n * 1.4e-45f;
-                    bool bit;
-                    if (!long_row && fabsf(tot[u]) > bound) {
-                        bit = tot[u] >= 0.0f;
-                    } else {
-                        // undecided: queue it for srp_recheck_kernel (bit left 0 here),
-                        // or recompute in line if the queue is full
-                        const uint32_t j = col0 + 4 * (t + g * T) + c;
-                        const unsigned long long slot = atomicAdd(&scratch->recheck_count, 1ull);
-                        if (slot < BLSH_RECHECK_CAP) {
-                            queue[slot] = make_uint2((uint32_t)row, j);
-                            bit = false;
-                        } else {
-                            const double d = srp_recheck_fp64<RT>(indices, values, s, e, R, dim, bits, j);
-                            bit = d >= 0.0;
-                            ++rechecked;
-                            zeros += d == 0.0;
-                        }
-                    }
-                    nib |= (uint32_t)bit << c;
-                }
-                uint32_t word = nib << (4 * (lane & 7));
-                word |= __shfl_xor_sync(kFull, word, 1);
-                word |= __shfl_xor_sync(kFull, word, 2);
-                word |= __shfl_xor_sync(kFull, word, 4);
-                if ((lane & 7) == 0) sig[(size_t)row * words + (col0 >> 5) + ((t + g * T) >> 3)] = word;
+                for (int o = 1; o < 32 / CPL; o <<= 1) word |= __shfl_xor_sync(kFull, word, o);
+                if ((lane & (32 / CPL - 1)) == 0)
+                    A.sig[(size_t)row * words + (col0 >> 5) + lane / (32 / CPL)] = word;
             }
         }
     }
-    if (bad) blsh_dev_error(scratch, BLSH_ERANGE, 0, bad);
-    if (rechecked) atomicAdd(&scratch->counters[2], rechecked);
-    if (zeros) atomicAdd(&scratch->counters[3], zeros);
+    if (bad) blsh_dev_error(A.scratch, BLSH_ERANGE, 0, bad);
+    if (rechecked) atomicAdd(&A.scratch->counters[2], rechecked);
+    if (zeros) atomicAdd(&A.scratch->counters[3], zeros);
+}
+
+// Rows of more than kSrpLongRow nonzeros: a CTA per (row, piece), handed out
+// from a counter, its eight warps taking every eighth block of 32 nonzeros; the
+// warps' sums and magnitudes (every column's own here) meet in shared memory,
+// added in warp order.  No product passes through more than 32 + ceil(n / 256)
+// + 8 roundings.
+template <typename RT, int CPL>
+__global__ void __launch_bounds__(256, 3) srp_long_kernel(const SrpArgs A, const RT *__restrict__ R) {
+    constexpr int PC = 32 * CPL;
+    __shared__ float s_tot[8][PC], s_mag[8][PC];
+    __shared__ unsigned long long s_item;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int words = A.bits >> 5, pieces = A.outer * A.inner;
+    const unsigned long long listed = A.scratch->work3;
+    const bool all = listed > BLSH_LITE_QUEUE_CAP;   // more than the list holds: every row is looked at
+    const unsigned long long items = (all ? (unsigned long long)A.N : listed) * pieces;
+    unsigned long long rechecked = 0, zeros = 0, bad = 0;
+    for (;;) {
+        __syncthreads();                              // the previous item and its sums have been read
+        if (threadIdx.x == 0) s_item = atomicAdd(&A.scratch->work2, 1ull);
+        __syncthreads();
+        const unsigned long long item = s_item;
+        if (item >= items) break;
+        const unsigned long long q = item / (unsigned)pieces;
+        const int p = (int)(item - q * (unsigned)pieces);
+        const long long row = (long long)(all ? q : A.longs[q]);
+        if (all && A.row_mask && !A.row_mask[row]) continue;
+        const long long s = __ldg(A.indptr + row), len = __ldg(A.indptr + row + 1) - s;
+        if (len <= kSrpLongRow) continue;
+        const int col0 = A.col_first + p * PC;
+        const RT *Rc = R + col0 + CPL * lane;
+        SrpCols<RT, CPL> c;
+        c.clear();
+        float mag[CPL];
+#pragma unroll
+        for (int i = 0; i < CPL; ++i) mag[i] = 0.0f;
+        [[maybe_unused]] unsigned long long mag2[CPL / 2];
+#pragma unroll
+        for (int i = 0; i < CPL / 2; ++i) mag2[i] = 0ull;
+        for (long long k0 = 32 * warp; k0 < len; k0 += 256) {
+            uint32_t my_ix = 0;
+            float my_v = 0.0f;
+            if (k0 + lane < len) {
+                my_ix = __ldg(A.indices + s + k0 + lane);
+                my_v = __ldg(A.values + s + k0 + lane);
+                if (my_ix >= A.dim) {
+                    bad += p == 0;
+                    my_ix = 0;
+                    my_v = 0.0f;
+                }
+            }
+            const int cnt = len - k0 < 32 ? (int)(len - k0) : 32;
+            for (int u0 = 0; u0 < cnt; u0 += kSrpBatch) {
+                float vb[kSrpBatch];
+#pragma unroll
+                for (int b = 0; b < kSrpBatch; ++b) {
+                    const uint32_t ix = __shfl_sync(kFull, my_ix, (u0 + b) & 31);
+                    vb[b] = __shfl_sync(kFull, my_v, (u0 + b) & 31);
+                    c.load(b, Rc + (size_t)ix * A.bits);
+                }
+#pragma unroll
+                for (int b = 0; b < kSrpBatch; ++b) {
+                    if constexpr (sizeof(RT) == 2) c.add(b, vb[b], mag2);
+                    else c.add(b, vb[b], mag);
+                }
+            }
+            c.end_block();
+        }
+        float t[CPL];
+        c.totals(t);
+        if constexpr (sizeof(RT) == 2) {
+#pragma unroll
+            for (int i = 0; i < CPL / 2; ++i) f2_unpack(mag2[i], mag[2 * i], mag[2 * i + 1]);
+        }
+#pragma unroll
+        for (int i = 0; i < CPL; ++i) {
+            s_tot[warp][CPL * lane + i] = t[i];
+            s_mag[warp][CPL * lane + i] = mag[i];
+        }
+        __syncthreads();
+        if (threadIdx.x < PC) {
+            float tt = 0.0f, mm = 0.0f;
+#pragma unroll
+            for (int w = 0; w < 8; ++w) {
+                tt = __fadd_rn(tt, s_tot[w][threadIdx.x]);
+                mm = __fadd_rn(mm, s_mag[w][threadIdx.x]);
+            }
+            // the row length through a 32-bit integer; rows past 2^30 count as 2^30, which is too long
+            const int len32 = (int)(len < (1ll << 30) ? len : (1ll << 30));
+            const float n = (float)len32;
+            const bool too_long = n * 5.9604644775390625e-8f > 0.05f;   // the 1.25 slack needs n u <= 0.05
+            const float chain = 40.0f + (float)((len32 + 255) >> 8);
+            bool bit = tt >= 0.0f;
+            if (too_long || !(fabsf(tt) > srp_bound(chain, mm, n)))
+                bit = srp_undecided<RT>(A, R, row, s, s + len, col0 + (int)threadIdx.x, rechecked, zeros);
+            const unsigned word = __ballot_sync(kFull, bit);
+            if (lane == 0) A.sig[(size_t)row * words + (col0 >> 5) + warp] = word;
+        }
+    }
+    if (bad) blsh_dev_error(A.scratch, BLSH_ERANGE, 0, bad);
+    if (rechecked) atomicAdd(&A.scratch->counters[2], rechecked);
+    if (zeros) atomicAdd(&A.scratch->counters[3], zeros);
 }
 
 // The queued signs: one warp per (row, bit).  The lanes form the row's exact
@@ -660,10 +812,6 @@ __global__ void __launch_bounds__(256) srp_recheck_kernel(const uint2 *__restric
     if (lane == 0 && done) atomicAdd(&scratch->counters[2], done);
     if (lane == 0 && zeros) atomicAdd(&scratch->counters[3], zeros);
 }
-
-// Sign random projections with R stored in two bytes per entry (Section 4.3,
-// "Cheaper storage of hash functions").  Thread t owns the groups of 8 bits
-// t, t+T, ...: one 16-byte load brings the 8 codes of a group for a nonzero.
 
 // Two-byte codes of Gaussian samples (Section 4.3): q = floor((x + 8) 2^12),
 // formed as floor(x 2^12) + 2^15 (exact in FP32).  Codes outside [0, 65535]
@@ -846,77 +994,67 @@ __global__ void __launch_bounds__(256) srp_dense_simt_kernel(const float *__rest
     if (zeros) atomicAdd(&scratch->counters[3], zeros);
 }
 
-// Columns [col0, col0 + ncols) of the sparse projection (multiples of 128)
-// for the rows row_mask selects, on the 16-byte path (R float or two-byte
-// codes); -1 when that path does not take the shape.
-template <typename RT>
-int srp_sparse_cols(blsh_ctx *ctx, const int64_t *indptr, const uint32_t *indices, const float *values, int64_t N,
-                    const RT *R, int64_t dim, int bits, int col0, int ncols, const uint8_t *row_mask,
-                    uint32_t *sig, cudaStream_t s) {
-    // selected rows (usually few): pieces of 512 columns, one per CTA; all
-    // rows: the whole range per CTA.  T4 = 32 wt threads, V = groups / T4
-    // groups of four columns per thread: for two-byte codes the fewest warps
-    // that give every thread at most two groups (each nonzero's shuffles and
-    // address then serve eight columns: measured faster, e.g. one warp per
-    // row for 256 columns), otherwise the largest divisor of groups/32 up to 8
-    const int piece = row_mask && ncols % 512 == 0 ? 512 : ncols;
-    const int pieces = ncols / piece;
-    const int groups = piece / 4;
-    int wt = 0;
-    if (sizeof(RT) == 2)
-        for (int c = 1; c <= 8 && !wt; ++c)
-            if ((groups / 32) % c == 0 && groups / (32 * c) <= 2) wt = c;
-    if (!wt) {
-        wt = 8;
-        while ((groups / 32) % wt) --wt;
-    }
-    const int T4 = 32 * wt, V = groups / T4;
-    if (V < 1 || V > 4) return -1;
-    // many small CTAs (rows have very different lengths): 32 per SM measured best
-    const long long cap = (long long)ctx->sm_count * 32;
-    const unsigned grid = (unsigned)(N * pieces < cap ? N * pieces : cap);
-    // items from a counter where each CTA has many of them (at least 256;
-    // otherwise a fixed share per CTA): kSrpGrab per grab, eight times as
-    // many when a row mask selects the rows (most items of a grab are then
-    // skipped at once)
-    const int grab = N * pieces >= 256ll * grid ? (row_mask ? 8 * kSrpGrab : kSrpGrab) : 0;
-    BLSH_CUDA(ctx, cudaMemsetAsync(&ctx->scratch->recheck_count, 0, sizeof(unsigned long long), s));
-    BLSH_CUDA(ctx, cudaMemsetAsync(&ctx->scratch->hash_work, 0, sizeof(unsigned long long), s));
-    uint2 *q = ctx->recheck_queue;
+// Columns [col0, col0 + ncols) of the sparse projection (multiples of 128) for
+// the rows row_mask selects, on the aligned path.
+template <typename RT, int CPL>
+int srp_sparse_pieces(blsh_ctx *ctx, const int64_t *indptr, const uint32_t *indices, const float *values, int64_t N,
+                      const RT *R, int64_t dim, int bits, int col0, int ncols, const uint8_t *row_mask,
+                      uint32_t *sig, cudaStream_t s) {
+    const int pieces = ncols / (32 * CPL);
+    const long long warps = (long long)ctx->sm_count * 32;   // about the resident ones
+    SrpArgs A;
+    A.indptr = indptr;
+    A.indices = indices;
+    A.values = values;
+    A.N = N;
+    A.dim = dim;
+    A.bits = bits;
+    A.col_first = col0;
+    A.row_mask = row_mask;
+    A.sig = sig;
+    A.scratch = ctx->scratch;
+    A.queue = ctx->recheck_queue;
+    A.longs = ctx->lite_queue;
+    // piece by piece over all the rows where R's columns exceed half of L2, or
+    // where there are too few rows to give every warp several
+    const bool by_piece = (!row_mask && (double)dim * ncols * sizeof(RT) > 64e6) || N < 8 * warps;
+    A.outer = by_piece ? pieces : 1;
+    A.inner = by_piece ? 1 : pieces;
+    // rows a grab: up to 32, at least eight grabs a warp
+    int G = 32;
+    while (G > 1 && (N / G) * A.outer < 8 * warps) G >>= 1;
     blsh_dev_scratch *scr = ctx->scratch;
+    // work2 (next long row), work3 (long rows listed), recheck_count .. hash_work
+    BLSH_CUDA(ctx, cudaMemsetAsync(&scr->work2, 0, offsetof(blsh_dev_scratch, norm2_valid) -
+                                                       offsetof(blsh_dev_scratch, work2), s));
     const char *name = sizeof(RT) == 2 ? "srp_sparse4_kernel (two-byte codes)" : "srp_sparse4_kernel";
+    const long long blocks = ((N + G - 1) / G * A.outer + 7) / 8, most = (long long)ctx->sm_count * 8;
     blsh_time_start(ctx, s);
-    switch (V) {
-    case 1: srp_sparse4_kernel<1, RT><<<grid, T4, 0, s>>>(indptr, indices, values, N, R, dim, bits, col0, pieces, row_mask, sig, scr, q, grab); break;
-    case 2: srp_sparse4_kernel<2, RT><<<grid, T4, 0, s>>>(indptr, indices, values, N, R, dim, bits, col0, pieces, row_mask, sig, scr, q, grab); break;
-    case 3: srp_sparse4_kernel<3, RT><<<grid, T4, 0, s>>>(indptr, indices, values, N, R, dim, bits, col0, pieces, row_mask, sig, scr, q, grab); break;
-    default: srp_sparse4_kernel<4, RT><<<grid, T4, 0, s>>>(indptr, indices, values, N, R, dim, bits, col0, pieces, row_mask, sig, scr, q, grab); break;
-    }
+    srp_sparse4_kernel<RT, CPL><<<(unsigned)(blocks < most ? blocks : most), 256, 0, s>>>(A, R, G);
     BLSH_LAUNCHED(ctx, name);
     blsh_time_start(ctx, s);
-    srp_recheck_kernel<RT><<<ctx->sm_count * 4, 256, 0, s>>>(q, indptr, indices, values, R, dim, bits, sig, scr);
+    srp_long_kernel<RT, CPL><<<ctx->sm_count * 4, 256, 0, s>>>(A, R);
+    BLSH_LAUNCHED(ctx, name);
+    blsh_time_start(ctx, s);
+    srp_recheck_kernel<RT><<<ctx->sm_count * 4, 256, 0, s>>>(ctx->recheck_queue, indptr, indices, values, R, dim, bits,
+                                                             sig, scr);
     BLSH_LAUNCHED(ctx, "srp_recheck_kernel");
     return BLSH_OK;
 }
 
-// Column ranges the kernel cannot take in one launch (col_count / 128 with no
-// divisor in 1..8 that leaves at most 4 groups per thread) are split: the
-// largest piece it can take first, and so on (128 columns always can).
-template <typename RT>
-int srp_sparse_range(blsh_ctx *ctx, const int64_t *indptr, const uint32_t *indices, const float *values, int64_t N,
-                     const RT *R, int64_t dim, int bits, int col_begin, int col_count, const uint8_t *row_mask,
-                     uint32_t *sig, cudaStream_t s) {
-    for (int c0 = col_begin, left = col_count; left > 0;) {
-        int rc = -1, piece = left;
-        for (; piece > 0; piece -= 128) {
-            rc = srp_sparse_cols<RT>(ctx, indptr, indices, values, N, R, dim, bits, c0, piece, row_mask, sig, s);
-            if (rc != -1) break;
-        }
-        if (rc != BLSH_OK) return rc == -1 ? blsh_fail(ctx, BLSH_EINVAL, "no launch shape") : rc;
-        c0 += piece;
-        left -= piece;
-    }
-    return BLSH_OK;
+int srp_sparse_cols(blsh_ctx *ctx, const int64_t *indptr, const uint32_t *indices, const float *values, int64_t N,
+                    const float *R, int64_t dim, int bits, int col0, int ncols, const uint8_t *row_mask,
+                    uint32_t *sig, cudaStream_t s) {
+    return srp_sparse_pieces<float, 4>(ctx, indptr, indices, values, N, R, dim, bits, col0, ncols, row_mask, sig, s);
+}
+int srp_sparse_cols(blsh_ctx *ctx, const int64_t *indptr, const uint32_t *indices, const float *values, int64_t N,
+                    const uint16_t *R, int64_t dim, int bits, int col0, int ncols, const uint8_t *row_mask,
+                    uint32_t *sig, cudaStream_t s) {
+    // eight codes a lane where the pieces and the alignment allow it
+    if (ncols % 256 == 0 && blsh_aligned(R, 16))
+        return srp_sparse_pieces<uint16_t, 8>(ctx, indptr, indices, values, N, R, dim, bits, col0, ncols, row_mask, sig,
+                                              s);
+    return srp_sparse_pieces<uint16_t, 4>(ctx, indptr, indices, values, N, R, dim, bits, col0, ncols, row_mask, sig, s);
 }
 
 int srp_threads(int bits, int *per_thread) {
@@ -998,10 +1136,8 @@ extern "C" int blsh_srp_sparse(blsh_ctx *ctx, const int64_t *indptr, const uint3
     // many small CTAs (rows have very different lengths): 32 per SM measured best
     const long long cap = (long long)ctx->sm_count * 32;
     const unsigned grid = (unsigned)(N < cap ? N : cap);
-    if (bits % 128 == 0 && blsh_aligned(R, 16)) {
-        const int rc = srp_sparse_cols<float>(ctx, indptr, indices, values, N, R, dim, bits, 0, bits, nullptr, sig, s);
-        if (rc != -1) return rc;
-    }
+    if (bits % 128 == 0 && blsh_aligned(R, 16))
+        return srp_sparse_cols(ctx, indptr, indices, values, N, R, dim, bits, 0, bits, nullptr, sig, s);
     blsh_time_start(ctx, s);
     srp_sparse_kernel<float><<<grid, T, 0, s>>>(indptr, indices, values, N, R, dim, bits, per_thread, sig, ctx->scratch);
     BLSH_LAUNCHED(ctx, "srp_sparse_kernel");
@@ -1071,7 +1207,7 @@ extern "C" int blsh_srp_sparse_cols(blsh_ctx *ctx, const int64_t *indptr, const 
     if (!blsh_aligned(indptr, 8) || !blsh_aligned(R, 16)) return blsh_fail(ctx, BLSH_EINVAL, "misaligned pointer");
     if (N == 0) return BLSH_OK;
     blsh_device_guard g(ctx->device);
-    return srp_sparse_range<float>(ctx, indptr, indices, values, N, R, dim, bits, col_begin, col_count, row_mask,
+    return srp_sparse_cols(ctx, indptr, indices, values, N, R, dim, bits, col_begin, col_count, row_mask,
                                    sig, blsh_stream(stream));
 }
 
@@ -1088,7 +1224,7 @@ extern "C" int blsh_srp_sparse_q16_cols(blsh_ctx *ctx, const int64_t *indptr, co
     if (!blsh_aligned(indptr, 8) || !blsh_aligned(Rq, 8)) return blsh_fail(ctx, BLSH_EINVAL, "misaligned pointer");
     if (N == 0) return BLSH_OK;
     blsh_device_guard g(ctx->device);
-    return srp_sparse_range<uint16_t>(ctx, indptr, indices, values, N, Rq, dim, bits, col_begin, col_count, row_mask,
+    return srp_sparse_cols(ctx, indptr, indices, values, N, Rq, dim, bits, col_begin, col_count, row_mask,
                                       sig, blsh_stream(stream));
 }
 
@@ -1107,7 +1243,7 @@ extern "C" int blsh_srp_sparse_q16(blsh_ctx *ctx, const int64_t *indptr, const u
     const long long cap = (long long)ctx->sm_count * 32;
     const unsigned grid = (unsigned)(N < cap ? N : cap);
     if (bits % 128 == 0 && blsh_aligned(Rq, 8))   // 8-byte loads of four codes
-        return srp_sparse_range<uint16_t>(ctx, indptr, indices, values, N, Rq, dim, bits, 0, bits, nullptr, sig, s);
+        return srp_sparse_cols(ctx, indptr, indices, values, N, Rq, dim, bits, 0, bits, nullptr, sig, s);
     int per_thread;
     const int T = srp_threads(bits, &per_thread);
     if (per_thread > kSrpMaxPerThread) return blsh_fail(ctx, BLSH_EINVAL, "bits/32 needs a divisor in 2..8");

@@ -1,0 +1,54 @@
+"""GPU parity of the sparse projection on both sides of its rules: rows around
+the lengths at which a block of 32 and the long rows' kernel begin, few rows
+(handed out singly, piece by piece) and many (several a grab, all pieces of a
+row together), four and eight columns a lane, and malformed indices, which
+contribute nothing and are reported.  Bit-exact against the CPU oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+import synth
+
+pytestmark = pytest.mark.gpu
+dev = torch.device("cuda")
+EDGES = [0, 1, 7, 8, 9, 31, 32, 33, 64, 65, 255, 256, 257, 287, 511, 512, 513, 2049, 9000]
+
+
+def rows(n, dim, seed):
+    rng = np.random.default_rng(seed)
+    lens = rng.integers(0, 6, n)
+    lens[rng.choice(n, len(EDGES), replace=False)] = EDGES
+    indptr = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    ix = rng.integers(0, dim, indptr[-1]).astype(np.uint32)
+    return synth.CSR(indptr, ix, rng.standard_normal(indptr[-1]).astype(np.float32), dim)
+
+
+@pytest.mark.parametrize("n", [60, 40_000, 90_000])
+@pytest.mark.parametrize("form, bits", [("float", 256), ("codes", 384), ("codes", 512), ("codes on 8 bytes", 512)])
+def test_srp_rows(B, ctx, n, form, bits):
+    dim = 3000
+    csr = rows(n, dim, n + bits)
+    bad = csr.indices.copy()
+    drop = np.zeros(len(bad), bool)
+    drop[::97] = True
+    drop[int(csr.indptr[np.argmax(np.diff(csr.indptr))]) + 300] = True   # past a long row's first round of blocks
+    bad[drop] = np.where(np.arange(drop.sum()) % 2, dim, 2**32 - 1).astype(np.uint32)
+    kept = np.concatenate([[0], np.cumsum(~drop)])[csr.indptr].astype(np.int64)
+    clean = synth.CSR(kept, csr.indices[~drop], csr.values[~drop], dim)
+    ip, val = torch.from_numpy(csr.indptr).to(dev), torch.from_numpy(csr.values).to(dev)
+    sig = torch.zeros((n, bits // 32), dtype=torch.int32, device=dev)
+    if form == "float":
+        R = synth.gaussian_matrix(dim, bits, seed=5)
+        Rd, oracle, call = torch.from_numpy(R).to(dev), O.srp_sparse, B.blsh_srp_sparse
+    else:
+        R = O.gaussian_codes(5, dim, bits)
+        off = 4 if form.endswith("8 bytes") else 0
+        store = torch.zeros(R.size + off, dtype=torch.int16, device=dev)
+        Rd = store[off:].view(dim, bits)
+        Rd.copy_(torch.from_numpy(R.view(np.int16)))
+        oracle, call = O.srp_sparse_q16, B.blsh_srp_sparse_q16
+    for indices, want, rc in ((csr.indices, oracle(csr, R), 0), (bad, oracle(clean, R), B.ERANGE)):
+        call(ctx, ip, torch.from_numpy(indices.view(np.int32)).to(dev), val, Rd, sig)
+        assert B.blsh_status(ctx) == rc
+        assert np.array_equal(sig.cpu().numpy().view(np.uint32), want)
