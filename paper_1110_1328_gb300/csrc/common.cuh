@@ -154,6 +154,28 @@ struct blsh_device_guard {
 
 static inline cudaStream_t blsh_stream(void *s) { return (cudaStream_t)s; }
 
+// Paired FP32 arithmetic (two lanes of a 64-bit register per instruction,
+// each an IEEE single-precision operation rounded to nearest).
+__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void f2_unpack(unsigned long long p, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p));
+}
+__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
+                                                     unsigned long long c) {
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 // Statuses (one byte each) equal to `val` among the 16 bytes of v: bit i of
 // the result for byte i.  Per 32-bit word, x = w ^ (val in every byte); the
 // high bit of a byte of ~(((x & 0x7f..) + 0x7f..) | x) is set exactly when

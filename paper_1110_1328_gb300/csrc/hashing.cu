@@ -315,28 +315,6 @@ __device__ __noinline__ double srp_recheck_fp64(const uint32_t *__restrict__ ind
     return d;
 }
 
-// Paired FP32 arithmetic (two lanes of a 64-bit register per instruction,
-// each an IEEE single-precision operation rounded to nearest): the two-byte
-// projection's decode, sum and magnitude for two columns at a time.
-__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-    return r;
-}
-__device__ __forceinline__ void f2_unpack(unsigned long long p, float &lo, float &hi) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p));
-}
-__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
-                                                     unsigned long long c) {
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
 // The two codes of a 32-bit word as the pair (2^23 + low code, 2^23 + high
 // code): each code's bits placed under the exponent of 2^23.
 __device__ __forceinline__ unsigned long long f2_codes(uint32_t w) {

@@ -14,8 +14,9 @@
 //      thread issues tcgen05.mma (BF16 x BF16 -> FP32 in tensor memory) for
 //      hi*hi, hi*lo and lo*hi into one of two accumulators; four epilogue
 //      warps read the other accumulator back (tcgen05.ld) and set a bit
-//      wherever |p| > margin * |x_i| * |r_j|, queueing every other sign.
-//   3. srp_dense_recheck_kernel: each queued sign is recomputed in FP32 with a
+//      wherever |p| > margin * |x_i| * |r_j|, marking every other sign in a
+//      bit map.
+//   3. srp_dense_recheck_kernel: each marked sign is recomputed in FP32 with a
 //      rigorous error bound, then in FP64 with one, and, if neither can decide
 //      it, as the FP64 sum over coordinates 0..d-1 in order -- the oracle's
 //      definition -- so every bit is exact whenever the margin bounds the
@@ -28,7 +29,7 @@
 // A width that is no multiple of 64 takes the same path since the padding
 // costs at most one K stage, while the CUDA cores need 2 d operations a sign
 // at 1/50 of the tensor rate: 99,991 x 300 x 1,024 bits took 36.4 ms on the
-// CUDA cores' kernel of that time, 332 us here.
+// CUDA cores' kernel of that time, 297 us here.
 //
 // Every other shape uses srp_dense_simt_kernel (hashing.cu): FP32 sums with
 // the same kind of bound and an FP64 recheck.
@@ -62,8 +63,7 @@ __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)_
 
 // ---- preparation --------------------------------------------------------------
 
-// One launch prepares both operands and clears the recheck queue's count: the
-// first r_blocks CTAs take 32 columns of R each, the others the rows of X.
+// One launch prepares both operands: the first r_blocks CTAs take 32 columns of R each, the others the rows of X.
 //
 // R: a CTA walks K in stages of 64: a 64 x 32 tile is read in 128-byte rows,
 // turned in shared memory, and each thread writes eight K values of a column
@@ -76,14 +76,16 @@ __device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)_
 // consecutive values a lane at a time (VEC: d a multiple of 4, so that every
 // row starts on 16 bytes).
 // xnorm, rnorm: |x_i|, |r_j| in FP32 rounded up, infinity outside
-// [1e-15, 1e18] (norm_or_inf): inside it no partial sum of the tensor cores
-// can overflow (each is at most |x_i| |r_j| <= 1e36) and no underflow of a
-// split or a product comes near margin |x_i| |r_j| >= 3e-34; outside it an
-// infinite bound sends every sign to the recheck.
+// [1e-30, 1e18] (norm_or_inf), where an infinite bound sends every sign to the
+// recheck.  Up to 1e18 no partial sum of the tensor cores can overflow (each is
+// at most |x_i| |r_j| <= 1e36); down to 1e-30 what an operand's split loses to
+// underflow is below 2^-20 of its norm.  A product's underflow stays far below
+// margin |x_i| |r_j| while |x_i| |r_j| >= 1e-30 (margin >= 3e-4: 3e-34), which
+// the epilogue asks of a row and the smallest column.
 constexpr int kPrepCols = 32;
 __device__ __forceinline__ float norm_or_inf(float ss) {
-    const float n = __fsqrt_ru(ss) * 1.0001f;
-    return n >= 1e-15f && n <= 1e18f ? n : INFINITY;
+    const float n = __fsqrt_ru(ss) * 1.0001f;   // (ss: squares added upwards, so never too small)
+    return n >= 1e-30f && n <= 1e18f ? n : INFINITY;
 }
 
 template <bool VEC>
@@ -91,11 +93,10 @@ __global__ void __launch_bounds__(256) srp_dense_prep(
     const float *__restrict__ X, long long N, long long Npad, int d, int KT, unsigned char *__restrict__ Xh,
     unsigned char *__restrict__ Xl, float *__restrict__ xnorm, const float *__restrict__ R, int bits,
     unsigned char *__restrict__ Rh, unsigned char *__restrict__ Rl, float *__restrict__ rnorm,
-    float *__restrict__ Rt, int r_blocks, unsigned long long *qcount) {
+    float *__restrict__ Rt, int r_blocks) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if ((int)blockIdx.x < r_blocks) {
         __shared__ float tile[BK][kPrepCols + 1];
-        if (blockIdx.x == 0 && threadIdx.x == 0) *qcount = 0ull;
         const int j0 = blockIdx.x * kPrepCols;
         const int c = threadIdx.x >> 3, q = threadIdx.x & 7;   // this thread's column and 16-byte chunk
         const int j = j0 + c;
@@ -244,25 +245,6 @@ __device__ __forceinline__ void tmem_ld32(unsigned taddr, float (&v)[32]) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// A sign the tensor-core margin cannot decide, when the recheck queue is
-// full: FP32 with its bound, else the FP64 sum in coordinate order.
-__device__ __noinline__ bool sign_in_line(const float *__restrict__ x, const float *__restrict__ R, int d, int bits,
-                                          int col, blsh_dev_scratch *scratch) {
-    atomicAdd(&scratch->counters[2], 1ull);
-    float acc = 0.0f, mag = 0.0f;
-    for (int c = 0; c < d; ++c) {
-        const float a = __ldg(x + c), b = __ldg(R + (size_t)c * bits + col);
-        acc = __fmaf_rn(a, b, acc);
-        mag = __fmaf_rn(fabsf(a), fabsf(b), mag);
-    }
-    const float bound = 1.25f * (float)d * 5.9604644775390625e-8f * mag + (float)d * 1.4e-45f;
-    if (fabsf(acc) > bound) return acc >= 0.0f;
-    double s = 0.0;
-    for (int c = 0; c < d; ++c) s += (double)__ldg(x + c) * (double)__ldg(R + (size_t)c * bits + col);
-    if (s == 0.0) atomicAdd(&scratch->counters[3], 1ull);
-    return s >= 0.0;
-}
-
 // ---- the persistent, warp-specialised tensor-core kernel -------------------------
 //
 // One CTA per SM walks the tiles t = blockIdx.x, blockIdx.x + gridDim.x, ...
@@ -275,7 +257,7 @@ __device__ __noinline__ bool sign_in_line(const float *__restrict__ x, const flo
 //   warps 2-9 epilogue: warp w reads TMEM lanes 32 (w % 4) .. +31 (rows of
 //           the tile) in columns 128 ((w - 2) / 4) .. +127, tests each value
 //           against margin |x_i| |r_j| (margin |r_j| staged in shared memory
-//           for all bits), writes the decided bits and queues the others.
+//           for all bits), writes the decided bits and marks the others.
 // Barriers: full/empty per ring stage (bulk-copy bytes / MMA commit), and
 // acc_full/acc_empty per accumulator (MMA commit / 128 epilogue arrivals).
 // Every wait is bounded; a role that gives up records the failure and
@@ -290,8 +272,7 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long *bar) {
 __global__ void __launch_bounds__(kTcThreads, 1) srp_dense_tc_persistent(
     const unsigned char *__restrict__ Xh, const unsigned char *__restrict__ Xl, const unsigned char *__restrict__ Rh,
     const unsigned char *__restrict__ Rl, const float *__restrict__ xnorm, const float *__restrict__ rnorm,
-    long long N, int d, int bits, float margin, uint32_t *__restrict__ sig, uint2 *__restrict__ queue,
-    unsigned long long qcap, unsigned long long *qcount, const float *__restrict__ X, const float *__restrict__ R,
+    long long N, int d, int bits, float margin, uint32_t *__restrict__ sig, uint32_t *__restrict__ und,
     long long tiles_total, blsh_dev_scratch *scratch) {
     extern __shared__ __align__(1024) unsigned char dyn_smem[];
     unsigned char *ring = reinterpret_cast<unsigned char *>(((uintptr_t)dyn_smem + 1023) & ~(uintptr_t)1023);
@@ -403,6 +384,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) srp_dense_tc_persistent(
         const int ew = warp & 3;                  // TMEM lanes 32 ew .. 32 ew + 31
         const int half = (warp - 2) >> 2;         // columns 128 half .. 128 half + 127
         const int words = bits >> 5;
+        const bool sig16 = ((uintptr_t)sig & 15) == 0;
+        float mr_min = INFINITY;
+        for (int j = lane; j < bits; j += 32) mr_min = fminf(mr_min, s_mr[j]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mr_min = fminf(mr_min, __shfl_xor_sync(kFull, mr_min, o));
         long long tc = 0;
         for (long long t = blockIdx.x; t < tiles_total && !s_fail; t += gridDim.x, ++tc) {
             const long long mt = t / tiles_n;
@@ -415,57 +401,37 @@ __global__ void __launch_bounds__(kTcThreads, 1) srp_dense_tc_persistent(
             }
             fence_after();
             const long long row = mt * BM + ew * 32 + lane;
-            const float xn = row < N ? __ldg(xnorm + row) : 0.0f;
-            constexpr int kBuf = 8;
-            unsigned short pend[kBuf];
-            int npend = 0;
-            for (int c = half * 4; c < half * 4 + 4; ++c) {
+            float xn = row < N ? __ldg(xnorm + row) : 0.0f;
+            if (!(xn * mr_min >= margin * 1e-30f)) xn = INFINITY;
+            uint32_t word[4], mark[4];
+#pragma unroll
+            for (int cc = 0; cc < 4; ++cc) {
+                const int c = half * 4 + cc;
                 float v[32];
                 tmem_ld32(tmem + ((unsigned)(ew * 32) << 16) + (unsigned)(buf * BN + c * 32), v);
                 const float *mr = s_mr + nt * BN + c * 32;
-                uint32_t word = 0, und = 0;
+                uint32_t w = 0, u = 0;
 #pragma unroll
                 for (int i = 0; i < 32; ++i) {
-                    word |= (uint32_t)(v[i] >= 0.0f) << i;
-                    und |= (uint32_t)!(fabsf(v[i]) > xn * mr[i]) << i;   // inside the margin (or NaN): recheck
+                    w |= (uint32_t)(v[i] >= 0.0f) << i;
+                    u |= (uint32_t)!(fabsf(v[i]) > xn * mr[i]) << i;   // inside the margin (or NaN): recheck
                 }
-                if (row < N) {
-                    word &= ~und;
-                    for (uint32_t u = und; u; u &= u - 1) {
-                        const int i = __ffs(u) - 1;
-                        if (npend < kBuf) {
-                            pend[npend++] = (unsigned short)(c * 32 + i);
-                        } else {
-                            word |= (uint32_t)sign_in_line(X + (size_t)row * d, R, d, bits, nt * BN + c * 32 + i,
-                                                           scratch) << i;
-                        }
-                    }
-                    sig[(size_t)row * words + nt * (BN / 32) + c] = word;
+                word[cc] = w & ~u;
+                mark[cc] = u;
+            }
+            if (row < N) {
+                const size_t at = (size_t)row * words + nt * (BN / 32) + half * 4;
+                if (sig16) {
+                    *reinterpret_cast<uint4 *>(sig + at) = make_uint4(word[0], word[1], word[2], word[3]);
+                } else {
+#pragma unroll
+                    for (int cc = 0; cc < 4; ++cc) sig[at + cc] = word[cc];
                 }
+                *reinterpret_cast<uint4 *>(und + at) = make_uint4(mark[0], mark[1], mark[2], mark[3]);
             }
             // the accumulator may be overwritten now
             fence_before();
             mbar_arrive(&acc_empty[buf]);
-            // warp-aggregated append of the undecided signs: one atomic per warp
-            int incl = npend;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(kFull, incl, o);
-                if (lane >= o) incl += y;
-            }
-            const int wtotal = __shfl_sync(kFull, incl, 31);
-            unsigned long long base = 0;
-            if (lane == 0 && wtotal) base = atomicAdd(qcount, (unsigned long long)wtotal);
-            base = __shfl_sync(kFull, base, 0);
-            for (int p = 0; p < npend; ++p) {
-                const unsigned long long slot = base + (unsigned long long)(incl - npend + p);
-                const int col = nt * BN + pend[p];
-                if (slot < qcap) {
-                    queue[slot] = make_uint2((uint32_t)row, (uint32_t)col);
-                } else if (sign_in_line(X + (size_t)row * d, R, d, bits, col, scratch)) {
-                    atomicOr(sig + (size_t)row * words + (col >> 5), 1u << (col & 31));
-                }
-            }
         }
     }
     fence_before();
@@ -475,130 +441,282 @@ __global__ void __launch_bounds__(kTcThreads, 1) srp_dense_tc_persistent(
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
 }
 
-// Queued signs: eight lanes per (row, bit).  Three stages, each with a
-// rigorous bound:
-//   FP32 partial sums, lane g of the group taking the 16-byte pieces 8i + g
-//   of both rows into four chains of at most ceil(d/32) FMAs, joined by two
-//   and then three additions: no term passes through more than
-//   ceil(d/32) + 5 roundings, so the sum errs by at most that many u sum|p|;
-//   if undecided, FP64 partial sums of the exact products, lane g owning
-//   coordinates [g per, (g+1) per), per = ceil(d/8) (error at most
-//   (d+8) 2^-53 sum|p|, so a sign it decides is the sign of the exact sum and
-//   of the oracle's sum, which errs by less);
-//   if still undecided (exact ties such as zero rows), the FP64 sum over
-//   coordinates 0..d-1 in order, lane g continuing lane g-1's running sum --
-//   exactly the oracle's sum.
-// The FP64 stage costs a warp about fifty times the FP32 one (the FP64 pipe is
-// narrow) and runs when any of its four signs needs it, so the first bound
-// decides the time: counting the chains' own lengths instead of d + 8
-// roundings leaves 1/19 as many signs at d = 256.  1e6 x 256 x 1,024 bits with
-// the margin 1e-3 (1.3e7 queued signs): 2,374 us before, 2,077 now (the gathers of 2 KB a sign are left).
-// VEC: d a multiple of 4 (16-byte loads of X).
-template <bool VEC>
-__global__ void __launch_bounds__(256) srp_dense_recheck_kernel(const uint2 *__restrict__ queue,
-                                                                unsigned long long qcap,
-                                                                const unsigned long long *qcount,
-                                                                const float *__restrict__ X,
-                                                                const float *__restrict__ Rt, int d, int ldr, int bits,
-                                                                uint32_t *__restrict__ sig,
-                                                                blsh_dev_scratch *scratch) {
-    const unsigned long long total = *qcount;
-    const unsigned long long n = total < qcap ? total : qcap;
-    const int lane = threadIdx.x & 31, g = lane & 7;
-    const int per = (d + 7) >> 3;   // coordinates per lane of the FP64 stages
-    const int lo = g * per < d ? g * per : d, hi = lo + per < d ? lo + per : d;
-    const float roundings = (float)((d + 31) / 32 + 6);
-    const unsigned long long groups = (unsigned long long)gridDim.x * (blockDim.x >> 3);
-    unsigned long long done = 0, zeros = 0;
-    const unsigned long long warp_first = (((unsigned long long)blockIdx.x * blockDim.x + threadIdx.x) >> 3) & ~3ull;
-    for (unsigned long long it0 = warp_first; it0 < n; it0 += groups) {
-        const unsigned long long it = it0 + (unsigned long long)(lane >> 3);
-        const bool live = it < n;
-        uint2 rj = make_uint2(0u, 0u);
-        if (live) rj = queue[it];
-        const float *xr = X + (size_t)rj.x * d, *rr = Rt + (size_t)rj.y * ldr;
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f;
-        // the group's eight lanes read 128 contiguous bytes of each row per
-        // step (lane g the 16 bytes at 4 (8 i + g))
-        if (live)
-#pragma unroll 4
-            for (int c = 4 * g; c < d; c += 32) {
-                float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (VEC) {
-                    u = __ldg(reinterpret_cast<const float4 *>(xr + c));
-                } else {
-                    u.x = __ldg(xr + c);
-                    if (c + 1 < d) u.y = __ldg(xr + c + 1);
-                    if (c + 2 < d) u.z = __ldg(xr + c + 2);
-                    if (c + 3 < d) u.w = __ldg(xr + c + 3);
-                }
-                const float4 v = __ldg(reinterpret_cast<const float4 *>(rr + c));   // zeros past d
-                a0 = __fmaf_rn(u.x, v.x, a0); a1 = __fmaf_rn(u.y, v.y, a1);
-                a2 = __fmaf_rn(u.z, v.z, a2); a3 = __fmaf_rn(u.w, v.w, a3);
-                m0 = __fmaf_rn(fabsf(u.x), fabsf(v.x), m0); m1 = __fmaf_rn(fabsf(u.y), fabsf(v.y), m1);
-                m2 = __fmaf_rn(fabsf(u.z), fabsf(v.z), m2); m3 = __fmaf_rn(fabsf(u.w), fabsf(v.w), m3);
-            }
-        float acc = (a0 + a1) + (a2 + a3), mag = (m0 + m1) + (m2 + m3);
+// The marked signs.  An item is the marks of kPartRows rows in kPartWords
+// words (kPartCols columns): a lane a word.  They are listed in shared memory
+// row by row, and the warp forms four sums at a time: lane l takes coordinates
+// 4 l .. 4 l + 3 of every 128 of x_i (kept in registers for all of the row's
+// signs where d <= 256) and of the four columns, paired FMAs, and the four sums
+// meet in six shuffles.  Three stages, each with a rigorous bound:
+//   FP32: no term passes through more than 2 ceil(d/128) + 6 roundings, so the
+//   sum errs by at most that many u |x_i| |r_j| (norms rounded up; infinite
+//   where they could over- or underflow), or, if that does not decide, u sum|p|
+//   of the same chains;
+//   then FP64 partial sums of the exact products, a lane's coordinates l, l + 32, ...
+//   (error at most (d/32 + 6) 2^-53 sum|p|: a sign it decides is the sign of
+//   the exact sum and of the oracle's sum, which errs by less than d 2^-53
+//   sum|p|); a sum that is not finite, or of products that are all zero, is the
+//   same in every order;
+//   the rest, exact ties, as the FP64 sum over coordinates 0..d-1 in order --
+//   exactly the oracle's sum -- a lane each.  A zero row's sums need no FP64.
+//
+// What bounds it: the reads of the columns, 4 d bytes a sign, from L2 and L1.
+// A queue of (row, bit) entries, eight lanes each, read x_i as well for every
+// sign: 2,077 us for the 1.3e7 signs that 1e6 x 256 x 1,024 bits leave inside
+// the margin 1e-3, and the queue's appends cost the tensor-core kernel 200 us
+// (1,049 us, with marks 840 us); where most signs were ties it overflowed and
+// the epilogue summed them itself (1% zero rows among 1e5: 51 ms, now 0.3 ms).
+// Here x_i is read once, and the sums take 1,090 us (13 TB/s of columns).
+// Items of 8 words of 4 rows, so that an SM's L1 holds its part of the columns,
+// take 1,695 us: a row's few signs no longer fill a batch.  24 warps of 80
+// registers: with 32 of 64 1,230 us, with 28 1,263 us, with 20 1,137 us; four
+// sums at a time instead of eight 1,311 us.
+constexpr int kReWarps = 24;
+constexpr int kReList = 512;   // signs listed at a time
+
+struct RecheckArgs {
+    const uint32_t *und;
+    const float *X, *Rt, *xnorm, *rnorm;
+    long long N;
+    int d, ldr, bits;
+    int part_words;   // words of a row an item covers: 8, 16 or 32
+    uint32_t *sig;
+    blsh_dev_scratch *scratch;
+};
+
+// coordinates c .. c + 3 of x (zeros past d), as two pairs (CG: not kept in L1)
+template <bool VEC, bool CG>
+__device__ __forceinline__ ulonglong2 x_pairs(const float *__restrict__ x, int c, int d) {
+    ulonglong2 v = make_ulonglong2(0ull, 0ull);
+    if (VEC) {
+        if (c < d) v = CG ? __ldcg(reinterpret_cast<const ulonglong2 *>(x + c)) : __ldg(reinterpret_cast<const ulonglong2 *>(x + c));
+    } else {
+        float a[4];
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) {
-            acc += __shfl_xor_sync(kFull, acc, o);
-            mag += __shfl_xor_sync(kFull, mag, o);
-        }
-        const float bound = 1.25f * roundings * 5.9604644775390625e-8f * mag + (float)(d + 8) * 1.4e-45f;
-        bool decided = !live || fabsf(acc) > bound;
-        bool bit = acc >= 0.0f;
-        if (__any_sync(kFull, !decided)) {
-            double p = 0.0, q = 0.0;
-            if (!decided)
-                for (int c = lo; c < hi; ++c) {
-                    const double t = (double)__ldg(xr + c) * (double)__ldg(rr + c);
-                    p += t;
-                    q += fabs(t);
-                }
-#pragma unroll
-            for (int o = 4; o > 0; o >>= 1) {
-                p += __shfl_xor_sync(kFull, p, o);
-                q += __shfl_xor_sync(kFull, q, o);
-            }
-            const double bound64 = 1.25 * (double)(d + 8) * 1.1102230246251565e-16 * q + (double)(d + 8) * 5e-324;
-            const bool decided64 = decided || fabs(p) > bound64;
-            if (!decided && decided64) bit = p >= 0.0;
-            if (__any_sync(kFull, !decided64)) {
-                double s = 0.0;
-                for (int step = 0; step < 8; ++step) {
-                    if (g == step && !decided64)
-                        for (int c = lo; c < hi; ++c) s += (double)__ldg(xr + c) * (double)__ldg(rr + c);
-                    s = __shfl_sync(kFull, s, (lane & 24) | step);
-                }
-                if (!decided64) {
-                    bit = s >= 0.0;
-                    zeros += (g == 0 && s == 0.0);
-                }
-            }
-        }
-        if (g == 0 && live) {
-            if (bit) atomicOr(sig + (size_t)rj.x * (bits >> 5) + (rj.y >> 5), 1u << (rj.y & 31));
-            ++done;
-        }
+        for (int i = 0; i < 4; ++i) a[i] = c + i >= d ? 0.0f : CG ? __ldcg(x + c + i) : __ldg(x + c + i);
+        v = make_ulonglong2(f2_pack(a[0], a[1]), f2_pack(a[2], a[3]));
     }
-    if (done) atomicAdd(&scratch->counters[2], done);
-    if (zeros) atomicAdd(&scratch->counters[3], zeros);
+    return v;
+}
+
+// The warp's sign of x . r where the norms did not decide it: +1, -1, or 0 for
+// a tie (the ordered sum is needed).  zero: the exact sum is zero.
+template <bool VEC>
+__device__ __noinline__ int sign_by_magnitude(const float *__restrict__ x, const float *__restrict__ r, int d, int ldr,
+                                              float acc, float roundings, bool *zero) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long m2 = 0ull;
+    for (int c = 4 * lane; c < ldr; c += 128) {
+        const ulonglong2 u = x_pairs<VEC, false>(x, c, d), v = __ldg(reinterpret_cast<const ulonglong2 *>(r + c));
+        constexpr unsigned long long kAbs = 0x7fffffff7fffffffull;
+        m2 = f2_fma(u.x & kAbs, v.x & kAbs, m2);
+        m2 = f2_fma(u.y & kAbs, v.y & kAbs, m2);
+    }
+    float m0, m1;
+    f2_unpack(m2, m0, m1);
+    float mag = m0 + m1;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mag += __shfl_xor_sync(kFull, mag, o);
+    if (fabsf(acc) > 1.25f * roundings * 5.9604644775390625e-8f * mag + (float)(d + 8) * 1.4e-45f)
+        return acc > 0.0f ? 1 : -1;
+    double p = 0.0, q = 0.0;
+    for (int c = lane; c < d; c += 32) {
+        const double t = (double)__ldg(x + c) * (double)__ldg(r + c);
+        p += t;
+        q += fabs(t);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        p += __shfl_xor_sync(kFull, p, o);
+        q += __shfl_xor_sync(kFull, q, o);
+    }
+    *zero = q == 0.0;
+    if (!(fabs(p) <= 1.7976931348623157e308) || q == 0.0) return p >= 0.0 ? 1 : -1;   // NaN: no bit
+    if (fabs(p) > 1.25 * (double)(d + 8) * 1.1102230246251565e-16 * q + (double)(d + 8) * 5e-324)
+        return p > 0.0 ? 1 : -1;
+    return 0;
+}
+
+template <bool VEC, bool REG>
+__global__ void __launch_bounds__(32 * kReWarps, 1) srp_dense_recheck_kernel(const RecheckArgs A) {
+    __shared__ __align__(16) uint16_t s_list[kReWarps][kReList + 8];   // columns within the part, padded to eight
+    __shared__ uint32_t s_bits[kReWarps][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int W = A.part_words, rows = 32 / W, words = A.bits >> 5, parts = words / W, d = A.d, ldr = A.ldr;
+    const int part = blockIdx.x % parts;
+    const long long groups = (A.N + rows - 1) / rows;
+    const long long stride = (long long)(gridDim.x / parts) * kReWarps;
+    const float *__restrict__ Rt = A.Rt + (size_t)part * W * 32 * ldr;
+    const float *__restrict__ rn = A.rnorm + part * W * 32;
+    const unsigned ldr4 = 4u * ldr;
+    // this lane's coordinates of a column (those past its end: x is zero there)
+    const char *r0 = reinterpret_cast<const char *>(Rt + (4 * lane < ldr ? 4 * lane : 0));
+    const char *r1 = reinterpret_cast<const char *>(Rt + (128 + 4 * lane < ldr ? 128 + 4 * lane : 0));
+    const float roundings = (float)(2 * ((d + 127) / 128) + 6);
+    const float tiny = (float)(d + 8) * 1.4e-45f;
+    constexpr unsigned long long kAbs = 0x7fffffff7fffffffull;
+    uint16_t *list = s_list[warp];
+    uint32_t *bits = s_bits[warp];
+    unsigned long long done = 0;
+    unsigned zeros = 0;
+    const int wrow = lane / W, wword = part * W + lane % W;
+    auto marks = [&](long long g) -> uint32_t {
+        const long long row = g * rows + wrow;
+        return g < groups && row < A.N ? __ldcs(A.und + (size_t)row * words + wword) : 0u;
+    };
+    long long g = (long long)(blockIdx.x / parts) * kReWarps + warp;
+    uint32_t next = marks(g);
+    for (; g < groups; g += stride) {
+        const uint32_t u = next;
+        next = marks(g + stride);
+        if (!__any_sync(kFull, u != 0)) continue;
+        done += __popc(u);
+        bits[lane] = 0;
+        int tie_at = 0, ties = 0;   // this lane's pending tie (16 bits of column, the row above), and how many in all
+        auto settle = [&] {
+            if (lane < ties) {
+                const int l = tie_at >> 16, col = tie_at & 0xffff;
+                const float *x = A.X + (size_t)(g * rows + l) * d, *r = Rt + (size_t)col * ldr;
+                double sum = 0.0;
+#pragma unroll 4
+                for (int c = 0; c < d; ++c) sum += (double)__ldg(x + c) * (double)__ldg(r + c);
+                if (sum >= 0.0) atomicOr(&bits[l * W + (col >> 5)], 1u << (col & 31));
+                zeros += sum == 0.0;
+            }
+            ties = 0;
+            __syncwarp();
+        };
+        for (int l = 0; l < rows; ++l) {
+            uint32_t m = wrow == l ? u : 0u;   // row l's marks not yet listed
+            if (!__any_sync(kFull, m != 0)) continue;
+            const long long row = g * rows + l;
+            const float *__restrict__ x = A.X + (size_t)row * d;
+            ulonglong2 u0, u1;
+            bool zero_row = false;
+            if (REG) {
+                u0 = x_pairs<VEC, true>(x, 4 * lane, d);
+                u1 = x_pairs<VEC, true>(x, 128 + 4 * lane, d);
+                zero_row = !__any_sync(kFull, ((u0.x | u0.y | u1.x | u1.y) & kAbs) != 0);
+            }
+            const float xb = 1.25f * roundings * 5.9604644775390625e-8f * __ldg(A.xnorm + row);
+            do {
+                int hi = 0;
+                for (unsigned b; hi <= kReList - 32 && (b = __ballot_sync(kFull, m != 0)) != 0;) {   // one of each word
+                    if (m) list[hi + __popc(b & ((1u << lane) - 1u))] = (uint16_t)((lane % W) * 32 + __ffs(m) - 1);
+                    m &= m - 1;
+                    hi += __popc(b);
+                }
+                __syncwarp();
+                if (lane < 8) list[hi + lane] = list[hi - 1];
+                __syncwarp();
+                for (int lo = 0; lo < hi; lo += 8) {
+                    const uint4 e8 = *reinterpret_cast<const uint4 *>(list + lo);
+                    const unsigned e2[4] = {e8.x, e8.y, e8.z, e8.w};
+                    const int my_col = list[lo + (lane >> 2)];
+                    const float my_rn = __ldg(rn + my_col);
+                    float t[8] = {};
+                    unsigned long long any = 0;
+    #pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        if (h && lo + 4 >= hi) break;   // (t[4..7] are not looked at)
+                        unsigned off[4];
+    #pragma unroll
+                        for (int i = 0; i < 4; ++i) off[i] = (i & 1 ? e2[2 * h + i / 2] >> 16 : e2[2 * h + i / 2] & 0xffffu) * ldr4;
+                        unsigned long long acc[4];
+    #pragma unroll
+                        for (int i = 0; i < 4; ++i) acc[i] = 0ull;
+                        if (REG) {
+                            ulonglong2 a[4], b[4];
+    #pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                a[i] = __ldg(reinterpret_cast<const ulonglong2 *>(r0 + off[i]));
+                                b[i] = __ldg(reinterpret_cast<const ulonglong2 *>(r1 + off[i]));
+                            }
+    #pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                acc[i] = f2_fma(u0.x, a[i].x, acc[i]);
+                                acc[i] = f2_fma(u0.y, a[i].y, acc[i]);
+                                acc[i] = f2_fma(u1.x, b[i].x, acc[i]);
+                                acc[i] = f2_fma(u1.y, b[i].y, acc[i]);
+                            }
+                        } else {
+    #pragma unroll 2
+                            for (int c = 4 * lane; c < ldr; c += 128) {
+                                const ulonglong2 xv = x_pairs<VEC, false>(x, c, d);
+                                any |= xv.x | xv.y;
+                                const char *rc = reinterpret_cast<const char *>(Rt + c);
+    #pragma unroll
+                                for (int i = 0; i < 4; ++i) {
+                                    const ulonglong2 a = __ldg(reinterpret_cast<const ulonglong2 *>(rc + off[i]));
+                                    acc[i] = f2_fma(xv.x, a.x, acc[i]);
+                                    acc[i] = f2_fma(xv.y, a.y, acc[i]);
+                                }
+                            }
+                        }
+    #pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            float e, f;
+                            f2_unpack(acc[i], e, f);
+                            t[4 * h + i] = e + f;
+                        }
+                    }
+                    if (!REG) zero_row = !__any_sync(kFull, (any & kAbs) != 0);
+                    // lane l is left with sum l / 4
+    #pragma unroll
+                    for (int o = 16, k = 4; o >= 4; o >>= 1, k >>= 1) {
+                        const bool high = lane & o;
+    #pragma unroll
+                        for (int i = 0; i < k; ++i)
+                            t[i] = (high ? t[i + k] : t[i]) + __shfl_xor_sync(kFull, high ? t[i] : t[i + k], o);
+                    }
+                    float s = t[0];
+                    s += __shfl_xor_sync(kFull, s, 2);
+                    s += __shfl_xor_sync(kFull, s, 1);
+                    const bool lead = (lane & 3) == 0 && lo + (lane >> 2) < hi;
+                    bool bit = s >= 0.0f;
+                    // (a zero row's sum over a finite column is zero: every product is)
+                    const unsigned open = __ballot_sync(kFull, lead && !(fabsf(s) > xb * my_rn + tiny));
+                    if (open) {
+                        if (zero_row && s == 0.0f) zeros += lead;
+                        for (unsigned o = __ballot_sync(kFull, (open >> lane & 1u) && !(zero_row && s == 0.0f)); o; o &= o - 1) {
+                            const int from = __ffs(o) - 1, c = __shfl_sync(kFull, my_col, from);
+                            bool zero = false;
+                            const int sg = sign_by_magnitude<VEC>(x, Rt + (size_t)c * ldr, d, ldr,
+                                                                  __shfl_sync(kFull, s, from), roundings, &zero);
+                            if (lane == from) {
+                                bit = sg > 0;
+                                zeros += zero;
+                            }
+                            if (sg == 0) {
+                                if (lane == ties) tie_at = l << 16 | c;
+                                if (++ties == 32) settle();
+                            }
+                        }
+                    }
+                    if (lead && bit) atomicOr(&bits[l * W + (my_col >> 5)], 1u << (my_col & 31));
+                }
+                __syncwarp();   // the list has been read
+            } while (__any_sync(kFull, m != 0));
+        }
+        if (ties) settle();
+        const uint32_t w = bits[lane];
+        if (w) A.sig[(size_t)(g * rows + wrow) * words + wword] |= w;
+        __syncwarp();
+    }
+    unsigned long long zs = zeros;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        done += __shfl_xor_sync(kFull, done, o);
+        zs += __shfl_xor_sync(kFull, zs, o);
+    }
+    if (lane == 0 && done) atomicAdd(&A.scratch->counters[2], done);
+    if (lane == 0 && zs) atomicAdd(&A.scratch->counters[3], zs);
 }
 
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct DenseLayout {
-    size_t xh, xl, rh, rl, rt, xn, rn, qc, q, total;
-    unsigned long long qcap;
+    size_t xh, xl, rh, rl, rt, xn, rn, und, total;
 };
-
-// Recheck queue capacity: 1/16 of the signs (at least 2^20); signs beyond it
-// are decided in line by the tensor-core kernel itself.
-unsigned long long queue_cap(long long N, int bits) {
-    const unsigned long long all = (unsigned long long)N * bits;
-    const unsigned long long c = all / 16;
-    return c < (1ull << 20) ? ((1ull << 20) < all ? (1ull << 20) : all) : c;
-}
 
 DenseLayout dense_layout(long long N, int d0, int bits) {
     const int d = (d0 + BK - 1) / BK * BK;   // K padded to whole stages
@@ -612,9 +730,7 @@ DenseLayout dense_layout(long long N, int d0, int bits) {
     L.rt = o; o = up256(o + (size_t)bits * d * 4);
     L.xn = o; o = up256(o + (size_t)Npad * 4);
     L.rn = o; o = up256(o + (size_t)bits * 4);
-    L.qc = o; o = up256(o + 8);
-    L.qcap = queue_cap(N, bits);
-    L.q = o; o = up256(o + (size_t)L.qcap * 8);
+    L.und = o; o = up256(o + (size_t)N * (bits / 8));
     L.total = o;
     return L;
 }
@@ -655,15 +771,14 @@ extern "C" int blsh_srp_dense(blsh_ctx *ctx, const float *X, int64_t N, int32_t 
     const float m = margin > rigorous ? margin : rigorous;
     unsigned char *ws = (unsigned char *)workspace;
     const long long Npad = (N + BM - 1) / BM * BM;
-    unsigned long long *qcount = (unsigned long long *)(ws + L.qc);
-    uint2 *queue = (uint2 *)(ws + L.q);
+    uint32_t *und = (uint32_t *)(ws + L.und);
     const int r_blocks = bits / kPrepCols;
     const unsigned x_blocks = (unsigned)((Npad + 7) / 8 < 65535ll * 8 ? (Npad + 7) / 8 : 65535ll * 8);
     const bool vec = d % 4 == 0;
     blsh_time_start(ctx, s);
     (vec ? srp_dense_prep<true> : srp_dense_prep<false>)<<<r_blocks + x_blocks, 256, 0, s>>>(
         X, N, Npad, d, KT, ws + L.xh, ws + L.xl, (float *)(ws + L.xn), R, bits, ws + L.rh, ws + L.rl,
-        (float *)(ws + L.rn), (float *)(ws + L.rt), r_blocks, qcount);
+        (float *)(ws + L.rn), (float *)(ws + L.rt), r_blocks);
     BLSH_LAUNCHED(ctx, "srp_dense_prep");
     const size_t smem = (size_t)STAGES * STAGE_BYTES + 1024 + (size_t)bits * sizeof(float);
     const size_t smem_max = (size_t)STAGES * STAGE_BYTES + 1024 + 4096 * sizeof(float);   // bits <= 4096
@@ -678,11 +793,21 @@ extern "C" int blsh_srp_dense(blsh_ctx *ctx, const float *X, int64_t N, int32_t 
     blsh_time_start(ctx, s);
     srp_dense_tc_persistent<<<grid, kTcThreads, smem, s>>>(ws + L.xh, ws + L.xl, ws + L.rh, ws + L.rl,
                                                           (float *)(ws + L.xn), (float *)(ws + L.rn), N, d, bits, m,
-                                                          sig, queue, L.qcap, qcount, X, R, tiles, ctx->scratch);
+                                                          sig, und, tiles, ctx->scratch);
     BLSH_LAUNCHED(ctx, "srp_dense_tc_persistent");
     blsh_time_start(ctx, s);
-    (vec ? srp_dense_recheck_kernel<true> : srp_dense_recheck_kernel<false>)<<<ctx->sm_count * 8, 256, 0, s>>>(
-        queue, L.qcap, qcount, X, (float *)(ws + L.rt), d, KT * BK, bits, sig, ctx->scratch);
+    const int part_words = bits % 1024 == 0 ? 32 : bits % 512 == 0 ? 16 : 8, parts = bits / (32 * part_words);
+    const RecheckArgs A = {und, X, (const float *)(ws + L.rt), (const float *)(ws + L.xn), (const float *)(ws + L.rn), N,
+                           d, KT * BK, bits, part_words, sig, ctx->scratch};
+    const long long groups = (N * part_words + 31) / 32, share = (groups + kReWarps - 1) / kReWarps;
+    const long long copies = ctx->sm_count / parts > 0 ? ctx->sm_count / parts : 1;   // CTAs a part
+    const unsigned re_grid = (unsigned)((share < copies ? share : copies) * parts);
+    if (d <= 256)
+        (vec ? srp_dense_recheck_kernel<true, true> : srp_dense_recheck_kernel<false, true>)<<<re_grid, 32 * kReWarps, 0,
+                                                                                             s>>>(A);
+    else
+        (vec ? srp_dense_recheck_kernel<true, false> : srp_dense_recheck_kernel<false, false>)<<<
+            re_grid, 32 * kReWarps, 0, s>>>(A);
     BLSH_LAUNCHED(ctx, "srp_dense_recheck_kernel");
     return BLSH_OK;
 }
