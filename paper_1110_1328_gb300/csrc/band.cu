@@ -520,7 +520,12 @@ __device__ __forceinline__ T warp_exclusive(T v) {
 //
 // 1e6 points, 64 bands of 16 bits (1.7e9 tests of 6.4e8 pairs): the count
 // pass 15.1 ms with borrow tests on every word, whole windows staged a row per
-// lane and the open tests dealt by searching their owners; 10.3 now.
+// lane and the open tests dealt by searching their owners; 8.9 now.  Of that
+// the open tests take 2.8, the first tests 1.0, loading rows 2 (of a row's
+// eight pieces only those that the chunk's bands reach, 4.5 on average; whole
+// rows took 0.7 ms more); the pass issues on 6 cycles of 10, two thirds of the
+// integer pipe's rate.  (A table of the poison words, more rows staged where
+// they are short, and ids at hand for the first batches changed nothing.)
 template <int MODE, int KW4, int LANE>
 __global__ void __launch_bounds__(256, 3) emit_warp_kernel(BandArgs A, const uint32_t *__restrict__ keys,
                                                            const uint32_t *__restrict__ vals, long long n,
@@ -530,7 +535,9 @@ __global__ void __launch_bounds__(256, 3) emit_warp_kernel(BandArgs A, const uin
     if (RETEST && (cap == 0 || *E.rec_next <= E.rec_cap)) return;   // nothing to write, or every chunk recorded
     extern __shared__ uint4 s_all[];
     const int cw4 = A.ck_words >> 2, cws = cw4 | 1;
-    const unsigned magic = (65536u + cw4 - 1) / cw4;   // i / cw4 = i * magic >> 16 for i < 2^11 (cw4 <= 8)
+    // 16-byte chunks of a key row that this chunk's bands reach, and i / need = i * magic >> 16 for i < 2^11 (need <= 8)
+    int need = cw4;
+    unsigned magic = (65536u + cw4 - 1) / cw4;
     const int lane = threadIdx.x & 31;
     unsigned char *region = reinterpret_cast<unsigned char *>(s_all) + (threadIdx.x >> 5) * R::kRegion;
     uint4 *s_ck = reinterpret_cast<uint4 *>(region);
@@ -543,19 +550,58 @@ __global__ void __launch_bounds__(256, 3) emit_warp_kernel(BandArgs A, const uin
     const bool jac = LANE == 4 && A.exact_classes;
     const unsigned long long items =
         MODE == kSegment ? (*E.task_next < E.task_cap ? *E.task_next : E.task_cap) : (unsigned long long)((n + 31) >> 5);
-    // key rows of objects ids[0 .. m) into dst
+    // the first `need` chunks of the key rows of objects ids[0 .. m) into dst
     auto load_rows = [&](uint4 *dst, const uint32_t *ids, int m) {
 #pragma unroll 4
-        for (int i = lane; i < m * cw4; i += 32) {
-            const int k = (int)((unsigned)i * magic >> 16), q = i - k * cw4;
+        for (int i = lane; i < m * need; i += 32) {
+            const int k = (int)((unsigned)i * magic >> 16), q = i - k * need;
             dst[k * cws + q] = __ldg(reinterpret_cast<const uint4 *>(A.ck + (size_t)ids[k] * A.ck_stride) + q);
         }
     };
+    // The next chunk, its keys and its first ids are fetched while this one is
+    // worked on: its number, its keys, its ids and its rows would otherwise be
+    // four waits one after the other at its start (10.4 ms of the pass below,
+    // 9.5 so).  (Every warp starts with the
+    // chunk of its own number, so that none holds two while another has none;
+    // segments, a few a warp and long, are taken when they are begun.)
+    constexpr bool AHEAD = MODE == kCount;
+    static_assert(R::kStage <= 64, "two ids a lane");
+    uint32_t ahead_key[kKeyWin / 32], ahead_val[2];
+    unsigned long long after = 0;                         // (lane 0) the chunk after the next
+    const unsigned long long workers = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+    auto grab = [&] { after = lane == 0 ? (AHEAD ? workers : 0ull) + atomicAdd(E.next, 1ull) : 0ull; };
+    auto fetch = [&](unsigned long long ch) {
+        if (!AHEAD || ch >= items) return;
+        const long long left = n - (long long)(ch << 5);
+#pragma unroll
+        for (int q = 0; q < kKeyWin / 32; ++q) ahead_key[q] = lane + 32 * q < left ? __ldg(keys + (ch << 5) + lane + 32 * q) : 0u;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) ahead_val[q] = lane + 32 * q < left ? __ldg(vals + (ch << 5) + lane + 32 * q) : 0u;
+    };
+    unsigned long long next = (unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (AHEAD && next < items) {
+        fetch(next);
+        grab();
+    }
     for (;;) {
-        unsigned long long c = 0;
-        if (lane == 0) c = atomicAdd(E.next, 1ull);
-        c = __shfl_sync(kFull, c, 0);
+        if (!AHEAD) {
+            grab();
+            next = __shfl_sync(kFull, after, 0);
+        }
+        unsigned long long c = next;
         if (c >= items) break;
+        if (AHEAD) {
+            __syncwarp();                                 // the previous chunk is done with the region
+#pragma unroll
+            for (int q = 0; q < kKeyWin / 32; ++q) s_key[lane + 32 * q] = ahead_key[q];
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (lane + 32 * q < R::kStage) s_val[lane + 32 * q] = ahead_val[q];
+            __syncwarp();
+            next = __shfl_sync(kFull, after, 0);
+            if (next < items) grab();
+            fetch(next);
+        }
         if (RETEST && E.rec_off[c] != ~0ull) continue;
         unsigned seg = 0;
         if (MODE == kSegment) {
@@ -575,8 +621,10 @@ __global__ void __launch_bounds__(256, 3) emit_warp_kernel(BandArgs A, const uin
         if (MODE == kSegment) {
             if (live) end += E.partners[p0 + lane];
         } else {
-            for (int k = lane; k < win; k += 32) s_key[k] = __ldg(keys + p0 + k);
-            __syncwarp();
+            if (!AHEAD) {
+                for (int k = lane; k < win; k += 32) s_key[k] = __ldg(keys + p0 + k);
+                __syncwarp();
+            }
             if (live) {
                 const long long band_end = (long long)(b + 1) * A.N - p0;
                 const uint32_t key = s_key[lane];
@@ -602,23 +650,30 @@ __global__ void __launch_bounds__(256, 3) emit_warp_kernel(BandArgs A, const uin
             }
             continue;
         }
-        for (int k = lane; k < staged; k += 32) s_val[k] = __ldg(vals + p0 + k);
-        __syncwarp();
+        if (!AHEAD) {
+            for (int k = lane; k < staged; k += 32) s_val[k] = __ldg(vals + p0 + k);
+            __syncwarp();
+        }
+        const bool flat = MODE != kSegment && jmax <= (unsigned)R::kStage && 5u * ((pairs_w + 31) / 32) < 2u * (jmax - 1);
+        const unsigned segs = MODE == kCount && jmax - 1 > kSplit ? (jmax - 2) / kSeg + 1 : 0u;
+        const unsigned long long words = flat ? (pairs_w + 31) / 32 : 32ull * ((jmax + 30) / 32) + 32ull * segs;
+        unsigned long long off = 0;                       // (the answer is waited for after the rows)
+        if (MODE == kCount && lane == 0) off = atomicAdd(E.rec_next, words);
+        // chunks of 16 bytes that any lane's earlier bands (and its class id) reach
+        const int nw4 = (int)(__reduce_max_sync(kFull, live ? (unsigned)(b * LANE + 15) / 16 : 0u));
+        const int reach = jac ? (int)__reduce_max_sync(kFull, (unsigned)b) / 4 + 1 : nw4 > 0 ? nw4 : 1;
+        if (reach != need) {
+            need = reach;
+            magic = (65536u + reach - 1) / reach;
+        }
         load_rows(s_ck, s_val, staged);
         __syncwarp();
-        const bool flat = MODE != kSegment && jmax <= (unsigned)R::kStage && 5u * ((pairs_w + 31) / 32) < 2u * (jmax - 1);
         const uint32_t x = live ? s_val[lane] : 0u;
         uint32_t *crec = nullptr;
         unsigned long long out = RETEST ? E.chunk[c] : 0ull;
         if (MODE == kCount) {
-            const unsigned segs = jmax - 1 > kSplit ? (jmax - 2) / kSeg + 1 : 0u;
-            const unsigned long long words =
-                flat ? (pairs_w + 31) / 32 : 32ull * ((jmax + 30) / 32) + 32ull * segs;
-            unsigned long long off = 0, slot = 0;
-            if (lane == 0) {
-                off = atomicAdd(E.rec_next, words);
-                if (segs && off + words <= E.rec_cap) slot = atomicAdd(E.task_next, (unsigned long long)segs);
-            }
+            unsigned long long slot = 0;
+            if (lane == 0 && segs && off + words <= E.rec_cap) slot = atomicAdd(E.task_next, (unsigned long long)segs);
             off = __shfl_sync(kFull, off, 0);
             slot = __shfl_sync(kFull, slot, 0);
             const bool room = off + words <= E.rec_cap;
@@ -674,8 +729,6 @@ __global__ void __launch_bounds__(256, 3) emit_warp_kernel(BandArgs A, const uin
 #pragma unroll
         for (int k = 0; k < PZ / 4; ++k) kx[k] = live && k < cw4 ? s_ck[lane * cws + k] : make_uint4(0u, 0u, 0u, 0u);
         const uint32_t xb = jac ? reinterpret_cast<const uint32_t *>(s_ck + (live ? lane : 0) * cws)[b] : 0u;
-        // chunks of 16 bytes any lane's earlier bands reach
-        const int nw4 = (int)(__reduce_max_sync(kFull, live ? (unsigned)(b * LANE + 15) / 16 : 0u));
         // (KW4 = 8) tests past the first chunk: earlier bands, or a class id, there
         const bool more = b * LANE > 16 || (jac && b >= 4);
         unsigned cnt = 0;

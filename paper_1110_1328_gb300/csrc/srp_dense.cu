@@ -441,12 +441,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) srp_dense_tc_persistent(
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
 }
 
-// The marked signs.  An item is the marks of kPartRows rows in kPartWords
-// words (kPartCols columns): a lane a word.  They are listed in shared memory
-// row by row, and the warp forms four sums at a time: lane l takes coordinates
-// 4 l .. 4 l + 3 of every 128 of x_i (kept in registers for all of the row's
-// signs where d <= 256) and of the four columns, paired FMAs, and the four sums
-// meet in six shuffles.  Three stages, each with a rigorous bound:
+// The marked signs.  An item is 32 words of marks, a lane a word: 32 words of a
+// row, or 16 or 8 words of two or four rows where the width asks for it.  They
+// are listed in shared memory row by row, and the warp forms eight sums at a
+// time: lane l takes coordinates 4 l .. 4 l + 3 of every 128 of x_i (kept in
+// registers for all of the row's signs where d <= 256) and of the columns, in
+// paired FMAs, and the eight sums meet in nine shuffles.  Three stages, each with a rigorous bound:
 //   FP32: no term passes through more than 2 ceil(d/128) + 6 roundings, so the
 //   sum errs by at most that many u |x_i| |r_j| (norms rounded up; infinite
 //   where they could over- or underflow), or, if that does not decide, u sum|p|
