@@ -15,7 +15,8 @@
 //
 // Two launch forms:
 //   PLAIN      -- one group per pair, grid covers all pairs; a warp lives as
-//                 long as its slowest pair.  For cosine with k = 32 it runs
+//                 long as its slowest pair.  Jaccard with eight lanes: a lane per
+//                 pair for the tests (verify_sets_kernel).  For cosine with k = 32 it runs
 //                 in two passes: every pair's first four chunks, then the
 //                 pairs still open (verify_tile_kernel does both, tile by
 //                 tile; verify_first_kernel then verify_kernel's OPEN form
@@ -539,6 +540,167 @@ __global__ void __launch_bounds__(512) verify_kernel(const VerifyArgs A) {
         }
     }
 
+    __syncthreads();
+    if (A.stop_hist)
+        for (int i = threadIdx.x; i < A.levels; i += blockDim.x)
+            if (s_hist[i]) atomicAdd(A.stop_hist + i, (unsigned long long)s_hist[i]);
+}
+
+// Jaccard, plain form, eight lanes a pair (k a multiple of 32).  A lane owns a
+// pair for its decisions and shares the comparing: a warp takes 32 pairs, lane
+// l that at 4 (l % 8) + l / 8, and compares them four at a time, the eight
+// lanes l / 8 = i reading 16 bytes each of the 128 that hold 32 hashes of pair
+// 4 u + i's rows.  A lane's counts of the eight rounds lie in the bytes of two
+// words; three shuffle steps add them over the eight lanes, and lane l finds
+// its own pair's in byte l % 8.  Decisions and outputs are then made once for
+// 32 pairs.  Pairs still open wait in the warp's part of shared memory and are
+// continued 32 at a time, each at its own chunk.
+//
+// With four lanes a pair (verify_kernel) the tests, outputs and histogram of
+// every chunk are issued for eight pairs: 200 instructions a step, 70% of the
+// issue slots, 428 us for 1.38e7 pairs of 32 hashes (the rows' bytes, 3.5 GB
+// through L1, take a third of that).  Here a step of 32 pairs takes
+// 190 instructions, and the call 269 us.
+struct SetsQueue {          // pairs waiting for their next chunk: at most 31, and the 32 of a step
+    long long q[64];
+    uint2 pair[64];
+    int m[64];
+    uint32_t state[64];     // chunk | Algorithm 1 open << 30 | Algorithm 2 open << 31
+};
+
+__global__ void __launch_bounds__(256, 4) verify_sets_kernel(const VerifyArgs A) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    SetsQueue &Q = reinterpret_cast<SetsQueue *>(smem)[threadIdx.x >> 5];
+    int32_t *s_mm = reinterpret_cast<int32_t *>(smem + (blockDim.x >> 5) * sizeof(SetsQueue));
+    unsigned *s_hist = reinterpret_cast<unsigned *>(s_mm + A.levels);
+    for (int i = threadIdx.x; i < A.levels; i += blockDim.x) {
+        s_mm[i] = A.min_matches[i];
+        s_hist[i] = 0;
+    }
+    __syncthreads();
+    long long P = A.P;
+    if (A.P_dev) {
+        const long long pd = *A.P_dev;
+        P = pd < 0 ? 0 : (pd < P ? pd : P);
+    }
+    const int lane = threadIdx.x & 31, oct = lane & 24, mine = 4 * (lane & 7) + (lane >> 3);
+    const unsigned lt = (1u << lane) - 1u;
+    unsigned first_stops = 0;   // this lane's stops at level 0
+    int waiting = 0;
+
+    // the agreements of every lane's pair in its chunk j (a lane without one: row 0 against itself)
+    auto agreements = [&](auto first, uint2 pr, int j) {
+        uint32_t lo = 0, hi = 0;
+        for (int w = 0; w < A.chunk_words; w += 32) {   // (k <= 128: a byte holds a count)
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const uint32_t x = __shfl_sync(kFull, pr.x, oct | u), y = __shfl_sync(kFull, pr.y, oct | u);
+                int off = w + 4 * (lane & 7);
+                if (!decltype(first)::value) off += __shfl_sync(kFull, j, oct | u) * A.chunk_words;
+                const uint4 a = ldg4(A.sig + (size_t)x * A.W + off), b = ldg4(A.sig + (size_t)y * A.W + off);
+                const uint32_t e = (a.x == b.x) + (a.y == b.y) + (a.z == b.z) + (a.w == b.w);
+                if (u < 4) lo += e << (8 * u);
+                else hi += e << (8 * (u - 4));
+            }
+        }
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) {
+            lo += __shfl_xor_sync(kFull, lo, o);
+            hi += __shfl_xor_sync(kFull, hi, o);
+        }
+        return (int)(((lane & 4 ? hi : lo) >> (8 * (lane & 3))) & 0xffu);
+    };
+    // a step of the warp: chunk j of every lane's pair (a1, al: which algorithms are open)
+    auto step = [&](auto first, long long q, uint2 pr, int m, int j, bool a1, bool al) {
+        const bool was = a1 || al;
+        if (!__any_sync(kFull, was)) return;
+        m += agreements(first, was ? pr : make_uint2(0u, 0u), was ? j : 0);
+        if (was) {
+            const bool pruned = m < s_mm[j];                             // Pr[S >= t | M] < eps
+            if (a1) {
+                int st = -1;
+                if (pruned) st = BLSH_PRUNED;
+                else if (!A.lite && ((__ldg(A.conc_bits + j * A.conc_words + (m >> 5)) >> (m & 31)) & 1u)) st = BLSH_ACCEPT;
+                else if (j + 1 == A.levels) st = A.lite ? BLSH_LITE_SURVIVOR : BLSH_ACCEPT_AT_MAX;
+                else if (j + 1 == A.cap_levels) st = BLSH_NEEDS_HASHES;
+                if (st >= 0) {
+                    A.status[q] = (uint8_t)st;
+                    if (A.n_used) A.n_used[q] = (uint16_t)((j + 1) * A.k);
+                    if (A.m_out) A.m_out[q] = (uint16_t)m;
+                    if (st == BLSH_NEEDS_HASHES) {                       // Algorithm 1 needs hashes not yet computed
+                        A.need[pr.x] = 1;
+                        A.need[pr.y] = 1;
+                    } else {
+                        // the estimate is an output only for pairs that are kept
+                        if (A.est_out && st != BLSH_PRUNED)
+                            A.est_out[q] = __ldg(A.est_tab + (size_t)j * A.est_stride + m);
+                        if (j == 0) ++first_stops;
+                        else atomicAdd(&s_hist[j], 1u);
+                    }
+                    a1 = false;
+                }
+            }
+            if (al && (pruned || j + 1 == A.lite_levels)) {              // Algorithm 2: the same test, h hashes
+                A.lstatus[q] = pruned ? BLSH_PRUNED : BLSH_LITE_SURVIVOR;
+                if (A.ln_used) A.ln_used[q] = (uint16_t)((j + 1) * A.k);
+                al = false;
+            }
+        }
+        const bool open = a1 || al;
+        const unsigned o = __ballot_sync(kFull, open);
+        if (open) {
+            const int e = waiting + __popc(o & lt);
+            Q.q[e] = q;
+            Q.pair[e] = pr;
+            Q.m[e] = m;
+            Q.state[e] = (uint32_t)(j + 1) | (uint32_t)a1 << 30 | (uint32_t)al << 31;
+        }
+        waiting += __popc(o);
+        __syncwarp();
+    };
+    auto go_on = [&](int n) {   // the last n waiting pairs' next chunk
+        long long q = 0;
+        uint2 pr = make_uint2(0u, 0u);
+        int m = 0;
+        uint32_t state = 0;
+        if (lane < n) {
+            const int e = waiting - n + lane;
+            q = Q.q[e];
+            pr = Q.pair[e];
+            m = Q.m[e];
+            state = Q.state[e];
+        }
+        waiting -= n;
+        __syncwarp();
+        step(std::false_type{}, q, pr, m, (int)(state & 0x3fffffffu), (state >> 30) & 1u, state >> 31);
+    };
+
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    long long base = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31);
+    uint2 next = make_uint2(0u, 0u);
+    if (base + mine < P) next = __ldg(A.pairs + base + mine);
+    for (; base < P; base += stride) {
+        const uint2 pr = next;
+        const long long q = base + mine;
+        if (q + stride < P) next = __ldg(A.pairs + q + stride);
+        const bool good = (long long)pr.x < A.N && (long long)pr.y < A.N;
+        if (q < P && !good) {
+            A.status[q] = BLSH_BAD_PAIR;
+            if (A.n_used) A.n_used[q] = 0;
+            if (A.m_out) A.m_out[q] = 0;
+            if (A.lite_levels) {
+                A.lstatus[q] = BLSH_BAD_PAIR;
+                if (A.ln_used) A.ln_used[q] = 0;
+            }
+            blsh_dev_error(A.scratch, BLSH_ERANGE, 0, 1ull);
+        }
+        step(std::true_type{}, q, pr, 0, 0, q < P && good, q < P && good && A.lite_levels > 0);
+        while (waiting >= 32) go_on(32);
+    }
+    while (waiting > 0) go_on(waiting < 32 ? waiting : 32);
+
+    const unsigned z = __reduce_add_sync(kFull, first_stops);
+    if (lane == 0 && z) atomicAdd(&s_hist[0], z);
     __syncthreads();
     if (A.stop_hist)
         for (int i = threadIdx.x; i < A.levels; i += blockDim.x)
@@ -1080,6 +1242,20 @@ int launch_kernel(blsh_ctx *ctx, const VerifyArgs &A, const blsh_plan &plan, cud
     return BLSH_OK;
 }
 
+int launch_sets(blsh_ctx *ctx, const VerifyArgs &A, const blsh_plan &plan, cudaStream_t s) {
+    if (A.P == 0) return BLSH_OK;
+    const int block = plan.block < 256 ? plan.block : 256;
+    const size_t smem = (block / 32) * sizeof(SetsQueue) + 2ull * A.levels * sizeof(int32_t);
+    int occ = 0;
+    BLSH_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, verify_sets_kernel, block, smem));
+    // one wave of resident CTAs: a warp's last open pairs leave lanes idle once
+    const long long blocks = (A.P + block - 1) / block, cap = (long long)ctx->sm_count * (occ > 0 ? occ : 1);
+    blsh_time_start(ctx, s);
+    verify_sets_kernel<<<(unsigned)(blocks < cap ? blocks : cap), block, smem, s>>>(A);
+    BLSH_LAUNCHED(ctx, "verify_sets_kernel");
+    return BLSH_OK;
+}
+
 template <bool PERSIST>
 int dispatch(blsh_ctx *ctx, const VerifyArgs &A, const blsh_plan &plan, int kind, cudaStream_t s) {
     if (kind == BLSH_COSINE) {
@@ -1133,7 +1309,9 @@ int dispatch(blsh_ctx *ctx, const VerifyArgs &A, const blsh_plan &plan, int kind
     switch (plan.group) {
     case 1: return launch_kernel<BLSH_JACCARD, 1, 8, PERSIST>(ctx, A, plan, s);
     case 4: return launch_kernel<BLSH_JACCARD, 4, 2, PERSIST>(ctx, A, plan, s);
-    case 8: return launch_kernel<BLSH_JACCARD, 8, 1, PERSIST>(ctx, A, plan, s);
+    case 8:
+        if constexpr (PERSIST) return launch_kernel<BLSH_JACCARD, 8, 1, true>(ctx, A, plan, s);
+        else return launch_sets(ctx, A, plan, s);
     case 16: return launch_kernel<BLSH_JACCARD, 16, 1, PERSIST>(ctx, A, plan, s);
     case 32: return launch_kernel<BLSH_JACCARD, 32, 1, PERSIST>(ctx, A, plan, s);
     }
@@ -1145,16 +1323,20 @@ int dispatch(blsh_ctx *ctx, const VerifyArgs &A, const blsh_plan &plan, int kind
 // The plan of a caller who has not tuned one, for up to P pairs: the plain
 // form, the fastest for every k, size and kind measured (Algorithms 1 and 2
 // together, plain against persistent: 2.7e7 cosine pairs, k = 32: 240 against
-// 471 us, k = 64: 334 / 448, k = 128: 319 / 444; 6e5 pairs 54 / 58; 1.4e7
-// Jaccard pairs, k = 32: four lanes a pair 467 / 524, one 542, eight 775 / 865;
-// k = 64: 555 / 638, 913, 938 / 1,079; 176 pairs 31 / 41).  Cosine calls over
-// fewer than 65,536 pairs, where the two forms take the same time, keep the
-// persistent one.
+// 471 us, k = 64: 334 / 448, k = 128: 319 / 444; 6e5 pairs 54 / 58).  Cosine
+// calls over fewer than 65,536 pairs, where the two forms take the same time,
+// keep the persistent one.  Jaccard pairs take eight lanes a pair
+// (verify_sets_kernel: 1.4e7 pairs, k = 32: 269 us, four lanes a pair 428; 8e6
+// random ones 288 / 350, k = 64 490 / 715, k = 128 900 / 1,395; 5e5 pairs
+// 34 / 37), fewer than 2^18 of them four: the two take the same time there,
+// and where a few hundred pairs leave most warps idle a step of eight pairs is
+// shorter than one of 32 (176 pairs: 13 us, 20 with eight lanes).
 blsh_plan blsh_default_plan(int kind, long long P) {
     blsh_plan p;
     p.mode = kind == BLSH_COSINE && P < 65536 ? BLSH_PLAN_PERSISTENT : BLSH_PLAN_PLAIN;
-    p.group = kind == BLSH_COSINE ? 1 : 4;
-    p.block = kind == BLSH_COSINE ? 256 : 128;
+    const bool few_sets = kind == BLSH_JACCARD && P < (1ll << 18);
+    p.group = kind == BLSH_COSINE ? 1 : few_sets ? 4 : 8;
+    p.block = few_sets ? 128 : 256;
     p.grab = kind == BLSH_COSINE ? 128 : 32;
     p.ctas_per_sm = 0;
     return p;
