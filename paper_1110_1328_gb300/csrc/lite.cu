@@ -76,6 +76,18 @@ __device__ __forceinline__ long long fixed_term(float u, float v) {
     return ((bu ^ bv) >> 31) ? -(long long)r : (long long)r;
 }
 
+// fixed_term(v, v) with one rounded shift where v lies in the range of a unit
+// vector's entries: the product, moved up 15 bits, is shifted down by 1 to 63.
+__device__ __forceinline__ long long fixed_square(float v) {
+    const uint32_t b = __float_as_uint(v) & 0x7fffffffu;
+    uint32_t e = b >> 23, m = b & 0x7fffffu;
+    if (e) m |= 0x800000u; else e = 1;
+    const int down = 15 - (2 * (int)e - 240);
+    if (down < 1 || down > 63) return fixed_term(v, v);
+    const unsigned long long t = ((unsigned long long)m * m) << 15;
+    return (long long)((t + ((1ull << (down - 1)) - 1ull) + ((t >> down) & 1ull)) >> down);   // half to even
+}
+
 __device__ __forceinline__ long long warp_sum(long long v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
@@ -589,9 +601,10 @@ __device__ __forceinline__ void lite_batch(const LiteArgs &A, long long my_q, bo
 // four rows a warp; the lanes' sums meet in three shuffle steps.  (A warp over
 // 128 consecutive elements with a search for every element's row and a
 // segmented scan took 147 instructions per 32 elements: 1.27 ms for 1.4e8
-// nonzeros, 0.97 here.)  Formed only when there are more survivors than
+// nonzeros; eight lanes for the longest rows too, 0.97; 0.56 here.)  Formed only when there are more survivors than
 // half the rows (the collection pass has counted them); otherwise each
 // survivor forms its two norms itself, which is less work.
+constexpr int kNormLong = 256;   // (a row of 30,000 took eight lanes longer than all the others together)
 __global__ void __launch_bounds__(256) row_norm2_kernel(const int64_t *__restrict__ indptr,
                                                         const float *__restrict__ values, long long N,
                                                         long long *__restrict__ norm2,
@@ -611,13 +624,30 @@ __global__ void __launch_bounds__(256) row_norm2_kernel(const int64_t *__restric
             e = __ldg(indptr + row + 1);
         }
         long long sum = 0;
+        // long rows: all of the warp's lanes, eight loads each
+        const bool is_long = e - s > kNormLong;
+        for (unsigned rows = __ballot_sync(kFull, is_long && g == 0); rows; rows &= rows - 1) {
+            const int from = __ffs(rows) - 1;
+            const long long ls = __shfl_sync(kFull, s, from), le = __shfl_sync(kFull, e, from);
+            long long part = 0;
+            for (long long i = ls + (threadIdx.x & 31); i < le; i += 256) {
+                float v[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) v[u] = i + 32 * u < le ? __ldg(values + i + 32 * u) : 0.0f;
+#pragma unroll
+                for (int u = 0; u < 8; ++u) part += fixed_square(v[u]);   // (0 past the end)
+            }
+            part = warp_sum(part);
+            if ((int)(threadIdx.x & 31) == from) sum = part;
+        }
+        if (is_long) s = e;
         for (long long i = s + g; i < e; i += 32) {
             float v[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) v[u] = i + 8 * u < e ? __ldg(values + i + 8 * u) : 0.0f;
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-                if (i + 8 * u < e) sum += fixed_term(v[u], v[u]);
+                if (i + 8 * u < e) sum += fixed_square(v[u]);
         }
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(kFull, sum, o);
@@ -693,9 +723,13 @@ __global__ void __launch_bounds__(256, 4) lite_exact_kernel(const LiteArgs A) {
 }
 
 // Survivors into a queue (the context's survivor queue, BLSH_LITE_QUEUE_CAP
-// entries): warps scan groups of four 512-status tiles in grid-stride order
-// and append their survivors' indices with one atomic per group.  Survivors
-// beyond the queue are left for lite_exact_kernel.
+// entries): warps scan T tiles of 512 statuses at a time in grid-stride order,
+// four loads in flight, and append their survivors' indices with one atomic
+// for all T.  Survivors beyond the queue are left for lite_exact_kernel.
+// T = 16 where every warp has such a group: with an atomic for every
+// four tiles the counter's one address (and a load in flight less often) 1e9 statuses
+// took 495 us, 271 so.
+template <int T>
 __global__ void __launch_bounds__(256) lite_collect_kernel(const LiteArgs A, unsigned long long *queue) {
     long long P = A.P;
     if (A.P_dev) {
@@ -704,23 +738,30 @@ __global__ void __launch_bounds__(256) lite_collect_kernel(const LiteArgs A, uns
     }
     const int lane = threadIdx.x & 31;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    // four tiles of 512 statuses per warp at a time: their 16-byte loads are
-    // in flight together, and one atomic reserves queue slots for all four
-    for (long long q0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 2048; q0 < P;
-         q0 += nwarps * 2048) {
-        uint32_t surv[4];
+    for (long long q0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (512 * T); q0 < P;
+         q0 += nwarps * (512 * T)) {
+        uint32_t surv[T / 2];   // two tiles' 16 bits a word
+        unsigned c = 0;
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const long long qs = q0 + 512ll * t + 16ll * lane;
-            surv[t] = 0;
-            if (A.vec && qs + 16 <= P) {
-                surv[t] = blsh_eq16(__ldg(reinterpret_cast<const uint4 *>(A.status + qs)), BLSH_LITE_SURVIVOR);
+        for (int t0 = 0; t0 < T; t0 += 4) {
+            const long long qs = q0 + 512ll * t0 + 16ll * lane;
+            uint32_t b[4] = {0u, 0u, 0u, 0u};
+            if (A.vec && qs + 512 * 3 + 16 <= P) {
+                uint4 v[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) v[t] = __ldg(reinterpret_cast<const uint4 *>(A.status + qs + 512 * t));
+#pragma unroll
+                for (int t = 0; t < 4; ++t) b[t] = blsh_eq16(v[t], BLSH_LITE_SURVIVOR);
             } else {
-                for (int i = 0; i < 16; ++i)
-                    if (qs + i < P && A.status[qs + i] == BLSH_LITE_SURVIVOR) surv[t] |= 1u << i;
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    for (int i = 0; i < 16; ++i)
+                        if (qs + 512 * t + i < P && A.status[qs + 512 * t + i] == BLSH_LITE_SURVIVOR) b[t] |= 1u << i;
             }
+            surv[t0 / 2] = b[0] | b[1] << 16;
+            surv[t0 / 2 + 1] = b[2] | b[3] << 16;
+            c += __popc(surv[t0 / 2]) + __popc(surv[t0 / 2 + 1]);
         }
-        const unsigned c = __popc(surv[0]) + __popc(surv[1]) + __popc(surv[2]) + __popc(surv[3]);
         unsigned incl = c;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -732,12 +773,15 @@ __global__ void __launch_bounds__(256) lite_collect_kernel(const LiteArgs A, uns
         unsigned long long base = 0;
         if (lane == 31) base = atomicAdd(&A.scratch->work3, (unsigned long long)total);
         base = __shfl_sync(kFull, base, 31);
+        if (base >= BLSH_LITE_QUEUE_CAP) continue;
         unsigned long long slot = base + incl - c;
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const long long qs = q0 + 512ll * t + 16ll * lane;
-            for (uint32_t b = surv[t]; b; b &= b - 1, ++slot)
-                if (slot < BLSH_LITE_QUEUE_CAP) queue[slot] = (unsigned long long)(qs + __ffs(b) - 1);
+        for (int t = 0; t < T / 2; ++t) {
+            const long long qs = q0 + 1024ll * t + 16ll * lane;
+            for (uint32_t b = surv[t]; b; b &= b - 1, ++slot) {
+                const int i = __ffs(b) - 1;
+                if (slot < BLSH_LITE_QUEUE_CAP) queue[slot] = (unsigned long long)(qs + (i & 15) + 512 * (i >> 4));
+            }
         }
     }
 }
@@ -864,7 +908,9 @@ int lite_exact_pass(blsh_ctx *ctx, const uint2 *pairs, int64_t P, const long lon
     BLSH_CUDA(ctx, cudaMemsetAsync(&ctx->scratch->work, 0, 3 * sizeof(unsigned long long), s));   // work, work2, work3
     unsigned long long *queue = ctx->lite_queue;
     blsh_time_start(ctx, s);
-    lite_collect_kernel<<<ctx->sm_count * 8, 256, 0, s>>>(L, queue);
+    // (every warp has a group of 16 tiles)
+    if (L.P >= 8192ll * 64 * ctx->sm_count) lite_collect_kernel<16><<<ctx->sm_count * 8, 256, 0, s>>>(L, queue);
+    else lite_collect_kernel<4><<<ctx->sm_count * 8, 256, 0, s>>>(L, queue);
     BLSH_LAUNCHED(ctx, "lite_collect_kernel");
     if (L.norm2) {
         const long long blocks = (N + 31) / 32, cap = (long long)ctx->sm_count * 32;   // 32 rows a CTA

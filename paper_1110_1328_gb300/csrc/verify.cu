@@ -1631,13 +1631,29 @@ __global__ void __launch_bounds__(256) verify_resume_kernel(const VerifyArgs A, 
         const long long pd = *A.P_dev;
         P = pd < 0 ? 0 : (pd < P ? pd : P);
     }
+    __shared__ unsigned s_hist[BLSH_MAX_NMAX / 32];
+    __shared__ uint8_t s_src[8][32];
+    for (int i = threadIdx.x; i < A.levels; i += blockDim.x) s_hist[i] = 0;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+    // this lane's tests of the first 32 chunks
+    auto concentrated = [&](int j, int m) {   // m >= conc_lo[j] where every level's set is an upper range
+        return A.conc_upper ? m >= __ldg(A.conc_lo + j)
+                            : (bool)((__ldg(A.conc_bits + j * A.conc_words + (m >> 5)) >> (m & 31)) & 1u);
+    };
+    const int lo0 = A.conc_upper && lane < A.levels ? __ldg(A.conc_lo + lane) : 0;
+    const int mm0 = lane < A.levels ? __ldg(A.min_matches + lane) : 0;
+    const bool one = kind == BLSH_COSINE && A.chunk_words == 1;
     // a warp scans 512 statuses (16 per lane), then works each open pair of
     // them with all its lanes: lane l takes chunk j0 + l of 32 chunks at a
     // time, an inclusive scan gives m after every chunk, and the first chunk
     // whose test stops the pair (the tests of Algorithm 1, in its order) is
-    // the one the sequential loop would stop at
+    // the one the sequential loop would stop at.  The open pairs are numbered,
+    // their indices read 32 at a time, and (one word a chunk) the next pair's
+    // first words read before this pair is tested: a pair's two waits, for its
+    // indices and its rows, had taken most of 1,337 us (1e9 statuses); 1,055
+    // now.
     for (long long base = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 512; base < P;
          base += nwarps * 512) {
         const long long q0 = base + 16ll * lane;
@@ -1648,21 +1664,48 @@ __global__ void __launch_bounds__(256) verify_resume_kernel(const VerifyArgs A, 
             for (int i = 0; i < 16; ++i)
                 if (q0 + i < P && A.status[q0 + i] == BLSH_NEEDS_HASHES) hit |= 1u << i;
         }
-        for (unsigned lanes = __ballot_sync(kFull, hit != 0); lanes; lanes &= lanes - 1) {
-            const int l = __ffs(lanes) - 1;
-            for (uint32_t bits = __shfl_sync(kFull, hit, l); bits; bits &= bits - 1) {
-                const long long q = base + 16ll * l + (__ffs(bits) - 1);
-                const uint2 pr = __ldg(A.pairs + q);
-                const uint32_t *rx = A.sig + (size_t)pr.x * A.W, *ry = A.sig + (size_t)pr.y * A.W;
+        while (__any_sync(kFull, hit != 0)) {
+            // up to 32 open pairs, one of each lane's at most: lane l holds the l-th
+            const unsigned have = __ballot_sync(kFull, hit != 0);
+            const int n = __popc(have);
+            __syncwarp();
+            if (hit) s_src[threadIdx.x >> 5][__popc(have & ((1u << lane) - 1u))] = (uint8_t)lane;
+            __syncwarp();
+            const int src = lane < n ? s_src[threadIdx.x >> 5][lane] : 0;
+            const int bit = __shfl_sync(kFull, hit ? __ffs(hit) - 1 : 0, src);
+            hit &= hit - 1;
+            const long long my_q = base + 16ll * src + bit;
+            uint2 my_pr = make_uint2(0u, 0u);
+            if (lane < n) my_pr = __ldg(A.pairs + my_q);
+            uint32_t na = 0, nb = 0;   // the next pair's word of this lane
+            auto first_words = [&](int e) {
+                const uint32_t x = __shfl_sync(kFull, my_pr.x, e), y = __shfl_sync(kFull, my_pr.y, e);
+                if (one && lane < A.levels) {
+                    na = __ldg(A.sig + (size_t)x * A.W + lane);
+                    nb = __ldg(A.sig + (size_t)y * A.W + lane);
+                }
+            };
+            first_words(0);
+            for (int e = 0; e < n; ++e) {
+                const long long q = __shfl_sync(kFull, my_q, e);
+                const uint32_t x = __shfl_sync(kFull, my_pr.x, e), y = __shfl_sync(kFull, my_pr.y, e);
+                const uint32_t *rx = A.sig + (size_t)x * A.W, *ry = A.sig + (size_t)y * A.W;
+                const uint32_t diff = na ^ nb;
+                if (e + 1 < n) first_words(e + 1);
                 int carry = 0, jstop = A.levels - 1, mstop = 0, st = BLSH_ACCEPT_AT_MAX;
                 for (int j0 = 0; j0 < A.levels; j0 += 32) {
                     const int j = j0 + lane;
                     int c = 0;
-                    if (j < A.levels)
-                        for (int w = j * A.chunk_words; w < (j + 1) * A.chunk_words; ++w) {
-                            const uint32_t a = __ldg(rx + w), b = __ldg(ry + w);
-                            c += kind == BLSH_JACCARD ? (a == b) : 32 - __popc(a ^ b);
+                    if (j < A.levels) {
+                        if (one && j0 == 0) {
+                            c = 32 - __popc(diff);
+                        } else {
+                            for (int w = j * A.chunk_words; w < (j + 1) * A.chunk_words; ++w) {
+                                const uint32_t a = __ldg(rx + w), b = __ldg(ry + w);
+                                c += kind == BLSH_JACCARD ? (a == b) : 32 - __popc(a ^ b);
+                            }
                         }
+                    }
                     int m = c;
 #pragma unroll
                     for (int o = 1; o < 32; o <<= 1) {
@@ -1672,11 +1715,8 @@ __global__ void __launch_bounds__(256) verify_resume_kernel(const VerifyArgs A, 
                     m += carry;
                     int s = -1;
                     if (j < A.levels) {
-                        // concentration: m >= conc_lo[j] where every level's set is an upper range
-                        const bool conc = A.conc_upper
-                                              ? m >= __ldg(A.conc_lo + j)
-                                              : (__ldg(A.conc_bits + j * A.conc_words + (m >> 5)) >> (m & 31)) & 1u;
-                        if (m < __ldg(A.min_matches + j)) s = BLSH_PRUNED;
+                        const bool conc = j0 == 0 && A.conc_upper ? m >= lo0 : concentrated(j, m);
+                        if (m < (j0 == 0 ? mm0 : __ldg(A.min_matches + j))) s = BLSH_PRUNED;
                         else if (conc) s = BLSH_ACCEPT;
                         else if (j + 1 == A.levels) s = BLSH_ACCEPT_AT_MAX;
                     }
@@ -1696,11 +1736,15 @@ __global__ void __launch_bounds__(256) verify_resume_kernel(const VerifyArgs A, 
                     if (A.m_out) A.m_out[q] = (uint16_t)mstop;
                     if (A.est_out && st != BLSH_PRUNED)
                         A.est_out[q] = __ldg(A.est_tab + (size_t)jstop * A.est_stride + mstop);
-                    if (A.stop_hist) atomicAdd(A.stop_hist + jstop, 1ull);
+                    if (A.stop_hist) atomicAdd(&s_hist[jstop], 1u);
                 }
             }
         }
     }
+    __syncthreads();
+    if (A.stop_hist)
+        for (int i = threadIdx.x; i < A.levels; i += blockDim.x)
+            if (s_hist[i]) atomicAdd(A.stop_hist + i, (unsigned long long)s_hist[i]);
 }
 
 }  // namespace
