@@ -32,10 +32,11 @@
 // rows of every feature are listed in any order, and a CTA per row x sets bit
 // y of an N-bit map in shared memory for every y > x in the lists of x's
 // indexed features; the map's set bits, in order, are x's candidates (counted
-// first, then written at scanned offsets).  A map costs N / 32 words per row
+// first, then written at scanned offsets; the write pass reads the counted maps
+// again where N^2 / 8 bytes fit the place of the key buffers).  A map costs N / 32 words per row
 // and pass (0.3 ps a word), the sort about 50 ps a key, which is where the
 // line lies.  20,000 tf-idf rows (2.4e7 keys, 1.7e7 pairs): 1.96 ms by sorting,
-// 0.55 ms with the maps.
+// 0.38 ms with the maps.
 #include <type_traits>
 
 #include "common.cuh"
@@ -87,13 +88,24 @@ __device__ __forceinline__ unsigned long long ap_key(const ApArgs &A, uint32_t f
     return ((unsigned long long)(0xffffffffu - A.df[f]) << 32) | f;
 }
 
-__global__ void __launch_bounds__(256) ap_stats_kernel(ApArgs A, long long nnz) {
+// df and max |value| of every feature; with `place`, also each element's number
+// among its feature's (in no particular order: where ap_post_kernel puts it).
+// Bound by the atomics on the most frequent features' addresses (20,000 rows:
+// one feature stands in most of them); the largest value is looked at before
+// it is replaced, and the numbers save ap_post_kernel the same atomics again
+// (20,000 rows, 1.15e6 elements: 35 us and 51 us, now 46 and 19: an
+// atomic whose answer is waited for costs more, two of them most).
+__global__ void __launch_bounds__(256) ap_stats_kernel(ApArgs A, long long nnz, uint32_t *place) {
     unsigned long long bad = 0;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nnz; e += (long long)gridDim.x * blockDim.x) {
         const uint32_t f = __ldg(A.indices + e);
         if (f >= A.dim) { ++bad; continue; }
-        atomicAdd(&A.df[f], 1u);
-        if (A.cosine) atomicMax(&A.maxabs[f], __float_as_uint(fabsf(__ldg(A.values + e))));
+        const uint32_t at = atomicAdd(&A.df[f], 1u);
+        if (place) place[e] = at;
+        if (A.cosine) {
+            const uint32_t v = __float_as_uint(fabsf(__ldg(A.values + e)));
+            if (v > __ldcg(&A.maxabs[f])) atomicMax(&A.maxabs[f], v);
+        }
     }
     if (bad) blsh_dev_error(A.scratch, BLSH_ERANGE, 0, bad);
 }
@@ -360,7 +372,7 @@ __global__ void __launch_bounds__(256) ap_write_kernel(const unsigned long long 
 // ---- candidates by bit maps ---------------------------------------------------
 
 // Every feature's rows, in any order: post[fstart[f] .. fstart[f + 1]).
-__global__ void __launch_bounds__(256) ap_post_kernel(ApArgs A, const uint32_t *fstart, uint32_t *cursor,
+__global__ void __launch_bounds__(256) ap_post_kernel(ApArgs A, const uint32_t *fstart, const uint32_t *place,
                                                       uint32_t *post) {
     const int lane = threadIdx.x & 31;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -368,7 +380,7 @@ __global__ void __launch_bounds__(256) ap_post_kernel(ApArgs A, const uint32_t *
         const long long s = __ldg(A.indptr + row), e = __ldg(A.indptr + row + 1);
         for (long long i = s + lane; i < e; i += 32) {
             const uint32_t f = __ldg(A.indices + i);
-            if (f < A.dim) post[__ldg(fstart + f) + atomicAdd(cursor + f, 1u)] = (uint32_t)row;
+            if (f < A.dim) post[__ldg(fstart + f) + __ldg(place + i)] = (uint32_t)row;
         }
     }
 }
@@ -378,13 +390,15 @@ __global__ void __launch_bounds__(256) ap_post_kernel(ApArgs A, const uint32_t *
 // y > x in the lists of x's indexed features.  MAP_WRITE: the pairs (x, y), y
 // increasing, from offset cnt[x] (after the scan).  Both MAP_COUNT and
 // MAP_DUPS (which forms no map) add the number of (feature, y) met to
-// *dup_total, the number of keys the sorting form would have.
+// *dup_total, the number of keys the sorting form would have.  With `kept`
+// MAP_COUNT leaves every row's map there (word x words + i, words from that of
+// x + 1 on) for ap_map_write_kernel.
 enum { MAP_DUPS, MAP_COUNT, MAP_WRITE };
 template <int MODE>
 __global__ void __launch_bounds__(256) ap_map_kernel(ApArgs A, const uint32_t *fstart, const uint32_t *post,
                                                      unsigned long long *cnt, unsigned long long *dup_total,
                                                      long long max_dups, uint32_t *pairs, long long cap,
-                                                     unsigned *next_row) {
+                                                     unsigned *next_row, uint32_t *kept) {
     extern __shared__ uint32_t map[];   // [(N + 31) / 32], zero between rows
     __shared__ unsigned s_cnt, s_row[2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -434,8 +448,10 @@ __global__ void __launch_bounds__(256) ap_map_kernel(ApArgs A, const uint32_t *f
         if (MODE == MAP_COUNT) {
             unsigned c = 0;
             for (int i = w0 + threadIdx.x; i < words; i += blockDim.x) {
-                c += __popc(map[i]);
+                const uint32_t m = map[i];
+                c += __popc(m);
                 map[i] = 0;
+                if (kept) kept[(size_t)x * words + i] = m;
             }
             c = __reduce_add_sync(kFull, c);
             if (lane == 0 && c) atomicAdd(&s_cnt, c);
@@ -466,6 +482,49 @@ __global__ void __launch_bounds__(256) ap_map_kernel(ApArgs A, const uint32_t *f
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) dups += __shfl_xor_sync(kFull, dups, o);
         if (lane == 0 && dups) atomicAdd(dup_total, dups);
+    }
+}
+
+// The pairs of the kept maps: a warp per row, 32 words at a time, put in order in
+// shared memory so that they leave in coalesced stores.  20,000 rows, 1.6e7
+// pairs: MAP_WRITE, which forms every map again, 172 us, 47 here.
+constexpr int kKeptWarps = 8;
+__global__ void __launch_bounds__(32 * kKeptWarps) ap_map_write_kernel(long long N, const uint32_t *kept,
+                                                                       const unsigned long long *cnt,
+                                                                       const unsigned long long *dup_total,
+                                                                       long long max_dups, uint32_t *pairs,
+                                                                       long long cap) {
+    __shared__ uint32_t s_y[kKeptWarps][1024];
+    if ((long long)*dup_total > max_dups) return;   // no pairs: the buffer was too small
+    const int lane = threadIdx.x & 31;
+    uint32_t *ys = s_y[threadIdx.x >> 5];
+    const int words = (int)((N + 31) >> 5);
+    const long long nw = (long long)gridDim.x * kKeptWarps;
+    for (long long x = (long long)blockIdx.x * kKeptWarps + (threadIdx.x >> 5); x < N; x += nw) {
+        long long base = (long long)cnt[x];
+        const long long end = (long long)cnt[x + 1];
+        const uint32_t *row = kept + (size_t)x * words;
+        int i = (int)((x + 1) >> 5) + lane;
+        uint32_t next = i < words && base < end ? __ldcs(row + i) : 0u;
+        for (; base < end; i += 32) {
+            const uint32_t m = next;
+            next = i + 32 < words ? __ldcs(row + i + 32) : 0u;
+            const int c = __popc(m);
+            int incl = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += v;
+            }
+            const int total = __shfl_sync(kFull, incl, 31);
+            int at = incl - c;
+            for (uint32_t b = m; b; b &= b - 1) ys[at++] = 32u * i + __ffs(b) - 1u;
+            __syncwarp();
+            for (int k = lane; k < total; k += 32)
+                if (base + k < cap) reinterpret_cast<uint2 *>(pairs)[base + k] = make_uint2((uint32_t)x, ys[k]);
+            __syncwarp();
+            base += total;
+        }
     }
 }
 
@@ -599,8 +658,13 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
     // 1. statistics
     BLSH_CUDA(ctx, cudaMemsetAsync(A.df, 0, L.indexed - L.df, s));   // df and maxabs
     BLSH_CUDA(ctx, cudaMemsetAsync(ws + L.grand, 0, 64, s));         // the totals and counters
+    // bit maps where they cost less than sorting the keys (see the top of the
+    // file), and for a count-only call, which then forms no map
+    const bool count_only = cap == 0 || max_dups == 0;
+    const bool maps = N <= kMapRows && nnz < (1ll << 31) && (count_only || N * N <= 4096 * max_dups);
+    uint32_t *place = (uint32_t *)(ws + L.iv0);
     blsh_time_start(ctx, s);
-    ap_stats_kernel<<<grid_for(nnz, 256), 256, 0, s>>>(A, nnz);
+    ap_stats_kernel<<<grid_for(nnz, 256), 256, 0, s>>>(A, nnz, maps ? place : nullptr);
     BLSH_LAUNCHED(ctx, "ap_stats_kernel");
     // 2. indexed features
     blsh_time_start(ctx, s);
@@ -611,22 +675,17 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
     blsh_time_start(ctx, s);
     ap_prefix_cta_kernel<<<(unsigned)sms * 4, kCtaThreads, 0, s>>>(A, mid, n_mid);
     BLSH_LAUNCHED(ctx, "ap_prefix_cta_kernel");
-    // bit maps where they cost less than sorting the keys (see the top of the
-    // file), and for a count-only call, which then forms no map
-    const bool count_only = cap == 0 || max_dups == 0;
-    if (N <= kMapRows && nnz < (1ll << 31) && (count_only || N * N <= 4096 * max_dups)) {
-        uint32_t *fstart = (uint32_t *)(ws + L.fcnt), *cursor = fstart + dim + 1;   // in the (dim + 1) * 8 bytes
-        uint32_t *post = (uint32_t *)(ws + L.ik0);
-        BLSH_CUDA(ctx, cudaMemsetAsync(cursor, 0, dim * 4, s));
+    if (maps) {
+        uint32_t *fstart = (uint32_t *)(ws + L.fcnt), *post = (uint32_t *)(ws + L.ik0);
         if (const int rc = blsh_scan::run<uint32_t>(ctx, A.df, fstart, dim, (uint32_t *)partial64, fstart + dim, s)) return rc;
         blsh_time_start(ctx, s);
-        ap_post_kernel<<<grid_for(N, 8), 256, 0, s>>>(A, fstart, cursor, post);
+        ap_post_kernel<<<grid_for(N, 8), 256, 0, s>>>(A, fstart, place, post);
         BLSH_LAUNCHED(ctx, "ap_post_kernel");
         const unsigned grid = (unsigned)(N < (long long)sms * 8 ? N : (long long)sms * 8);
         if (count_only) {
             blsh_time_start(ctx, s);
             ap_map_kernel<MAP_DUPS><<<grid, 256, 0, s>>>(A, fstart, post, nullptr, dup_total, 0, nullptr, 0,
-                                                                n_mid + 1);
+                                                                n_mid + 1, nullptr);
             BLSH_LAUNCHED(ctx, "ap_map_kernel (keys)");
             ap_count_only_kernel<<<1, 1, 0, s>>>(dup_total, n_pairs, n_dups);
             BLSH_LAUNCHED(ctx, "ap_count_only_kernel");
@@ -639,14 +698,20 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
             BLSH_CUDA(ctx, cudaFuncSetAttribute(ap_map_kernel<MAP_WRITE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)(kMapRows / 8)));
         }
+        // the maps are kept for the write pass where they fit the key buffers' place (N^2 / 8 of 32 max_dups bytes)
+        uint32_t *kept = (size_t)N * smem <= L.hist - L.k0 ? (uint32_t *)(ws + L.k0) : nullptr;
         blsh_time_start(ctx, s);
         ap_map_kernel<MAP_COUNT><<<grid, 256, smem, s>>>(A, fstart, post, ycnt, dup_total, max_dups, nullptr, 0,
-                                                             n_mid + 1);
+                                                             n_mid + 1, kept);
         BLSH_LAUNCHED(ctx, "ap_map_kernel (count pass)");
         if (const int rc = blsh_scan::run<unsigned long long>(ctx, ycnt, ycnt, N, partial64, ycnt + N, s)) return rc;
         blsh_time_start(ctx, s);
-        ap_map_kernel<MAP_WRITE><<<grid, 256, smem, s>>>(A, fstart, post, ycnt, dup_total, max_dups, pairs, cap,
-                                                             n_mid + 2);
+        if (kept)
+            ap_map_write_kernel<<<grid_for(N, kKeptWarps), 32 * kKeptWarps, 0, s>>>(N, kept, ycnt, dup_total, max_dups,
+                                                                                     pairs, cap);
+        else
+            ap_map_kernel<MAP_WRITE><<<grid, 256, smem, s>>>(A, fstart, post, ycnt, dup_total, max_dups, pairs, cap,
+                                                             n_mid + 2, nullptr);
         BLSH_LAUNCHED(ctx, "ap_map_kernel (write pass)");
         ap_finish_kernel<<<1, 1, 0, s>>>(ycnt + N, dup_total, max_dups, cap, n_pairs, n_dups, ctx->scratch);
         BLSH_LAUNCHED(ctx, "ap_finish_kernel");

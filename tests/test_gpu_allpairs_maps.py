@@ -84,3 +84,19 @@ def test_truncated_map_output(B, ctx):
     less = dups - len(want) + 11
     got, k, _ = candidates(B, ctx, csr, 0.5, O.JACCARD, cap_less=less)
     assert k == len(want) and np.array_equal(got, want[:-11])
+
+
+@pytest.mark.parametrize("dim, kept", [(700, True), (4500, False)])
+@pytest.mark.parametrize("kind", [O.JACCARD, O.COSINE])
+@pytest.mark.parametrize("cap_less", [0, 1000])
+def test_maps_kept_or_formed_again(B, ctx, dim, kept, kind, cap_less):
+    """The write pass from the maps the count pass kept, and where they do not
+    fit the place of the key buffers (32 bytes a key)."""
+    n = 6001
+    csr = rows_csr(np.full(n, 3), dim, dim, kind == O.COSINE)
+    want = O.allpairs_candidates(csr, 0.01, kind)   # every feature indexed: 4.5 n^2 / dim keys
+    got, k, names = candidates(B, ctx, csr, 0.01, kind, cap_less)
+    assert k == len(want) and "ap_map_kernel (write pass)" in names
+    m = min(k, len(got))
+    assert np.array_equal(got[:m], want[:m]) and np.all(got[m:] == 2**32 - 1)
+    assert (n * n <= 256 * (len(got) + cap_less)) == kept
