@@ -1146,7 +1146,7 @@ __global__ void __launch_bounds__(32 * kSmallWarps) band_small_kernel(BandArgs A
     for (int bit = 0; bit < key_bits; bit += 8) {
         for (int d = lane; d < 256; d += 32) cnt[w][d] = 0;
         __syncwarp();
-        blsh_radix::warp_ranks<ROUNDS>(cnt[w], rank, [&](int r, bool &ok) {
+        blsh_radix::warp_ranks<8, ROUNDS>(cnt[w], rank, [&](int r, bool &ok) {
             ok = r < rounds && base + 32 * r < N;
             return (key[r] >> bit) & 255u;
         });
