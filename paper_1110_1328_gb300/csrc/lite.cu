@@ -4,13 +4,13 @@
 // pruning loop over at most h hashes, no concentration test; an unpruned
 // pair is marked as a survivor in its status byte.  Pass 2 (this file) gives
 // every survivor its exact similarity: the survivors are collected into a
-// queue (one atomic per tile of 512 statuses) and warps take them in
-// grid-stride order, so the many survivors of one bucket of near-duplicates
-// spread over the GPU; a warp computes a survivor's similarity
-// cooperatively by intersecting the two sorted index lists (each lane
-// binary-searches elements of the shorter row in the longer one, staged in
-// shared memory when it is short).  Survivors beyond the queue's capacity
-// are found by a scan of the statuses in tiles handed out by a counter.
+// queue (one atomic per 4 or 16 tiles of 512 statuses) and warps take batches
+// of up to 32 from a counter, so the many survivors of one bucket of
+// near-duplicates spread over the GPU; a warp intersects a batch's sorted
+// index lists together, the elements of the shorter rows dealt over its lanes
+// and searched in the longer ones in shared memory (lite_flat), or a few
+// survivors one by one (lite_few).  Survivors beyond the queue's capacity are
+// found by a scan of the statuses in tiles handed out by a counter.
 //
 //   Jaccard: s = |A n B| / |A u B|, one FP64 division.
 //   Cosine:  s = D / sqrt(Nx * Ny) with D = sum over common indices of
@@ -116,7 +116,8 @@ constexpr int kLiteStage = 512;   // half the elements a warp stages in shared m
 // staged in the warp's shared memory, a tile at a time.  (Searching rows of
 // more than 512 elements in global memory, two lookups in flight, took 62 us
 // for 3,600 survivors whose longest rows have some 900 elements; 42 now.)
-template <bool COSINE>
+// KEEP: x's elements are looked up in y, whichever is shorter.
+template <bool COSINE, bool KEEP = false>
 __device__ __forceinline__ void lite_exact_one(const LiteArgs &A, long long ax, long long na, long long ay,
                                                long long nb, bool have_norms, uint32_t *w_idx,
                                                long long &D_out, long long &Nx_out, long long &Ny_out) {
@@ -124,9 +125,9 @@ __device__ __forceinline__ void lite_exact_one(const LiteArgs &A, long long ax, 
     // the shorter row S, the longer row L (the sums below do not depend on
     // which row is which)
     long long s0 = ax, ns = na, l0 = ay, nl = nb;
-    if (nb < na) { s0 = ay; ns = nb; l0 = ax; nl = na; }
+    if (!KEEP && nb < na) { s0 = ay; ns = nb; l0 = ax; nl = na; }
     long long inter = 0, D = 0, Ns = 0, Nl = 0;
-    if (nl <= 32) {
+    if (!KEEP && nl <= 32) {
         // lane e holds element e of both rows
         uint32_t si = 0, li = 0;
         float sv = 0.0f, lv = 0.0f;
@@ -169,6 +170,11 @@ __device__ __forceinline__ void lite_exact_one(const LiteArgs &A, long long ax, 
         // forms one survivor has nothing else to wait behind)
         constexpr int kTile = 2 * kLiteStage;
         long long sp = 0;                                  // the shorter row's elements done
+        if (KEEP && COSINE && !have_norms && nl == 0)      // no tile to look them up in
+            for (long long i = lane; i < ns; i += 32) {
+                const float v = __ldg(A.values + s0 + i);
+                Ns += fixed_term(v, v);
+            }
         for (long long tb = 0; tb < nl && (sp < ns || (COSINE && !have_norms)); tb += kTile) {
             const int tn = (int)(nl - tb < kTile ? nl - tb : kTile);
             __syncwarp();                                  // the previous tile is done with the stage
@@ -222,7 +228,7 @@ __device__ __forceinline__ void lite_exact_one(const LiteArgs &A, long long ax, 
     // and the two squared norms (which row is which does not matter: the
     // similarity uses their product)
     if (!COSINE) {
-        D_out = nl > 32 ? warp_sum(inter) : inter;
+        D_out = KEEP || nl > 32 ? warp_sum(inter) : inter;
     } else {
         D_out = warp_sum(D);
         if (!have_norms) {
@@ -565,9 +571,17 @@ __device__ __forceinline__ LiteSums lite_few(const LiteArgs &A, unsigned todo, l
 // those dependent loads overlap across the batch; then the warp forms their
 // sums, and finally every lane turns its own survivor's sums into the
 // similarity and writes it with the verdict.
+//
+// heavy (or NULL): survivors both of whose rows have more than kLiteHeavy
+// elements are put there instead, while it has room, for lite_heavy: one of
+// them takes a warp as long as dozens of batches, and a batch of 32 (a long row's
+// survivors follow each other) held its warp 0.3 ms after all others had
+// ended (a search over 6e5 vectors: queue 478 us, with the list 202 + 38; 256
+// elements 184 + 39, 1,024 237 + 37).
+constexpr int kLiteHeavy = 512;
 template <bool COSINE>
 __device__ __forceinline__ void lite_batch(const LiteArgs &A, long long my_q, bool have_norms, uint32_t *w_idx,
-                                           uint32_t *flat) {
+                                           uint32_t *flat, unsigned long long *heavy = nullptr) {
     long long ax = 0, ex = 0, ay = 0, ey = 0;
     LiteSums my = {0, 0, 0};
     if (my_q >= 0) {
@@ -579,6 +593,13 @@ __device__ __forceinline__ void lite_batch(const LiteArgs &A, long long my_q, bo
         if (have_norms) {
             my.Nx = __ldg(A.norm2 + pr.x);
             my.Ny = __ldg(A.norm2 + pr.y);
+        }
+    }
+    if (heavy && ex - ax > kLiteHeavy && ey - ay > kLiteHeavy) {
+        const unsigned long long slot = atomicAdd(&A.scratch->recheck_count, 1ull);
+        if (slot < BLSH_RECHECK_CAP) {
+            heavy[slot] = (unsigned long long)my_q;
+            my_q = -1;
         }
     }
     unsigned todo = __ballot_sync(kFull, my_q >= 0);
@@ -659,14 +680,74 @@ __global__ void __launch_bounds__(256) row_norm2_kernel(const int64_t *__restric
 constexpr int kLiteWarpWords = 2 * kLiteStage + kFlatWords + 272;
 static_assert(kLiteWarpWords % 4 == 0, "16-byte rows");
 
+// The listed survivors of two long rows, a CTA each: warp w takes the w-th eighth
+// of the shorter row and the part of the longer one that its elements can lie
+// in (the parts cover it), and the warps' sums are added.
 template <bool COSINE>
-__global__ void __launch_bounds__(256, 4) lite_exact_kernel(const LiteArgs A) {
+__device__ __forceinline__ void lite_heavy(const LiteArgs &A, const unsigned long long *heavy, bool have_norms,
+                                           uint32_t *w_idx) {
+    __shared__ long long s_sum[8][3];
+    __shared__ unsigned long long s_item;
+    const int warp = threadIdx.x >> 5;
+    const unsigned long long listed = A.scratch->recheck_count;
+    const unsigned long long n = listed < BLSH_RECHECK_CAP ? listed : BLSH_RECHECK_CAP;
+    if (n == 0) return;
+    for (;;) {
+        __syncthreads();                                   // the previous survivor's sums have been read
+        if (threadIdx.x == 0) s_item = atomicAdd(&A.scratch->hash_work, 1ull);
+        __syncthreads();
+        if (s_item >= n) break;
+        const long long q = (long long)heavy[s_item];
+        const uint2 pr = __ldg(A.pairs + q);
+        const long long ax = __ldg(A.indptr + pr.x), na = __ldg(A.indptr + pr.x + 1) - ax;
+        const long long ay = __ldg(A.indptr + pr.y), nb = __ldg(A.indptr + pr.y + 1) - ay;
+        const bool swap = nb < na;
+        const long long s0 = swap ? ay : ax, ns = swap ? nb : na, l0 = swap ? ax : ay, nl = swap ? na : nb;
+        // where this warp's parts of the two rows begin, and the next one's (equal indices stay together)
+        long long at[2], cut[2];
+#pragma unroll 1
+        for (int e = 0; e < 2; ++e) {
+            const int w = warp + e;
+            long long i = ns * w / 8;
+            while (i > 0 && i < ns && __ldg(A.indices + s0 + i) == __ldg(A.indices + s0 + i - 1)) ++i;
+            at[e] = i;
+            cut[e] = w == 0 ? 0 : i >= ns ? nl : lower_bound(A.indices + l0, nl, __ldg(A.indices + s0 + i));
+        }
+        const long long sa = at[0], sn = at[1] - sa, ln = cut[1] - cut[0];
+        long long D = 0, Ns = 0, Nl = 0;
+        lite_exact_one<COSINE, true>(A, s0 + sa, sn, l0 + cut[0], ln, have_norms, w_idx, D, Ns, Nl);
+        if ((threadIdx.x & 31) == 0) {
+            s_sum[warp][0] = D;
+            s_sum[warp][1] = Ns;
+            s_sum[warp][2] = Nl;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            long long d = 0, nx = 0, ny = 0;
+            for (int w = 0; w < 8; ++w) {
+                d += s_sum[w][0];
+                nx += s_sum[w][1];
+                ny += s_sum[w][2];
+            }
+            if (have_norms) {
+                nx = __ldg(A.norm2 + pr.x);
+                ny = __ldg(A.norm2 + pr.y);
+            }
+            const double sim = lite_similarity<COSINE>(d, nx, ny, na, nb);
+            A.sim[q] = sim;
+            A.status[q] = sim > A.t ? BLSH_LITE_ACCEPT : BLSH_LITE_REJECT;
+        }
+    }
+    __syncthreads();
+}
+
+template <bool COSINE>
+__global__ void __launch_bounds__(256, 4) lite_exact_kernel(const LiteArgs A, const unsigned long long *heavy) {
     long long P = A.P;
     if (A.P_dev) {
         const long long pd = *A.P_dev;
         P = pd < 0 ? 0 : (pd < P ? pd : P);
     }
-    if (A.scratch->work3 <= BLSH_LITE_QUEUE_CAP) return;   // every survivor was queued
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     // per warp: the stage for longer rows' indices, lite_flat's area, and the
@@ -676,6 +757,8 @@ __global__ void __launch_bounds__(256, 4) lite_exact_kernel(const LiteArgs A) {
     uint32_t *flat = w_idx + 2 * kLiteStage;
     uint16_t *w_list = reinterpret_cast<uint16_t *>(flat + kFlatWords);
     const bool have_norms = COSINE && A.norm2 && A.scratch->norm2_valid;
+    lite_heavy<COSINE>(A, heavy, have_norms, w_idx);
+    if (A.scratch->work3 <= BLSH_LITE_QUEUE_CAP) return;   // every survivor was queued
     // A warp takes kLiteGrab tiles of 512 statuses per grab of the work
     // counter; a lane reads 16 statuses with one 16-byte load; the tiles'
     // survivors are listed in shared memory and computed 32 at a time, what is
@@ -730,12 +813,7 @@ __global__ void __launch_bounds__(256, 4) lite_exact_kernel(const LiteArgs A) {
 // four tiles the counter's one address (and a load in flight less often) 1e9 statuses
 // took 495 us, 271 so.
 template <int T>
-__global__ void __launch_bounds__(256) lite_collect_kernel(const LiteArgs A, unsigned long long *queue) {
-    long long P = A.P;
-    if (A.P_dev) {
-        const long long pd = *A.P_dev;
-        P = pd < 0 ? 0 : (pd < P ? pd : P);
-    }
+__device__ __forceinline__ void lite_collect(const LiteArgs &A, long long P, unsigned long long *queue) {
     const int lane = threadIdx.x & 31;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
     for (long long q0 = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * (512 * T); q0 < P;
@@ -786,11 +864,22 @@ __global__ void __launch_bounds__(256) lite_collect_kernel(const LiteArgs A, uns
     }
 }
 
+__global__ void __launch_bounds__(256) lite_collect_kernel(const LiteArgs A, unsigned long long *queue) {
+    long long P = A.P;
+    if (A.P_dev) {
+        const long long pd = *A.P_dev;
+        P = pd < 0 ? 0 : (pd < P ? pd : P);
+    }
+    if (P >= 8192ll * ((long long)gridDim.x * blockDim.x >> 5)) lite_collect<16>(A, P, queue);
+    else lite_collect<4>(A, P, queue);
+}
+
 // The queued survivors, a batch per warp at a time from a counter: the
 // survivors of one dense tile (a bucket of near-duplicates) spread over many
 // warps, and a warp with long rows takes fewer batches.
 template <bool COSINE>
-__global__ void __launch_bounds__(256, 4) lite_queue_kernel(const LiteArgs A, const unsigned long long *queue) {
+__global__ void __launch_bounds__(256, 4) lite_queue_kernel(const LiteArgs A, const unsigned long long *queue,
+                                                            unsigned long long *heavy) {
     const unsigned long long total = A.scratch->work3;
     const unsigned long long n = total < BLSH_LITE_QUEUE_CAP ? total : BLSH_LITE_QUEUE_CAP;
     extern __shared__ uint32_t lite_smem[];
@@ -810,7 +899,7 @@ __global__ void __launch_bounds__(256, 4) lite_queue_kernel(const LiteArgs A, co
         base = __shfl_sync(kFull, base, 0);
         if (base >= n) break;
         const long long q = lane < bs && base + lane < n ? (long long)queue[base + lane] : -1;
-        lite_batch<COSINE>(A, q, have_norms, w_idx, flat);
+        lite_batch<COSINE>(A, q, have_norms, w_idx, flat, heavy);
     }
 }
 
@@ -905,12 +994,13 @@ int lite_exact_pass(blsh_ctx *ctx, const uint2 *pairs, int64_t P, const long lon
     // two sums itself (no allocation here: this is a hot call)
     if (values && N > 0 && ctx->norm2_cap >= N) L.norm2 = (const long long *)ctx->norm2;
     // survivors: queued (balanced over warps), then any beyond the queue in place
-    BLSH_CUDA(ctx, cudaMemsetAsync(&ctx->scratch->work, 0, 3 * sizeof(unsigned long long), s));   // work, work2, work3
+    // work, work2, work3, recheck_count (survivors of two long rows) .. hash_work (the next of them)
+    BLSH_CUDA(ctx, cudaMemsetAsync(&ctx->scratch->work, 0, offsetof(blsh_dev_scratch, norm2_valid) -
+                                                              offsetof(blsh_dev_scratch, work), s));
     unsigned long long *queue = ctx->lite_queue;
+    unsigned long long *heavy = reinterpret_cast<unsigned long long *>(ctx->recheck_queue);   // [BLSH_RECHECK_CAP]
     blsh_time_start(ctx, s);
-    // (every warp has a group of 16 tiles)
-    if (L.P >= 8192ll * 64 * ctx->sm_count) lite_collect_kernel<16><<<ctx->sm_count * 8, 256, 0, s>>>(L, queue);
-    else lite_collect_kernel<4><<<ctx->sm_count * 8, 256, 0, s>>>(L, queue);
+    lite_collect_kernel<<<ctx->sm_count * 8, 256, 0, s>>>(L, queue);
     BLSH_LAUNCHED(ctx, "lite_collect_kernel");
     if (L.norm2) {
         const long long blocks = (N + 31) / 32, cap = (long long)ctx->sm_count * 32;   // 32 rows a CTA
@@ -928,10 +1018,10 @@ int lite_exact_pass(blsh_ctx *ctx, const uint2 *pairs, int64_t P, const long lon
                                             (int)smem));
         BLSH_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, lite_queue_kernel<true>, 256, smem));
         blsh_time_start(ctx, s);
-        lite_queue_kernel<true><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L, queue);
+        lite_queue_kernel<true><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L, queue, heavy);
         BLSH_LAUNCHED(ctx, "lite_queue_kernel");
         blsh_time_start(ctx, s);
-        lite_exact_kernel<true><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L);
+        lite_exact_kernel<true><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L, heavy);
         BLSH_LAUNCHED(ctx, "lite_exact_kernel");
     } else {
         BLSH_CUDA(ctx, cudaFuncSetAttribute(lite_queue_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -940,10 +1030,10 @@ int lite_exact_pass(blsh_ctx *ctx, const uint2 *pairs, int64_t P, const long lon
                                             (int)smem));
         BLSH_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, lite_queue_kernel<false>, 256, smem));
         blsh_time_start(ctx, s);
-        lite_queue_kernel<false><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L, queue);
+        lite_queue_kernel<false><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L, queue, heavy);
         BLSH_LAUNCHED(ctx, "lite_queue_kernel");
         blsh_time_start(ctx, s);
-        lite_exact_kernel<false><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L);
+        lite_exact_kernel<false><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L, heavy);
         BLSH_LAUNCHED(ctx, "lite_exact_kernel");
     }
     return BLSH_OK;
