@@ -52,3 +52,34 @@ def test_srp_rows(B, ctx, n, form, bits):
         call(ctx, ip, torch.from_numpy(indices.view(np.int32)).to(dev), val, Rd, sig)
         assert B.blsh_status(ctx) == rc
         assert np.array_equal(sig.cpu().numpy().view(np.uint32), want)
+
+
+@pytest.mark.parametrize("form", ["float", "codes"])
+def test_rechecked_long_rows(B, ctx, form):
+    """Rows whose every sum is zero, or cancels to its last entry, at the
+    lengths where a recheck takes more entries at a time."""
+    dim, bits = 4000, 256
+    half = dim // 2
+    if form == "float":
+        R = synth.gaussian_matrix(dim, bits, seed=9)
+        R[half:] = -R[:half]
+        Rd, oracle, call = torch.from_numpy(R).to(dev), O.srp_sparse, B.blsh_srp_sparse
+    else:
+        R = np.maximum(O.gaussian_codes(9, dim, bits), 1)
+        R[half:] = (65536 - R[:half].astype(np.int64)).astype(np.uint16)   # decoded: the negatives
+        Rd, oracle, call = torch.from_numpy(R.view(np.int16)).to(dev), O.srp_sparse_q16, B.blsh_srp_sparse_q16
+    rng = np.random.default_rng(4)
+    rows, vals = [], []
+    for n in (1, 15, 63, 64, 65, 255, 256, 257, 512, 1000):   # pairs of entries that cancel
+        f = np.sort(rng.choice(half, n, replace=False))
+        v = rng.standard_normal(n).astype(np.float32)
+        rows += [np.concatenate([f, f + half])] * 2
+        vals += [np.concatenate([v, v]), np.concatenate([v, v[:-1], np.nextafter(v[-1:], np.float32(9))])]
+    csr = synth.CSR(np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int64),
+                    np.concatenate(rows).astype(np.uint32), np.concatenate(vals).astype(np.float32), dim)
+    sig = torch.zeros((csr.n, bits // 32), dtype=torch.int32, device=dev)
+    call(ctx, torch.from_numpy(csr.indptr).to(dev), torch.from_numpy(csr.indices.view(np.int32)).to(dev),
+         torch.from_numpy(csr.values).to(dev), Rd, sig)
+    rc, c = B.blsh_status(ctx, counters=True)
+    assert rc == 0 and c[2] >= csr.n * bits // 2
+    assert np.array_equal(sig.cpu().numpy().view(np.uint32), oracle(csr, R))
