@@ -401,7 +401,7 @@ class ClockSampler:
 # dram__bytes_write.sum of the bench step under --profile-step); reported as
 # the roofline's traffic for the workload it was taken on (per step, like the
 # algorithmic bytes), and to be taken again whenever the kernel changes.
-NCU_TRAFFIC = {("large-mixed", "srp_sparse4_kernel (two-byte codes)"): (20874986240 + 163516160) + (6676972544 + 165890816)}
+NCU_TRAFFIC = {}
 
 
 def load_tensor_peak():
@@ -537,13 +537,41 @@ def verification_totals(work, timed):
     if "verify_first_kernel" in timed:
         work["verify_first_kernel"] = (first, "B")
         work["verify_kernel"] = (total - first, "B")
-    if "verify_tile_kernel" in timed:     # both passes in one kernel
-        work["verify_tile_kernel"] = (total, "B")
-    names = [n for n in ("verify_tile_kernel", "verify_first_kernel", "verify_kernel", "verify_resume_kernel")
-             if n in timed]
+    for name in ("verify_tile_kernel", "verify_sets_kernel"):   # all of it in one kernel
+        if name in timed:
+            work[name] = (total, "B")
+    names = [n for n in ("verify_tile_kernel", "verify_sets_kernel", "verify_first_kernel", "verify_kernel",
+                         "verify_resume_kernel") if n in timed]
     vbytes = total + work.get("verify_resume_kernel", (0, "B"))[0]
     v_ms = sum(timed[n][1] for n in names)
     return vbytes, v_ms, " + ".join(names)
+
+
+def banding_work(kind, N, P, rows, bands):
+    """Algorithmic bytes of the banding kernels: n = N * bands (object, band)
+    entries, P pairs.  Key rows of up to 128 bytes are staged: 32-bit keys sorted
+    band by band, eight or nine bits a pass, an object's id its position at
+    first; longer ones take 64-bit keys with the band in them."""
+    n = N * bands
+    if kind == 1:
+        lane = 1 if rows <= 8 else 2 if rows <= 16 else 4
+        staged, obj_rows = rows <= 32 and bands * lane <= 128, N * bands * ((rows + 7) // 8)
+        sig_bytes, bits = N * bands * rows // 8, rows
+    else:
+        staged, obj_rows = ((bands + 3) & ~3) <= 32, N * bands * 4
+        sig_bytes, bits = N * bands * rows * 4, 32 - max(1, (bands - 1).bit_length())
+    if staged:
+        kb, ids = 4, 0
+        passes = min((bits + 7) // 8, (bits + 8) // 9)
+    else:
+        kb, ids = 8, 4
+        passes = 8 if kind == 0 else (max(1, (bands - 1).bit_length()) + rows + 7) // 8
+    return {"band_keys_kernel": (sig_bytes + n * (kb + ids) + obj_rows, "B"),
+            "band_small_kernel": (sig_bytes + n * 8 + obj_rows, "B"),   # keys and sort in one launch
+            "digit_hist_kernel": (passes * n * kb, "B"),
+            "digit_scatter_kernel": (passes * 2 * n * (kb + 4) - (n * 4 if staged else 0), "B"),
+            "emit_warp_kernel (count pass)": (n * (kb + 4) + obj_rows + n * 8, "B"),
+            "emit_warp_kernel (write pass)": (n * (4 + 8) + P * 8, "B")}
 
 
 def kernel_work(B, pipe, w, objs, st, nu, lst, need):
@@ -601,21 +629,8 @@ def kernel_work(B, pipe, w, objs, st, nu, lst, need):
         nnz = int(objs.indptr[-1])
         work["minhash_kernel"] = (nnz * 4 + N * (8 + 4 * w["n_hashes"]), "B")
     # banding: n = N * bands (object, band) entries
-    n, rows, bands = N * w["bands"], w["rows"], w["bands"]
-    if w["kind"] == 1:
-        kb = 4 if max(1, (bands - 1).bit_length()) + rows <= 32 else 8
-        obj_rows = N * bands * ((rows + 7) // 8)
-    else:   # 32-bit class keys while a row of class ids fits the staging (32 words), else 64-bit band hashes
-        kb = 4 if ((bands + 3) & ~3) <= 32 else 8
-        obj_rows = N * bands * 4
+    work.update(banding_work(w["kind"], N, P, w["rows"], w["bands"]))
     emit = "emit_warp_kernel"
-    passes = (8 * kb + 7) // 8 if w["kind"] == 0 else (max(1, (bands - 1).bit_length()) + rows + 7) // 8
-    sig_bytes = N * bands * rows // 8 if w["kind"] == 1 else N * bands * rows * 4   # the banded hashes
-    work["band_keys_kernel"] = (sig_bytes + n * (kb + 4) + obj_rows, "B")
-    work["digit_hist_kernel"] = (passes * n * kb, "B")
-    work["digit_scatter_kernel"] = (passes * 2 * n * (kb + 4), "B")
-    work[emit + " (count pass)"] = (n * (kb + 4) + obj_rows + n * 8, "B")
-    work[emit + " (write pass)"] = (n * (kb + 4 + 8) + obj_rows + P * 8, "B")
     for ps in (" (count pass)", " (write pass)"):    # the unstaged form
         work["emit_kernel" + ps] = work[emit + ps]
     if getattr(pipe, "allpairs", False):
@@ -629,11 +644,16 @@ def kernel_work(B, pipe, w, objs, st, nu, lst, need):
         p_idx = (xb + max(1, int(dim).bit_length()) + 1 + 7) // 8
         p_key = (32 + xb + 1 + 7) // 8
         for name in list(work):
-            if name.startswith(("band_keys", "digit_", "emit_", "class_id")):
+            if name.startswith(("band_", "digit_", "emit_", "class_id")):
                 del work[name]
         work["ap_stats_kernel"] = (nnz * 8 + dim * 8, "B")
         work["ap_prefix_warp_kernel"] = (nnz * 9, "B")
         work["ap_prefix_cta_kernel"] = (nnz * 9, "B")
+        if N <= 1 << 19 and N * N <= 4096 * dups:   # bit maps: every feature's rows listed, the maps of N^2 / 2 bits kept
+            work["ap_post_kernel"] = (nnz * 12, "B")
+            kept_maps = N * N // 16 if N * N <= 256 * dups else 0
+            work["ap_map_kernel (count pass)"] = (nnz * 5 + dups * 4 + kept_maps, "B")
+            work["ap_map_kernel (write pass)"] = ((kept_maps or nnz * 5 + dups * 4) + P * 8, "B")
         work["ap_index_keys_kernel"] = (nnz * (5 + 8) + N * 16, "B")
         work["digit_hist_kernel"] = (p_idx * nnz * 8 + p_key * dups * 8, "B")
         work["digit_scatter_kernel"] = (p_idx * 2 * nnz * 12 + p_key * 2 * dups * 12, "B")
@@ -644,6 +664,7 @@ def kernel_work(B, pipe, w, objs, st, nu, lst, need):
     n_keep = int(kept.sum())
     work["compact_count"] = ((2 if pipe.with_lite else 1) * P, "B")
     work["compact_write"] = ((2 if pipe.with_lite else 1) * P + 8 * n_keep, "B")
+    work["compact_few"] = work["compact_write"]    # one launch for few statuses
     return work
 
 
@@ -1074,7 +1095,8 @@ def run_verify_large(args, w):
     kept = int(((stn == B.ACCEPT) | (stn == B.ACCEPT_AT_MAX)).sum())
     alg = P * (8 + 5) + 4 * kept + chunks * (w["k"] // 4)
     sector = P * (8 + 9) + P * 2 * 32
-    v_names = [n for n in ("verify_tile_kernel", "verify_first_kernel", "verify_kernel") if n in kern]
+    v_names = [n for n in ("verify_tile_kernel", "verify_sets_kernel", "verify_first_kernel", "verify_kernel")
+               if n in kern]
     vk = sum(kern[n] for n in v_names) or ms
     print(json.dumps({"metric": METRIC, "value": round(P / (ms / 1e3), 1), "unit": "pairs/s", "n_gpus": 1,
                       "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(ms, 4),
@@ -1489,16 +1511,7 @@ def large_kernel_work(pipe):
     work["lite_exact_kernel"] = (scale * (n_last + (ns - n_q) * per_surv), "B")
     work["row_norm2_kernel"] = (nnz * 4 + N * 8, "B")
     # banding (cosine: packed band keys, LSD radix passes, emission)
-    rows, bands = w["rows"], w["bands"]
-    n = N * bands
-    kb = 4 if max(1, (bands - 1).bit_length()) + rows <= 32 else 8
-    obj_rows = N * bands * ((rows + 7) // 8)
-    passes = (max(1, (bands - 1).bit_length()) + rows + 7) // 8
-    work["band_keys_kernel"] = (N * bands * rows // 8 + n * (kb + 4) + obj_rows, "B")
-    work["digit_hist_kernel"] = (passes * n * kb, "B")
-    work["digit_scatter_kernel"] = (passes * 2 * n * (kb + 4), "B")
-    work["emit_warp_kernel (count pass)"] = (n * (kb + 4) + obj_rows + n * 8, "B")
-    work["emit_warp_kernel (write pass)"] = (n * (kb + 4 + 8) + obj_rows + P * 8, "B")
+    work.update(banding_work(1, N, P, w["rows"], w["bands"]))
     n_keep = scale * int(kept.sum()) + scale * int((lst == B.LITE_ACCEPT).sum())
     work["compact_count"] = (2 * P, "B")
     work["compact_write"] = (2 * P + 8 * n_keep, "B")

@@ -1622,9 +1622,9 @@ extern "C" int blsh_autotune_k(blsh_ctx *ctx, const blsh_params *params, const i
 
 namespace {
 
-// Pairs left at BLSH_NEEDS_HASHES, finished over all n_max hashes: one
-// thread per pair (they are few), Algorithm 1 from its first chunk, the
-// decisions of verify_kernel.  Statuses are read 16 at a time.
+// Pairs left at BLSH_NEEDS_HASHES, finished over all n_max hashes: a warp
+// per pair, a lane per chunk, Algorithm 1 from its first chunk, the decisions
+// of verify_kernel.  Statuses are read 16 at a time.
 __global__ void __launch_bounds__(256) verify_resume_kernel(const VerifyArgs A, int kind, int vec) {
     long long P = A.P;
     if (A.P_dev) {
