@@ -1359,7 +1359,9 @@ int staged_candidates(blsh_ctx *ctx, BandArgs &A, const Layout &L, char *ws, siz
     E.task_next = work + 6;
     E.tasks = (uint2 *)(ws + L.hist + 256);                   // (the chunk totals of a tiny n may reach into hist)
     E.task_cap = (L.partial - L.hist - 256) / sizeof(uint2);  // n / 32 of them
-    const bool long_walks = N - 1 > kSplit;                   // a bucket may be long enough to be split
+    // a chunk may be split: its partners end up to 31 positions past a whole
+    // bucket of N, where the band begins on the chunk's last lane
+    const bool long_walks = N + 30 > kSplit;
     E.next = work;
     int rc = emit_dispatch<kCount>(ctx, A, keys[cur], vals[cur], n, E, nullptr, 0, s);
     if (rc) return rc;

@@ -102,3 +102,25 @@ def test_long_buckets(B, ctx, kind, rows, bands):
     assert len(got) == len(want) and np.array_equal(np.sort(packed(got)), np.sort(packed(want)))
     for rec in (0, 64 * N):   # no record: every chunk by its own warp, in the same order
         assert np.array_equal(candidates(B, ctx, sig, kind, rows, bands, rec), got)
+
+
+@pytest.mark.parametrize("N", [2019, 2028, 2035, 2040, 2047, 2049, 2050])
+@pytest.mark.parametrize("kind,rows,band", [(1, 16, 1), (1, 16, 2), (0, 2, 1), (0, 2, 2)])
+def test_long_bucket_past_a_band_edge(B, ctx, N, kind, rows, band):
+    """About as many objects as a chunk may have partners before it is cut into
+    segments, nearly all of them in one bucket of a band whose first position
+    lies inside a chunk of 32: the bucket's end is N + (N * band) % 32
+    positions from the chunk's start."""
+    rng = np.random.default_rng(N)
+    sig = rng.permutation(1 << 16)[: N * 8].reshape(N, 8).astype(np.uint32) if kind == 0 else \
+        np.stack([rng.permutation(1 << 16)[:N] for _ in range(8)], 1).astype(np.uint16).view(np.uint32)
+    if kind == 0:
+        sig[3:, band * rows:(band + 1) * rows] = 7
+    else:
+        sig.view(np.uint16)[3:, band] = 7
+    want = O.lsh_candidates(sig, O.COSINE if kind else O.JACCARD, rows, 3)
+    assert len(want) >= (N - 3) * (N - 4) // 2
+    got = candidates(B, ctx, sig, kind, rows, 3, 1 << 40)
+    assert len(got) == len(want) and np.array_equal(np.sort(packed(got)), np.sort(packed(want)))
+    for rec in (0, 8 * N):
+        assert np.array_equal(candidates(B, ctx, sig, kind, rows, 3, rec), got)
