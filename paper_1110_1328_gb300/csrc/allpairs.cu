@@ -692,12 +692,11 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
             return BLSH_OK;
         }
         const size_t smem = (size_t)((N + 31) / 32) * 4;
-        if (smem > 48 * 1024) {
-            BLSH_CUDA(ctx, cudaFuncSetAttribute(ap_map_kernel<MAP_COUNT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)(kMapRows / 8)));
-            BLSH_CUDA(ctx, cudaFuncSetAttribute(ap_map_kernel<MAP_WRITE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                (int)(kMapRows / 8)));
-        }
+        // (always: the launch default of 48 KB holds a kernel's own shared memory too)
+        BLSH_CUDA(ctx, cudaFuncSetAttribute(ap_map_kernel<MAP_COUNT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)(kMapRows / 8)));
+        BLSH_CUDA(ctx, cudaFuncSetAttribute(ap_map_kernel<MAP_WRITE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)(kMapRows / 8)));
         // the maps are kept for the write pass where they fit the key buffers' place (N^2 / 8 of 32 max_dups bytes)
         uint32_t *kept = (size_t)N * smem <= L.hist - L.k0 ? (uint32_t *)(ws + L.k0) : nullptr;
         blsh_time_start(ctx, s);

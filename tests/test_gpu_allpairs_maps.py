@@ -100,3 +100,24 @@ def test_maps_kept_or_formed_again(B, ctx, dim, kept, kind, cap_less):
     m = min(k, len(got))
     assert np.array_equal(got[:m], want[:m]) and np.all(got[m:] == 2**32 - 1)
     assert (n * n <= 256 * (len(got) + cap_less)) == kept
+
+
+@pytest.mark.parametrize("n", [392_200, 393_200])
+@pytest.mark.parametrize("kept", [True, False])
+def test_maps_at_the_default_shared_memory(B, n, kept):
+    """Maps of just under 48 KB, which with the kernels' own shared memory pass
+    the launch default: kept for the write pass, and formed again."""
+    i = np.arange(n)
+    feats = np.sort(np.stack([i // 2, n // 2 + (i * 7919) % 190_000], 1), 1)
+    csr = synth.CSR(np.arange(n + 1, dtype=np.int64) * 2, feats.ravel().astype(np.uint32), None, n // 2 + 190_000)
+    want = O.allpairs_candidates(csr, 0.4, O.JACCARD)
+    assert len(want) > n // 2
+    max_dups = n * n // (256 if kept else 4096) + 1
+    ip, ix = torch.from_numpy(csr.indptr).to(dev), torch.from_numpy(csr.indices.view(np.int32)).to(dev)
+    ws = torch.empty(B.blsh_allpairs_workspace(n, 2 * n, csr.dim, max_dups), dtype=torch.uint8, device=dev)
+    pairs = torch.full((len(want) + 5, 2), -1, dtype=torch.int32, device=dev)
+    n_pairs = torch.zeros(1, dtype=torch.int64, device=dev)
+    ctx = B.Context(0)
+    B.blsh_allpairs_candidates(ctx, ip, ix, None, csr.dim, 0.4, O.JACCARD, pairs, n_pairs, ws, max_dups)
+    assert B.blsh_status(ctx) == 0 and int(n_pairs.item()) == len(want)
+    assert np.array_equal(pairs[: len(want)].cpu().numpy().view(np.uint32), want)
