@@ -339,7 +339,9 @@ BLSH_API int blsh_lsh_candidates(blsh_ctx *ctx, const uint32_t *sig, int64_t N, 
  * order of (x, y), their number to *n_pairs (device int64).
  * Rows: indptr int64 [N+1] (indptr[N] = nnz, passed from the host too),
  * indices uint32 sorted and distinct within a row, features < dim; values
- * float [nnz] for cosine, NULL for sets.
+ * float [nnz] for cosine, NULL for sets.  (A part of a larger indptr over the
+ * whole index array is taken too, nnz then at least indptr[N]: elements
+ * outside the rows count for nothing.)
  * The pairs are formed by sorting the candidate keys of every (row, shared
  * indexed feature), duplicates included: max_dups is the capacity of that
  * key buffer (a part of the workspace).  A call with cap = 0 is a count-only

@@ -88,8 +88,16 @@ __device__ __forceinline__ unsigned long long ap_key(const ApArgs &A, uint32_t f
     return ((unsigned long long)(0xffffffffu - A.df[f]) << 32) | f;
 }
 
+// The elements of the rows: those before indptr[0] or past indptr[N] (some
+// rows of a larger CSR) are no row's, so nothing counts them.
+__device__ __forceinline__ void ap_elements(const ApArgs &A, long long nnz, long long &s, long long &e) {
+    s = __ldg(A.indptr);
+    e = min(nnz, (long long)__ldg(A.indptr + A.N));
+}
+
 // df and max |value| of every feature; with `place`, also each element's number
-// among its feature's (in no particular order: where ap_post_kernel puts it).
+// among its feature's (in no particular order: where ap_post_kernel puts it, so
+// the elements counted are those it places, and every entry is filled).
 // Bound by the atomics on the most frequent features' addresses (20,000 rows:
 // one feature stands in most of them); the largest value is looked at before
 // it is replaced, and the numbers save ap_post_kernel the same atomics again
@@ -97,7 +105,9 @@ __device__ __forceinline__ unsigned long long ap_key(const ApArgs &A, uint32_t f
 // atomic whose answer is waited for costs more, two of them most).
 __global__ void __launch_bounds__(256) ap_stats_kernel(ApArgs A, long long nnz, uint32_t *place) {
     unsigned long long bad = 0;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < nnz; e += (long long)gridDim.x * blockDim.x) {
+    long long s, end;
+    ap_elements(A, nnz, s, end);
+    for (long long e = s + (long long)blockIdx.x * blockDim.x + threadIdx.x; e < end; e += (long long)gridDim.x * blockDim.x) {
         const uint32_t f = __ldg(A.indices + e);
         if (f >= A.dim) { ++bad; continue; }
         const uint32_t at = atomicAdd(&A.df[f], 1u);
@@ -250,10 +260,18 @@ __global__ void __launch_bounds__(kCtaThreads) ap_prefix_cta_kernel(ApArgs A, co
 }
 
 // Index keys: (feature << xbits) | row for indexed nonzeros, the padding key
-// (all ones) for the others; per-feature counts of indexed nonzeros.
-__global__ void __launch_bounds__(256) ap_index_keys_kernel(ApArgs A, int xbits, unsigned long long *keys,
-                                                            unsigned long long *fcnt) {
+// (all ones) for the others and for elements of no row; per-feature counts of
+// indexed nonzeros.
+__global__ void __launch_bounds__(256) ap_index_keys_kernel(ApArgs A, long long nnz, int xbits,
+                                                            unsigned long long *keys, unsigned long long *fcnt) {
     const int lane = threadIdx.x & 31;
+    {
+        const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
+        long long first, end;
+        ap_elements(A, nnz, first, end);
+        for (long long i = t; i < first && i < nnz; i += nt) keys[i] = ~0ull;
+        for (long long i = end + t; i < nnz; i += nt) keys[i] = ~0ull;
+    }
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
     for (long long row = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; row < A.N; row += nw) {
         const long long s = __ldg(A.indptr + row), e = __ldg(A.indptr + row + 1);
@@ -723,7 +741,7 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
     uint32_t *iv[2] = {(uint32_t *)(ws + L.iv0), (uint32_t *)(ws + L.iv1)};
     BLSH_CUDA(ctx, cudaMemsetAsync(fcnt, 0, (dim + 1) * 8, s));
     blsh_time_start(ctx, s);
-    ap_index_keys_kernel<<<grid_for(N, 8), 256, 0, s>>>(A, xbits, ik[0], fcnt);
+    ap_index_keys_kernel<<<grid_for(N, 8), 256, 0, s>>>(A, nnz, xbits, ik[0], fcnt);
     BLSH_LAUNCHED(ctx, "ap_index_keys_kernel");
     int cur = 0;
     {

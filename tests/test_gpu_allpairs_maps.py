@@ -121,3 +121,38 @@ def test_maps_at_the_default_shared_memory(B, n, kept):
     B.blsh_allpairs_candidates(ctx, ip, ix, None, csr.dim, 0.4, O.JACCARD, pairs, n_pairs, ws, max_dups)
     assert B.blsh_status(ctx) == 0 and int(n_pairs.item()) == len(want)
     assert np.array_equal(pairs[: len(want)].cpu().numpy().view(np.uint32), want)
+
+
+@pytest.mark.parametrize("first,last", [(300, 1200), (0, 1000), (250, 1100), (1199, 1200)])
+@pytest.mark.parametrize("kind", [O.JACCARD, O.COSINE])
+@pytest.mark.parametrize("sparse", [False, True])
+def test_some_rows_of_a_larger_csr(B, ctx, first, last, kind, sparse):
+    """indptr a part of a larger one over the whole index array: the elements of
+    the other rows, before indptr[0] and past indptr[N], count for nothing, in
+    the bit maps as in the sorted keys."""
+    csr = rows_csr(np.full(1200, 6), 60_000, 8, kind == O.COSINE) if sparse else \
+        rows_csr(np.random.default_rng(9).integers(0, 30, 1200), 300, 9, kind == O.COSINE)
+    part = csr.indptr[first:last + 1]
+    s, e = part[0], part[-1]
+    sub = synth.CSR(part - s, csr.indices[s:e], None if csr.values is None else csr.values[s:e], csr.dim)
+    want = O.allpairs_candidates(sub, 0.3, kind)
+    ip, ix = torch.from_numpy(part.copy()).to(dev), torch.from_numpy(csr.indices.view(np.int32)).to(dev)
+    val = None if csr.values is None else torch.from_numpy(csr.values).to(dev)
+    n_pairs, n_dups = (torch.zeros(1, dtype=torch.int64, device=dev) for _ in range(2))
+    dups, names = 0, []
+    for counted in (False, True):
+        ws = torch.full((B.blsh_allpairs_workspace(last - first, ix.numel(), csr.dim, dups),), 0xEE, dtype=torch.uint8,
+                        device=dev)
+        pairs = torch.full((max(1, dups), 2), -1, dtype=torch.int32, device=dev) if counted else None
+        B.blsh_timing_begin(ctx)
+        B.blsh_allpairs_candidates(ctx, ip, ix, val, csr.dim, 0.3, kind, pairs, n_pairs, ws, dups, n_dups)
+        names = [n for n, _ in B.blsh_timing_end(ctx)]
+        assert B.blsh_status(ctx) == 0
+        if not counted:
+            dups = int(n_dups.item())
+        if dups == 0:
+            assert len(want) == 0
+            return
+    assert int(n_dups.item()) == dups and int(n_pairs.item()) == len(want)
+    assert np.array_equal(pairs[: len(want)].cpu().numpy().view(np.uint32), want)
+    assert ("digit_scatter_kernel" in names) == sparse
