@@ -752,7 +752,7 @@ __global__ void __launch_bounds__(256, 4) lite_exact_kernel(const LiteArgs A, co
     const int warp = threadIdx.x >> 5;
     // per warp: the stage for longer rows' indices, lite_flat's area, and the
     // survivors of the current tile (offsets within it)
-    extern __shared__ uint32_t lite_smem[];
+    extern __shared__ __align__(16) uint32_t lite_smem[];   // (read and filled 16 bytes at a time)
     uint32_t *w_idx = lite_smem + warp * kLiteWarpWords;
     uint32_t *flat = w_idx + 2 * kLiteStage;
     uint16_t *w_list = reinterpret_cast<uint16_t *>(flat + kFlatWords);
@@ -882,7 +882,7 @@ __global__ void __launch_bounds__(256, 4) lite_queue_kernel(const LiteArgs A, co
                                                             unsigned long long *heavy) {
     const unsigned long long total = A.scratch->work3;
     const unsigned long long n = total < BLSH_LITE_QUEUE_CAP ? total : BLSH_LITE_QUEUE_CAP;
-    extern __shared__ uint32_t lite_smem[];
+    extern __shared__ __align__(16) uint32_t lite_smem[];   // (read and filled 16 bytes at a time)
     const int lane = threadIdx.x & 31;
     uint32_t *w_idx = lite_smem + (threadIdx.x >> 5) * kLiteWarpWords;
     uint32_t *flat = w_idx + 2 * kLiteStage;
