@@ -578,7 +578,13 @@ __device__ __forceinline__ LiteSums lite_few(const LiteArgs &A, unsigned todo, l
 // survivors follow each other) held its warp 0.3 ms after all others had
 // ended (a search over 6e5 vectors: queue 478 us, with the list 202 + 38; 256
 // elements 184 + 39, 1,024 237 + 37).
+// Their status is set apart from a survivor's until lite_heavy writes the
+// verdict, so that the scan for survivors beyond the queue, which other CTAs
+// run meanwhile, does not take them again.
 constexpr int kLiteHeavy = 512;
+constexpr uint8_t kHeavyStatus = 251;
+static_assert(kHeavyStatus != BLSH_LITE_SURVIVOR && kHeavyStatus != BLSH_NEEDS_HASHES && kHeavyStatus != BLSH_BAD_PAIR,
+              "the listed pairs' status must differ from every other status");
 template <bool COSINE>
 __device__ __forceinline__ void lite_batch(const LiteArgs &A, long long my_q, bool have_norms, uint32_t *w_idx,
                                            uint32_t *flat, unsigned long long *heavy = nullptr) {
@@ -599,6 +605,7 @@ __device__ __forceinline__ void lite_batch(const LiteArgs &A, long long my_q, bo
         const unsigned long long slot = atomicAdd(&A.scratch->recheck_count, 1ull);
         if (slot < BLSH_RECHECK_CAP) {
             heavy[slot] = (unsigned long long)my_q;
+            A.status[my_q] = kHeavyStatus;
             my_q = -1;
         }
     }
@@ -762,7 +769,8 @@ __global__ void __launch_bounds__(256, 4) lite_exact_kernel(const LiteArgs A, co
     // A warp takes kLiteGrab tiles of 512 statuses per grab of the work
     // counter; a lane reads 16 statuses with one 16-byte load; the tiles'
     // survivors are listed in shared memory and computed 32 at a time, what is
-    // left of a tile with the next one's.
+    // left of a tile with the next one's.  (Not through the read-only path:
+    // statuses are written in this kernel, lite_heavy's among them.)
     for (;;) {
         unsigned long long grab = 0;
         if (lane == 0) grab = atomicAdd(&A.scratch->work2, 1ull);
@@ -776,7 +784,7 @@ __global__ void __launch_bounds__(256, 4) lite_exact_kernel(const LiteArgs A, co
             const long long qs = q0 + 16ll * lane;
             uint32_t surv = 0;
             if (A.vec && qs + 16 <= P) {
-                surv = blsh_eq16(__ldg(reinterpret_cast<const uint4 *>(A.status + qs)), BLSH_LITE_SURVIVOR);
+                surv = blsh_eq16(__ldcg(reinterpret_cast<const uint4 *>(A.status + qs)), BLSH_LITE_SURVIVOR);
             } else {
                 for (int i = 0; i < 16; ++i)
                     if (qs + i < P && A.status[qs + i] == BLSH_LITE_SURVIVOR) surv |= 1u << i;

@@ -67,3 +67,28 @@ def test_repeated_indices_stay_together(B):
     term = 2.0**50   # 0.03125 squared, times 2^60
     want = (200 * term) / np.sqrt((len(a) * term) * (len(b) * term))
     assert np.array_equal(sim, [want, want])
+
+
+@pytest.mark.parametrize("kind", [0, 1])
+@pytest.mark.parametrize("long_share", [0.01, 0.3])
+def test_past_the_queue_and_the_list(B, kind, long_share):
+    """More survivors than the queue holds (2^23), and fewer or more pairs of
+    long rows among the queued ones than their list holds (2^20)."""
+    rng = np.random.default_rng(11 + kind)
+    dim = 2000
+    ln = np.concatenate([rng.integers(513, 560, 24), rng.integers(3, 30, 400)])
+    rows = [np.sort(rng.choice(dim, n, replace=False)) for n in ln]
+    vals = np.concatenate([rng.standard_normal(n) / np.sqrt(n) for n in ln]).astype(np.float32)
+    csr = synth.CSR(np.concatenate([[0], np.cumsum(ln)]).astype(np.int64), np.concatenate(rows).astype(np.uint32),
+                    vals if kind else None, dim)
+    some = 4001
+    heavy = rng.random(some) < long_share
+    few = np.where(heavy[:, None], rng.integers(0, 24, (some, 2)), rng.integers(24, csr.n, (some, 2))).astype(np.uint32)
+    reps = (1 << 23) // some + 40
+    assert ((1 << 23) * long_share > 1.2 * (1 << 20)) == (long_share > 0.2)
+    W = 64 if kind == 0 else 8
+    want = O.verify_lite(O.tables(O.Params(kind=kind, t=0.3, n_max=64 if kind == 0 else 256, h=64)), few,
+                         np.zeros((csr.n, W), np.uint32), csr)
+    st, sim = run(B, csr, np.tile(few, (reps, 1)), kind, True)
+    assert np.array_equal(st.reshape(reps, some), np.broadcast_to(want.status, (reps, some)))
+    assert np.array_equal(sim.reshape(reps, some), np.broadcast_to(want.sim, (reps, some)))
