@@ -49,6 +49,14 @@ constexpr unsigned kFull = 0xffffffffu;
 constexpr int kShortRow = 128;
 constexpr int kLongRow = 4096;
 constexpr long long kMapRows = 1ll << 19;   // bit maps of up to 64 KB
+// A count-only call walks the lists where every element's list of every row
+// (nnz N entries, a bound known on the host) has at most 2^28 entries, else it
+// sorts the index and searches it, whose time does not grow with the keys.  Rows
+// that share nearly every feature, lists / sort: 2^27.2 entries 165 / 264 us,
+// 2^28.3 233 / 274 and 164 / 158, 2^30.9 734 / 346.  (Always by lists: 250,000
+// tf-idf rows 8.8 ms, sorted 2.5; between, where the lists are far shorter than
+// their bound, the sort costs up to twice the time: 20,000 rows 288 / 415.)
+constexpr double kListReads = 268435456.0;
 constexpr double kTwo48 = 281474976710656.0;
 constexpr long long kTermCap = 1ll << 50;
 
@@ -677,9 +685,11 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
     BLSH_CUDA(ctx, cudaMemsetAsync(A.df, 0, L.indexed - L.df, s));   // df and maxabs
     BLSH_CUDA(ctx, cudaMemsetAsync(ws + L.grand, 0, 64, s));         // the totals and counters
     // bit maps where they cost less than sorting the keys (see the top of the
-    // file), and for a count-only call, which then forms no map
+    // file); a count-only call forms neither map nor key, and walks the lists
+    // only where all of them for every element are few
     const bool count_only = cap == 0 || max_dups == 0;
-    const bool maps = N <= kMapRows && nnz < (1ll << 31) && (count_only || N * N <= 4096 * max_dups);
+    const bool maps = N <= kMapRows && nnz < (1ll << 31) &&
+                      (count_only ? (double)nnz * (double)N <= kListReads : N * N <= 4096 * max_dups);
     uint32_t *place = (uint32_t *)(ws + L.iv0);
     blsh_time_start(ctx, s);
     ap_stats_kernel<<<grid_for(nnz, 256), 256, 0, s>>>(A, nnz, maps ? place : nullptr);

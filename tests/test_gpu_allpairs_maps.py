@@ -156,3 +156,29 @@ def test_some_rows_of_a_larger_csr(B, ctx, first, last, kind, sparse):
     assert int(n_dups.item()) == dups and int(n_pairs.item()) == len(want)
     assert np.array_equal(pairs[: len(want)].cpu().numpy().view(np.uint32), want)
     assert ("digit_scatter_kernel" in names) == sparse
+
+
+@pytest.mark.parametrize("n,length,by_lists", [(2000, 65, True), (2000, 69, False), (6000, 7, True), (6000, 8, False)])
+@pytest.mark.parametrize("kind", [O.JACCARD, O.COSINE])
+def test_count_only_by_lists_or_by_sorting(B, ctx, n, length, by_lists, kind):
+    """The number of keys from either form of a count-only call, which walks
+    lists only where n rows' every list is short enough in the worst case."""
+    csr = rows_csr(np.full(n, length), 400, n + length, kind == O.COSINE)
+    nnz = csr.indices.size
+    assert (nnz * n <= 2**28) == by_lists
+    indexed = O.allpairs_indexed(csr, 0.4, kind).astype(bool)
+    # the keys: (row x, indexed feature f of x, row y > x with f)
+    row = np.repeat(np.arange(n), length)
+    has = np.zeros((n, csr.dim), bool)
+    has[row, csr.indices] = True
+    later = has[::-1].cumsum(0)[::-1] - has
+    want = int(later[row[indexed], csr.indices[indexed]].sum())
+    ip, ix = torch.from_numpy(csr.indptr).to(dev), torch.from_numpy(csr.indices.view(np.int32)).to(dev)
+    val = None if kind == O.JACCARD else torch.from_numpy(csr.values).to(dev)
+    n_pairs, n_dups = (torch.full((1,), 7, dtype=torch.int64, device=dev) for _ in range(2))
+    ws = torch.full((B.blsh_allpairs_workspace(n, nnz, csr.dim, 0),), 0xEE, dtype=torch.uint8, device=dev)
+    B.blsh_timing_begin(ctx)
+    B.blsh_allpairs_candidates(ctx, ip, ix, val, csr.dim, 0.4, kind, None, n_pairs, ws, 0, n_dups)
+    names = [k for k, _ in B.blsh_timing_end(ctx)]
+    assert B.blsh_status(ctx) == 0 and int(n_pairs.item()) == 0 and int(n_dups.item()) == want > 0
+    assert ("ap_map_kernel (keys)" in names) == by_lists and ("digit_scatter_kernel" in names) != by_lists
