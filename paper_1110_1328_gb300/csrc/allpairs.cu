@@ -28,15 +28,19 @@
 //   5. the keys are radix-sorted, and the distinct ones are written as pairs
 //      (x, y) in increasing order.
 //
-// Where N^2 <= 4096 max_dups (and N <= 2^19) steps 3 to 5 need no sort: the
+// Where N^2 <= 4096 max_dups and N^2 <= 2^31 + 512 max_dups (and N <= 2^19)
+// steps 3 to 5 need no sort: the
 // rows of every feature are listed in any order, and a CTA per row x sets bit
 // y of an N-bit map in shared memory for every y > x in the lists of x's
 // indexed features; the map's set bits, in order, are x's candidates (counted
 // first, then written at scanned offsets; the write pass reads the counted maps
-// again where N^2 / 8 bytes fit the place of the key buffers).  A map costs N / 32 words per row
-// and pass (0.3 ps a word), the sort about 50 ps a key, which is where the
-// line lies.  20,000 tf-idf rows (2.4e7 keys, 1.7e7 pairs): 1.96 ms by sorting,
-// 0.38 ms with the maps.
+// again where N^2 / 8 bytes fit the place of the key buffers).  20,000 tf-idf
+// rows (2.4e7 keys, 1.7e7 pairs): 1.96 ms by sorting, 0.38 ms with the maps.
+// The line: a row's map of N / 32 words takes 0.4 ps a word to count and, not
+// kept, 1.3 to 2.1 ps to form and write again; the sort takes about 50 ps a key
+// of max_dups and 0.2 ms of launches.  Rows of 10 features, maps / sort:
+// 8,000 rows, 1.6e4 keys 0.11 / 0.24 ms; 60,000, 9e5 0.46 / 0.45; 250,000,
+// 1.6e7 3.5 / 1.5; 500,000, 6.3e7 20 / 4.0; 500,000, 6.3e8 26 / 27.
 #include <type_traits>
 
 #include "common.cuh"
@@ -689,7 +693,8 @@ extern "C" int blsh_allpairs_candidates(blsh_ctx *ctx, const int64_t *indptr, co
     // only where all of them for every element are few
     const bool count_only = cap == 0 || max_dups == 0;
     const bool maps = N <= kMapRows && nnz < (1ll << 31) &&
-                      (count_only ? (double)nnz * (double)N <= kListReads : N * N <= 4096 * max_dups);
+                      (count_only ? (double)nnz * (double)N <= kListReads
+                                  : N * N <= 4096 * max_dups && N * N <= (1ll << 31) + 512 * max_dups);
     uint32_t *place = (uint32_t *)(ws + L.iv0);
     blsh_time_start(ctx, s);
     ap_stats_kernel<<<grid_for(nnz, 256), 256, 0, s>>>(A, nnz, maps ? place : nullptr);

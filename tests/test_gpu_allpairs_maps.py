@@ -112,7 +112,7 @@ def test_maps_at_the_default_shared_memory(B, n, kept):
     csr = synth.CSR(np.arange(n + 1, dtype=np.int64) * 2, feats.ravel().astype(np.uint32), None, n // 2 + 190_000)
     want = O.allpairs_candidates(csr, 0.4, O.JACCARD)
     assert len(want) > n // 2
-    max_dups = n * n // (256 if kept else 4096) + 1
+    max_dups = n * n // (256 if kept else 400) + 1
     ip, ix = torch.from_numpy(csr.indptr).to(dev), torch.from_numpy(csr.indices.view(np.int32)).to(dev)
     ws = torch.empty(B.blsh_allpairs_workspace(n, 2 * n, csr.dim, max_dups), dtype=torch.uint8, device=dev)
     pairs = torch.full((len(want) + 5, 2), -1, dtype=torch.int32, device=dev)
@@ -182,3 +182,18 @@ def test_count_only_by_lists_or_by_sorting(B, ctx, n, length, by_lists, kind):
     names = [k for k, _ in B.blsh_timing_end(ctx)]
     assert B.blsh_status(ctx) == 0 and int(n_pairs.item()) == 0 and int(n_dups.item()) == want > 0
     assert ("ap_map_kernel (keys)" in names) == by_lists and ("digit_scatter_kernel" in names) != by_lists
+
+
+@pytest.mark.parametrize("n,maps", [(46_000, True), (60_000, False)])
+def test_many_rows_of_few_keys(B, ctx, n, maps):
+    """Around the number of rows from which maps that the key buffers' place
+    cannot hold cost more than sorting the few keys there are."""
+    length, dim = 10, 190_000
+    rng = np.random.default_rng(n)
+    feats = rng.integers(0, dim // length, (n, length)) + np.arange(length) * (dim // length)
+    csr = synth.CSR(np.arange(n + 1, dtype=np.int64) * length, feats.ravel().astype(np.uint32), None, dim)
+    want = O.allpairs_candidates(csr, 0.05, O.JACCARD)
+    got, k, names = candidates(B, ctx, csr, 0.05, O.JACCARD)
+    assert n * n <= 4096 * len(got) and n * n > 256 * len(got)
+    assert k == len(want) and np.array_equal(got[:k], want)
+    assert ("ap_map_kernel (write pass)" in names) == maps and ("digit_scatter_kernel" in names) != maps
