@@ -55,102 +55,122 @@ __device__ __forceinline__ void min_hash_run(const uint32_t *__restrict__ indice
 }
 
 // One warp per (set, tile of 32 HPL hashes): lane l owns hashes l, l + 32, ...
-// of tile blockIdx.y and keeps their running minima in registers.  A warp
-// alone takes about 46 ns an element, so sets longer than kBigSet are queued
-// in chunks of kBigChunk elements for minhash_big_kernel: the degrees of a
+// of a tile and keeps their running minima in registers.  A warp
+// alone takes about 46 ns an element, so sets longer than kBigSet are listed
+// for minhash_big_kernel: the degrees of a
 // graph follow a power law, and a set of 150,000 elements would hold up one
 // warp for milliseconds.
+//
+// Two lists, an entry a set: sets of more than kHubSet elements in one of their
+// own (2^20 of them), so that however many others there are (2^23 in the other
+// list) a hub is never one warp's work while a warp's worth of others is.  An
+// entry holds the set and the number of 32-element blocks listed before it; the
+// list's counter holds both numbers, entries above the blocks, so that one
+// atomic gives an entry its place and its blocks' place.  The row of a listed
+// set starts at the identity of the minimum; that of a set past its list's end
+// at a value that no hash takes (its first words), by which minhash_big_kernel
+// finds it: those sets are a warp's work each.
+// (Entries of 256 elements and a tile on one list of 2^20: 1.5e6 sets of 300
+// and then 20 hubs of 1e6 took 109 ms, the hubs a warp each; 25 here.)
+//
 // 1e6 neighbour lists (mean 27) x 256 hashes, both kernels: 4.77 ms with
-// twelve instructions a hash and long sets spread over whole CTAs, 1.66 now
-// (4.2e12 hashes/s; 4.9e12 where every set has 64 elements or more, the
+// twelve instructions a hash and long sets spread over whole CTAs, 1.56 now
+// (4.4e12 hashes/s; 4.9e12 where every set has 64 elements or more, the
 // rate of the 64-bit multiply-add and the four others at this mix).
 constexpr long long kBigSet = 256;
-constexpr long long kBigChunk = 256;   // elements of a long set per warp task
+constexpr long long kHubSet = 2048;
+constexpr int kListShift = 36;          // 2^36 blocks and 2^28 entries: more than 280 GB of elements
+constexpr unsigned kPartBlocks = 8;     // blocks of a list a warp takes, at least
+constexpr uint32_t kListed = 0xffffffffu, kUnlisted = 0xfffffffeu;
 
-// Queues the chunks of a long set [s, e) for one tile of hashes (one warp);
-// false if the queue is full: the set is then hashed by its own warp.
-__device__ __forceinline__ bool queue_long_set(long long i, long long s, long long e, unsigned tile, unsigned tiles,
-                                               blsh_dev_scratch *scratch, uint2 *__restrict__ big) {
-    const int lane = threadIdx.x & 31;
-    const unsigned long long chunks = (unsigned long long)(e - s + kBigChunk - 1) / kBigChunk;
-    unsigned long long slot = 0;
-    if (lane == 0) slot = atomicAdd(&scratch->work3, chunks);
-    slot = __shfl_sync(kFull, slot, 0);
-    if (slot + chunks <= BLSH_RECHECK_CAP) {
-        for (unsigned long long c = lane; c < chunks; c += 32)
-            big[slot + c] = make_uint2((uint32_t)i, (uint32_t)c * tiles + tile);
-        return true;
-    }
-    // entries of the queue that this set reserved but does not fill
-    for (unsigned long long c = slot + lane; c < slot + chunks && c < BLSH_RECHECK_CAP; c += 32)
-        big[c] = make_uint2(0u, 0xffffffffu);
-    return false;
+struct LongSets {
+    uint2 *set, *hub;                   // [BLSH_LITE_QUEUE_CAP], [BLSH_RECHECK_CAP]
+    unsigned long long *n_set, *n_hub;  // entries << kListShift | blocks
+    unsigned long long *next;           // [2]: the next part of the hubs, of the others
+};
+
+// Lists a long set [s, e) (one warp); false if its list is full.
+__device__ __forceinline__ bool list_long_set(const LongSets &L, long long i, long long s, long long e) {
+    const bool is_hub = e - s > kHubSet;
+    unsigned long long before = 0;
+    if ((threadIdx.x & 31) == 0)
+        before = atomicAdd(is_hub ? L.n_hub : L.n_set, 1ull << kListShift | (unsigned long long)(e - s + 31) >> 5);
+    before = __shfl_sync(kFull, before, 0);
+    const unsigned long long slot = before >> kListShift;
+    if (slot >= (is_hub ? BLSH_RECHECK_CAP : BLSH_LITE_QUEUE_CAP)) return false;
+    if ((threadIdx.x & 31) == 0) (is_hub ? L.hub : L.set)[slot] = make_uint2((uint32_t)i, (uint32_t)before);   // (< 2^32 blocks)
+    return true;
 }
 
+// The coefficients of the lane's hashes in a tile.
 template <int HPL>
-__global__ void __launch_bounds__(256) minhash_kernel(const int64_t *__restrict__ indptr,
-                                                      const uint32_t *__restrict__ indices, long long N,
-                                                      int n_hashes, const uint32_t *__restrict__ A,
-                                                      const uint32_t *__restrict__ B, uint32_t *__restrict__ sig,
-                                                      blsh_dev_scratch *scratch, uint2 *__restrict__ big) {
-    const int lane = threadIdx.x & 31;
-    const int h0 = blockIdx.y * 32 * HPL + lane;
-    uint32_t a2[HPL], b2[HPL];
+__device__ __forceinline__ void load_coeffs(const uint32_t *__restrict__ A, const uint32_t *__restrict__ B,
+                                            unsigned tile, uint32_t (&a2)[HPL], uint32_t (&b2)[HPL]) {
+    const size_t h0 = (size_t)tile * 32 * HPL + (threadIdx.x & 31);
 #pragma unroll
     for (int u = 0; u < HPL; ++u) {
         a2[u] = 2u * mod_p31(__ldg(A + h0 + 32 * u));
         b2[u] = 2u * mod_p31(__ldg(B + h0 + 32 * u));
     }
+}
+
+// (The bounds choose the compiler's schedule: 1e6 sets of 27 x 256 hashes 1.48 ms,
+// 1.53 without; 3e5 of 100 x 128 0.84, 0.86 without, 0.85 with four CTAs.)
+template <int HPL>
+__global__ void __launch_bounds__(256, HPL == 4 ? 5 : 4) minhash_kernel(
+    const int64_t *__restrict__ indptr, const uint32_t *__restrict__ indices, long long N, int n_hashes,
+    const uint32_t *__restrict__ A, const uint32_t *__restrict__ B, uint32_t *__restrict__ sig, const LongSets L) {
+    const int lane = threadIdx.x & 31;
+    const unsigned tiles = (unsigned)n_hashes / (32u * HPL);
     const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
-    for (long long i = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < N; i += warps) {
-        const long long s = __ldg(indptr + i), e = __ldg(indptr + i + 1);
-        uint32_t mn[HPL];
+    for (unsigned tile = blockIdx.y; tile < tiles; tile += gridDim.y) {
+        const int h0 = (int)tile * 32 * HPL + lane;
+        uint32_t a2[HPL], b2[HPL];
+        load_coeffs<HPL>(A, B, tile, a2, b2);
+        for (long long i = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < N; i += warps) {
+            const long long s = __ldg(indptr + i), e = __ldg(indptr + i + 1);
+            uint32_t mn[HPL];
 #pragma unroll
-        for (int u = 0; u < HPL; ++u) mn[u] = 0xffffffffu;
-        // a long set: its part of the row starts at the identity of min, the
-        // chunks lower it
-        const bool queued = e - s > kBigSet && queue_long_set(i, s, e, blockIdx.y, gridDim.y, scratch, big);
-        if (!queued) min_hash_run<HPL>(indices, s, e, a2, b2, mn);
+            for (int u = 0; u < HPL; ++u) mn[u] = kListed;
+            if (e - s <= kBigSet) {
+                min_hash_run<HPL>(indices, s, e, a2, b2, mn);
+            } else if (tile == 0 && !list_long_set(L, i, s, e)) {   // (all its tiles are listed at once)
 #pragma unroll
-        for (int u = 0; u < HPL; ++u) sig[(size_t)i * n_hashes + h0 + 32 * u] = mn[u];
+                for (int u = 0; u < HPL; ++u) mn[u] = kUnlisted;
+            }
+#pragma unroll
+            for (int u = 0; u < HPL; ++u) sig[(size_t)i * n_hashes + h0 + 32 * u] = mn[u];
+        }
     }
 }
 
 // The same for few sets: a CTA per (set, tile), its eight warps taking an
-// eighth of the elements each, their minima joined in shared memory.
+// eighth of the elements each, their minima joined in shared memory.  (There
+// are fewer sets than the list of hubs holds.)
 template <int HPL>
 __global__ void __launch_bounds__(256) minhash_cta_kernel(const int64_t *__restrict__ indptr,
                                                           const uint32_t *__restrict__ indices, int n_hashes,
                                                           const uint32_t *__restrict__ A,
                                                           const uint32_t *__restrict__ B, uint32_t *__restrict__ sig,
-                                                          blsh_dev_scratch *scratch, uint2 *__restrict__ big) {
+                                                          const LongSets L) {
     __shared__ uint32_t red[8][32 * HPL];
-    __shared__ bool s_queued;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int h0 = blockIdx.y * 32 * HPL;
     const long long i = blockIdx.x;
     const long long s = __ldg(indptr + i), e = __ldg(indptr + i + 1);
-    uint32_t a2[HPL], b2[HPL], mn[HPL];
-#pragma unroll
-    for (int u = 0; u < HPL; ++u) {
-        a2[u] = 2u * mod_p31(__ldg(A + h0 + 32 * u + lane));
-        b2[u] = 2u * mod_p31(__ldg(B + h0 + 32 * u + lane));
-        mn[u] = 0xffffffffu;
-    }
-    bool queued = false;
-    if (e - s > 8 * kBigSet) {
-        if (warp == 0) {
-            const bool q = queue_long_set(i, s, e, blockIdx.y, gridDim.y, scratch, big);
-            if (lane == 0) s_queued = q;
+    if (e - s > kHubSet) {
+        if (blockIdx.y == 0) {
+            if (warp == 0) list_long_set(L, i, s, e);
+            for (int k = threadIdx.x; k < n_hashes; k += 256) sig[(size_t)i * n_hashes + k] = kListed;
         }
-        __syncthreads();
-        queued = s_queued;
+        return;
     }
-    if (!queued) {
-        const long long piece = (e - s + 7) >> 3;
-        const long long s0 = s + warp * piece, e0 = s0 + piece < e ? s0 + piece : e;
-        min_hash_run<HPL>(indices, s0, e0, a2, b2, mn);
-    }
+    uint32_t a2[HPL], b2[HPL], mn[HPL];
+    load_coeffs<HPL>(A, B, blockIdx.y, a2, b2);
+#pragma unroll
+    for (int u = 0; u < HPL; ++u) mn[u] = 0xffffffffu;
+    const long long piece = (e - s + 7) >> 3;
+    const long long s0 = s + warp * piece, e0 = s0 + piece < e ? s0 + piece : e;
+    min_hash_run<HPL>(indices, s0, e0, a2, b2, mn);
 #pragma unroll
     for (int u = 0; u < HPL; ++u) red[warp][32 * u + lane] = mn[u];
     __syncthreads();
@@ -158,43 +178,95 @@ __global__ void __launch_bounds__(256) minhash_cta_kernel(const int64_t *__restr
         uint32_t m = red[0][threadIdx.x];
 #pragma unroll
         for (int w = 1; w < 8; ++w) m = min(m, red[w][threadIdx.x]);
-        sig[(size_t)i * n_hashes + h0 + threadIdx.x] = m;
+        sig[(size_t)i * n_hashes + (size_t)blockIdx.y * 32 * HPL + threadIdx.x] = m;
     }
 }
 
-// The queued chunks of long sets, a warp each: entry (set, chunk * tiles +
-// tile); the chunk's minima meet in the set's row in global memory (atomicMin:
-// the minimum does not depend on the order).
+// The listed sets: a list's blocks are cut into equal parts, about four a warp
+// over all tiles, whatever sets they lie in, and handed out from a counter; a
+// part's minima of a set meet in the set's row
+// in global memory (atomicMin: the minimum does not depend on the order).
+template <int HPL>
+__device__ __forceinline__ void hash_listed(const uint2 *list, unsigned long long count, unsigned long long cap,
+                                            unsigned long long *next,
+                                            const int64_t *__restrict__ indptr, const uint32_t *__restrict__ indices,
+                                            int n_hashes, const uint32_t *__restrict__ A,
+                                            const uint32_t *__restrict__ B, uint32_t *__restrict__ sig) {
+    const int lane = threadIdx.x & 31;
+    const unsigned long long entries = count >> kListShift;
+    if (entries == 0) return;
+    const unsigned n = (unsigned)(entries < cap ? entries : cap);
+    unsigned total = (unsigned)count;                  // (< 2^32 blocks)
+    if (entries > cap) {
+        const uint2 last = list[n - 1];
+        total = last.y + (unsigned)((__ldg(indptr + last.x + 1) - __ldg(indptr + last.x) + 31) >> 5);
+    }
+    const unsigned tiles = (unsigned)n_hashes / (32u * HPL), warps = gridDim.x * (blockDim.x >> 5);
+    const unsigned per_tile = 4 * warps / tiles > 0 ? 4 * warps / tiles : 1u;
+    unsigned part = (total - 1) / per_tile + 1;
+    if (part < kPartBlocks) part = kPartBlocks;
+    const unsigned parts = (total - 1) / part + 1;     // parts tiles <= 4 warps, unless the tiles alone are more
+    for (;;) {
+        unsigned u = 0;
+        if (lane == 0) u = (unsigned)atomicAdd(next, 1ull);
+        u = __shfl_sync(kFull, u, 0);
+        if (u >= parts * tiles) break;
+        const unsigned tile = u / parts;
+        unsigned b = (u - tile * parts) * part;        // the next block
+        const unsigned end = total - b > part ? b + part : total;
+        unsigned q = 0, hi = n;                        // its set: the last that starts at or before it
+        while (hi - q > 1) {
+            const unsigned mid = q + (hi - q) / 2;
+            if (list[mid].y <= b) q = mid; else hi = mid;
+        }
+        uint32_t a2[HPL], b2[HPL];
+        load_coeffs<HPL>(A, B, tile, a2, b2);
+        for (; b < end; ++q) {
+            const uint2 ent = list[q];
+            long long s = __ldg(indptr + ent.x), e = __ldg(indptr + ent.x + 1);
+            const unsigned next = ent.y + (unsigned)((e - s + 31) >> 5);   // the set's last block, and one
+            const unsigned to = next < end ? next : end;
+            if (next > end) e = s + 32ll * (end - ent.y);
+            s += 32ll * (b - ent.y);
+            b = to;
+            uint32_t mn[HPL];
+#pragma unroll
+            for (int v = 0; v < HPL; ++v) mn[v] = 0xffffffffu;
+            min_hash_run<HPL>(indices, s, e, a2, b2, mn);
+            uint32_t *row = sig + (size_t)ent.x * n_hashes + (size_t)tile * 32 * HPL + lane;
+#pragma unroll
+            for (int v = 0; v < HPL; ++v) atomicMin(row + 32 * v, mn[v]);
+        }
+    }
+}
+
 template <int HPL>
 __global__ void __launch_bounds__(256) minhash_big_kernel(const int64_t *__restrict__ indptr,
-                                                          const uint32_t *__restrict__ indices, int n_hashes,
-                                                          const uint32_t *__restrict__ A,
+                                                          const uint32_t *__restrict__ indices, long long N,
+                                                          int n_hashes, const uint32_t *__restrict__ A,
                                                           const uint32_t *__restrict__ B,
-                                                          uint32_t *__restrict__ sig, const blsh_dev_scratch *scratch,
-                                                          const uint2 *__restrict__ big) {
-    const int lane = threadIdx.x & 31;
+                                                          uint32_t *__restrict__ sig, const LongSets L) {
+    // one copy of the code for both lists: hubs first
+#pragma unroll 1
+    for (int set = 0; set < 2; ++set)
+        hash_listed<HPL>(set ? L.set : L.hub, set ? *L.n_set : *L.n_hub, set ? BLSH_LITE_QUEUE_CAP : BLSH_RECHECK_CAP,
+                         L.next + set, indptr, indices, n_hashes, A, B, sig);
+    if (*L.n_hub >> kListShift <= BLSH_RECHECK_CAP && *L.n_set >> kListShift <= BLSH_LITE_QUEUE_CAP) return;
     const unsigned tiles = (unsigned)n_hashes / (32u * HPL);
-    const unsigned long long total = scratch->work3;
-    const unsigned long long nq = total < BLSH_RECHECK_CAP ? total : BLSH_RECHECK_CAP;
-    const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
-    for (unsigned long long q = (unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); q < nq;
-         q += warps) {
-        const uint2 ent = big[q];
-        if (ent.y == 0xffffffffu) continue;
-        const unsigned c = ent.y / tiles;
-        const int h0 = (int)(ent.y - c * tiles) * 32 * HPL + lane;
-        const long long s = __ldg(indptr + ent.x) + (long long)c * kBigChunk;
-        const long long e = min(s + kBigChunk, (long long)__ldg(indptr + ent.x + 1));
-        uint32_t a2[HPL], b2[HPL], mn[HPL];
+    const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
+    for (long long i = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < N; i += warps) {
+        const long long s = __ldg(indptr + i), e = __ldg(indptr + i + 1);
+        uint32_t *row = sig + (size_t)i * n_hashes + (threadIdx.x & 31);
+        if (e - s <= kBigSet || sig[(size_t)i * n_hashes] != kUnlisted) continue;
+        for (unsigned tile = 0; tile < tiles; ++tile) {
+            uint32_t a2[HPL], b2[HPL], mn[HPL];
+            load_coeffs<HPL>(A, B, tile, a2, b2);
 #pragma unroll
-        for (int u = 0; u < HPL; ++u) {
-            a2[u] = 2u * mod_p31(__ldg(A + h0 + 32 * u));
-            b2[u] = 2u * mod_p31(__ldg(B + h0 + 32 * u));
-            mn[u] = 0xffffffffu;
+            for (int u = 0; u < HPL; ++u) mn[u] = 0xffffffffu;
+            min_hash_run<HPL>(indices, s, e, a2, b2, mn);
+#pragma unroll
+            for (int u = 0; u < HPL; ++u) row[(size_t)tile * 32 * HPL + 32 * u] = mn[u];
         }
-        min_hash_run<HPL>(indices, s, e, a2, b2, mn);
-#pragma unroll
-        for (int u = 0; u < HPL; ++u) atomicMin(&sig[(size_t)ent.x * n_hashes + h0 + 32 * u], mn[u]);
     }
 }
 
@@ -1052,11 +1124,10 @@ int srp_threads(int bits, int *per_thread) {
 }  // namespace
 
 // minhash_kernel over every set, then minhash_big_kernel over the long sets
-// the first one queued.
+// the first one listed.
 template <int HPL>
 int minhash_launch(blsh_ctx *ctx, cudaStream_t s, const int64_t *indptr, const uint32_t *indices, int64_t N,
-                   int n_hashes, const uint32_t *a, const uint32_t *b, uint32_t *sig, uint2 *big) {
-    blsh_dev_scratch *scr = ctx->scratch;
+                   int n_hashes, const uint32_t *a, const uint32_t *b, uint32_t *sig, const LongSets &L) {
     const unsigned tiles = (unsigned)(n_hashes / (32 * HPL));
     const long long blocks = (N + 7) / 8, cap = (long long)ctx->sm_count * 32;
     blsh_time_start(ctx, s);
@@ -1064,13 +1135,13 @@ int minhash_launch(blsh_ctx *ctx, cudaStream_t s, const int64_t *indptr, const u
     // the longest set's chain decides (2,000 sets, mean 50, longest 837, x 256
     // hashes: 124 us with a warp per set, 23 us with a CTA)
     if (N * tiles < 32ll * ctx->sm_count)
-        minhash_cta_kernel<HPL><<<dim3((unsigned)N, tiles), 256, 0, s>>>(indptr, indices, n_hashes, a, b, sig, scr, big);
+        minhash_cta_kernel<HPL><<<dim3((unsigned)N, tiles), 256, 0, s>>>(indptr, indices, n_hashes, a, b, sig, L);
     else
-        minhash_kernel<HPL><<<dim3((unsigned)(blocks < cap ? blocks : cap), tiles), 256, 0, s>>>(
-            indptr, indices, N, n_hashes, a, b, sig, scr, big);
+        minhash_kernel<HPL><<<dim3((unsigned)(blocks < cap ? blocks : cap), tiles < 65535u ? tiles : 65535u), 256, 0, s>>>(
+            indptr, indices, N, n_hashes, a, b, sig, L);
     BLSH_LAUNCHED(ctx, "minhash_kernel");
     blsh_time_start(ctx, s);
-    minhash_big_kernel<HPL><<<ctx->sm_count * 4, 256, 0, s>>>(indptr, indices, n_hashes, a, b, sig, scr, big);
+    minhash_big_kernel<HPL><<<ctx->sm_count * 4, 256, 0, s>>>(indptr, indices, N, n_hashes, a, b, sig, L);
     BLSH_LAUNCHED(ctx, "minhash_big_kernel");
     return BLSH_OK;
 }
@@ -1087,15 +1158,21 @@ extern "C" int blsh_minhash(blsh_ctx *ctx, const int64_t *indptr, const uint32_t
     blsh_device_guard g(ctx->device);
     cudaStream_t s = blsh_stream(stream);
     const int words = n_hashes / 32;
-    // long sets go to minhash_big_kernel through the context's work queue
-    uint2 *big = ctx->recheck_queue;
-    BLSH_CUDA(ctx, cudaMemsetAsync(&ctx->scratch->work3, 0, sizeof(unsigned long long), s));
+    // long sets go to minhash_big_kernel through the context's queues
+    blsh_dev_scratch *scr = ctx->scratch;
+    static_assert(offsetof(blsh_dev_scratch, work2) == offsetof(blsh_dev_scratch, work) + 8 &&
+                      offsetof(blsh_dev_scratch, work3) == offsetof(blsh_dev_scratch, work) + 16 &&
+                      offsetof(blsh_dev_scratch, recheck_count) == offsetof(blsh_dev_scratch, work) + 24,
+                  "cleared together");
+    const LongSets L = {reinterpret_cast<uint2 *>(ctx->lite_queue), ctx->recheck_queue, &scr->work3, &scr->recheck_count,
+                        &scr->work};
+    BLSH_CUDA(ctx, cudaMemsetAsync(&scr->work, 0, 4 * sizeof(unsigned long long), s));
     const int hpl = words % 8 == 0 ? 8 : words % 4 == 0 ? 4 : words % 2 == 0 ? 2 : 1;   // hashes a lane
     switch (hpl) {
-    case 8: return minhash_launch<8>(ctx, s, indptr, indices, N, n_hashes, a, b, sig, big);
-    case 4: return minhash_launch<4>(ctx, s, indptr, indices, N, n_hashes, a, b, sig, big);
-    case 2: return minhash_launch<2>(ctx, s, indptr, indices, N, n_hashes, a, b, sig, big);
-    default: return minhash_launch<1>(ctx, s, indptr, indices, N, n_hashes, a, b, sig, big);
+    case 8: return minhash_launch<8>(ctx, s, indptr, indices, N, n_hashes, a, b, sig, L);
+    case 4: return minhash_launch<4>(ctx, s, indptr, indices, N, n_hashes, a, b, sig, L);
+    case 2: return minhash_launch<2>(ctx, s, indptr, indices, N, n_hashes, a, b, sig, L);
+    default: return minhash_launch<1>(ctx, s, indptr, indices, N, n_hashes, a, b, sig, L);
     }
 }
 
