@@ -1,8 +1,8 @@
 // compact.cu -- the output set O of Algorithms 1 and 2: a stable compaction
 // of the retained pair indices.
 //
-// A fixed grid of C CTAs splits [0, P) into C contiguous ranges (starting
-// at multiples of 16 statuses, read 16 at a time).  Pass 1
+// Few statuses take one launch (compact_few).  Otherwise a fixed grid of C CTAs
+// splits [0, P) into C contiguous ranges, read 16 statuses at a time.  Pass 1
 // counts the kept items of each range (1e9 statuses: 0.30 ms at one load in
 // flight a thread, 0.19 with eight; pass 2 0.52 and 0.39); pass 2 gives each CTA the sum of the
 // counts of the ranges before it and writes its range's indices in order,
@@ -26,18 +26,36 @@ __device__ __forceinline__ long long resolve_p(long long P, const long long *P_d
     return pd < 0 ? 0 : (pd < P ? pd : P);
 }
 
-// CTA b owns [lo, hi): P * b / C rounded down to a multiple of 16, so that
-// with a 16-byte aligned status array every thread reads its 16 statuses
-// with one 16-byte load.
-__device__ __forceinline__ void cta_range(long long P, long long &lo, long long &hi) {
-    lo = (P * blockIdx.x / gridDim.x) & ~15ll;
-    hi = blockIdx.x + 1 == gridDim.x ? P : (P * (blockIdx.x + 1) / gridDim.x) & ~15ll;
+// The status array may start anywhere: `off` is its address modulo 16, and
+// ranges and tiles begin at multiples of 16 of the index plus off, so that every
+// 16 statuses but the first ones are one 16-byte load.
+// CTA b owns [lo, hi), about P b / C on; the first begins at -off (statuses
+// below 0 are none).
+__device__ __forceinline__ void cta_range(long long P, int off, long long &lo, long long &hi) {
+    lo = ((P * blockIdx.x / gridDim.x + off) & ~15ll) - off;
+    hi = blockIdx.x + 1 == gridDim.x ? P : ((P * (blockIdx.x + 1) / gridDim.x + off) & ~15ll) - off;
 }
 
-// Bit i of the result: status i of v is kept.
+// Bit i: status i (a byte of v) is kept (a shift past 31 gives 0): about four
+// operations a status, whatever the mask.
+__device__ __forceinline__ uint32_t kept4(uint32_t v, uint32_t mask) {
+    uint32_t r = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        uint32_t k;
+        asm("shr.u32 %0, %1, %2;" : "=r"(k) : "r"(mask), "r"((v >> (8 * i)) & 0xffu));   // (clamped at 32)
+        r |= (k & 1u) << i;
+    }
+    return r;
+}
+
+// Bit i of the result: status i of v is kept.  One or two kept statuses are
+// matched in all 16 bytes at once, about 45 operations each; more cost what
+// kept4 does.
 __device__ __forceinline__ uint32_t kept16(uint4 v, uint32_t mask) {
+    if (__popc(mask) > 2) return kept4(v.x, mask) | kept4(v.y, mask) << 4 | kept4(v.z, mask) << 8 | kept4(v.w, mask) << 12;
     uint32_t bits = 0;
-    for (uint32_t m = mask; m; m &= m - 1) bits |= blsh_eq16(v, (uint32_t)(__ffs(m) - 1));   // each kept status
+    for (uint32_t m = mask; m; m &= m - 1) bits |= blsh_eq16(v, (uint32_t)(__ffs(m) - 1));
     return bits;
 }
 
@@ -47,8 +65,8 @@ __device__ __forceinline__ uint32_t kept16(uint4 v, uint32_t mask) {
 // 1e9 statuses were read at 3.3 TB/s.
 template <int U>
 __device__ __forceinline__ void kept_tiles(const uint8_t *status, long long q0, long long step, long long hi,
-                                           uint32_t mask, bool vec, uint32_t (&bits)[U]) {
-    if (vec && q0 + (U - 1) * step + 16 <= hi) {
+                                           uint32_t mask, uint32_t (&bits)[U]) {
+    if (q0 >= 0 && q0 + (U - 1) * step + 16 <= hi) {
         uint4 v[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) v[u] = __ldg(reinterpret_cast<const uint4 *>(status + q0 + u * step));
@@ -60,90 +78,90 @@ __device__ __forceinline__ void kept_tiles(const uint8_t *status, long long q0, 
             const long long q = q0 + u * step;
             bits[u] = 0;
             if (q >= hi) continue;
-            if (vec && q + 16 <= hi) {
+            if (q >= 0 && q + 16 <= hi) {
                 bits[u] = kept16(__ldg(reinterpret_cast<const uint4 *>(status + q)), mask);
             } else {
                 for (int i = 0; i < 16; ++i)
-                    if (q + i < hi) bits[u] |= (uint32_t)kept(status[q + i], mask) << i;
+                    if (q + i >= 0 && q + i < hi) bits[u] |= (uint32_t)kept(status[q + i], mask) << i;
             }
         }
     }
 }
 
-// Up to kFew statuses: one CTA, every load in flight, one prefix sum over the
-// warps' counts of all its tiles.  No count pass: the second launch costs more
-// than the rest (50,000 statuses, 200 of them in use: 12.6 us in two launches,
-// 7.5 in one).
-constexpr int kFewThreads = 1024, kFewTiles = 8;
-constexpr long long kFew = (long long)kFewThreads * kPer * kFewTiles;
+// Up to kFew statuses: one launch.  CTA b writes the indices of 4,096 statuses,
+// in order from shared memory so that the stores are coalesced, and counts the
+// kept ones before them itself (at most 128 KB, from L2, every load in flight)
+// instead of waiting for a count pass: the second launch costs more.  Those
+// past the device's count end at once.  (One CTA for all of them wrote its
+// indices a lane each: 131,072 statuses, all kept, 79 us, 12.0 in two launches;
+// 8.7 here.  200 in use: 12.6 in two launches, 8.7 here.)
+constexpr int kFewThreads = 1024, kFewTile = 4 * kFewThreads, kFewLoads = 8;
+constexpr long long kFew = (long long)kFewThreads * kPer * kFewLoads;
 __global__ void __launch_bounds__(kFewThreads) compact_few(const uint8_t *status, long long P_cap,
-                                                           const long long *P_dev, uint32_t mask, bool vec,
+                                                           const long long *P_dev, uint32_t mask, int off,
                                                            int64_t *out, long long cap, long long *n_out,
                                                            blsh_dev_scratch *scratch) {
-    static_assert(kFewTiles * (kFewThreads / 32) == 256, "eight counts a lane of the warp that adds them");
-    __shared__ int s_cnt[256];   // [tile][warp]: kept, then kept before
-    const long long P = resolve_p(P_cap, P_dev);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    uint32_t bits[kFewTiles];
-    kept_tiles<kFewTiles>(status, (long long)threadIdx.x * kPer, kFewThreads * kPer, P, mask, vec, bits);
-    int before[kFewTiles];
+    __shared__ int s_before[32], s_own[32];
+    __shared__ uint16_t s_list[kFewTile];
+    const int P = (int)resolve_p(P_cap, P_dev), lo = (int)blockIdx.x * kFewTile - off;   // (the first begins at -off)
+    if (lo >= P && blockIdx.x > 0) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, t = threadIdx.x;
+    auto by_one = [&](int q, int n) {   // statuses q .. q + n - 1, those that are there
+        uint32_t b = 0;
+        for (int i = 0; i < n; ++i)
+            if (q + i >= 0 && q + i < P) b |= (uint32_t)kept(status[q + i], mask) << i;
+        return b;
+    };
+    uint4 v[kFewLoads];   // the statuses before this CTA's, chunks of 16 from -off on
 #pragma unroll
-    for (int u = 0; u < kFewTiles; ++u) {
-        const int c = __popc(bits[u]);
-        int incl = c;
+    for (int u = 0; u < kFewLoads; ++u) {
+        const int q = (t + u * kFewThreads) * kPer - off;
+        v[u] = q >= 0 && q < lo ? __ldg(reinterpret_cast<const uint4 *>(status + q)) : make_uint4(~0u, ~0u, ~0u, ~0u);
+    }
+    const int q = lo + 4 * t;   // its own, four a thread
+    const uint32_t own = q >= 0 && q + 4 <= P ? kept4(__ldg(reinterpret_cast<const uint32_t *>(status + q)), mask)
+                                              : by_one(q, 4);
+    int before = t == 0 && off && lo > 0 ? __popc(by_one(-off, kPer)) : 0;   // the first chunk, where it is not whole
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        before[u] = incl - c;
-        if (lane == 31) s_cnt[u * (kFewThreads / 32) + warp] = incl;
+    for (int u = 0; u < kFewLoads; ++u)
+        before += __popc(kept16(v[u], mask));
+    before = __reduce_add_sync(0xffffffffu, before);
+    const int c = __popc(own);
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) {
+        s_before[warp] = before;
+        s_own[warp] = incl;
     }
     __syncthreads();
-    if (warp == 0) {
-        int v[8], sum = 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            v[i] = s_cnt[8 * lane + i];
-            sum += v[i];
-        }
-        int incl = sum;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
-        }
-        int at = incl - sum;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            s_cnt[8 * lane + i] = at;
-            at += v[i];
-        }
-        if (lane == 31) {
-            *n_out = incl;
-            if (incl > cap) blsh_dev_error(scratch, BLSH_ETRUNC, 1, (unsigned long long)(incl - cap));
-        }
-    }
+    const int base = __reduce_add_sync(0xffffffffu, s_before[lane]);
+    const int total = __reduce_add_sync(0xffffffffu, s_own[lane]);
+    int at = incl - c + __reduce_add_sync(0xffffffffu, lane < warp ? s_own[lane] : 0);
+    for (uint32_t b = own; b; b &= b - 1) s_list[at++] = (uint16_t)(4 * t + __ffs(b) - 1);
     __syncthreads();
-#pragma unroll
-    for (int u = 0; u < kFewTiles; ++u) {
-        long long o = s_cnt[u * (kFewThreads / 32) + warp] + before[u];
-        const long long q0 = (long long)u * kFewThreads * kPer + (long long)threadIdx.x * kPer;
-        for (uint32_t b = bits[u]; b; b &= b - 1, ++o)
-            if (o < cap) out[o] = q0 + __ffs(b) - 1;
+    for (int i = t; i < total; i += kFewThreads)
+        if ((long long)base + i < cap) out[base + i] = lo + s_list[i];
+    if (lo + kFewTile >= P && t == 0) {   // the last of them
+        const long long n = (long long)base + total;
+        *n_out = n;
+        if (n > cap) blsh_dev_error(scratch, BLSH_ETRUNC, 1, (unsigned long long)(n - cap));
     }
 }
 
 __global__ void __launch_bounds__(kThreads) compact_count(const uint8_t *status, long long P_cap,
-                                                          const long long *P_dev, uint32_t mask, bool vec,
+                                                          const long long *P_dev, uint32_t mask, int off,
                                                           blsh_dev_scratch *scratch) {
     const long long P = resolve_p(P_cap, P_dev);
     long long lo, hi;
-    cta_range(P, lo, hi);
+    cta_range(P, off, lo, hi);
     long long c = 0;
     for (long long q0 = lo + 16ll * threadIdx.x; q0 < hi; q0 += (long long)kBatch * kTile) {
         uint32_t bits[kBatch];
-        kept_tiles<kBatch>(status, q0, kTile, hi, mask, vec, bits);
+        kept_tiles<kBatch>(status, q0, kTile, hi, mask, bits);
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) c += __popc(bits[u]);
     }
@@ -152,14 +170,22 @@ __global__ void __launch_bounds__(kThreads) compact_count(const uint8_t *status,
     if (threadIdx.x == 0) scratch->cta_counts[blockIdx.x] = total;
 }
 
+// The indices of a warp's 512 statuses are written in order from shared memory,
+// 32 at a time, where more than kFewKept are kept, else by the lanes that hold
+// them (1e8 statuses, all kept, a lane writing its own 16: 926 us, 210 here; a
+// sixth kept 110, 117 through shared memory).
+constexpr int kFewKept = 128;
 __global__ void __launch_bounds__(kThreads) compact_write(const uint8_t *status, long long P_cap,
-                                                          const long long *P_dev, uint32_t mask, bool vec,
+                                                          const long long *P_dev, uint32_t mask, int off,
                                                           int64_t *out, long long cap, long long *n_out,
                                                           blsh_dev_scratch *scratch) {
     __shared__ long long s_base;
+    __shared__ uint16_t s_list[kThreads / 32][32 * kPer];
+    const int lane = threadIdx.x & 31;
+    uint16_t *list = s_list[threadIdx.x >> 5];
     const long long P = resolve_p(P_cap, P_dev);
     long long lo, hi;
-    cta_range(P, lo, hi);
+    cta_range(P, off, lo, hi);
     long long before = 0;
     for (int c = threadIdx.x; c < (int)blockIdx.x; c += kThreads) before += scratch->cta_counts[c];
     long long tot;
@@ -171,16 +197,26 @@ __global__ void __launch_bounds__(kThreads) compact_write(const uint8_t *status,
     // tile gets its block-wide prefix sum and writes its indices in order
     for (long long t0 = lo; t0 < hi; t0 += (long long)kBatch * kTile) {
         uint32_t bits[kBatch];
-        kept_tiles<kBatch>(status, t0 + (long long)threadIdx.x * kPer, kTile, hi, mask, vec, bits);
+        kept_tiles<kBatch>(status, t0 + (long long)threadIdx.x * kPer, kTile, hi, mask, bits);
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
             if (t0 + (long long)u * kTile >= hi) break;      // uniform across the CTA
-            const long long q0 = t0 + (long long)u * kTile + (long long)threadIdx.x * kPer;
             long long tile_total;
-            long long o = base + blsh_scan::block_exclusive<long long>((long long)__popc(bits[u]), &tile_total);
-            for (uint32_t b = bits[u]; b; b &= b - 1) {
-                if (o < cap) out[o] = q0 + __ffs(b) - 1;
-                ++o;
+            const int c = __popc(bits[u]);
+            const long long mine = base + blsh_scan::block_exclusive<long long>((long long)c, &tile_total);
+            const long long first = __shfl_sync(0xffffffffu, mine, 0);
+            int at = (int)(mine - first);
+            const int n = __shfl_sync(0xffffffffu, at + c, 31);
+            const long long q0 = t0 + (long long)u * kTile + (long long)(threadIdx.x - lane) * kPer;
+            if (n <= kFewKept) {
+                for (uint32_t b = bits[u]; b; b &= b - 1, ++at)
+                    if (first + at < cap) out[first + at] = q0 + kPer * lane + __ffs(b) - 1;
+            } else {
+                for (uint32_t b = bits[u]; b; b &= b - 1) list[at++] = (uint16_t)(kPer * lane + __ffs(b) - 1);
+                __syncwarp();
+                for (int i = lane; i < n; i += 32)
+                    if (first + i < cap) out[first + i] = q0 + list[i];
+                __syncwarp();
             }
             base += tile_total;
         }
@@ -208,20 +244,21 @@ extern "C" int blsh_compact(blsh_ctx *ctx, const uint8_t *status, int64_t P, con
                                                                                  : BLSH_COMPACT_MAX_CTAS;
     if (ctas > most) ctas = most;
     if (ctas < 1) ctas = 1;
-    const bool vec = blsh_aligned(status, 16);
+    const int off = (int)((uintptr_t)status & 15);
     if (P <= kFew) {
+        const unsigned few = (unsigned)((P + off + kFewTile - 1) / kFewTile);
         blsh_time_start(ctx, s);
-        compact_few<<<1, kFewThreads, 0, s>>>(status, P, (const long long *)P_dev, keep_mask, vec, out_idx, cap,
-                                              (long long *)n_out, ctx->scratch);
+        compact_few<<<few > 0 ? few : 1u, kFewThreads, 0, s>>>(status, P, (const long long *)P_dev, keep_mask, off,
+                                                               out_idx, cap, (long long *)n_out, ctx->scratch);
         BLSH_LAUNCHED(ctx, "compact_few");
         return BLSH_OK;
     }
     blsh_time_start(ctx, s);
-    compact_count<<<(unsigned)ctas, kThreads, 0, s>>>(status, P, (const long long *)P_dev, keep_mask, vec,
+    compact_count<<<(unsigned)ctas, kThreads, 0, s>>>(status, P, (const long long *)P_dev, keep_mask, off,
                                                       ctx->scratch);
     BLSH_LAUNCHED(ctx, "compact_count");
     blsh_time_start(ctx, s);
-    compact_write<<<(unsigned)ctas, kThreads, 0, s>>>(status, P, (const long long *)P_dev, keep_mask, vec, out_idx,
+    compact_write<<<(unsigned)ctas, kThreads, 0, s>>>(status, P, (const long long *)P_dev, keep_mask, off, out_idx,
                                                       cap, (long long *)n_out, ctx->scratch);
     BLSH_LAUNCHED(ctx, "compact_write");
     return BLSH_OK;

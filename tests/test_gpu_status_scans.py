@@ -91,3 +91,73 @@ def test_resumed_pairs(B, ctx, kind, k, P):
     for a, b in zip(got, want):
         assert torch.equal(a, b)
     assert opened > P // 50 or P == 1
+
+
+@pytest.mark.parametrize("P", [0, 1, 4095, 4096, 4097, 8193, 126_977, 131_072])
+@pytest.mark.parametrize("keep", [0, 1 << 4, 0xffffffff])
+@pytest.mark.parametrize("offset", [0, 1, 15])
+def test_compaction_in_one_launch(B, ctx, P, keep, offset):
+    """Tiles of 4,096 statuses from a 16-byte boundary on, all kept, some and
+    none, and a device count at and past the end of a tile."""
+    st = (np.arange(P) * 7 % 37).astype(np.uint8)   # 32 .. 36 are never kept
+    store = torch.full((P + offset + 16,), 4, dtype=torch.uint8, device=dev)   # kept, but outside
+    dst = store[offset:offset + P]
+    dst.copy_(torch.from_numpy(st))
+    for used in sorted({0, min(P, 5), max(0, 4096 - offset) if P >= 4096 else 0, P // 2 // 4096 * 4096, P // 2, P}):
+        want = O.compact(st[:used], keep)
+        out = torch.full((P,), -1, dtype=torch.int64, device=dev)
+        n_out = torch.full((1,), 5, dtype=torch.int64, device=dev)
+        B.blsh_compact(ctx, dst, keep, out, n_out, P_dev=torch.tensor([used], dtype=torch.int64, device=dev))
+        assert B.blsh_status(ctx) == 0 and int(n_out) == len(want)
+        assert np.array_equal(out[: len(want)].cpu().numpy(), want) and bool((out[len(want):] == -1).all())
+
+
+@pytest.mark.parametrize("P", [60_000, 131_072])
+def test_compaction_of_kept_statuses_takes_no_single_block(B, ctx, P):
+    """Everything kept: 8 bytes a status written by all the blocks (a single one
+    takes 40 to 80 us, two launches 12)."""
+    st = torch.full((P,), 3, dtype=torch.uint8, device=dev)
+    out, n_out = torch.zeros(P, dtype=torch.int64, device=dev), torch.zeros(1, dtype=torch.int64, device=dev)
+    times = []
+    for _ in range(4):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(20):
+            B.blsh_compact(ctx, st, 1 << 3, out, n_out)
+        b.record()
+        b.synchronize()
+        times.append(a.elapsed_time(b) / 20)
+    assert int(n_out) == P and torch.equal(out, torch.arange(P, device=dev))
+    assert min(times) < 0.025, times
+
+
+@pytest.mark.parametrize("offset", [0, 1, 15])
+@pytest.mark.parametrize("P", [131_073, 2_500_000])
+def test_compaction_from_any_address(B, ctx, P, offset):
+    st = (np.arange(P) * 11 % 41).astype(np.uint8)
+    store = torch.full((P + offset + 16,), 4, dtype=torch.uint8, device=dev)
+    dst = store[offset:offset + P]
+    dst.copy_(torch.from_numpy(st))
+    for used in (0, 3, 700, P - 1, P):
+        want = O.compact(st[:used], 0x80000015)
+        out = torch.full((P,), -1, dtype=torch.int64, device=dev)
+        n_out = torch.full((1,), 5, dtype=torch.int64, device=dev)
+        B.blsh_compact(ctx, dst, 0x80000015, out, n_out, P_dev=torch.tensor([used], dtype=torch.int64, device=dev))
+        assert B.blsh_status(ctx) == 0 and int(n_out) == len(want)
+        assert np.array_equal(out[: len(want)].cpu().numpy(), want) and bool((out[len(want):] == -1).all())
+
+
+@pytest.mark.parametrize("offset", [0, 1, 15])
+@pytest.mark.parametrize("P", [131_073, 2_500_000])
+def test_compaction_from_any_address(B, ctx, P, offset):
+    st = (np.arange(P) * 11 % 41).astype(np.uint8)
+    store = torch.full((P + offset + 16,), 4, dtype=torch.uint8, device=dev)
+    dst = store[offset:offset + P]
+    dst.copy_(torch.from_numpy(st))
+    for used in (0, 3, 700, P - 1, P):
+        want = O.compact(st[:used], 0x80000015)
+        out = torch.full((P,), -1, dtype=torch.int64, device=dev)
+        n_out = torch.full((1,), 5, dtype=torch.int64, device=dev)
+        B.blsh_compact(ctx, dst, 0x80000015, out, n_out, P_dev=torch.tensor([used], dtype=torch.int64, device=dev))
+        assert B.blsh_status(ctx) == 0 and int(n_out) == len(want)
+        assert np.array_equal(out[: len(want)].cpu().numpy(), want) and bool((out[len(want):] == -1).all())
