@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kFewThreads) compact_few(const uint8_t *status
     int before = t == 0 && off && lo > 0 ? __popc(by_one(-off, kPer)) : 0;   // the first chunk, where it is not whole
 #pragma unroll
     for (int u = 0; u < kFewLoads; ++u)
-        before += __popc(kept16(v[u], mask));
+        if (u * kFewThreads * kPer < lo + off) before += __popc(kept16(v[u], mask));   // (the CTA has any there)
     before = __reduce_add_sync(0xffffffffu, before);
     const int c = __popc(own);
     int incl = c;
