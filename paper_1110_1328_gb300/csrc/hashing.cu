@@ -554,7 +554,9 @@ __device__ __forceinline__ bool srp_undecided(const SrpArgs &A, const RT *R, lon
     return d >= 0.0;
 }
 
-template <typename RT, int CPL>
+// ONCE: no more items than warps, a warp's is that of its number (the counter
+// takes about 0.9 ns a grab, the last and vain one of every warp included).
+template <typename RT, int CPL, bool ONCE>
 __global__ void __launch_bounds__(256, 4) srp_sparse4_kernel(const SrpArgs A, const RT *__restrict__ R, int G) {
     constexpr bool Q16 = sizeof(RT) == 2;
     constexpr int PC = 32 * CPL;   // columns of a piece
@@ -565,8 +567,12 @@ __global__ void __launch_bounds__(256, 4) srp_sparse4_kernel(const SrpArgs A, co
     const unsigned long long items = (unsigned long long)groups * A.outer;
     for (;;) {
         unsigned long long item = 0;
-        if (lane == 0) item = atomicAdd(&A.scratch->hash_work, 1ull);
-        item = __shfl_sync(kFull, item, 0);
+        if constexpr (ONCE) {
+            item = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+        } else {
+            if (lane == 0) item = atomicAdd(&A.scratch->hash_work, 1ull);
+            item = __shfl_sync(kFull, item, 0);
+        }
         if (item >= items) break;
         const int outer = A.outer == 1 ? 0 : (int)(item / (unsigned long long)groups);
         const long long r0 = ((long long)item - outer * groups) * G;
@@ -678,6 +684,7 @@ __global__ void __launch_bounds__(256, 4) srp_sparse4_kernel(const SrpArgs A, co
                     A.sig[(size_t)row * words + (col0 >> 5) + lane / (32 / CPL)] = word;
             }
         }
+        if constexpr (ONCE) break;
     }
     if (bad) blsh_dev_error(A.scratch, BLSH_ERANGE, 0, bad);
     if (rechecked) atomicAdd(&A.scratch->counters[2], rechecked);
@@ -1080,17 +1087,23 @@ int srp_sparse_pieces(blsh_ctx *ctx, const int64_t *indptr, const uint32_t *indi
     const bool by_piece = (!row_mask && (double)dim * ncols * sizeof(RT) > 64e6) || N < 8 * warps;
     A.outer = by_piece ? pieces : 1;
     A.inner = by_piece ? 1 : pieces;
-    // rows a grab: up to 32, at least eight grabs a warp
+    // rows a grab: up to 32, at least eight grabs a warp.  With a mask a grab may
+    // hold few rows or none and the counter be most of the time (no row of
+    // 100,000 left: 47 us, 13 so), so there a warp's first grab is all it takes
+    // while that is at most 32 rows.
     int G = 32;
-    while (G > 1 && (N / G) * A.outer < 8 * warps) G >>= 1;
+    if (row_mask) G = (int)((N * A.outer + warps - 1) / warps < 32 ? (N * A.outer + warps - 1) / warps : 32);
+    else
+        while (G > 1 && (N / G) * A.outer < 8 * warps) G >>= 1;
     blsh_dev_scratch *scr = ctx->scratch;
     // work2 (next long row), work3 (long rows listed), recheck_count .. hash_work
     BLSH_CUDA(ctx, cudaMemsetAsync(&scr->work2, 0, offsetof(blsh_dev_scratch, norm2_valid) -
                                                        offsetof(blsh_dev_scratch, work2), s));
     const char *name = sizeof(RT) == 2 ? "srp_sparse4_kernel (two-byte codes)" : "srp_sparse4_kernel";
-    const long long blocks = ((N + G - 1) / G * A.outer + 7) / 8, most = (long long)ctx->sm_count * 8;
+    const long long items = (N + G - 1) / G * A.outer, blocks = (items + 7) / 8, most = (long long)ctx->sm_count * 8;
     blsh_time_start(ctx, s);
-    srp_sparse4_kernel<RT, CPL><<<(unsigned)(blocks < most ? blocks : most), 256, 0, s>>>(A, R, G);
+    if (items <= 2 * warps) srp_sparse4_kernel<RT, CPL, true><<<(unsigned)blocks, 256, 0, s>>>(A, R, G);
+    else srp_sparse4_kernel<RT, CPL, false><<<(unsigned)(blocks < most ? blocks : most), 256, 0, s>>>(A, R, G);
     BLSH_LAUNCHED(ctx, name);
     blsh_time_start(ctx, s);
     srp_long_kernel<RT, CPL><<<ctx->sm_count * 3, 256, 0, s>>>(A, R);

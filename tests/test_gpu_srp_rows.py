@@ -83,3 +83,52 @@ def test_rechecked_long_rows(B, ctx, form):
     rc, c = B.blsh_status(ctx, counters=True)
     assert rc == 0 and c[2] >= csr.n * bits // 2
     assert np.array_equal(sig.cpu().numpy().view(np.uint32), oracle(csr, R))
+
+
+@pytest.mark.parametrize("n", [1, 700, 20_000, 160_000])
+@pytest.mark.parametrize("share", [0.0, 0.03, 1.0])
+@pytest.mark.parametrize("form", ["float", "codes"])
+def test_masked_rows(B, ctx, n, share, form):
+    """Some rows' columns 128 .. 383: a warp's first rows all it takes, and more
+    rows than that; the others stay as they are."""
+    dim, bits = 500, 512
+    csr = rows(n, dim, n) if n > 100 else synth.CSR(np.array([0, 40], np.int64), np.arange(40, dtype=np.uint32) * 3,
+                                                    np.linspace(-1, 1, 40).astype(np.float32), dim)
+    mask = np.random.default_rng(n).random(n) < share
+    ip, val = torch.from_numpy(csr.indptr).to(dev), torch.from_numpy(csr.values).to(dev)
+    ix = torch.from_numpy(csr.indices.view(np.int32)).to(dev)
+    if form == "float":
+        R = synth.gaussian_matrix(dim, bits, seed=5)
+        want, Rd, call = O.srp_sparse(csr, R), torch.from_numpy(R).to(dev), B.blsh_srp_sparse_cols
+    else:
+        R = O.gaussian_codes(5, dim, bits)
+        want, Rd, call = O.srp_sparse_q16(csr, R), torch.from_numpy(R.view(np.int16)).to(dev), B.blsh_srp_sparse_q16_cols
+    for first, count in ((128, 256), (256, 128)):
+        sig = torch.full((n, bits // 32), 0x5A5A5A5A, dtype=torch.int32, device=dev)
+        call(ctx, ip, ix, val, Rd, sig, first, count, row_mask=torch.from_numpy(mask.astype(np.uint8)).to(dev))
+        assert B.blsh_status(ctx) == 0
+        got = sig.cpu().numpy().view(np.uint32)
+        there = np.zeros_like(got, bool)
+        there[mask, first // 32:(first + count) // 32] = True
+        assert np.array_equal(got, np.where(there, want, 0x5A5A5A5A))
+
+
+def test_an_empty_mask_costs_no_grabs(B, ctx):
+    """100,000 rows, none of them left: one look at the mask (a grab of a few rows
+    at a time takes 47 us for the counter alone)."""
+    n, dim, bits = 100_000, 300, 256
+    csr = rows(n, dim, 4)
+    ip, val = torch.from_numpy(csr.indptr).to(dev), torch.from_numpy(csr.values).to(dev)
+    ix = torch.from_numpy(csr.indices.view(np.int32)).to(dev)
+    R = torch.from_numpy(synth.gaussian_matrix(dim, bits, seed=5)).to(dev)
+    sig, mask = torch.zeros((n, bits // 32), dtype=torch.int32, device=dev), torch.zeros(n, dtype=torch.uint8, device=dev)
+    times = []
+    for _ in range(4):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(20):
+            B.blsh_srp_sparse_cols(ctx, ip, ix, val, R, sig, 128, 128, row_mask=mask)
+        b.record()
+        b.synchronize()
+        times.append(a.elapsed_time(b) / 20)
+    assert min(times) < 0.03, times
