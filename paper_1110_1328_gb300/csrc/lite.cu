@@ -19,6 +19,8 @@
 //            integer (formed with integer arithmetic) and added in int64, so
 //            the sums do not depend on the order the lanes add them in.
 // A pair is kept iff s > t.
+#include <type_traits>
+
 #include "verify.cuh"
 
 namespace {
@@ -189,26 +191,28 @@ __device__ __forceinline__ void lite_exact_one(const LiteArgs &A, long long ax, 
             __syncwarp();
             const uint32_t last = w_idx[tn - 1];
             const bool final_tile = tb + tn >= nl;
-            for (bool more = sp < ns; more;) {
-                uint32_t v[4];
-                bool in[4];
-                int pos[4];
+            // U elements a lane against a tile of fewer than 2 TOP
+            auto round = [&](auto width, auto top) {
+                constexpr int U = decltype(width)::value, TOP = decltype(top)::value;
+                uint32_t v[U];
+                bool in[U];
+                int pos[U];
                 unsigned taken = 0;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
+                for (int u = 0; u < U; ++u) {
                     const long long i = sp + 32 * u + lane;
                     v[u] = i < ns ? __ldg(A.indices + s0 + i) : 0u;
                     in[u] = i < ns && (final_tile || v[u] <= last);
                     pos[u] = 0;
                 }
 #pragma unroll
-                for (int u = 0; u < 4; ++u) taken += __popc(__ballot_sync(kFull, in[u]));
-                for (int step = kTile / 2; step > 0; step >>= 1)
+                for (int u = 0; u < U; ++u) taken += __popc(__ballot_sync(kFull, in[u]));
+                for (int step = TOP; step > 0; step >>= 1)
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
+                    for (int u = 0; u < U; ++u)
                         if (pos[u] + step <= tn && w_idx[pos[u] + step - 1] < v[u]) pos[u] += step;
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
+                for (int u = 0; u < U; ++u) {
                     const bool hit = in[u] && pos[u] < tn && w_idx[pos[u]] == v[u];
                     if (!COSINE) {
                         inter += hit;
@@ -220,7 +224,13 @@ __device__ __forceinline__ void lite_exact_one(const LiteArgs &A, long long ax, 
                     }
                 }
                 sp += taken;
-                more = taken == 128 && sp < ns;            // the rest lies past this tile, or none is left
+                return taken == 32 * U && sp < ns;         // the rest lies past this tile, or none is left
+            };
+            if (!KEEP && tn < 128 && ns - sp <= 64) {
+                if (sp < ns) round(std::integral_constant<int, 2>{}, std::integral_constant<int, 64>{});
+            } else {
+                for (bool more = sp < ns; more;)
+                    more = round(std::integral_constant<int, 4>{}, std::integral_constant<int, kTile / 2>{});
             }
         }
     }
@@ -1017,34 +1027,22 @@ int lite_exact_pass(blsh_ctx *ctx, const uint2 *pairs, int64_t P, const long lon
             indptr, values, N, const_cast<long long *>(L.norm2), ctx->scratch);
         BLSH_LAUNCHED(ctx, "row_norm2_kernel");
     }
-    int occ = 0;
+    // (four CTAs an SM: their launch bounds' registers, and 55 KB of shared memory)
     const size_t smem = 8 * kLiteWarpWords * sizeof(uint32_t);
-    if (values) {
-        BLSH_CUDA(ctx, cudaFuncSetAttribute(lite_queue_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)smem));
-        BLSH_CUDA(ctx, cudaFuncSetAttribute(lite_exact_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)smem));
-        BLSH_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, lite_queue_kernel<true>, 256, smem));
+    const unsigned grid = 4u * ctx->sm_count;
+    auto run = [&](auto queue_kernel, auto exact_kernel) -> int {
+        BLSH_CUDA(ctx, cudaFuncSetAttribute(queue_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        BLSH_CUDA(ctx, cudaFuncSetAttribute(exact_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         blsh_time_start(ctx, s);
-        lite_queue_kernel<true><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L, queue, heavy);
+        queue_kernel<<<grid, 256, smem, s>>>(L, queue, heavy);
         BLSH_LAUNCHED(ctx, "lite_queue_kernel");
         blsh_time_start(ctx, s);
-        lite_exact_kernel<true><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L, heavy);
+        exact_kernel<<<grid, 256, smem, s>>>(L, heavy);
         BLSH_LAUNCHED(ctx, "lite_exact_kernel");
-    } else {
-        BLSH_CUDA(ctx, cudaFuncSetAttribute(lite_queue_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)smem));
-        BLSH_CUDA(ctx, cudaFuncSetAttribute(lite_exact_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)smem));
-        BLSH_CUDA(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, lite_queue_kernel<false>, 256, smem));
-        blsh_time_start(ctx, s);
-        lite_queue_kernel<false><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L, queue, heavy);
-        BLSH_LAUNCHED(ctx, "lite_queue_kernel");
-        blsh_time_start(ctx, s);
-        lite_exact_kernel<false><<<(occ > 0 ? occ : 1) * ctx->sm_count, 256, smem, s>>>(L, heavy);
-        BLSH_LAUNCHED(ctx, "lite_exact_kernel");
-    }
-    return BLSH_OK;
+        return BLSH_OK;
+    };
+    return values ? run(lite_queue_kernel<true>, lite_exact_kernel<true>)
+                  : run(lite_queue_kernel<false>, lite_exact_kernel<false>);
 }
 
 }  // namespace

@@ -83,3 +83,14 @@ def test_sums_past_the_limbs(B, ctx):
     x, y = np.triu_indices(40, 1)
     pairs = np.tile(np.stack([x, y], 1).astype(np.uint32), (200, 1))
     lite(B, ctx, csr, pairs, 1, 2, reserve=True)
+
+
+@pytest.mark.parametrize("kind", [0, 1])
+def test_rows_of_a_small_tile_one_by_one(B, ctx, kind):
+    """Survivors formed singly whose longer row is one tile of fewer than 128
+    elements and whose shorter one has up to 64, and just past both."""
+    csr = csr_of([1, 31, 33, 63, 64, 65, 96, 126, 127, 128, 129, 64, 65, 40], 200, 8, kind == 1)
+    x, y = np.triu_indices(csr.n, 1)
+    pairs = np.stack([x, y], 1).astype(np.uint32)
+    lite(B, ctx, csr, pairs, kind, 1)
+    lite(B, ctx, csr, np.tile(pairs, (400, 1)), kind)   # batches of them, no norms formed
