@@ -435,6 +435,7 @@ __device__ __forceinline__ unsigned long long f2_codes(uint32_t w) {
 // own before); 20,000 rows x 2,048 columns of floats (R of 820 MB) 607 us, now
 // 506 us + 54 us; 7,000 rows x 128 codes 33 us a call, 44 with three launches.
 constexpr int kSrpLongRow = 256;
+constexpr int kSrpLongMost = 1024;
 
 // Where a call's rows and columns lie, and its queues.
 struct SrpArgs {
@@ -443,12 +444,24 @@ struct SrpArgs {
     const float *values;
     long long N, dim;
     int bits, col_first, outer, inner;
+    int many;                  // (row, piece) items enough to fill the GPU several times
     const uint8_t *row_mask;   // rows to project (NULL: all)
     uint32_t *sig;
     blsh_dev_scratch *scratch;
     uint2 *queue;              // undecided signs, for srp_long_kernel
     unsigned long long *longs; // rows of more than kSrpLongRow nonzeros (BLSH_LITE_QUEUE_CAP of them)
 };
+
+// From how many nonzeros on a row is a CTA's: kSrpLongRow, but where there are
+// rows for every warp anyway, four times the average row, up to kSrpLongMost.  A
+// CTA's eight warps are half idle on a row of 300, and where most rows are as
+// long that is most of the work (20,000 rows of 200 on average x 1,024 columns,
+// R of 1,000 rows: 791 us with 256 for all, 677 here).
+__device__ __forceinline__ int srp_long_row(const SrpArgs &A) {
+    if (!A.many) return kSrpLongRow;
+    const float four = 4.0f * (float)(__ldg(A.indptr + A.N) - __ldg(A.indptr)) / (float)A.N;
+    return four > (float)kSrpLongMost ? kSrpLongMost : four > (float)kSrpLongRow ? (int)four : kSrpLongRow;
+}
 
 // A lane's CPL columns: their sums of a block, then of the row.
 template <typename RT, int CPL>
@@ -563,6 +576,7 @@ __global__ void __launch_bounds__(256, 4) srp_sparse4_kernel(const SrpArgs A, co
     const int lane = threadIdx.x & 31;
     const int words = A.bits >> 5;
     unsigned long long rechecked = 0, zeros = 0, bad = 0;
+    const int long_row = srp_long_row(A);
     const long long groups = (A.N + G - 1) / G;
     const unsigned long long items = (unsigned long long)groups * A.outer;
     for (;;) {
@@ -583,7 +597,7 @@ __global__ void __launch_bounds__(256, 4) srp_sparse4_kernel(const SrpArgs A, co
         if (lane < G && r0 + lane < A.N && (!A.row_mask || A.row_mask[r0 + lane])) {
             my_s = __ldg(A.indptr + r0 + lane);
             const long long len = __ldg(A.indptr + r0 + lane + 1) - my_s;
-            sel = len <= kSrpLongRow;
+            sel = len <= long_row;
             my_len = sel ? (int)len : 0;
             if (!sel && outer == 0) {
                 const unsigned long long slot = atomicAdd(&A.scratch->work3, 1ull);
@@ -773,6 +787,7 @@ __global__ void __launch_bounds__(256, 3) srp_long_kernel(const SrpArgs A, const
     const bool all = listed > BLSH_LITE_QUEUE_CAP;   // more than the list holds: every row is looked at
     const unsigned long long items = (all ? (unsigned long long)A.N : listed) * pieces;
     unsigned long long rechecked = 0, zeros = 0, bad = 0;
+    const int long_row = srp_long_row(A);
     for (;;) {
         __syncthreads();                              // the previous item and its sums have been read
         if (threadIdx.x == 0) s_item = atomicAdd(&A.scratch->work2, 1ull);
@@ -784,7 +799,7 @@ __global__ void __launch_bounds__(256, 3) srp_long_kernel(const SrpArgs A, const
         const long long row = (long long)(all ? q : A.longs[q]);
         if (all && A.row_mask && !A.row_mask[row]) continue;
         const long long s = __ldg(A.indptr + row), len = __ldg(A.indptr + row + 1) - s;
-        if (len <= kSrpLongRow) continue;
+        if (len <= long_row) continue;
         const int col0 = A.col_first + p * PC;
         const RT *Rc = R + col0 + CPL * lane;
         SrpCols<RT, CPL> c;
@@ -1087,6 +1102,7 @@ int srp_sparse_pieces(blsh_ctx *ctx, const int64_t *indptr, const uint32_t *indi
     const bool by_piece = (!row_mask && (double)dim * ncols * sizeof(RT) > 64e6) || N < 8 * warps;
     A.outer = by_piece ? pieces : 1;
     A.inner = by_piece ? 1 : pieces;
+    A.many = N * pieces >= 4 * warps && !row_mask;
     // rows a grab: up to 32, at least eight grabs a warp.  With a mask a grab may
     // hold few rows or none and the counter be most of the time (no row of
     // 100,000 left: 47 us, 13 so), so there a warp's first grab is all it takes

@@ -132,3 +132,32 @@ def test_an_empty_mask_costs_no_grabs(B, ctx):
         b.synchronize()
         times.append(a.elapsed_time(b) / 20)
     assert min(times) < 0.03, times
+
+
+@pytest.mark.parametrize("form", ["float", "codes"])
+@pytest.mark.parametrize("mean", [20, 150, 400])
+def test_long_rows_by_the_average(B, ctx, form, mean):
+    """20,000 rows, enough for every warp: a CTA's rows begin at four times the
+    average, at least 256 and at most 1,024."""
+    n, dim = 20_000, 4000
+    bits = 128 if form == "float" else 256
+    rng = np.random.default_rng(mean)
+    lens = np.full(n, mean)
+    edge = [255, 256, 257, 4 * mean - 2, 4 * mean - 1, 4 * mean, 4 * mean + 1, 4 * mean + 2, 1023, 1024, 1025, 3000, 0, 1]
+    lens[rng.choice(n, len(edge), replace=False)] = edge
+    indptr = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    csr = synth.CSR(indptr, rng.integers(0, dim, indptr[-1]).astype(np.uint32),
+                    rng.standard_normal(indptr[-1]).astype(np.float32), dim)
+    ip, val = torch.from_numpy(csr.indptr).to(dev), torch.from_numpy(csr.values).to(dev)
+    ix = torch.from_numpy(csr.indices.view(np.int32)).to(dev)
+    sig = torch.zeros((n, bits // 32), dtype=torch.int32, device=dev)
+    if form == "float":
+        R = synth.gaussian_matrix(dim, bits, seed=6)
+        B.blsh_srp_sparse(ctx, ip, ix, val, torch.from_numpy(R).to(dev), sig)
+        want = O.srp_sparse(csr, R)
+    else:
+        R = O.gaussian_codes(6, dim, bits)
+        B.blsh_srp_sparse_q16(ctx, ip, ix, val, torch.from_numpy(R.view(np.int16)).to(dev), sig)
+        want = O.srp_sparse_q16(csr, R)
+    assert B.blsh_status(ctx) == 0
+    assert np.array_equal(sig.cpu().numpy().view(np.uint32), want)
