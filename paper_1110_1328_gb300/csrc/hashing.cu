@@ -787,7 +787,6 @@ __global__ void __launch_bounds__(256, 3) srp_long_kernel(const SrpArgs A, const
     const bool all = listed > BLSH_LITE_QUEUE_CAP;   // more than the list holds: every row is looked at
     const unsigned long long items = (all ? (unsigned long long)A.N : listed) * pieces;
     unsigned long long rechecked = 0, zeros = 0, bad = 0;
-    const int long_row = srp_long_row(A);
     for (;;) {
         __syncthreads();                              // the previous item and its sums have been read
         if (threadIdx.x == 0) s_item = atomicAdd(&A.scratch->work2, 1ull);
@@ -799,7 +798,7 @@ __global__ void __launch_bounds__(256, 3) srp_long_kernel(const SrpArgs A, const
         const long long row = (long long)(all ? q : A.longs[q]);
         if (all && A.row_mask && !A.row_mask[row]) continue;
         const long long s = __ldg(A.indptr + row), len = __ldg(A.indptr + row + 1) - s;
-        if (len <= long_row) continue;
+        if (all && len <= srp_long_row(A)) continue;   // (a listed row is long)
         const int col0 = A.col_first + p * PC;
         const RT *Rc = R + col0 + CPL * lane;
         SrpCols<RT, CPL> c;
