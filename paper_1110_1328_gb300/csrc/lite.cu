@@ -979,7 +979,7 @@ extern "C" int blsh_verify_lite(blsh_ctx *ctx, const blsh_tables *tab, const uin
     A.lsim = nullptr;
     A.cap_levels = A.levels;
     A.need = nullptr;
-    const blsh_plan plan = blsh_plan_for(ctx, tab, P);
+    const blsh_plan plan = blsh_plan_for(ctx, tab, P, blsh_packed_outputs(pairs, status, n_used, nullptr, nullptr, nullptr));
     A.grab = (plan.grab + 31) / 32 * 32;
     int rc = blsh_launch_verify(ctx, A, plan, s);
     if (rc) return rc;
@@ -1077,7 +1077,8 @@ int verify_both(blsh_ctx *ctx, const blsh_tables *tab, int32_t hash_limit, const
     A.lsim = sim;
     A.cap_levels = hash_limit / p.k;
     A.need = need;
-    const blsh_plan plan = blsh_plan_for(ctx, tab, P);
+    const blsh_plan plan =
+        blsh_plan_for(ctx, tab, P, blsh_packed_outputs(pairs, status, n_used, m, lite_status, lite_n_used));
     A.grab = (plan.grab + 31) / 32 * 32;
     blsh_device_guard g(ctx->device);
     cudaStream_t s = blsh_stream(stream);

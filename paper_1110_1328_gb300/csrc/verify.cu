@@ -1267,9 +1267,8 @@ int dispatch(blsh_ctx *ctx, const VerifyArgs &A, const blsh_plan &plan, int kind
             // then the pairs Algorithm 1 leaves open (a few percent)
             if (!PERSIST && A.lite_levels <= 4 && (A.lite_levels == 0 || A.lite_levels <= A.levels)) {
                 // four pairs a lane where the outputs take the packed stores
-                const bool quad = A.P < (1ll << 31) && blsh_aligned(A.pairs, 16) && blsh_aligned(A.status, 4) &&
-                                  blsh_aligned(A.n_used, 8) && blsh_aligned(A.m_out, 8) &&
-                                  (!A.lite_levels || (blsh_aligned(A.lstatus, 4) && blsh_aligned(A.ln_used, 8)));
+                const bool quad = A.P < (1ll << 31) && blsh_packed_outputs(A.pairs, A.status, A.n_used, A.m_out, A.lstatus,
+                                                                           A.ln_used);
                 if (quad) {
                     // both passes in one kernel (verify_tile_kernel): one wave
                     // of resident CTAs, warps taking tiles from a counter
@@ -1325,15 +1324,19 @@ int dispatch(blsh_ctx *ctx, const VerifyArgs &A, const blsh_plan &plan, int kind
 // together, plain against persistent: 2.7e7 cosine pairs, k = 32: 240 against
 // 471 us, k = 64: 334 / 448, k = 128: 319 / 444; 6e5 pairs 54 / 58).  Cosine
 // calls over fewer than 65,536 pairs, where the two forms take the same time,
-// keep the persistent one.  Jaccard pairs take eight lanes a pair
+// keep the persistent one, and so do those with k = 32 whose outputs take no
+// packed stores (blsh_packed_outputs; the plain form is then two kernels) up to
+// 2^22 pairs: 3e5 pairs 31.9 us plain, 18.6 persistent; 3e6 62 / 55; 1e7 135 / 166.
+// Jaccard pairs take eight lanes a pair
 // (verify_sets_kernel: 1.4e7 pairs, k = 32: 269 us, four lanes a pair 428; 8e6
 // random ones 288 / 350, k = 64 490 / 715, k = 128 900 / 1,395; 5e5 pairs
 // 34 / 37), fewer than 2^18 of them four: the two take the same time there,
 // and where a few hundred pairs leave most warps idle a step of eight pairs is
 // shorter than one of 32 (176 pairs: 13 us, 20 with eight lanes).
-blsh_plan blsh_default_plan(int kind, long long P) {
+blsh_plan blsh_default_plan(int kind, int k, long long P, bool packed) {
     blsh_plan p;
-    p.mode = kind == BLSH_COSINE && P < 65536 ? BLSH_PLAN_PERSISTENT : BLSH_PLAN_PLAIN;
+    const long long persistent = kind != BLSH_COSINE ? 0 : k == 32 && !packed ? 1ll << 22 : 65536;
+    p.mode = P < persistent ? BLSH_PLAN_PERSISTENT : BLSH_PLAN_PLAIN;
     const bool few_sets = kind == BLSH_JACCARD && P < (1ll << 18);
     p.group = kind == BLSH_COSINE ? 1 : few_sets ? 4 : 8;
     p.block = few_sets ? 128 : 256;
@@ -1442,8 +1445,8 @@ int blsh_make_verify_args(blsh_ctx *ctx, const blsh_tables *tab, const uint32_t 
 // The plan the autotuner chose for these tables, else the default.  (A
 // plan stored for destroyed tables whose address was reused may not fit the
 // new tables' kind and k; the default is used then.)
-blsh_plan blsh_plan_for(blsh_ctx *ctx, const blsh_tables *tab, long long P) {
-    blsh_plan plan = blsh_default_plan(tab->p.kind, P);
+blsh_plan blsh_plan_for(blsh_ctx *ctx, const blsh_tables *tab, long long P, bool packed) {
+    blsh_plan plan = blsh_default_plan(tab->p.kind, tab->p.k, P, packed);
     std::lock_guard<std::mutex> lk(ctx->mu);
     auto it = ctx->plans.find(tab);
     if (it != ctx->plans.end() && blsh_check_plan(it->second, tab->p.kind, tab->p.k) == BLSH_OK) plan = it->second;
@@ -1474,7 +1477,7 @@ extern "C" int blsh_verify(blsh_ctx *ctx, const blsh_tables *tab, const uint32_t
                            uint8_t *status, uint16_t *n_used, uint16_t *m, float *est, uint64_t *stop_hist,
                            void *stream) {
     if (!ctx || !tab) return BLSH_EINVAL;
-    const blsh_plan plan = blsh_plan_for(ctx, tab, P);
+    const blsh_plan plan = blsh_plan_for(ctx, tab, P, blsh_packed_outputs(pairs, status, n_used, m, nullptr, nullptr));
     return blsh_verify_plan(ctx, tab, &plan, pairs, P, P_dev, sig, N, sig_words, status, n_used, m, est,
                             stop_hist, stream);
 }
@@ -1522,7 +1525,7 @@ int tune_plans(blsh_ctx *ctx, const blsh_tables *tab, const uint32_t *pairs, int
     BLSH_CUDA(ctx, cudaEventCreate(&e0));
     BLSH_CUDA(ctx, cudaEventCreate(&e1));
     float best_ms = 1e30f;
-    blsh_plan best_plan = blsh_default_plan(kind, P);
+    blsh_plan best_plan = blsh_default_plan(kind, tab->p.k, P, true);
     int rc = BLSH_OK;
     for (const blsh_plan &p : cands) {
         rc = blsh_verify_plan(ctx, tab, &p, pairs, P, nullptr, sig, N, sig_words, status, n_used, m, est,
@@ -1581,7 +1584,7 @@ extern "C" int blsh_autotune_k(blsh_ctx *ctx, const blsh_params *params, const i
             return blsh_fail(ctx, BLSH_EINVAL, "chunk size %d: not 32, 64 or 128, or not dividing n_max", ks[i]);
     blsh_device_guard g(ctx->device);
     blsh_tables *best_tab = nullptr;
-    blsh_plan best_plan = blsh_default_plan(params->kind, P);
+    blsh_plan best_plan = blsh_default_plan(params->kind, params->k, P, true);
     float best_ms = 1e30f;
     int rc = BLSH_OK;
     for (int i = 0; i < n_ks && rc == BLSH_OK; ++i) {

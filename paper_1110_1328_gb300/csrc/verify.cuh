@@ -56,9 +56,17 @@ struct VerifyArgs {
 // those computed so far (blsh_verify_resume finishes it).
 
 int blsh_launch_verify(blsh_ctx *ctx, const VerifyArgs &A, const blsh_plan &plan, cudaStream_t s);
-blsh_plan blsh_default_plan(int kind, long long P);
+blsh_plan blsh_default_plan(int kind, int k, long long P, bool packed);
 int blsh_check_plan(const blsh_plan &plan, int kind, int k);
 int blsh_make_verify_args(blsh_ctx *ctx, const blsh_tables *tab, const uint32_t *pairs, int64_t P,
                           const int64_t *P_dev, const uint32_t *sig, int64_t N, int32_t sig_words, uint8_t *status,
                           uint16_t *n_used, uint16_t *m, float *est, uint64_t *stop_hist, VerifyArgs &A);
-blsh_plan blsh_plan_for(blsh_ctx *ctx, const blsh_tables *tab, long long P);
+blsh_plan blsh_plan_for(blsh_ctx *ctx, const blsh_tables *tab, long long P, bool packed);
+
+// Whether four consecutive pairs' indices and outputs can be read and stored
+// together (NULL outputs are not written).
+inline bool blsh_packed_outputs(const void *pairs, const void *status, const void *n_used, const void *m,
+                                const void *lstatus, const void *ln_used) {
+    return blsh_aligned(pairs, 16) && blsh_aligned(status, 4) && blsh_aligned(n_used, 8) && blsh_aligned(m, 8) &&
+           blsh_aligned(lstatus, 4) && blsh_aligned(ln_used, 8);
+}
