@@ -961,15 +961,17 @@ __global__ void __launch_bounds__(256) gaussian_codes_kernel(unsigned long long 
 // three 16-byte shared loads, and R is read from L2 once per 64 rows; the
 // former kernel (one row per CTA, R streamed from L2 for every row, a second
 // FMA per product for the error bound) was bound by those reads: 99,991 x 300
-// x 1,024 bits took 36.4 ms, 2.69 ms here; 1,659 x 100 x 512 bits 208 us, 34 us here.
+// x 1,024 bits took 36.4 ms, 2.61 ms here; 1,659 x 100 x 512 bits 208 us, 29 us here.
 //
 // Error bound: a stage's chain of at most 32 FMAs, then the stage totals
 // added in order, so no product passes through more than 32 + ceil(d/32)
 // roundings, and sum|x_i r_ij| <= |x| |r_j| (norms formed from the staged
 // values, every operation rounded up): a sum of magnitude above 1.25 times
 // that many u |x| |r_j| (plus the underflow terms) has the sign of the exact
-// sum.  The others, about 1 in 10^4, are summed in FP64 over coordinates
-// 0..d-1 in order, which is the definition.
+// sum.  The others, about 1 in 10^4, are listed and summed in FP64 over
+// coordinates 0..d-1 in order, which is the definition, a thread each: where a
+// tenth of the sums are ties (rows of +-1, 100 x 64 x 128 bits) a lane summing
+// its own took 223 us, 35 so.  Zero rows and columns need no sum.
 constexpr int kSimtK = 32;
 constexpr int kSimtCols = 128;
 
@@ -981,6 +983,7 @@ __global__ void __launch_bounds__(256) srp_dense_simt_kernel(const float *__rest
     __shared__ __align__(16) float xs[kSimtK][ROWS + 4];      // [k][row]
     __shared__ __align__(16) float rs[kSimtK][kSimtCols];
     __shared__ float xn[ROWS], rn[kSimtCols];
+    __shared__ int s_open;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const long long rt = blockIdx.x / col_tiles;
     const int j0 = (int)(blockIdx.x - rt * col_tiles) * kSimtCols;
@@ -992,46 +995,52 @@ __global__ void __launch_bounds__(256) srp_dense_simt_kernel(const float *__rest
 #pragma unroll
         for (int c = 0; c < 4; ++c) tot[i][c] = 0.0f;
     float nrm = 0.0f;   // threads 0 .. ROWS-1: their row's squared norm; 128 .. 255: their column's
+    if (t == 0) s_open = 0;
     for (int k0 = 0; k0 < d; k0 += kSimtK) {
+        const int kn = d - k0 < kSimtK ? (d - k0 + 7) & ~7 : kSimtK;   // (whole eights: the loops below)
         __syncthreads();
-        for (int r = w; r < ROWS; r += 8) {
-            const long long row = row0 + r;
-            xs[lane][r] = row < N && k0 + lane < d ? __ldg(X + (size_t)row * d + k0 + lane) : 0.0f;
-        }
-        for (int i = t; i < kSimtK * kSimtCols; i += 256) {
+        if (lane < kn)
+            for (int r = w; r < ROWS; r += 8) {
+                const long long row = row0 + r;
+                xs[lane][r] = row < N && k0 + lane < d ? __ldg(X + (size_t)row * d + k0 + lane) : 0.0f;
+            }
+        for (int i = t; i < kn * kSimtCols; i += 256) {
             const int k = i / kSimtCols, c = i % kSimtCols;
             rs[k][c] = k0 + k < d && c < ncols ? __ldg(R + (size_t)(k0 + k) * bits + j0 + c) : 0.0f;
         }
         __syncthreads();
         if (t < ROWS) {
+            for (int k8 = 0; k8 < kn; k8 += 8)
 #pragma unroll
-            for (int k = 0; k < kSimtK; ++k) nrm = __fmaf_ru(xs[k][t], xs[k][t], nrm);
+                for (int k = k8; k < k8 + 8; ++k) nrm = __fmaf_ru(xs[k][t], xs[k][t], nrm);
         } else if (t >= 128) {
+            for (int k8 = 0; k8 < kn; k8 += 8)
 #pragma unroll
-            for (int k = 0; k < kSimtK; ++k) nrm = __fmaf_ru(rs[k][t - 128], rs[k][t - 128], nrm);
+                for (int k = k8; k < k8 + 8; ++k) nrm = __fmaf_ru(rs[k][t - 128], rs[k][t - 128], nrm);
         }
         float acc[RT][4];
 #pragma unroll
         for (int i = 0; i < RT; ++i)
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[i][c] = 0.0f;
-#pragma unroll 8
-        for (int k = 0; k < kSimtK; ++k) {
-            const float4 r = *reinterpret_cast<const float4 *>(&rs[k][4 * lane]);
-            float x[RT];
+        for (int k8 = 0; k8 < kn; k8 += 8)
 #pragma unroll
-            for (int i = 0; i < RT; i += 4) {
-                const float4 v = *reinterpret_cast<const float4 *>(&xs[k][RT * w + i]);
-                x[i] = v.x; x[i + 1] = v.y; x[i + 2] = v.z; x[i + 3] = v.w;
-            }
+            for (int k = k8; k < k8 + 8; ++k) {
+                const float4 r = *reinterpret_cast<const float4 *>(&rs[k][4 * lane]);
+                float x[RT];
 #pragma unroll
-            for (int i = 0; i < RT; ++i) {
-                acc[i][0] = __fmaf_rn(x[i], r.x, acc[i][0]);
-                acc[i][1] = __fmaf_rn(x[i], r.y, acc[i][1]);
-                acc[i][2] = __fmaf_rn(x[i], r.z, acc[i][2]);
-                acc[i][3] = __fmaf_rn(x[i], r.w, acc[i][3]);
+                for (int i = 0; i < RT; i += 4) {
+                    const float4 v = *reinterpret_cast<const float4 *>(&xs[k][RT * w + i]);
+                    x[i] = v.x; x[i + 1] = v.y; x[i + 2] = v.z; x[i + 3] = v.w;
+                }
+#pragma unroll
+                for (int i = 0; i < RT; ++i) {
+                    acc[i][0] = __fmaf_rn(x[i], r.x, acc[i][0]);
+                    acc[i][1] = __fmaf_rn(x[i], r.y, acc[i][1]);
+                    acc[i][2] = __fmaf_rn(x[i], r.z, acc[i][2]);
+                    acc[i][3] = __fmaf_rn(x[i], r.w, acc[i][3]);
+                }
             }
-        }
 #pragma unroll
         for (int i = 0; i < RT; ++i)
 #pragma unroll
@@ -1044,32 +1053,68 @@ __global__ void __launch_bounds__(256) srp_dense_simt_kernel(const float *__rest
     const float u = 1.25f * (float)(kSimtK + (d + kSimtK - 1) / kSimtK) * 5.9604644775390625e-8f;
     const float tiny = (float)d * 2.9e-45f;
     const bool loose = (float)d * 5.9604644775390625e-8f > 0.05f;   // the 1.25 slack needs d u <= 0.05
+    // the decided bits into shared memory, the open signs (row of the tile << 7 |
+    // column) into a list there: one sum a thread, so that rows of ties are not
+    // one lane's sixteen or thirty-two sums one after the other
+    auto s_bits = reinterpret_cast<uint32_t(*)[kSimtCols / 32]>(&xs[0][0]);   // [ROWS][4]
+    uint16_t *s_list = reinterpret_cast<uint16_t *>(&rs[0][0]);               // [ROWS * 128]
+    static_assert(ROWS * kSimtCols * sizeof(uint16_t) <= sizeof(rs) && ROWS * 16 <= sizeof(xs), "the stage's place");
+    uint32_t open = 0;   // bit 4 i + c
     unsigned long long rechecked = 0, zeros = 0;
 #pragma unroll
     for (int i = 0; i < RT; ++i) {
         const long long row = row0 + RT * w + i;
-        const float ux = u * xn[RT * w + i];
+        const float xi = xn[RT * w + i], ux = u * xi;
         uint32_t nib = 0;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
             const int col = 4 * lane + c;
-            bool bit = tot[i][c] >= 0.0f;
-            if (row < N && col < ncols && (loose || !(fabsf(tot[i][c]) > ux * rn[col] + tiny))) {
-                double dd = 0.0;
-                for (int k = 0; k < d; ++k)
-                    dd += (double)__ldg(X + (size_t)row * d + k) * (double)__ldg(R + (size_t)k * bits + j0 + col);
-                bit = dd >= 0.0;
-                ++rechecked;
-                zeros += dd == 0.0;
+            const bool decided = !loose && fabsf(tot[i][c]) > ux * rn[col] + tiny;
+            // (zeros against finite values: every product is zero; no square is lost in the norms)
+            const bool zero = xi * rn[col] == 0.0f && (xi == 0.0f || rn[col] == 0.0f);
+            if (row < N && col < ncols && !decided) {
+                if (zero) ++zeros;
+                else open |= 1u << (4 * i + c);
             }
-            nib |= (uint32_t)bit << c;
+            nib |= (uint32_t)(zero || (decided && tot[i][c] >= 0.0f)) << c;
         }
         // eight lanes' nibbles form a word
         uint32_t word = nib << (4 * (lane & 7));
         word |= __shfl_xor_sync(kFull, word, 1);
         word |= __shfl_xor_sync(kFull, word, 2);
         word |= __shfl_xor_sync(kFull, word, 4);
-        if ((lane & 7) == 0 && row < N && 4 * lane < ncols) sig[(size_t)row * words + (j0 >> 5) + (lane >> 3)] = word;
+        if ((lane & 7) == 0) s_bits[RT * w + i][lane >> 3] = word;
+    }
+    const int mine = __popc(open);
+    int before = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(kFull, before, o);
+        if (lane >= o) before += y;
+    }
+    int at = 0;
+    if (lane == 31 && before) at = atomicAdd(&s_open, before);
+    at = __shfl_sync(kFull, at, 31) + before - mine;
+    for (; open; open &= open - 1) {
+        const int b = __ffs(open) - 1;
+        s_list[at++] = (uint16_t)((RT * w + (b >> 2)) << 7 | (4 * lane + (b & 3)));
+    }
+    __syncthreads();
+    rechecked = zeros;
+    for (int e = t; e < s_open; e += 256) {
+        const int r = s_list[e] >> 7, col = s_list[e] & 127;
+        const float *x = X + (size_t)(row0 + r) * d, *rc = R + j0 + col;
+        double dd = 0.0;
+#pragma unroll 4
+        for (int k = 0; k < d; ++k) dd += (double)__ldg(x + k) * (double)__ldg(rc + (size_t)k * bits);
+        if (dd >= 0.0) atomicOr(&s_bits[r][col >> 5], 1u << (col & 31));
+        ++rechecked;
+        zeros += dd == 0.0;
+    }
+    __syncthreads();
+    for (int i = t; i < ROWS * (kSimtCols / 32); i += 256) {
+        const int r = i >> 2, q = i & 3;
+        if (row0 + r < N && 32 * q < ncols) sig[(size_t)(row0 + r) * words + (j0 >> 5) + q] = s_bits[r][q];
     }
     if (rechecked) atomicAdd(&scratch->counters[2], rechecked);
     if (zeros) atomicAdd(&scratch->counters[3], zeros);

@@ -458,6 +458,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) srp_dense_tc_persistent(
 //   same in every order;
 //   the rest, exact ties, as the FP64 sum over coordinates 0..d-1 in order --
 //   exactly the oracle's sum -- a lane each.  A zero row's sums need no FP64.
+//   Three open signs or more among eight are taken for ties at once: the middle
+//   stages, the warp's for every sign, cost 3 to 5 us each where a lane's sum
+//   costs 2 us for 32 of them (100 x 64 x 256 bits of +-1, a tenth ties: 846 us,
+//   75 here).
 //
 // What bounds it: the reads of the columns, 4 d bytes a sign, from L2 and L1.
 // A queue of (row, bit) entries, eight lanes each, read x_i as well for every
@@ -563,7 +567,10 @@ __global__ void __launch_bounds__(32 * kReWarps, 1) srp_dense_recheck_kernel(con
         const long long row = g * rows + wrow;
         return g < groups && row < A.N ? __ldcs(A.und + (size_t)row * words + wword) : 0u;
     };
-    long long g = (long long)(blockIdx.x / parts) * kReWarps + warp;
+    // no more items than warps: in as many CTAs as can be; else a CTA's follow
+    // each other (spread over the CTAs 1e5 x 300 x 1,024 bits took 137 us, 131 so)
+    const long long ctas = gridDim.x / parts, cta = blockIdx.x / parts;
+    long long g = groups <= ctas * kReWarps ? (long long)warp * ctas + cta : cta * kReWarps + warp;
     uint32_t next = marks(g);
     for (; g < groups; g += stride) {
         const uint32_t u = next;
@@ -677,11 +684,13 @@ __global__ void __launch_bounds__(32 * kReWarps, 1) srp_dense_recheck_kernel(con
                     const unsigned open = __ballot_sync(kFull, lead && !(fabsf(s) > xb * my_rn + tiny));
                     if (open) {
                         if (zero_row && s == 0.0f) zeros += lead;
-                        for (unsigned o = __ballot_sync(kFull, (open >> lane & 1u) && !(zero_row && s == 0.0f)); o; o &= o - 1) {
+                        unsigned o = __ballot_sync(kFull, (open >> lane & 1u) && !(zero_row && s == 0.0f));
+                        for (const bool ties_likely = __popc(o) > 2; o; o &= o - 1) {
                             const int from = __ffs(o) - 1, c = __shfl_sync(kFull, my_col, from);
                             bool zero = false;
-                            const int sg = sign_by_magnitude<VEC>(x, Rt + (size_t)c * ldr, d, ldr,
-                                                                  __shfl_sync(kFull, s, from), roundings, &zero);
+                            const int sg = ties_likely ? 0
+                                                       : sign_by_magnitude<VEC>(x, Rt + (size_t)c * ldr, d, ldr,
+                                                                                __shfl_sync(kFull, s, from), roundings, &zero);
                             if (lane == from) {
                                 bit = sg > 0;
                                 zeros += zero;
@@ -799,9 +808,9 @@ extern "C" int blsh_srp_dense(blsh_ctx *ctx, const float *X, int64_t N, int32_t 
     const int part_words = bits % 1024 == 0 ? 32 : bits % 512 == 0 ? 16 : 8, parts = bits / (32 * part_words);
     const RecheckArgs A = {und, X, (const float *)(ws + L.rt), (const float *)(ws + L.xn), (const float *)(ws + L.rn), N,
                            d, KT * BK, bits, part_words, sig, ctx->scratch};
-    const long long groups = (N * part_words + 31) / 32, share = (groups + kReWarps - 1) / kReWarps;
+    const long long groups = (N * part_words + 31) / 32;
     const long long copies = ctx->sm_count / parts > 0 ? ctx->sm_count / parts : 1;   // CTAs a part
-    const unsigned re_grid = (unsigned)((share < copies ? share : copies) * parts);
+    const unsigned re_grid = (unsigned)((groups < copies ? groups : copies) * parts);
     if (d <= 256)
         (vec ? srp_dense_recheck_kernel<true, true> : srp_dense_recheck_kernel<false, true>)<<<re_grid, 32 * kReWarps, 0,
                                                                                              s>>>(A);
