@@ -121,9 +121,10 @@ __global__ void __launch_bounds__(1024) scan_small(const T *in, T *out, int n, T
     if (threadIdx.x == 0 && grand) *grand = carry;
 }
 
-// Up to this many entries one CTA scans in less time than three launches take
-// (about 1.5 us per 8,192 entries against 12 to 14 us).
-constexpr long long kSmallScan = 32768;
+// Up to this many entries one CTA scans in less time than three launches take:
+// 8,192 entries of 4 bytes 8.3 us against 12.3, of 8 bytes 10.3 / 13.4; 16,384
+// entries 14.5 / 12.3 and 16.5 / 13.4, 32,768 26.7 / 12.3 and 30.8 / 14.4.
+constexpr long long kSmallScan = 8192;
 
 inline long long tiles_for(long long n) { return (n + kTile - 1) / kTile; }
 
@@ -152,7 +153,7 @@ int run(blsh_ctx *ctx, const T *in, T *out, long long n, T *partial, T *grand, c
     blsh_time_start(ctx, s);
     BLSH_CUDA(ctx, exclusive_scan<T>(in, out, n, partial, grand, s, &launches));
     ctx->launches.fetch_add(launches, std::memory_order_relaxed);
-    blsh_time_stop(ctx, "exclusive scan (3 launches)");
+    blsh_time_stop(ctx, "exclusive scan");
     return BLSH_OK;
 }
 

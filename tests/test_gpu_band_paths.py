@@ -124,3 +124,18 @@ def test_long_bucket_past_a_band_edge(B, ctx, N, kind, rows, band):
     assert len(got) == len(want) and np.array_equal(np.sort(packed(got)), np.sort(packed(want)))
     for rec in (0, 8 * N):
         assert np.array_equal(candidates(B, ctx, sig, kind, rows, 3, rec), got)
+
+
+def test_scan_in_one_launch_up_to_8192_entries(B, ctx):
+    """The pairs' offsets are a scan of one entry per 32 positions: one launch up
+    to 8,192 of them, three from 8,193 on (all else is the same)."""
+    launches = []
+    for N in (32_768, 32_769):
+        sig = torch.from_numpy(np.random.default_rng(N).integers(0, 1 << 31, (N, 4)).astype(np.int32)).to(dev)
+        ws = torch.empty(B.blsh_lsh_candidates_workspace(N, 1, 16, 8), dtype=torch.uint8, device=dev)
+        n = torch.zeros(1, dtype=torch.int64, device=dev)
+        before = B.blsh_launch_count(ctx)
+        B.blsh_lsh_candidates(ctx, sig, 1, 16, 8, None, n, ws)
+        launches.append(B.blsh_launch_count(ctx) - before)
+        assert B.blsh_status(ctx) == B.ETRUNC and int(n) > 0
+    assert launches[1] - launches[0] == 2
