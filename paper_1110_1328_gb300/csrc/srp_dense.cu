@@ -604,6 +604,15 @@ __global__ void __launch_bounds__(32 * kReWarps, 1) srp_dense_recheck_kernel(con
                 u1 = x_pairs<VEC, true>(x, 128 + 4 * lane, d);
                 zero_row = !__any_sync(kFull, ((u0.x | u0.y | u1.x | u1.y) & kAbs) != 0);
             }
+            if (REG && zero_row) {   // against a column of finite values: zero, and not summed (a third of 1e5 x 256: 3.55 ms, 0.29 so)
+                uint32_t zero = 0;
+                for (uint32_t b = m; b; b &= b - 1)
+                    if (__ldg(rn + (lane % W) * 32 + __ffs(b) - 1) < INFINITY) zero |= b & (0u - b);
+                zeros += __popc(zero);
+                if (zero) atomicOr(&bits[l * W + lane % W], zero);
+                m &= ~zero;
+                if (!__any_sync(kFull, m != 0)) continue;
+            }
             const float xb = 1.25f * roundings * 5.9604644775390625e-8f * __ldg(A.xnorm + row);
             do {
                 int hi = 0;
