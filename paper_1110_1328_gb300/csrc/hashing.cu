@@ -80,7 +80,7 @@ __device__ __forceinline__ void min_hash_run(const uint32_t *__restrict__ indice
 constexpr long long kBigSet = 256;
 constexpr long long kHubSet = 2048;
 constexpr int kListShift = 36;          // 2^36 blocks and 2^28 entries: more than 280 GB of elements
-constexpr unsigned kPartBlocks = 8;     // blocks of a list a warp takes, at least
+constexpr unsigned kPartBlocks = 4;     // blocks of a list a warp takes, at least
 constexpr uint32_t kListed = 0xffffffffu, kUnlisted = 0xfffffffeu;
 
 struct LongSets {
