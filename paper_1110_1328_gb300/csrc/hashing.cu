@@ -437,6 +437,12 @@ __device__ __forceinline__ unsigned long long f2_codes(uint32_t w) {
 constexpr int kSrpLongRow = 256;
 constexpr int kSrpLongMost = 1024;
 
+// The items' counters, 256 bytes apart in the context's scratch area.
+constexpr unsigned kSrpCounters = 8;
+__host__ __device__ __forceinline__ unsigned long long *srp_counter(blsh_dev_scratch *s, unsigned c) {
+    return reinterpret_cast<unsigned long long *>(s->cta_counts) + 32 * c;
+}
+
 // Where a call's rows and columns lie, and its queues.
 struct SrpArgs {
     const int64_t *indptr;
@@ -567,9 +573,12 @@ __device__ __forceinline__ bool srp_undecided(const SrpArgs &A, const RT *R, lon
     return d >= 0.0;
 }
 
-// ONCE: no more items than warps, a warp's is that of its number (the counter
-// takes about 0.9 ns a grab, the last and vain one of every warp included).
-template <typename RT, int CPL, bool ONCE>
+// GRABS 0: no more items than warps, a warp's is that of its number.  1: items
+// from a counter.  8: counter c hands out items c, c + 8, ...  One counter takes
+// about 0.9 ns a grab, the last and vain one of every warp included, which had
+// been most of a masked call over 20,000 to 100,000 rows; rows that are all
+// projected hide it (and the eight counters' addresses cost 3% there).
+template <typename RT, int CPL, int GRABS>
 __global__ void __launch_bounds__(256, 4) srp_sparse4_kernel(const SrpArgs A, const RT *__restrict__ R, int G) {
     constexpr bool Q16 = sizeof(RT) == 2;
     constexpr int PC = 32 * CPL;   // columns of a piece
@@ -581,10 +590,13 @@ __global__ void __launch_bounds__(256, 4) srp_sparse4_kernel(const SrpArgs A, co
     const unsigned long long items = (unsigned long long)groups * A.outer;
     for (;;) {
         unsigned long long item = 0;
-        if constexpr (ONCE) {
+        if constexpr (GRABS == 0) {
             item = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-        } else {
+        } else if constexpr (GRABS == 1) {
             if (lane == 0) item = atomicAdd(&A.scratch->hash_work, 1ull);
+            item = __shfl_sync(kFull, item, 0);
+        } else {
+            if (lane == 0) item = GRABS * atomicAdd(srp_counter(A.scratch, blockIdx.x % GRABS), 1ull) + blockIdx.x % GRABS;
             item = __shfl_sync(kFull, item, 0);
         }
         if (item >= items) break;
@@ -698,7 +710,7 @@ __global__ void __launch_bounds__(256, 4) srp_sparse4_kernel(const SrpArgs A, co
                     A.sig[(size_t)row * words + (col0 >> 5) + lane / (32 / CPL)] = word;
             }
         }
-        if constexpr (ONCE) break;
+        if constexpr (GRABS == 0) break;
     }
     if (bad) blsh_dev_error(A.scratch, BLSH_ERANGE, 0, bad);
     if (rechecked) atomicAdd(&A.scratch->counters[2], rechecked);
@@ -787,7 +799,7 @@ __global__ void __launch_bounds__(256, 3) srp_long_kernel(const SrpArgs A, const
     const bool all = listed > BLSH_LITE_QUEUE_CAP;   // more than the list holds: every row is looked at
     const unsigned long long items = (all ? (unsigned long long)A.N : listed) * pieces;
     unsigned long long rechecked = 0, zeros = 0, bad = 0;
-    for (;;) {
+    while (items > 0) {                               // (no grab where no row is long)
         __syncthreads();                              // the previous item and its sums have been read
         if (threadIdx.x == 0) s_item = atomicAdd(&A.scratch->work2, 1ull);
         __syncthreads();
@@ -1147,23 +1159,21 @@ int srp_sparse_pieces(blsh_ctx *ctx, const int64_t *indptr, const uint32_t *indi
     A.outer = by_piece ? pieces : 1;
     A.inner = by_piece ? 1 : pieces;
     A.many = N * pieces >= 4 * warps && !row_mask;
-    // rows a grab: up to 32, at least eight grabs a warp.  With a mask a grab may
-    // hold few rows or none and the counter be most of the time (no row of
-    // 100,000 left: 47 us, 13 so), so there a warp's first grab is all it takes
-    // while that is at most 32 rows.
+    // rows a grab: up to 32, about eight grabs a warp, four where a mask may leave
+    // them next to nothing
+    const long long grabs = (row_mask ? 4 : 8) * warps;
     int G = 32;
-    if (row_mask) G = (int)((N * A.outer + warps - 1) / warps < 32 ? (N * A.outer + warps - 1) / warps : 32);
-    else
-        while (G > 1 && (N / G) * A.outer < 8 * warps) G >>= 1;
+    while (G > 1 && (N / G) * A.outer < grabs) G >>= 1;
     blsh_dev_scratch *scr = ctx->scratch;
-    // work2 (next long row), work3 (long rows listed), recheck_count .. hash_work
-    BLSH_CUDA(ctx, cudaMemsetAsync(&scr->work2, 0, offsetof(blsh_dev_scratch, norm2_valid) -
-                                                       offsetof(blsh_dev_scratch, work2), s));
+    // work2 (next long row), work3 (long rows listed), recheck_count .. the items' counters
+    BLSH_CUDA(ctx, cudaMemsetAsync(&scr->work2, 0, (char *)(srp_counter(scr, kSrpCounters - 1) + 1) - (char *)&scr->work2, s));
     const char *name = sizeof(RT) == 2 ? "srp_sparse4_kernel (two-byte codes)" : "srp_sparse4_kernel";
     const long long items = (N + G - 1) / G * A.outer, blocks = (items + 7) / 8, most = (long long)ctx->sm_count * 8;
     blsh_time_start(ctx, s);
-    if (items <= 2 * warps) srp_sparse4_kernel<RT, CPL, true><<<(unsigned)blocks, 256, 0, s>>>(A, R, G);
-    else srp_sparse4_kernel<RT, CPL, false><<<(unsigned)(blocks < most ? blocks : most), 256, 0, s>>>(A, R, G);
+    const unsigned grid = (unsigned)(blocks < most ? blocks : most);
+    if (items <= warps) srp_sparse4_kernel<RT, CPL, 0><<<grid, 256, 0, s>>>(A, R, G);
+    else if (!row_mask) srp_sparse4_kernel<RT, CPL, 1><<<grid, 256, 0, s>>>(A, R, G);
+    else srp_sparse4_kernel<RT, CPL, (int)kSrpCounters><<<grid, 256, 0, s>>>(A, R, G);
     BLSH_LAUNCHED(ctx, name);
     blsh_time_start(ctx, s);
     srp_long_kernel<RT, CPL><<<ctx->sm_count * 3, 256, 0, s>>>(A, R);
