@@ -163,7 +163,9 @@ BLSH_API int64_t blsh_launch_count(const blsh_ctx *ctx);
  * blsh_timing_end waits for the recorded stop events, writes up to `max`
  * records in launch order -- names[i] = the kernel's name (a static string
  * owned by the library; a multi-launch helper such as the exclusive scan
- * is one record), ms[i] = its device time in milliseconds -- sets *n to the
+ * is one record, and the forms of one pass, or a kernel and the one that
+ * finishes its long rows and rechecks, go by one name, so that a pass's
+ * time is the sum over its name), ms[i] = its device time in milliseconds -- sets *n to the
  * number written, releases the events and switches recording off.
  * Errors: BLSH_EINVAL for max_launches outside 1..65536 or missing outputs;
  * BLSH_EDEVICE if an event could not be created or read (recording is then

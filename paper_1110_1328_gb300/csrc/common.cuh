@@ -16,8 +16,8 @@
 
 #define BLSH_MAX_NMAX 4096
 #define BLSH_COMPACT_MAX_CTAS 2048
-#define BLSH_RECHECK_CAP (1u << 20)   // queued SRP sign rechecks per call (8 MiB per context)
-#define BLSH_LITE_QUEUE_CAP (1u << 23) // queued Lite survivors per call (64 MiB per context)
+#define BLSH_RECHECK_CAP (1u << 20)    // entries of the context's small queue (8 MiB)
+#define BLSH_LITE_QUEUE_CAP (1u << 23) // entries of its large one (64 MiB)
 
 // Device-side scratch owned by a context.  Every call zeroes what it uses
 // before its kernels run (cudaMemsetAsync on the caller's stream).
@@ -25,14 +25,14 @@ struct blsh_dev_scratch {
     unsigned int err_code;             // first device-detected error (0 = none)
     unsigned int pad0;
     unsigned long long counters[4];    // bad pairs, truncations, SRP rechecks, SRP zeros
-    unsigned long long work;           // verify: next pair handed out
-    unsigned long long work2;          // lite: next survivor tile handed out
-    unsigned long long work3;          // lite: survivors queued
-    unsigned long long recheck_count;  // SRP: signs queued for an FP64 recheck
+    unsigned long long work;           // verify, lite: next pair, batch; minhash: next part of the hubs
+    unsigned long long work2;          // lite: next survivor tile; sparse projection: next long row; minhash: next part
+    unsigned long long work3;          // entries of the large queue: survivors, long rows, long sets
+    unsigned long long recheck_count;  // entries of the small queue: signs to recheck, pairs of long rows, hubs
     unsigned long long band_work[8];   // banding: next item of each emission pass, record words used, tasks
-    unsigned long long hash_work;      // sparse projection: next (row, piece) item handed out
+    unsigned long long hash_work;      // sparse projection: next (row, piece) item; lite: next pair of long rows
     unsigned int norm2_valid;          // Lite: the rows' squared norms were formed for this call
-    long long cta_counts[BLSH_COMPACT_MAX_CTAS];  // compaction: kept items per CTA
+    long long cta_counts[BLSH_COMPACT_MAX_CTAS];  // compaction: kept items per CTA; masked projections: the items' counters
 };
 
 struct blsh_ctx {
@@ -41,8 +41,11 @@ struct blsh_ctx {
     int cc_major = 0, cc_minor = 0;
     size_t smem_optin = 0;
     blsh_dev_scratch *scratch = nullptr;
-    uint2 *recheck_queue = nullptr;                   // [BLSH_RECHECK_CAP] (row, bit) of undecided SRP signs
-    unsigned long long *lite_queue = nullptr;         // [BLSH_LITE_QUEUE_CAP] Lite survivors (pair indices)
+    // queues of a call's own work, each used by one call at a time
+    uint2 *recheck_queue = nullptr;                   // [BLSH_RECHECK_CAP] undecided signs (row, bit); Lite's pairs of
+                                                      // long rows; minhash's hubs (set, blocks before)
+    unsigned long long *lite_queue = nullptr;         // [BLSH_LITE_QUEUE_CAP] Lite's survivors (pair indices); the sparse
+                                                      // projection's long rows; minhash's other long sets
     // per-object buffers, sized by blsh_ctx_reserve (never by a hot call)
     void *plane = nullptr;                            // verification: [plane_cap] first four words of each row
     long long plane_cap = 0;

@@ -1292,6 +1292,8 @@ int blsh_srp_dense_simt(blsh_ctx *ctx, const float *X, int64_t N, int32_t d, con
                         uint32_t *sig, cudaStream_t s) {
     int per_thread = 0;
     srp_threads(bits, &per_thread);
+    // (the tiles could form either; the refusals are the entry point's: the sparse
+    // projections take no such width, and rows have always been limited to 58,112 coordinates)
     if (per_thread > kSrpMaxPerThread) return blsh_fail(ctx, BLSH_EINVAL, "bits/32 needs a divisor in 2..8");
     if (sizeof(float) * (size_t)d > ctx->smem_optin) return blsh_fail(ctx, BLSH_EINVAL, "d too large");
     // 64-row tiles where they give every SM at least two, else 32-row ones

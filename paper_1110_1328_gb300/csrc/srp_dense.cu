@@ -24,7 +24,12 @@
 // The error of step 2 is at most 3.1 * 2^-16 sum|x_i r_ij| from the split
 // plus the FP32 accumulation of 3 Kpad products; the rigorous margin used when
 // the caller passes margin <= 0 is (2^-14 + 3 Kpad 2^-22) * 1.25, applied to
-// |x| |r| >= sum|x_i r_ij|.
+// |x| |r| >= sum|x_i r_ij|.  That the accumulation errs by less than 2^-22 a
+// product is taken from measurement, not from a document: over widths of 1 to
+// 4,096 and Gaussian, one-signed, widely spread and outlying values the
+// accumulators differ from the FP64 products by at most 0.20 of the margin (one
+// coordinate: 2.7e-5 of 1.34e-4, the split), 0.06 at 64, 0.01 from 300 on (4,096
+// one-signed ones: 1.9e-5 of 3.7e-3), and every sign is that of the FP64 sum.
 //
 // A width that is no multiple of 64 takes the same path since the padding
 // costs at most one K stage, while the CUDA cores need 2 d operations a sign
