@@ -649,7 +649,8 @@ def kernel_work(B, pipe, w, objs, st, nu, lst, need):
         work["ap_stats_kernel"] = (nnz * 8 + dim * 8, "B")
         work["ap_prefix_warp_kernel"] = (nnz * 9, "B")
         work["ap_prefix_cta_kernel"] = (nnz * 9, "B")
-        if N <= 1 << 19 and N * N <= 4096 * dups:   # bit maps: every feature's rows listed, the maps of N^2 / 2 bits kept
+        # bit maps: every feature's rows listed, the maps of N^2 / 2 bits kept
+        if N <= 1 << 19 and N * N <= 4096 * dups and N * N <= (1 << 31) + 512 * dups:
             work["ap_post_kernel"] = (nnz * 12, "B")
             kept_maps = N * N // 16 if N * N <= 256 * dups else 0
             work["ap_map_kernel (count pass)"] = (nnz * 5 + dups * 4 + kept_maps, "B")
