@@ -170,19 +170,56 @@ __global__ void __launch_bounds__(kThreads) compact_count(const uint8_t *status,
     if (threadIdx.x == 0) scratch->cta_counts[blockIdx.x] = total;
 }
 
-// The indices of a warp's 512 statuses are written in order from shared memory,
-// 32 at a time, where more than kFewKept are kept, else by the lanes that hold
-// them (1e8 statuses, all kept, a lane writing its own 16: 926 us, 210 here; a
-// sixth kept 110, 117 through shared memory).
-constexpr int kFewKept = 128;
+// Writes the indices of [lo, hi) from out[base] on and returns the place after
+// them.  kBatch tiles at a time: their loads are issued together, then each tile
+// gets its block-wide prefix sum and its indices leave in order.  STAGED: a
+// warp's from shared memory, 32 at a time, else by the lanes that hold them.
+template <bool STAGED>
+__device__ __forceinline__ long long write_range(const uint8_t *status, long long lo, long long hi, uint32_t mask,
+                                                 long long base, int64_t *out, long long cap, uint16_t *list) {
+    for (long long t0 = lo; t0 < hi; t0 += (long long)kBatch * kTile) {
+        uint32_t bits[kBatch];
+        kept_tiles<kBatch>(status, t0 + (long long)threadIdx.x * kPer, kTile, hi, mask, bits);
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+            if (t0 + (long long)u * kTile >= hi) break;      // uniform across the CTA
+            const long long q0 = t0 + (long long)u * kTile + (long long)threadIdx.x * kPer;
+            long long tile_total;
+            long long o = base + blsh_scan::block_exclusive<long long>((long long)__popc(bits[u]), &tile_total);
+            if constexpr (STAGED) {
+                const int lane = threadIdx.x & 31;
+                const long long first = __shfl_sync(0xffffffffu, o, 0);
+                int at = (int)(o - first);
+                for (uint32_t b = bits[u]; b; b &= b - 1) list[at++] = (uint16_t)(kPer * lane + __ffs(b) - 1);
+                const int n = __shfl_sync(0xffffffffu, at, 31);
+                __syncwarp();
+                for (int i = lane; i < n; i += 32)
+                    if (first + i < cap) out[first + i] = q0 - kPer * lane + list[i];
+                __syncwarp();
+            } else {
+                for (uint32_t b = bits[u]; b; b &= b - 1) {
+                    if (o < cap) out[o] = q0 + __ffs(b) - 1;
+                    ++o;
+                }
+            }
+            base += tile_total;
+        }
+    }
+    return base;
+}
+
+// A CTA stages its indices where more than a kFewKept-th of its statuses are kept
+// (1e8 statuses, all kept, a lane writing its own 16: 894 us, 190 here; 30% 124,
+// 110).  The two loops are apart because one with both forms, chosen warp by warp
+// or tile by tile, took longer where few are kept (1e9 statuses: 464 and 454 us,
+// 442 here).
+constexpr int kFewKept = 4;
 __global__ void __launch_bounds__(kThreads) compact_write(const uint8_t *status, long long P_cap,
                                                           const long long *P_dev, uint32_t mask, int off,
                                                           int64_t *out, long long cap, long long *n_out,
                                                           blsh_dev_scratch *scratch) {
     __shared__ long long s_base;
     __shared__ uint16_t s_list[kThreads / 32][32 * kPer];
-    const int lane = threadIdx.x & 31;
-    uint16_t *list = s_list[threadIdx.x >> 5];
     const long long P = resolve_p(P_cap, P_dev);
     long long lo, hi;
     cta_range(P, off, lo, hi);
@@ -193,34 +230,9 @@ __global__ void __launch_bounds__(kThreads) compact_write(const uint8_t *status,
     if (threadIdx.x == 0) s_base = tot;
     __syncthreads();
     long long base = s_base;
-    // kBatch tiles at a time: their loads are issued together, then each
-    // tile gets its block-wide prefix sum and writes its indices in order
-    for (long long t0 = lo; t0 < hi; t0 += (long long)kBatch * kTile) {
-        uint32_t bits[kBatch];
-        kept_tiles<kBatch>(status, t0 + (long long)threadIdx.x * kPer, kTile, hi, mask, bits);
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-            if (t0 + (long long)u * kTile >= hi) break;      // uniform across the CTA
-            long long tile_total;
-            const int c = __popc(bits[u]);
-            const long long mine = base + blsh_scan::block_exclusive<long long>((long long)c, &tile_total);
-            const long long first = __shfl_sync(0xffffffffu, mine, 0);
-            int at = (int)(mine - first);
-            const int n = __shfl_sync(0xffffffffu, at + c, 31);
-            const long long q0 = t0 + (long long)u * kTile + (long long)(threadIdx.x - lane) * kPer;
-            if (n <= kFewKept) {
-                for (uint32_t b = bits[u]; b; b &= b - 1, ++at)
-                    if (first + at < cap) out[first + at] = q0 + kPer * lane + __ffs(b) - 1;
-            } else {
-                for (uint32_t b = bits[u]; b; b &= b - 1) list[at++] = (uint16_t)(kPer * lane + __ffs(b) - 1);
-                __syncwarp();
-                for (int i = lane; i < n; i += 32)
-                    if (first + i < cap) out[first + i] = q0 + list[i];
-                __syncwarp();
-            }
-            base += tile_total;
-        }
-    }
+    base = scratch->cta_counts[blockIdx.x] > (unsigned long long)(hi > lo ? hi - lo : 0) / kFewKept
+               ? write_range<true>(status, lo, hi, mask, base, out, cap, s_list[threadIdx.x >> 5])
+               : write_range<false>(status, lo, hi, mask, base, out, cap, nullptr);
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
         *n_out = base;
         if (base > cap) blsh_dev_error(scratch, BLSH_ETRUNC, 1, (unsigned long long)(base - cap));

@@ -147,17 +147,25 @@ def test_compaction_from_any_address(B, ctx, P, offset):
         assert np.array_equal(out[: len(want)].cpu().numpy(), want) and bool((out[len(want):] == -1).all())
 
 
-@pytest.mark.parametrize("offset", [0, 1, 15])
-@pytest.mark.parametrize("P", [131_073, 2_500_000])
-def test_compaction_from_any_address(B, ctx, P, offset):
-    st = (np.arange(P) * 11 % 41).astype(np.uint8)
-    store = torch.full((P + offset + 16,), 4, dtype=torch.uint8, device=dev)
+@pytest.mark.parametrize("offset", [0, 7])
+@pytest.mark.parametrize("P", [131_073, 1_300_000])
+@pytest.mark.parametrize("share", [0.2, 0.25, 0.3, 1.0])
+def test_compaction_of_full_and_empty_ranges(B, ctx, P, share, offset):
+    """Shares of kept statuses on both sides of the line between the two write
+    forms, next to ranges that keep few, and a buffer that ends inside a full
+    range."""
+    rng = np.random.default_rng(P + offset)
+    p = np.where(np.arange(P) // 50_000 % 2 == 0, share, 0.001)
+    st = np.where(rng.random(P) < p, 2, 1).astype(np.uint8)
+    store = torch.full((P + offset + 16,), 2, dtype=torch.uint8, device=dev)
     dst = store[offset:offset + P]
     dst.copy_(torch.from_numpy(st))
-    for used in (0, 3, 700, P - 1, P):
-        want = O.compact(st[:used], 0x80000015)
-        out = torch.full((P,), -1, dtype=torch.int64, device=dev)
+    want = O.compact(st, 1 << 2)
+    for cap in (P, len(want), 6_007):
+        out = torch.full((cap,), -1, dtype=torch.int64, device=dev)
         n_out = torch.full((1,), 5, dtype=torch.int64, device=dev)
-        B.blsh_compact(ctx, dst, 0x80000015, out, n_out, P_dev=torch.tensor([used], dtype=torch.int64, device=dev))
-        assert B.blsh_status(ctx) == 0 and int(n_out) == len(want)
-        assert np.array_equal(out[: len(want)].cpu().numpy(), want) and bool((out[len(want):] == -1).all())
+        B.blsh_compact(ctx, dst, 1 << 2, out, n_out)
+        assert int(n_out) == len(want)
+        assert (B.blsh_status(ctx) == 0) == (cap >= len(want))
+        got = out.cpu().numpy()
+        assert np.array_equal(got[: len(want)], want[:cap]) and (got[len(want):] == -1).all()
