@@ -35,7 +35,7 @@
 // indexed features; the map's set bits, in order, are x's candidates (counted
 // first, then written at scanned offsets; the write pass reads the counted maps
 // again where N^2 / 8 bytes fit the place of the key buffers).  20,000 tf-idf
-// rows (2.4e7 keys, 1.7e7 pairs): 1.96 ms by sorting, 0.38 ms with the maps.
+// rows (2.4e7 keys, 1.7e7 pairs): 1.96 ms by sorting, 0.37 ms with the maps.
 // The line: a row's map of N / 32 words takes 0.4 ps a word to count and, not
 // kept, 1.3 to 2.1 ps to form and write again; the sort takes about 50 ps a key
 // of max_dups and 0.2 ms of launches.  Rows of 10 features, maps / sort:
@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(256) ap_map_kernel(ApArgs A, const uint32_t *f
 
 // The pairs of the kept maps: a warp per row, 32 words at a time, put in order in
 // shared memory so that they leave in coalesced stores.  20,000 rows, 1.6e7
-// pairs: MAP_WRITE, which forms every map again, 172 us, 47 here.
+// pairs: MAP_WRITE, which forms every map again, 172 us, 49 here.
 constexpr int kKeptWarps = 8;
 __global__ void __launch_bounds__(32 * kKeptWarps) ap_map_write_kernel(long long N, const uint32_t *kept,
                                                                        const unsigned long long *cnt,

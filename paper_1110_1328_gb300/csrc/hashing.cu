@@ -430,10 +430,10 @@ __device__ __forceinline__ unsigned long long f2_codes(uint32_t w) {
 // by asynchronous copies 4.78 ms.
 //
 // 5e6 rows, 1.4e8 nonzeros, the first 256 columns of two-byte codes: 11.5 ms
-// with four codes a lane and long rows left to single warps, now 4.37 ms + 3.28
+// with four codes a lane and long rows left to single warps, now 4.41 ms + 3.36
 // ms for the rows of more than 256 nonzeros and the rechecks (a kernel of their
 // own before); 20,000 rows x 2,048 columns of floats (R of 820 MB) 607 us, now
-// 506 us + 54 us; 7,000 rows x 128 codes 33 us a call, 44 with three launches.
+// 518 us + 52 us; 7,000 rows x 128 codes 33 us a call, 44 with three launches.
 constexpr int kSrpLongRow = 256;
 constexpr int kSrpLongMost = 1024;
 

@@ -34,7 +34,7 @@
 // A width that is no multiple of 64 takes the same path since the padding
 // costs at most one K stage, while the CUDA cores need 2 d operations a sign
 // at 1/50 of the tensor rate: 99,991 x 300 x 1,024 bits took 36.4 ms on the
-// CUDA cores' kernel of that time, 297 us here.
+// CUDA cores' kernel of that time, 292 us here.
 //
 // Every other shape uses srp_dense_simt_kernel (hashing.cu): FP32 sums with
 // the same kind of bound and an FP64 recheck.
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) srp_dense_tc_persistent(
 // sign: 2,077 us for the 1.3e7 signs that 1e6 x 256 x 1,024 bits leave inside
 // the margin 1e-3, and the queue's appends cost the tensor-core kernel 200 us
 // (1,049 us, with marks 840 us); where most signs were ties it overflowed and
-// the epilogue summed them itself (1% zero rows among 1e5: 51 ms, now 0.3 ms).
+// the epilogue summed them itself (1e5 x 256, 1% of them zero: 51 ms, now 0.23 ms).
 // Here x_i is read once, and the sums take 1,090 us (13 TB/s of columns).
 // Items of 8 words of 4 rows, so that an SM's L1 holds its part of the columns,
 // take 1,695 us: a row's few signs no longer fill a batch.  24 warps of 80
