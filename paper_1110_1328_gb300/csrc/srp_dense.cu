@@ -34,7 +34,7 @@
 // A width that is no multiple of 64 takes the same path since the padding
 // costs at most one K stage, while the CUDA cores need 2 d operations a sign
 // at 1/50 of the tensor rate: 99,991 x 300 x 1,024 bits took 36.4 ms on the
-// CUDA cores' kernel of that time, 292 us here.
+// CUDA cores' kernel of that time, 289 us here.
 //
 // Every other shape uses srp_dense_simt_kernel (hashing.cu): FP32 sums with
 // the same kind of bound and an FP64 recheck.
